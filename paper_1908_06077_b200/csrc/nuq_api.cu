@@ -26,7 +26,7 @@ struct WsEntry {
     // (0: none).  The allocation is zeroed and every encode kernel leaves its scan state zeroed, but the bucket
     // norms of a wide-bucket call or of a histogram call stay behind, at a place that depends on that call's size.
     size_t dirty_to = 0;
-    uint32_t dec_epoch = 0;  // decode calls made on this workspace (see DecodeParams::epoch)
+    uint32_t dec_epoch = 0;  // fixed-width decode calls made on this workspace (see DecodeParams::epoch)
 };
 
 // One mutex guards the host-side bookkeeping below (maps, tables); it is held for the microseconds a
@@ -34,7 +34,8 @@ struct WsEntry {
 std::mutex g_mu;
 std::map<std::pair<int, cudaStream_t>, WsEntry> g_ws;
 std::map<int, int> g_sms;                 // device -> SM count
-std::set<int> g_lut_ready;                // devices whose constant LUT is uploaded
+std::set<int> g_lut_ready;                // devices whose constant LUT is uploaded ...
+std::set<int> g_token_tables_ready;       // ... and those that hold the decoder's token tables
 std::map<int, const float*> g_test_norms;   // device -> bucket norms of nuq_set_test_norms
 float g_levels[kMaxTableS + 2], g_inv_width[kMaxTableS + 2];   // the level table of nuq_set_level_table ...
 uint32_t g_levels_s = 0;                                       // ... and its number of interior levels (0: none set)
@@ -543,13 +544,13 @@ static nuq_status enqueue_decode(const void* const* streams, uint32_t K, uint64_
     }
     for (uint32_t k = K; k < kMaxK; ++k) P.streams[k] = nullptr;
     P.K = K;
-    P.group = K >= 8 ? 8u : K >= 3 ? 4u : K;            // 1, 2, 4 or 8 streams side by side
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess) return NUQ_ERR_CUDA;
-    // A small call with the widest units (32 / group sub-blocks per warp) gives only a few warps of the whole
-    // GPU something to do, and a warp's walk is a chain of dependent steps: narrower units (lanes left idle)
-    // put more warps to work.
-    while (P.group < 8u && 2u * P.geo.ntiles * P.group <= 8u * (uint64_t)device_sms(dev)) P.group *= 2u;
+    if (!g_token_tables_ready.count(dev)) {
+        if (upload_token_tables() != cudaSuccess) return NUQ_ERR_CUDA;
+        g_token_tables_ready.insert(dev);
+    }
+    P.unit_subs = 0;                                    // (chosen at the launch)
     P.after_fixed = w ? 0u : 1u;                        // all streams believed to be in the fixed-width mode? (sums only)
     for (uint32_t k = 0; k < K; ++k) {
         auto it = g_container_mode.find(std::make_pair(dev, streams[k]));
@@ -566,10 +567,10 @@ static nuq_status enqueue_decode(const void* const* streams, uint32_t K, uint64_
     nuq_status st = get_workspace(stream, sizeof(Workspace), &ws, &dev);
     if (st != NUQ_OK) return st;
     P.ws = ws;
-    // The ticket counter a decode call uses has been zeroed by the call before it (or by the allocation, or by an
-    // encode call, which leaves both zeroed): calls take the two counters in turn and each zeroes the other one.
+    // The ticket counter a fixed-width decode call uses has been zeroed by the one before it (or by the allocation, or
+    // by an encode call, which leaves both zeroed): such calls take the two counters in turn and each zeroes the other one.
     WsEntry& entry = g_ws[std::make_pair(dev, stream)];
-    if (++entry.dec_epoch == 0) entry.dec_epoch = 2;        // never 0, parity kept
+    if (P.after_fixed && ++entry.dec_epoch == 0) entry.dec_epoch = 2;       // never 0, parity kept
     P.epoch = entry.dec_epoch;
     P.pad = 0;
     if (launch_decode(P, device_sms(dev), stream) != cudaSuccess) return NUQ_ERR_CUDA;

@@ -92,7 +92,7 @@ struct DecodeParams {
     Geometry geo;
     const uint32_t* streams[kMaxK];
     uint32_t K;
-    uint32_t group;          // streams decoded side by side (1, 2, 4 or 8)
+    uint32_t unit_subs;      // token streams: sub-blocks a warp decodes at a time
     uint32_t after_fixed;    // the fixed-width kernel runs first; the general kernel returns if it did the work
     uint32_t epoch;          // number of this decode call on its workspace (never 0)
     uint32_t pad;

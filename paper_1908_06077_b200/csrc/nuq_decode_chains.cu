@@ -1,0 +1,800 @@
+// DECODE + aggregate (App. A decoding; Algorithm 1, aggregation line) of token streams: the K
+// workers' containers are decoded and summed into one fp32 vector.
+//
+// A warp takes a unit of S consecutive 256-element sub-blocks in all K streams (up to 32 streams at a
+// time), K S <= 32, and works in two passes:
+//
+//   walk   lane (j, q) walks the chain of tokens of stream j, sub-block q and writes the symbol of every
+//          token, one byte, to its place in the chain's row of 256 positions in shared memory.  All
+//          chains of a warp advance side by side; nothing is kept in lists, so the density of the
+//          symbols does not matter.
+//   add    the rows are read across: a lane takes four consecutive elements of all K streams, turns
+//          their symbols into values and adds them up in ascending stream order, starting from +0, so
+//          the sum equals ((0 + q_0) + q_1) + ... bit for bit.  It is stored (or applied to the
+//          parameters) once, 512 contiguous bytes per warp and step.
+//
+// The walk is a chain of dependent steps.  What a step waits for is one table look-up and two shifts:
+//
+//   table   the next 13 bits of the chain give a whole token: the bits it takes, its gap and its symbol.
+//           A token that is longer than 13 bits is taken in two steps: the code of a gap ends with the
+//           bit 0, which is itself the code of gap 1, so an entry that stands for the gap's code without
+//           its last bit and for a gap one smaller, without a symbol, leaves an ordinary token of gap 1
+//           behind.  What the table cannot resolve at all (gaps from 128 on, long level codes) takes
+//           Algorithm 2's loop.
+//   window  64 bits hi:lo, at least 32 of them valid, shifted by the token's length; the next table
+//           index needs only the 13 top bits, which are valid before the window is refilled.
+//   end     every lane has its own copy of its chain (cp.async, 112 bytes at a time) and puts ones
+//           behind the chain's last bit: thirteen ones are no token, the table says "0 bits, no gap, no
+//           symbol", and the lane stands still until all others have ended too.  So a step has no
+//           branches; the lanes look up every four steps.
+//
+// The copy of the next unit's chains runs during the add pass, the block offsets of the one after that
+// are on their way during the walk.  16 warps fit an SM (12 KB each: rows, chain copies).
+#include "nuq_async.cuh"
+#include "nuq_decode_common.cuh"
+#include "nuq_launch.h"
+
+namespace nuq {
+
+constexpr uint32_t kTokBits = 13;                       // prefix bits the token table resolves
+constexpr uint32_t kTokEntries = 1u << kTokBits;
+constexpr uint32_t kChainMaxWarps = 16;                 // warps per CTA, one CTA per SM
+constexpr uint32_t kChunkWords = 28;                    // words of its chain a lane holds at a time
+constexpr uint32_t kChunkSlack = 3;                     // of these, words it needs behind the chain's last one
+constexpr uint32_t kStreamTabBytes = 256 + 64;          // per stream: level code by 7-bit prefix, level table
+constexpr size_t kChainSmem = 227u * 1024u - 512u;      // (512 bytes: static)
+
+// A row of symbols: 256 positions and a place for what a malformed chain would write behind them.  Rows of
+// neighbouring lanes start in neighbouring banks.
+template <class Sym>
+struct Row {
+    static constexpr uint32_t kPitch = kSB * sizeof(Sym) + 4u;
+    static constexpr uint32_t kWarpBytes = 32u * kPitch + 128u + 32u * 4u * kChunkWords;   // rows, norms, chain copies
+};
+
+// Token table entries.  Bits 0-4: bits consumed (0: not resolved here); bits 8-15: gap; bits 22-31: symbol, signed
+// (0: none, only a part of the gap).  Symbols: for exponential levels the upper byte of the level (with its sign) as
+// an fp16 number, 2^(j-1-s) being one without mantissa bits; for uniform levels the signed index.
+constexpr uint32_t kLenMask = 31u, kGapShift = 8u, kSymShift = 22u;
+__device__ __forceinline__ uint32_t exp_symbol(uint32_t index, uint32_t negative, uint32_t s) {
+    return ((negative ? 0x80u : 0u) | ((14u + index - s) << 2)) << kSymShift;
+}
+__device__ __forceinline__ uint32_t uniform_symbol(uint32_t index, uint32_t negative) {
+    return (negative ? 0u - index : index) << kSymShift;
+}
+
+// Tables as kept in device memory: the symbol is the level index (1 .. 255), bit 31 of the entry the sign.
+enum : uint32_t { kTabErc = 0, kTabGaps = 1, kTabCoded = 2, kTabUniform = 3 };
+__device__ uint32_t g_token_tables[2][kTokEntries];
+
+// ERC^-1 of the nbits-bit prefix idx from bit `pos` on (Algorithm 2, decoding): false when the code does not end within it.
+static bool erc_of_prefix(uint32_t idx, uint32_t nbits, uint32_t* pos, uint32_t* value) {
+    uint32_t N = 1;
+    for (;;) {
+        if (*pos >= nbits) return false;
+        if (!((idx >> (nbits - 1u - *pos)) & 1u)) {
+            *pos += 1;
+            *value = N;
+            return true;
+        }
+        const uint32_t nb = N + 1u;
+        if (*pos + nb > nbits) return false;
+        N = (idx >> (nbits - *pos - nb)) & ((1u << nb) - 1u);
+        *pos += nb;
+    }
+}
+
+cudaError_t upload_token_tables() {
+    static uint32_t tab[2][kTokEntries];
+    for (uint32_t i = 0; i < kTokEntries; ++i) {
+        uint32_t pos = 0, gap = 0;
+        tab[kTabErc][i] = tab[kTabGaps][i] = 0;
+        if (!erc_of_prefix(i, kTokBits, &pos, &gap) || gap >= kSB) continue;
+        tab[kTabGaps][i] = pos | (gap << kGapShift);
+        uint32_t at = pos + 1u, index = 0;                  // behind the sign bit
+        if (at < kTokBits && erc_of_prefix(i, kTokBits, &at, &index) && index <= 255u)
+            tab[kTabErc][i] = at | (gap << kGapShift) | (index << kSymShift) | (((i >> (kTokBits - 1u - pos)) & 1u) << 31);
+        else if (pos > 1u)
+            tab[kTabErc][i] = (pos - 1u) | ((gap - 1u) << kGapShift);
+    }
+    return cudaMemcpyToSymbol(g_token_tables, tab, sizeof(tab));
+}
+
+__device__ __forceinline__ void copy_async16(uint32_t dst, const void* src) {
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src) : "memory");
+}
+__device__ __forceinline__ void copy_async4(uint32_t dst, const void* src) {
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(dst), "l"(src) : "memory");
+}
+__device__ __forceinline__ uint32_t lds_u32(uint32_t addr) {
+    uint32_t v;
+    asm volatile("ld.shared.u32 %0, [%1];" : "=r"(v) : "r"(addr) : "memory");
+    return v;
+}
+
+// One Elias-recursive integer from bit `at` of the 32-bit window on; false when it does not end within it.
+__device__ __forceinline__ bool erc_in_window(uint32_t win, uint32_t* at, uint32_t* value) {
+    uint32_t N = 1;
+#pragma unroll 1
+    for (int it = 0; it < 5; ++it) {
+        const uint32_t w = win << *at;
+        if (!(w >> 31)) {
+            *at += 1;
+            *value = N;
+            return true;
+        }
+        const uint32_t nb = N + 1u;
+        if (*at + nb > 31u) return false;
+        N = w >> (32u - nb);
+        *at += nb;
+    }
+    return false;
+}
+
+// A stream with coded level indices brings its own code: the level index and the word's length (<< 8) by the
+// next 7 bits, 0 where no word starts (possible only with an incomplete code).
+__device__ __forceinline__ uint32_t coded_entry(const StreamHead& hd, uint32_t s, uint32_t prefix) {
+    const uint32_t w0 = __ldg(hd.hdr + hd.hwords - 2u), w1 = __ldg(hd.hdr + hd.hwords - 1u);   // the lengths, one byte each
+    auto len_of = [&](uint32_t j) { return ((j < 4u ? w0 : w1) >> (8u * (j & 3u))) & 0xffu; };
+    for (uint32_t j = 0; j <= s; ++j) {
+        // canonical words: level indices by (length, index), the first word all zeros, each next one the
+        // previous plus one; so the word of j counts, in units of its own length, the words before it
+        const uint32_t lj = len_of(j);
+        uint32_t word = 0;
+        for (uint32_t k = 0; k <= s; ++k) {
+            const uint32_t lk = len_of(k);
+            if (lk < lj || (lk == lj && k < j)) word += 1u << (lj - lk);
+        }
+        if ((prefix >> (kMaxCodedS - lj)) == word) return (j + 1u) | (lj << 8);
+    }
+    return 0;
+}
+
+// A token the table does not resolve, by Algorithm 2's loop; a gap longer than 1 is taken on its own, as in the table.
+// Returns the entry the table would hold, 0 when the bits are no token.
+__device__ __noinline__ uint32_t long_token(uint32_t win, const StreamHead& hd, const uint16_t* code, bool gaps_only, uint32_t s) {
+    uint32_t at = 0, gap = 0, index = 0;
+    if (!erc_in_window(win, &at, &gap) || gap > kSB) return 0u;
+    if (at > 1u) return (at - 1u) | ((gap - 1u) << kGapShift);
+    at = 2u;
+    if (hd.mode == kModeCoded) {
+        if (!gaps_only) return 0u;                          // (such a token would be in the table)
+        const uint32_t c = code[(win << 2) >> (32u - kMaxCodedS)];
+        at += c >> 8;
+        index = c & 0xffu;
+    } else if (!erc_in_window(win, &at, &index)) {
+        return 0u;
+    }
+    if (index == 0u || index >= hd.nlev) return 0u;
+    const uint32_t negative = (win >> 30) & 1u;
+    return at | (1u << kGapShift) | (hd.levelset == kLevelsUniform ? uniform_symbol(index, negative) : exp_symbol(index, negative, s));
+}
+
+// What a lane knows of its chain.
+struct Chain {
+    const uint32_t* src;     // the 16-byte piece of the container that holds its first bit
+    uint64_t left;           // words of the container from there on
+    uint32_t bit, len;       // first bit behind src, bits (0: no chain here)
+    float norm;
+    bool good;               // what the container says about it makes sense
+};
+
+// One pass over the words a lane holds: walks `bits` bits from bit `from` of the copy on, or further up to the end of
+// the token that crosses that point.  LONG: the copy ends before the chain does (in some lane); else every chain is
+// followed by ones.  `row` is the address of the last position taken, and is moved on.
+// GAPS: the table holds gaps alone; the level index comes from the stream's own table (by the 7 bits behind the sign).
+template <class Sym, bool LONG, bool GAPS>
+__device__ __forceinline__ uint32_t walk_body(uint32_t copy, uint32_t from, uint32_t bits, uint32_t tab, uint32_t& row, uint32_t row_end,
+                                              const StreamHead& hd, const uint16_t* code, uint32_t s, bool& good) {
+    const uint32_t sh = from & 31u, w0 = copy + 4u * (from >> 5);
+    const uint32_t x0 = lds_u32(w0), x1 = lds_u32(w0 + 4u), x2 = lds_u32(w0 + 8u);
+    uint32_t hi = __funnelshift_l(x1, x0, sh);
+    uint32_t lo = sh ? x1 << sh : 0u, nxt = sh ? x2 : x1;
+    uint32_t next = w0 + (sh ? 12u : 8u);                   // where the word behind nxt lies
+    // q counts the bits down to c; its low five bits are those of the number of valid bits in hi:lo
+    const uint32_t c = (0u - sh - bits) & 31u;
+    uint32_t q = bits + c, e = 0, at = row;
+    auto look_up = [&] {
+        const uint32_t addr = tab + ((hi >> (32u - kTokBits)) << 2);
+        if (LONG) asm("{\n\t.reg .pred p;\n\tsetp.gt.s32 p, %1, %2;\n\tmov.b32 %0, 0;\n\t@p ld.shared.u32 %0, [%3];\n\t}"
+                      : "=r"(e) : "r"(q), "r"(c), "r"(addr));
+        else asm("ld.shared.u32 %0, [%1];" : "=r"(e) : "r"(addr));
+        if (GAPS) {
+            const uint32_t behind = hi << (e & kLenMask), cw = code[(behind << 1) >> (32u - kMaxCodedS)];
+            const uint32_t len = (e & kLenMask) + 1u + (cw >> 8), index = cw & 0xffu, negative = behind >> 31;
+            const uint32_t sym = hd.levelset == kLevelsUniform ? uniform_symbol(index, negative) : exp_symbol(index, negative, s);
+            e = e != 0u && cw != 0u ? len | (e & (0xffu << kGapShift)) | sym : 0u;
+        }
+    };
+    if (bits != 0u) {
+        look_up();
+        for (;;) {
+            if (e == 0u) {
+                if ((int32_t)(q - c) <= 0) break;
+                e = long_token(hi, hd, code, GAPS, s);
+                if (e == 0u) {
+                    good = false;
+                    break;
+                }
+            }
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                if (!GAPS && !LONG && sizeof(Sym) == 1) {
+                    asm volatile(
+                        "{\n\t.reg .pred p, r;\n\t.reg .b32 g, y, t, n;\n\t"
+                        "prmt.b32 g, %0, 0, 0x4441;\n\tadd.u32 %1, %1, g;\n\tmin.u32 %1, %1, %7;\n\t"
+                        "shr.u32 y, %0, 22;\n\tsetp.ne.u32 r, y, 0;\n\t@r st.shared.u8 [%1], y;\n\t"
+                        "shf.l.wrap.b32 %2, %3, %2, %0;\n\tshf.l.wrap.b32 %3, 0, %3, %0;\n\t"
+                        "and.b32 t, %0, 31;\n\tsub.u32 n, %6, t;\n\t"
+                        "shr.u32 g, %2, 19;\n\tshl.b32 g, g, 2;\n\tadd.u32 g, g, %8;\n\tld.shared.u32 %0, [g];\n\t"
+                        "xor.b32 t, n, %6;\n\tand.b32 t, t, 32;\n\tsetp.ne.u32 p, t, 0;\n\tmov.b32 %6, n;\n\t"
+                        "shf.r.wrap.b32 t, %4, 0, n;\n\t@p or.b32 %2, %2, t;\n\t@p shf.r.wrap.b32 %3, 0, %4, n;\n\t"
+                        "@p ld.shared.u32 %4, [%5];\n\t@p add.u32 %5, %5, 4;\n\t}"
+                        : "+r"(e), "+r"(at), "+r"(hi), "+r"(lo), "+r"(nxt), "+r"(next), "+r"(q)
+                        : "r"(row_end), "r"(tab) : "memory");
+                    continue;
+                }
+                at += __byte_perm(e, 0u, 0x4441) * (uint32_t)sizeof(Sym);
+                at = min(at, row_end);
+                // (no symbol: a part of a gap, or a lane that stands still)
+                if (sizeof(Sym) == 1)
+                    asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.u32 p, %1, 0;\n\t@p st.shared.u8 [%0], %1;\n\t}" ::"r"(at), "r"(e >> kSymShift) : "memory");
+                else
+                    asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.u32 p, %1, 0;\n\t@p st.shared.u16 [%0], %1;\n\t}" ::"r"(at), "r"((int32_t)e >> kSymShift) : "memory");
+                const uint32_t q_was = q;
+                hi = __funnelshift_l(lo, hi, e);
+                lo = __funnelshift_l(0u, lo, e);
+                q -= e & kLenMask;
+                if (!GAPS) look_up();                       // (at least 13 valid bits are left)
+                asm("{\n\t.reg .pred p;\n\t.reg .b32 t;\n\txor.b32 t, %4, %5;\n\tand.b32 t, t, 32;\n\tsetp.ne.u32 p, t, 0;\n\t"
+                    "shf.r.wrap.b32 t, %2, 0, %4;\n\t@p or.b32 %0, %0, t;\n\t@p shf.r.wrap.b32 %1, 0, %2, %4;\n\t"
+                    "@p ld.shared.u32 %2, [%3];\n\t@p add.u32 %3, %3, 4;\n\t}"
+                    : "+r"(hi), "+r"(lo), "+r"(nxt), "+r"(next) : "r"(q), "r"(q_was));
+                if (GAPS) look_up();
+            }
+        }
+    }
+    row = at;
+    return bits + c - q;                                    // bits taken
+}
+
+// (the common walk is part of the kernel's loop, the others are calls)
+template <class Sym, bool LONG, bool GAPS>
+__device__ __noinline__ uint32_t walk_rare(uint32_t copy, uint32_t from, uint32_t bits, uint32_t tab, uint32_t& row, uint32_t row_end,
+                                           const StreamHead& hd, const uint16_t* code, uint32_t s, bool& good) {
+    return walk_body<Sym, LONG, GAPS>(copy, from, bits, tab, row, row_end, hd, code, s, good);
+}
+
+__device__ __forceinline__ uint64_t pack2(float a, float b) {
+    uint64_t r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
+    return r;
+}
+__device__ __forceinline__ float2 unpack2(uint64_t v) {
+    float2 r;
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(v));
+    return r;
+}
+// two fp32 operations at once, each rounded like the single one
+__device__ __forceinline__ uint64_t fma2(uint64_t a, uint64_t b, uint64_t c) {
+    uint64_t r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+    return r;
+}
+__device__ __forceinline__ uint64_t mul2(uint64_t a, uint64_t b) {
+    uint64_t r;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+__device__ __forceinline__ uint64_t add2(uint64_t a, uint64_t b) {
+    uint64_t r;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+// two fp16 numbers given by their upper bytes, in the upper bytes of the halves
+__device__ __forceinline__ uint64_t halves(uint32_t h) {
+    uint64_t r;
+    asm("{\n\t.reg .b16 a, b;\n\t.reg .f32 x, y;\n\tmov.b32 {a, b}, %1;\n\tcvt.f32.f16 x, a;\n\tcvt.f32.f16 y, b;\n\tmov.b64 %0, {x, y};\n\t}" : "=l"(r) : "r"(h));
+    return r;
+}
+
+// Four symbols of one stream as level values: a pair each.
+template <class Sym, bool UNIFORM>
+__device__ __forceinline__ void four_levels(uint32_t row, uint32_t s, uint64_t* v01, uint64_t* v23) {
+    if (!UNIFORM) {
+        const uint32_t x = lds_u32(row), y = sizeof(Sym) == 1 ? x : lds_u32(row + 4u);
+        *v01 = halves(sizeof(Sym) == 1 ? __byte_perm(x, 0u, 0x1404) : __byte_perm(x, 0u, 0x2404));
+        *v23 = halves(sizeof(Sym) == 1 ? __byte_perm(x, 0u, 0x3424) : __byte_perm(y, 0u, 0x2404));
+        return;
+    }
+    const float step = __uint_as_float((127u - s) << 23);   // k 2^-s is exact
+    float k[4];
+    if (sizeof(Sym) == 1) {
+        const uint32_t x = lds_u32(row);
+#pragma unroll
+        for (int i = 0; i < 4; ++i) k[i] = (float)(int8_t)(x >> (8 * i));
+    } else {
+        const uint32_t x = lds_u32(row), y = lds_u32(row + 4u);
+        k[0] = (float)(int16_t)x; k[1] = (float)(int16_t)(x >> 16);
+        k[2] = (float)(int16_t)y; k[3] = (float)(int16_t)(y >> 16);
+    }
+    *v01 = mul2(pack2(k[0], k[1]), pack2(step, step));
+    *v23 = mul2(pack2(k[2], k[3]), pack2(step, step));
+}
+
+// Four fields of a fixed-width stream, elements e .. e + 3 of the vector (e a multiple of 4), as values.  Returns
+// false when a symbol does not exist.
+__device__ __noinline__ bool four_fields(const Geometry& G, const StreamHead& hd, uint64_t e, float4* out) {
+    const uint32_t wd = hd.width, smask = (1u << (wd - 1u)) - 1u;
+    const uint64_t b = e / G.bucket;
+    const uint32_t in_bucket = (uint32_t)(e - b * G.bucket), rec_words = 1u + (G.bucket * wd + 31u) / 32u;
+    const uint64_t blen = G.d - b * G.bucket < G.bucket ? G.d - b * G.bucket : G.bucket;
+    const uint32_t last = (uint32_t)((blen * wd + 31u) / 32u) - 1u, bit = in_bucket * wd, wi = bit >> 5;
+    const uint32_t* const rec = hd.hdr + hd.hwords + b * rec_words;
+    const float norm = __uint_as_float(__ldg(rec));
+    const uint32_t x0 = __ldg(rec + 1u + min(wi, last)), x1 = __ldg(rec + 1u + min(wi + 1u, last)), x2 = __ldg(rec + 1u + min(wi + 2u, last));
+    const uint64_t win = ((uint64_t)__funnelshift_l(x1, x0, bit) << 32) | __funnelshift_l(x2, x1, bit);   // 64 bits from the first field on
+    float v[4];
+    bool ok = true;
+#pragma unroll
+    for (uint32_t c = 0; c < 4; ++c) {
+        const uint32_t field = (uint32_t)(win >> (64u - (c + 1u) * wd)) & ((1u << wd) - 1u), sym = field & smask;
+        v[c] = 0.0f;
+        if (sym == 0u || e + c >= G.d) continue;
+        if (sym >= hd.nlev) ok = false;
+        else v[c] = level_times_norm(norm, hd.levelset, G.s, sym, hd.hdr);
+        if (field >> (wd - 1u)) v[c] = -v[c];
+    }
+    *out = make_float4(v[0], v[1], v[2], v[3]);
+    return ok;
+}
+
+// The add pass of a unit.
+struct AddPass {
+    const StreamHead* heads;           // of the group's streams
+    const unsigned char* stream_tabs;
+    uint32_t rows, norms;              // shared-memory addresses
+    uint32_t S, streams;
+    uint32_t alike;                    // all streams are tokens of exponential (0) or uniform (1) levels; else 2
+    bool exact;                        // norm times a power of two is exact for all the unit's norms
+    bool last, carried;                // the last group of streams; sums of earlier groups are in `carry`
+};
+
+// NB sub-blocks from sub-block q0 of the unit on; e: the lane's first element, 128 more for each half of a sub-block.
+template <class Sym, int NB>
+__device__ __forceinline__ void add_block(const DecodeParams& P, const AddPass& A, uint32_t q0, uint64_t e, uint64_t (&carry)[4]) {
+    const Geometry& G = P.geo;
+    const uint32_t lane = lane_id(), s = G.s;
+    uint64_t sum[4 * NB];                                   // two halves of each, four elements in two pairs
+#pragma unroll
+    for (int i = 0; i < 4 * NB; ++i) sum[i] = 0;
+    if (NB == 1 && A.carried) {
+#pragma unroll
+        for (int i = 0; i < 4; ++i) sum[i] = carry[i];
+    }
+    uint32_t nrm = A.norms + 4u * q0, at = A.rows + q0 * Row<Sym>::kPitch + 4u * lane * (uint32_t)sizeof(Sym);
+    auto add_rows = [&](auto value) {
+#pragma unroll
+        for (int h = 0; h < 2 * NB; ++h)
+            value(at + (h / 2) * Row<Sym>::kPitch + (h & 1) * 128u * (uint32_t)sizeof(Sym), __uint_as_float(lds_u32(nrm + 4u * (h / 2))),
+                  sum[2 * h], sum[2 * h + 1]);
+    };
+    auto add_exp = [&](uint32_t row, float nm, uint64_t& s01, uint64_t& s23) {
+        uint64_t a, b;
+        four_levels<Sym, false>(row, s, &a, &b);
+        s01 = fma2(a, pack2(nm, nm), s01);
+        s23 = fma2(b, pack2(nm, nm), s23);
+    };
+    auto add_uniform = [&](uint32_t row, float nm, uint64_t& s01, uint64_t& s23) {
+        uint64_t a, b;
+        four_levels<Sym, true>(row, s, &a, &b);
+        s01 = add2(s01, mul2(a, pack2(nm, nm)));
+        s23 = add2(s23, mul2(b, pack2(nm, nm)));
+    };
+    if (A.alike == 0u) {
+#pragma unroll 4 / NB
+        for (uint32_t j = 0; j < A.streams; ++j, nrm += 4u * A.S, at += A.S * Row<Sym>::kPitch) add_rows(add_exp);
+    } else if (A.alike == 1u) {
+#pragma unroll 4 / NB
+        for (uint32_t j = 0; j < A.streams; ++j, nrm += 4u * A.S, at += A.S * Row<Sym>::kPitch) add_rows(add_uniform);
+    } else {
+#pragma unroll 1
+        for (uint32_t j = 0; j < A.streams; ++j, nrm += 4u * A.S, at += A.S * Row<Sym>::kPitch) {
+            const StreamHead& hd = A.heads[j];
+            if (!hd.ok) continue;
+            if (hd.mode == kModeFixed) {
+                bool ok = true;
+#pragma unroll
+                for (int h = 0; h < 2 * NB; ++h) {
+                    if (e + 128u * h < G.d) {
+                        float4 v;
+                        ok = four_fields(G, hd, e + 128u * h, &v) && ok;
+                        sum[2 * h] = add2(sum[2 * h], pack2(v.x, v.y));
+                        sum[2 * h + 1] = add2(sum[2 * h + 1], pack2(v.z, v.w));
+                    }
+                }
+                if (!ok) latch_status(P.ws, kErrBadStream);
+            } else {
+                const float* const lv = reinterpret_cast<const float*>(A.stream_tabs + j * kStreamTabBytes + 256u);
+                add_rows([&](uint32_t row, float nm, uint64_t& s01, uint64_t& s23) {
+                    float v[4];
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) {
+                        int32_t b;
+                        if (sizeof(Sym) == 1) asm volatile("ld.shared.s8 %0, [%1];" : "=r"(b) : "r"(row + i) : "memory");
+                        else asm volatile("ld.shared.s16 %0, [%1];" : "=r"(b) : "r"(row + 2u * i) : "memory");
+                        float level = 0.0f;                 // (no product for an element without a symbol: the norm may not be finite)
+                        if (b) {
+                            const uint32_t field = ((uint32_t)b >> 2) & 31u;
+                            level = hd.levelset == kLevelsUniform ? (float)b * __uint_as_float((127u - s) << 23)
+                                    : hd.levelset == kLevelsTable ? lv[field + s - 15u] : __uint_as_float((field + 112u) << 23);
+                            level = __fmul_rn(nm, level);
+                            if (hd.levelset != kLevelsUniform && (b & 0x80)) level = -level;
+                        }
+                        v[i] = level;
+                    }
+                    s01 = add2(s01, pack2(v[0], v[1]));
+                    s23 = add2(s23, pack2(v[2], v[3]));
+                });
+            }
+        }
+    }
+    if (NB == 1 && !A.last) {
+#pragma unroll
+        for (int i = 0; i < 4; ++i) carry[i] = sum[i];
+        return;
+    }
+    auto value = [&](int h) {
+        const float2 a = unpack2(sum[2 * h]), b = unpack2(sum[2 * h + 1]);
+        return make_float4(a.x, a.y, b.x, b.y);
+    };
+    if (e + 128u * (2 * NB - 1) + 4u <= G.d) {
+        if (P.w == nullptr) {
+#pragma unroll
+            for (int h = 0; h < 2 * NB; ++h) *reinterpret_cast<float4*>(P.acc + e + 128 * h) = value(h);
+        } else {
+            constexpr int kAtOnce = NB == 1 ? 2 : 4;        // the loads of four steps are on their way together
+#pragma unroll
+            for (int h0 = 0; h0 < 2 * NB; h0 += kAtOnce) {
+                float4 w[kAtOnce], yl[kAtOnce];
+#pragma unroll
+                for (int h = 0; h < kAtOnce; ++h) {
+                    w[h] = *reinterpret_cast<const float4*>(P.w + e + 128 * (h0 + h));
+                    yl[h] = P.mu != 0.0f ? *reinterpret_cast<const float4*>(P.yl + e + 128 * (h0 + h)) : make_float4(0.f, 0.f, 0.f, 0.f);
+                }
+#pragma unroll
+                for (int h = 0; h < kAtOnce; ++h) step4(P, e + 128 * (h0 + h), value(h0 + h), w[h], yl[h]);
+            }
+        }
+    } else {                                                // the end of the vector
+#pragma unroll
+        for (int h = 0; h < 2 * NB; ++h) {
+            const uint64_t at_h = e + 128u * h;
+            if (at_h + 4u <= G.d) finish4(P, at_h, value(h));
+            else if (at_h < G.d) finish_part(P, at_h, value(h), (uint32_t)(G.d - at_h));
+        }
+    }
+}
+
+// Shared memory: the token table, the streams' tables and heads, then per warp its rows, norms and chain copies.
+__host__ __device__ inline size_t chain_fixed_bytes(uint32_t K) {
+    return (4u * kTokEntries + (size_t)K * (kStreamTabBytes + sizeof(StreamHead)) + 15u) & ~(size_t)15u;
+}
+
+template <class Sym>
+__global__ void __launch_bounds__(32 * kChainMaxWarps, 1) decode_chains_kernel(const __grid_constant__ DecodeParams P) {
+    extern __shared__ __align__(128) unsigned char dsm[];
+    __shared__ uint32_t s_kind, s_alike;
+    // Behind the fixed-width kernel this one is launched with programmatic stream serialization: its launch is
+    // worked off while that kernel still runs, and it waits here until that kernel's writes are visible.
+    if (P.after_fixed) asm volatile("griddepcontrol.wait;" ::: "memory");
+    if (P.after_fixed && *reinterpret_cast<volatile uint32_t*>(&P.ws->dec_done_epoch) == P.epoch) return;   // the fixed-width kernel did it all
+    const Geometry& G = P.geo;
+    const uint32_t K = P.K, tid = threadIdx.x, lane = tid & 31u, warp = tid >> 5;
+    uint32_t* const table = reinterpret_cast<uint32_t*>(dsm);
+    unsigned char* const stream_tabs = dsm + 4u * kTokEntries;
+    StreamHead* const heads = reinterpret_cast<StreamHead*>(stream_tabs + K * kStreamTabBytes);
+    const uint32_t rows = smem_u32(dsm) + (uint32_t)chain_fixed_bytes(K) + warp * Row<Sym>::kWarpBytes;
+    const uint32_t norms = rows + 32u * Row<Sym>::kPitch;   // one per lane's chain
+    const uint32_t copy = norms + 128u + lane * (4u * kChunkWords);   // this lane's words of its chain
+
+    // ---- headers against the call's arguments, once per stream; then the table that serves all the token streams ----
+    for (uint32_t k = tid; k < K; k += blockDim.x) {
+        heads[k] = read_head(G, P.streams[k]);
+        if (!heads[k].ok) latch_status(P.ws, kErrBadStream);
+    }
+    auto clear_rows = [&] {
+        for (uint32_t i = 16u * lane; i < 32u * Row<Sym>::kPitch; i += 512u)
+            asm volatile("st.shared.v4.u32 [%0], {%1, %1, %1, %1};" ::"r"(rows + i), "r"(0u) : "memory");
+    };
+    clear_rows();
+    __syncthreads();
+    if (tid == 0) {
+        bool coded = false, erc = false, uniform = false, other = false, same_code = true, odd = false;
+        uint32_t w0 = 0, w1 = 0;
+        for (uint32_t k = 0; k < K; ++k) {
+            odd = odd || !heads[k].ok || heads[k].mode == kModeFixed || heads[k].levelset == kLevelsTable;
+            if (!heads[k].ok || heads[k].mode == kModeFixed) continue;
+            if (heads[k].levelset == kLevelsUniform) uniform = true; else other = true;
+            if (heads[k].mode == kModeCoded) {
+                const uint32_t a = __ldg(heads[k].hdr + heads[k].hwords - 2u), b = __ldg(heads[k].hdr + heads[k].hwords - 1u);
+                same_code = same_code && (!coded || (a == w0 && b == w1));
+                w0 = a; w1 = b;
+                coded = true;
+            } else {
+                erc = true;
+            }
+        }
+        s_kind = coded ? (erc || !same_code ? kTabGaps : kTabCoded) : uniform ? (other ? kTabGaps : kTabUniform) : kTabErc;
+        s_alike = odd || (uniform && other) ? 2u : uniform ? 1u : 0u;
+    }
+    __syncthreads();
+    const uint32_t kind = s_kind, all_alike = s_alike;
+    for (uint32_t k = 0; k < K; ++k) {
+        const StreamHead& hd = heads[k];
+        if (!hd.ok || hd.mode == kModeFixed) continue;
+        uint16_t* const code = reinterpret_cast<uint16_t*>(stream_tabs + k * kStreamTabBytes);
+        if (kind == kTabGaps || hd.mode == kModeCoded) {    // level index by the next 7 bits
+            for (uint32_t i = tid; i < (1u << kMaxCodedS); i += blockDim.x) {
+                uint32_t c = 0, at = 0, index = 0;
+                if (hd.mode == kModeCoded) c = coded_entry(hd, G.s, i);
+                else if (erc_in_window(i << (32u - kMaxCodedS) | 0x01ffffffu, &at, &index) && at <= kMaxCodedS && index < hd.nlev) c = index | (at << 8);
+                code[i] = (uint16_t)c;
+            }
+        }
+        if (hd.levelset == kLevelsTable && tid <= G.s)
+            reinterpret_cast<float*>(stream_tabs + k * kStreamTabBytes + 256u)[tid] =
+                tid < G.s ? __uint_as_float(__ldg(hd.hdr + kHeaderWords + tid)) : 1.0f;
+    }
+    if (kind == kTabCoded) __syncthreads();
+    {
+        uint32_t first = 0;                                 // a token stream (all have the same code in the coded mode)
+        while (first + 1u < K && (!heads[first].ok || heads[first].mode == kModeFixed)) ++first;
+        const uint16_t* const code = reinterpret_cast<const uint16_t*>(stream_tabs + first * kStreamTabBytes);
+        const uint4* src = reinterpret_cast<const uint4*>(g_token_tables[kind == kTabErc || kind == kTabUniform ? kTabErc : kTabGaps]);
+        const uint32_t top = kind == kTabUniform ? 1u << G.s : G.s + 1u;
+        auto entry = [&](uint32_t e, uint32_t i) {
+            if (kind == kTabGaps) return e;
+            const uint32_t at = e & kLenMask, low = e & 0xffffu;
+            if (kind == kTabCoded) {                        // the gap's entry joined with the streams' level code
+                if (at == 0u) return 0u;
+                const uint32_t rest = i << (32u - kTokBits + at), c = code[(rest << 1) >> (32u - kMaxCodedS)];
+                const uint32_t len = at + 1u + (c >> 8);
+                if (c != 0u && len <= kTokBits) return len | (low & (0xffu << kGapShift)) | exp_symbol(c & 0xffu, rest >> 31, G.s);
+                return at > 1u ? (at - 1u) | ((low & (0xffu << kGapShift)) - (1u << kGapShift)) : 0u;
+            }
+            const uint32_t index = (e >> kSymShift) & 0x1ffu, negative = e >> 31;
+            if (index == 0u) return e;
+            if (index > top) return 0u;
+            return low | (kind == kTabUniform ? uniform_symbol(index, negative) : exp_symbol(index, negative, G.s));
+        };
+#pragma unroll 4
+        for (uint32_t i = tid; i < kTokEntries / 4u; i += blockDim.x) {
+            uint4 e = __ldg(src + i);
+            e.x = entry(e.x, 4u * i);
+            e.y = entry(e.y, 4u * i + 1u);
+            e.z = entry(e.z, 4u * i + 2u);
+            e.w = entry(e.w, 4u * i + 3u);
+            reinterpret_cast<uint4*>(table)[i] = e;
+        }
+    }
+    __syncthreads();
+    // from here on warps run alone
+
+    const uint32_t tab = smem_u32(table);
+    const uint32_t S = P.unit_subs;                         // sub-blocks of a unit
+    const uint64_t nsub = (G.d + kSB - 1u) / kSB, nunits = (nsub + S - 1u) / S, stride = (uint64_t)gridDim.x * (blockDim.x >> 5);
+    const uint32_t spb = G.bucket <= kBLK ? G.sb_per_block : 32u;   // sub-blocks of a coding block
+    const uint32_t lj = lane / S, lq = lane - lj * S;
+    const uint32_t ngroups = (K + 31u) / 32u;               // of up to 32 streams (S = 1 when there are several)
+
+    // An item is a unit of a group of streams.  The block offsets of an item's chains ...
+    struct Offsets {
+        uint64_t from, to;
+    };
+    auto load_offsets = [&](uint64_t unit, uint32_t g0) {
+        Offsets o;
+        o.from = o.to = 0;
+        const uint64_t sub = unit * S + lq;
+        const uint32_t k = g0 + lj;
+        if (unit < nunits && sub < nsub && k < K && lj * S + lq < 32u && heads[k].ok && heads[k].mode != kModeFixed) {
+            const uint64_t* at = reinterpret_cast<const uint64_t*>(heads[k].hdr + heads[k].hwords) + (uint32_t)sub / spb;
+            o.from = __ldg(at);
+            o.to = __ldg(at + 1);
+        }
+        return o;
+    };
+    // ... and, from them, where this lane's chain lies: the lengths of the sub-blocks before it in its block
+    auto describe = [&](uint64_t unit, uint32_t g0, const Offsets& o) {
+        Chain ch;
+        ch.src = nullptr;
+        ch.left = 0;
+        ch.bit = ch.len = 0;
+        ch.norm = 0.0f;
+        ch.good = true;
+        const uint64_t sub = unit * S + lq;
+        const uint32_t k = g0 + lj;
+        if (unit < nunits && sub < nsub && k < K && heads[k].ok && heads[k].mode != kModeFixed) {
+            const StreamHead& hd = heads[k];
+            const uint32_t blk = (uint32_t)sub / spb, sbi = (uint32_t)sub - blk * spb;
+            const uint64_t in_blk = nsub - (uint64_t)blk * spb;
+            const uint32_t nsb_blk = in_blk < spb ? (uint32_t)in_blk : spb, head_words = 1u + (nsb_blk + 1u) / 2u;
+            const uint64_t head = hd.hwords + 2 * (G.nblk + 1), words = (o.to - o.from) >> 5;
+            ch.good = ((o.from | o.to) & 31u) == 0 && o.from < o.to && (o.to >> 5) <= hd.cwords - head &&
+                      words >= head_words && words <= (1u << 20);
+            if (ch.good) {
+                const uint64_t rec = head + (o.from >> 5);
+                const uint32_t* const lens = hd.hdr + rec + 1u;
+                uint32_t start = 0;
+                const uint32_t last = sbi >> 1, pair = __ldg(lens + last);
+#pragma unroll 4
+                for (uint32_t w = 0; w < last; ++w) {
+                    const uint32_t v = __ldg(lens + w);
+                    start += (v & 0xffffu) + (v >> 16);
+                }
+                ch.norm = __uint_as_float(__ldg(lens - 1));
+                if (sbi & 1u) start += pair & 0xffffu;
+                const uint32_t len = sbi & 1u ? pair >> 16 : pair & 0xffffu;
+                ch.good = start + len <= 32u * ((uint32_t)words - head_words);
+                if (ch.good) {
+                    const uint64_t word = rec + head_words + (start >> 5), piece = word & ~(uint64_t)3u;
+                    ch.src = hd.hdr + piece;
+                    ch.left = hd.cwords - piece;
+                    ch.bit = 32u * (uint32_t)(word - piece) + (start & 31u);
+                    ch.len = len;
+                }
+            }
+        }
+        return ch;
+    };
+    // starts the copy of the lane's next words: those with bits [bit, bit + len) of ch.src, as many as there is room for
+    auto start_copy = [&](const Chain& ch) {
+        if (ch.len != 0u) {
+            const uint32_t n = min((ch.bit + ch.len + 31u) / 32u, kChunkWords);
+#pragma unroll
+            for (uint32_t i = 0; i < kChunkWords; i += 4u) {
+                if (i >= n) break;
+                if (i + 4u <= ch.left) copy_async16(copy + 4u * i, ch.src + i);
+                else for (uint32_t j = i; j < ch.left; ++j) copy_async4(copy + 4u * j, ch.src + j);   // the container ends here
+            }
+        }
+        asm volatile("cp.async.commit_group;" ::: "memory");
+    };
+    // the whole of the lane's chain is in its copy, with room for the ones behind it
+    auto fits = [&](const Chain& ch) { return (ch.bit + ch.len + 31u) / 32u + kChunkSlack <= kChunkWords; };
+
+    uint64_t unit = (uint64_t)warp * gridDim.x + blockIdx.x, unit1 = unit;
+    uint32_t group = 0, group1 = 0;
+    auto advance = [&](uint64_t& u, uint32_t& g) {
+        if (++g == ngroups) {
+            g = 0;
+            u += stride;
+        }
+    };
+    Chain ch = describe(unit, 0, load_offsets(unit, 0));
+    start_copy(ch);
+    advance(unit1, group1);
+    Offsets next = load_offsets(unit1, 32u * group1);
+    uint64_t carry[4] = {0, 0, 0, 0};                       // sums of the groups of streams before this one (S = 1)
+    while (unit < nunits) {
+        uint64_t unit2 = unit1;
+        uint32_t group2 = group1;
+        advance(unit2, group2);
+        const Offsets next2 = load_offsets(unit2, 32u * group2);
+        const uint32_t g0 = 32u * group, gcount = min(K - g0, 32u);
+        asm volatile("cp.async.wait_group 0;" ::: "memory");
+
+        // ================= walk =================
+        const StreamHead& my_head = heads[g0 + min(lj, gcount - 1u)];
+        const uint16_t* const my_code = reinterpret_cast<const uint16_t*>(stream_tabs + (g0 + min(lj, gcount - 1u)) * kStreamTabBytes);
+        const uint32_t row0 = rows + lane * Row<Sym>::kPitch - (uint32_t)sizeof(Sym), row_end = row0 + (kSB + 1u) * (uint32_t)sizeof(Sym);
+        uint32_t row = row0;
+        bool good = ch.good;
+        const float norm = ch.len != 0u ? ch.norm : 0.0f;
+        bool long_chain = __any_sync(0xffffffffu, !fits(ch));
+        auto put_ones = [&] {                               // behind the chain's last bit
+            if (ch.len != 0u) {
+                const uint32_t end = ch.bit + ch.len, w = copy + 4u * (end >> 5);
+                const uint32_t have = end & 31u ? lds_u32(w) : 0u;
+                asm volatile("st.shared.u32 [%0], %1;" ::"r"(w), "r"(have | 0xFFFFFFFFu >> (end & 31u)) : "memory");
+                asm volatile("st.shared.u32 [%0], %1;" ::"r"(w + 4u), "r"(0xFFFFFFFFu) : "memory");
+            }
+        };
+        uint32_t left = ch.len;
+        if (!long_chain) {
+            put_ones();
+            left -= kind == kTabGaps ? walk_rare<Sym, false, true>(copy, ch.bit, left, tab, row, row_end, my_head, my_code, G.s, good)
+                                     : walk_body<Sym, false, false>(copy, ch.bit, left, tab, row, row_end, my_head, my_code, G.s, good);
+        } else {
+            // chains longer than a lane's copy: one copy after the other, each walked up to 96 bits before its end
+            while (__any_sync(0xffffffffu, left != 0u)) {
+                const uint32_t room = 32u * kChunkWords - ch.bit;
+                const uint32_t bits = fits(ch) ? left : room - 96u;
+                uint32_t took = kind == kTabGaps ? walk_rare<Sym, true, true>(copy, ch.bit, bits, tab, row, row_end, my_head, my_code, G.s, good)
+                                                 : walk_rare<Sym, true, false>(copy, ch.bit, bits, tab, row, row_end, my_head, my_code, G.s, good);
+                if (!good || took > left) {
+                    good = false;
+                    took = left;
+                }
+                left -= took;
+                ch.len = left;
+                const uint32_t at = ch.bit + took, pieces = at / 128u;
+                ch.src += 4u * pieces;
+                ch.left -= 4u * pieces;
+                ch.bit = at - 128u * pieces;
+                start_copy(ch);
+                asm volatile("cp.async.wait_group 0;" ::: "memory");
+            }
+        }
+        // a well-formed chain ends exactly at its declared length, inside its sub-block
+        const uint64_t my_sub = unit * S + lq;
+        const uint32_t elems = (uint32_t)(G.d - min(G.d, my_sub * kSB) < kSB ? G.d - min(G.d, my_sub * kSB) : kSB);
+        good = good && left == 0u && row <= row0 + elems * (uint32_t)sizeof(Sym);
+        if (__any_sync(0xffffffffu, !good) && lane == 0) latch_status(P.ws, kErrBadStream);
+        asm volatile("st.shared.f32 [%0], %1;" ::"r"(norms + 4u * lane), "f"(norm) : "memory");
+        // norm times a power of two is exact for these norms (0 where there is no chain), so one fused operation does for two
+        const bool exact = __all_sync(0xffffffffu, norm == 0.0f || (norm >= 0x1p-100f && norm < 0x1p126f));
+        const Chain after = describe(unit1, 32u * group1, next);
+        __syncwarp();
+        start_copy(after);
+
+        // ================= add =================
+        const AddPass ap = {heads + g0, stream_tabs + g0 * kStreamTabBytes, rows, norms, S, gcount, exact ? all_alike : 2u,
+                            exact, group + 1u == ngroups, group != 0u};
+        const uint64_t e0 = unit * S * kSB + 4u * lane;
+        uint32_t q0 = 0;
+#pragma unroll 1
+        for (; q0 + 4u <= S; q0 += 4u) add_block<Sym, 4>(P, ap, q0, e0 + 256u * q0, carry);
+#pragma unroll 1
+        for (; q0 < S; ++q0) add_block<Sym, 1>(P, ap, q0, e0 + 256u * q0, carry);
+        __syncwarp();
+        clear_rows();
+        __syncwarp();
+        ch = after;
+        next = next2;
+        unit = unit1; group = group1;
+        unit1 = unit2; group1 = group2;
+    }
+}
+
+template <class Sym>
+static cudaError_t launch_chains(const DecodeParams& P, int sms, cudaStream_t stream) {
+    static bool attr_set = false;
+    if (!attr_set) {
+        const cudaError_t e = cudaFuncSetAttribute(decode_chains_kernel<Sym>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kChainSmem);
+        if (e != cudaSuccess) return e;
+        attr_set = true;
+    }
+    const size_t fixed = chain_fixed_bytes(P.K);
+    size_t warps = (kChainSmem - fixed) / Row<Sym>::kWarpBytes;
+    if (warps > kChainMaxWarps) warps = kChainMaxWarps;
+    const uint64_t nsub = (P.geo.d + kSB - 1u) / kSB;
+    DecodeParams Q = P;
+    // As many sub-blocks as give every lane a chain; in a small call no more than give every warp a unit (a walk
+    // lasts as long for one lane as for 32).
+    Q.unit_subs = P.K >= 32u ? 1u : 32u / P.K;
+    const uint64_t share = (nsub + (uint64_t)sms * warps - 1u) / ((uint64_t)sms * warps);
+    if (share < Q.unit_subs) Q.unit_subs = (uint32_t)share;
+    const uint64_t units = (nsub + Q.unit_subs - 1u) / Q.unit_subs;
+    cudaLaunchConfig_t cfg = cudaLaunchConfig_t{};
+    cudaLaunchAttribute attr[1];
+    cfg.gridDim = dim3((unsigned)(units < (uint64_t)sms ? units : (uint64_t)sms));
+    cfg.blockDim = dim3(32u * (unsigned)warps);
+    cfg.dynamicSmemBytes = fixed + warps * Row<Sym>::kWarpBytes;
+    cfg.stream = stream;
+    cfg.attrs = attr;
+    cfg.numAttrs = 0;
+    if (P.after_fixed) {
+        attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        attr[0].val.programmaticStreamSerializationAllowed = 1;
+        cfg.numAttrs = 1;
+    }
+    return cudaLaunchKernelEx(&cfg, decode_chains_kernel<Sym>, Q);
+}
+
+cudaError_t launch_decode_chains(const DecodeParams& P, int sms, cudaStream_t stream) {
+    // With s = 7 or 8 the streams may have uniform levels, whose indices up to 256 do not fit a byte with their sign.
+    return P.geo.s == 7u || P.geo.s == 8u ? launch_chains<int16_t>(P, sms, stream) : launch_chains<int8_t>(P, sms, stream);
+}
+
+}  // namespace nuq

@@ -1,0 +1,125 @@
+// Shared by the decode kernels: what a container's header says (checked on the device), the value of a symbol,
+// and what happens to the finished sum of an element (stored, or applied to the parameters at once).
+#pragma once
+#include "nuq_common.cuh"
+
+namespace nuq {
+
+// `hdr`: the container (a level-table stream carries its s interior levels behind the 16 header words)
+__device__ __forceinline__ float level_times_norm(float norm, uint32_t levelset, uint32_t s, uint32_t sym, const uint32_t* hdr) {
+    // exponential: l_j = 2^(j-1-s) (exact scaling);  uniform: l_k = k / 2^s;  table: l_j as stored, l_{s+1} = 1
+    float level;
+    if (levelset == kLevelsExp) level = __uint_as_float((126u + sym - s) << 23);
+    else if (levelset == kLevelsUniform) level = (float)sym * __uint_as_float((127u - s) << 23);
+    else level = sym <= s ? __uint_as_float(__ldg(hdr + kHeaderWords + sym - 1u)) : 1.0f;
+    return __fmul_rn(norm, level);
+}
+
+// ---------------------------------------------------------------------------
+// What happens to the finished sum G = sum_k DECODE(c_k) of an element: it is stored to acc (if there is
+// one) and, when the call carries the aggregation step of Algorithm 1, applied to the parameters at once,
+// so that the sum is not written out and read again by an optimizer kernel:
+//     y = w - (alpha / K) G,   y^l = w - l (alpha / K) G,   w <- y + mu (y^l - y^l_prev)
+// (Sec. 4, "NUQSGD with momentum"; mu = 0 is Algorithm 1's own line and leaves y^l alone).  fp32, each line
+// one fused multiply-add.
+// ---------------------------------------------------------------------------
+__device__ __forceinline__ float step_value(const DecodeParams& P, float w, float G, float* yl) {
+    const float y = __fmaf_rn(-P.step_c, G, w);
+    if (P.mu == 0.0f) return y;
+    const float yl_next = __fmaf_rn(-P.step_lc, G, w);
+    const float w_next = __fmaf_rn(P.mu, __fsub_rn(yl_next, *yl), y);
+    *yl = yl_next;
+    return w_next;
+}
+// element e (a multiple of 4) and the three behind it, with the parameters and y^l as they were
+__device__ __forceinline__ void step4(const DecodeParams& P, uint64_t e, float4 G, float4 w, float4 yl) {
+    if (P.acc) *reinterpret_cast<float4*>(P.acc + e) = G;
+    w.x = step_value(P, w.x, G.x, &yl.x);
+    w.y = step_value(P, w.y, G.y, &yl.y);
+    w.z = step_value(P, w.z, G.z, &yl.z);
+    w.w = step_value(P, w.w, G.w, &yl.w);
+    *reinterpret_cast<float4*>(P.w + e) = w;
+    if (P.mu != 0.0f) *reinterpret_cast<float4*>(P.yl + e) = yl;
+}
+__device__ __forceinline__ void finish4(const DecodeParams& P, uint64_t e, float4 G) {
+    if (!P.w) {
+        *reinterpret_cast<float4*>(P.acc + e) = G;
+        return;
+    }
+    float4 yl = make_float4(0.f, 0.f, 0.f, 0.f);
+    const float4 w = *reinterpret_cast<const float4*>(P.w + e);
+    if (P.mu != 0.0f) yl = *reinterpret_cast<const float4*>(P.yl + e);
+    step4(P, e, G, w, yl);
+}
+__device__ __forceinline__ void finish1(const DecodeParams& P, uint64_t e, float G) {
+    if (P.acc) P.acc[e] = G;
+    if (P.w) {
+        float yl = P.mu != 0.0f ? P.yl[e] : 0.0f;
+        P.w[e] = step_value(P, P.w[e], G, &yl);
+        if (P.mu != 0.0f) P.yl[e] = yl;
+    }
+}
+
+// the first n < 4 elements from e on
+__device__ __forceinline__ void finish_part(const DecodeParams& P, uint64_t e, float4 G, uint32_t n) {
+    if (n > 0u) finish1(P, e, G.x);
+    if (n > 1u) finish1(P, e + 1, G.y);
+    if (n > 2u) finish1(P, e + 2, G.z);
+}
+
+// Per stream of the call: what its header says, checked once per CTA.
+struct StreamHead {
+    const uint32_t* hdr;
+    uint64_t cwords;         // container words the header declares
+    uint32_t ok, mode, levelset, nlev, width;
+    uint32_t hwords;         // header words: 16, plus the level table of a level-table stream
+};
+
+// A container's header checked against the call's arguments.
+__device__ __forceinline__ StreamHead read_head(const Geometry& G, const uint32_t* hdr) {
+    const uint32_t flags = __ldg(hdr + 6);
+    const uint32_t levelset = (flags >> 8) & 0xffu, mode = (flags >> 16) & 0xffu;
+    const uint64_t hd = (uint64_t)__ldg(hdr + 2) | ((uint64_t)__ldg(hdr + 3) << 32);
+    const uint64_t hnblk = (uint64_t)__ldg(hdr + 8) | ((uint64_t)__ldg(hdr + 9) << 32);
+    const uint64_t cbits = (uint64_t)__ldg(hdr + 10) | ((uint64_t)__ldg(hdr + 11) << 32);
+    bool ok = __ldg(hdr) == kMagic && __ldg(hdr + 1) == kVersion && hd == G.d && __ldg(hdr + 4) == G.bucket &&
+              __ldg(hdr + 5) == G.s && __ldg(hdr + 7) == kSB && levelset <= 2u && mode <= 2u &&
+              (flags & 0xffu) <= 1u && !(levelset == kLevelsUniform && G.s > 8u) && (cbits & 31u) == 0;
+    const uint32_t nlev = levelset == kLevelsUniform ? (1u << G.s) + 1u : G.s + 2u;
+    const uint32_t hwords = kHeaderWords + (levelset == kLevelsTable ? ((G.s + 1u) & ~1u) : 0u) + (mode == kModeCoded ? 2u : 0u);
+    if (ok && mode == kModeCoded) {                         // the lengths must be those of a prefix code of at most 7 bits
+        ok = levelset != kLevelsUniform && G.s <= kMaxCodedS;
+        uint32_t kraft = 0;
+        for (uint32_t j = 0; ok && j <= G.s; ++j) {
+            const uint32_t len = (__ldg(hdr + hwords - 2u + (j >> 2)) >> (8u * (j & 3u))) & 0xffu;
+            ok = len >= 1u && len <= kMaxCodedS;
+            kraft += ok ? 1u << (kMaxCodedS - len) : 0u;
+        }
+        ok = ok && kraft <= (1u << kMaxCodedS);
+    }
+    if (ok && levelset == kLevelsTable) {                   // the levels must increase strictly inside (0, 1)
+        float below = 0.0f;
+        for (uint32_t j = 0; j < G.s; ++j) {
+            const float l = __uint_as_float(__ldg(hdr + kHeaderWords + j));
+            ok = ok && below < l;
+            below = l;
+        }
+        ok = ok && below < 1.0f;
+    }
+    const uint32_t width = 1u + (32u - __clz(nlev - 1u));                   // fixed mode: sign bit + ceil(log2(levels))
+    const uint64_t cwords = cbits >> 5;
+    if (ok && mode != kModeFixed) {
+        ok = hnblk == G.nblk && cwords > hwords + 2 * (G.nblk + 1);
+    } else if (ok) {
+        const uint32_t rec_words = 1u + (G.bucket * width + 31u) / 32u;
+        const uint64_t last_len = G.d - (G.nb - 1) * G.bucket;
+        ok = hnblk == G.nb &&
+             cwords == hwords + (G.nb - 1) * (uint64_t)rec_words + 1 + (last_len * width + 31) / 32;
+    }
+    StreamHead h;
+    h.hdr = hdr; h.cwords = cwords; h.ok = ok ? 1u : 0u; h.mode = mode; h.levelset = levelset;
+    h.nlev = nlev; h.width = width; h.hwords = hwords;
+    return h;
+}
+
+}  // namespace nuq

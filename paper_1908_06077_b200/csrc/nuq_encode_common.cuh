@@ -2,6 +2,7 @@
 // exponential level set, the bulk asynchronous copy with its mbarrier, tile geometry, and the end-of-CTA
 // bookkeeping that writes the container header.
 #pragma once
+#include "nuq_async.cuh"
 #include "nuq_common.cuh"
 
 namespace nuq {
@@ -54,44 +55,6 @@ __device__ __forceinline__ uint32_t quantize_exp(float v, float inv, float top, 
     const uint32_t hi = (__float_as_uint(fmaxf(y, 1.0f)) + (0x007FFFFFu - 0x3F000000u) - (word >> 9)) >> 23;
     const bool up = __uint2float_rn(word >> 8) < __fmul_rn(y, 16777216.0f);
     return up ? hi : 0u;                                    // no round-up: y < 1 and the index is 0
-}
-
-// ---------------------------------------------------------------------------
-// Bulk asynchronous copy (TMA, untiled form) and its mbarrier.  CTA-local barriers only.
-// ---------------------------------------------------------------------------
-__device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
-
-__device__ __forceinline__ void mbar_init(uint64_t* bar, uint32_t count) {
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(bar)), "r"(count) : "memory");
-    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-}
-
-// Announces `bytes` to the barrier and starts the copy global -> shared.  Both addresses
-// 16-byte aligned, `bytes` a positive multiple of 16.
-__device__ __forceinline__ void bulk_load(void* dst_smem, const void* src_gmem, uint32_t bytes, uint64_t* bar) {
-    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // earlier generic writes to dst are ordered first
-    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(bar)), "r"(bytes) : "memory");
-    asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
-                     smem_u32(dst_smem)),
-                 "l"(src_gmem), "r"(bytes), "r"(smem_u32(bar))
-                 : "memory");
-}
-
-// Waits until the phase with the given parity has completed.  Bounded: false after ~tens of ms.
-__device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity) {
-    const uint32_t addr = smem_u32(bar);
-    // the hardware parks the thread for up to the hinted time (ns), so a wait costs a handful of
-    // instructions; the number of tries bounds the wait (a fraction of a second at most)
-    for (uint32_t polls = 0; polls < (1u << 17); ++polls) {
-        uint32_t done;
-        asm volatile(
-            "{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2, %3;\n\tselp.u32 %0, 1, 0, p;\n\t}"
-            : "=r"(done)
-            : "r"(addr), "r"(parity), "r"(2000u)
-            : "memory");
-        if (done) return true;
-    }
-    return false;
 }
 
 // ---------------------------------------------------------------------------
