@@ -375,9 +375,12 @@ __device__ __forceinline__ void add_block(const DecodeParams& P, const AddPass& 
     uint32_t nrm = A.norms + 4u * q0, at = A.rows + q0 * Row<Sym>::kPitch + 4u * lane * (uint32_t)sizeof(Sym);
     auto add_rows = [&](auto value) {
 #pragma unroll
-        for (int h = 0; h < 2 * NB; ++h)
-            value(at + (h / 2) * Row<Sym>::kPitch + (h & 1) * 128u * (uint32_t)sizeof(Sym), __uint_as_float(lds_u32(nrm + 4u * (h / 2))),
-                  sum[2 * h], sum[2 * h + 1]);
+        for (int b = 0; b < NB; ++b) {
+            const float nm = __uint_as_float(lds_u32(nrm + 4u * b));
+#pragma unroll
+            for (int h = 2 * b; h < 2 * b + 2; ++h)
+                value(at + b * Row<Sym>::kPitch + (h & 1) * 128u * (uint32_t)sizeof(Sym), nm, sum[2 * h], sum[2 * h + 1]);
+        }
     };
     auto add_exp = [&](uint32_t row, float nm, uint64_t& s01, uint64_t& s23) {
         uint64_t a, b;
