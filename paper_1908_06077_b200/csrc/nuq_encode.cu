@@ -55,10 +55,57 @@ void build_erc_lut(uint32_t* lut) {
     }
 }
 
+// What the ERC encoder writes for a lane's eight consecutive elements when all their symbols are 0 or 1 (index 1: its
+// word is the single bit 0), by the mask of the nonzero ones (first element in bit 7).  A token is ERC(gap), sign, 0.
+//   body[m].x  the tokens behind the first one's gap code, sign bits zero: left aligned (at most 23 bits) | length
+//   body[m].y  the bit of the first sign of elements 4-7 (byte 0), first and last nonzero element (bytes 1, 2)
+//   sign[n | s << 4]   where the signs s of the nonzero ones n among four elements go, from the first sign on, left aligned
+struct EmitTables {
+    uint2 body[256];
+    uint32_t sign[256];
+};
+__device__ EmitTables g_emit_tables;
+
+static void build_emit_tables(const uint32_t* lut, EmitTables* t) {
+    for (uint32_t m = 0; m < 256; ++m) {
+        uint32_t bits = 0, len = 0, first = 0, last = 0, off_b = 0;
+        int prev = -1;
+        for (int k = 0; k < 8; ++k) {
+            if (!((m >> (7 - k)) & 1u)) continue;
+            if (prev < 0) first = k;
+            else {
+                const uint32_t e = lut[k - prev - 1];
+                bits = (bits << (e >> 16)) | (e & 0xffffu);
+                len += e >> 16;
+            }
+            if (k >= 4 && prev < 4) off_b = len;
+            bits <<= 2;                                     // sign, index
+            len += 2;
+            prev = k;
+            last = k;
+        }
+        t->body[m] = make_uint2(len ? (bits << (32u - len)) | len : 0u, off_b | (first << 8) | (last << 16));
+    }
+    for (uint32_t i = 0; i < 256; ++i) {
+        uint32_t pattern = 0, at = 0;
+        int prev = -1;
+        for (int k = 0; k < 4; ++k) {
+            if (!((i >> (3 - k)) & 1u)) continue;
+            if (prev >= 0) at += 2u + (lut[k - prev - 1] >> 16);
+            if ((i >> (7 - k)) & 1u) pattern |= 0x80000000u >> at;
+            prev = k;
+        }
+        t->sign[i] = pattern;
+    }
+}
+
 cudaError_t upload_erc_lut() {
     uint32_t lut[256];
+    static EmitTables emit;
     build_erc_lut(lut);
-    return cudaMemcpyToSymbol(c_erc_lut, lut, sizeof(lut));
+    build_emit_tables(lut, &emit);
+    const cudaError_t e = cudaMemcpyToSymbol(g_emit_tables, &emit, sizeof(emit));
+    return e == cudaSuccess ? cudaMemcpyToSymbol(c_erc_lut, lut, sizeof(lut)) : e;
 }
 
 // Uniform levels k / 2^s:  p = y - floor(y).
@@ -133,6 +180,131 @@ __device__ __forceinline__ uint32_t warp_incl_scan(uint32_t v) {
             : "r"(o));
     }
     return v;
+}
+
+// Appends the upper n bits of v to the right-aligned bit string hi:lo, n being the low five bits of v (a bit string
+// in v, left aligned, is shorter than 28 bits).
+__device__ __forceinline__ void append_bits(uint32_t& hi, uint32_t& lo, uint32_t v) {
+    hi = __funnelshift_l(lo, hi, v);
+    lo = __funnelshift_l(v, lo, v);
+}
+
+// ORs the right-aligned bit string hi:lo into the MSB-first bit string `dst`, so that it ends before bit `end`.
+__device__ __forceinline__ void or_bits_ending(uint32_t* dst, uint32_t end, uint32_t hi, uint32_t lo) {
+    const uint32_t sh = 0u - end;
+    const uint32_t w0 = __funnelshift_l(0u, lo, sh), w1 = __funnelshift_l(lo, hi, sh), w2 = __funnelshift_l(hi, 0u, sh);
+    uint32_t* const w = dst + (int32_t)(end - 1u >> 5);
+    if (w0) atomicOr(w, w0);
+    if (w1) atomicOr(w - 1, w1);
+    if (w2) atomicOr(w - 2, w2);
+}
+
+// One sub-block in the ERC and coded modes: quantizes (Definition 1) a lane's eight consecutive elements `x` with the
+// draws `r` and appends the warp's tokens ERC(gap) sign index to its bit window (`bits` so far, `nnz` counts this
+// lane's nonzero symbols).
+//
+// Every lane puts the tokens of its eight elements together in registers, one scan over the lengths gives all of
+// them their places, and every lane ORs its bits into the window: the work does not depend on how many symbols
+// are nonzero.  A lane's first gap reaches back to the last nonzero element of the nearest lane below that has one.
+// Where no element of the sub-block reaches the lowest level (most of them, for large buckets), every nonzero symbol
+// is 1 and a lane's bits follow from its eight-bit mask by table: one look-up for the tokens, two for their signs.
+template <uint32_t LEVELSET>
+__device__ __forceinline__ void emit_sub_block(const float (&x)[8], const uint32_t (&r)[8], float inv, float top, uint32_t s, bool one_bit,
+                                               const float* levels, const float* invw, const uint32_t* lut, const uint32_t* index_word,
+                                               const uint2* body, const uint32_t* sign_place, uint32_t* window, uint32_t window_bits,
+                                               uint32_t lane, Workspace* ws, uint32_t& bits, uint32_t& nnz) {
+    constexpr bool kExp = LEVELSET == kLevelsExp;
+    uint32_t nz = 0, sg = 0;                                // masks of the nonzero and the negative elements, the first in bit 7
+    uint32_t idx[8];
+    float y[8];
+    bool all_one = false;                                   // every nonzero symbol of the warp's sub-block is 1
+    if (kExp) {
+        float most = 0.0f;
+#pragma unroll
+        for (int k = 0; k < 8; ++k) {
+            // see quantize_exp: nonzero iff m < y 2^24, m the upper 24 bits of the draw (the difference is exact in its sign)
+            y[k] = __fmul_rn(fabsf(x[k]), inv);
+            const float d = __fmaf_rn(-16777216.0f, y[k], __uint2float_rn(r[k] >> 8));
+            nz = __funnelshift_l(__float_as_uint(d), nz, 1);
+            sg = __funnelshift_l(__float_as_uint(x[k]), sg, 1);
+            most = fmaxf(most, y[k]);
+        }
+        all_one = !__any_sync(0xffffffffu, most >= 1.0f) && one_bit;
+    } else {
+#pragma unroll
+        for (int k = 0; k < 8; ++k) {
+            idx[k] = LEVELSET == kLevelsTable ? quantize_table(x[k], inv, s, r[k], levels, invw) : quantize_uniform(x[k], inv, top, r[k]);
+            nz = (nz << 1) | (idx[k] ? 1u : 0u);
+        }
+    }
+    nnz += __popc(nz);
+    const uint2 bd = body[nz];
+    const uint32_t first = __byte_perm(bd.y, 0u, 0x4441), last = __byte_perm(bd.y, 0u, 0x4442);
+    // the last nonzero element before this lane's: position, -1 if there is none
+    const uint32_t below = __ballot_sync(0xffffffffu, nz != 0u) & ((1u << lane) - 1u);
+    int prev = (int)__shfl_sync(0xffffffffu, 8u * lane + last, 31 - __clz((int)(below | 1u)));
+    if (below == 0u) prev = -1;
+
+    if (kExp && all_one) {
+        const uint32_t neg = sg & nz;
+        const uint32_t ia = (nz >> 4) | (neg & 0xF0u), ib = (nz & 15u) | ((neg & 15u) << 4);
+        uint32_t gap = 0, hi = 0, lo = 0;
+        if (nz) gap = lut[8u * lane + first - (uint32_t)prev - 1u];
+        const uint32_t b = bd.x | sign_place[ia] | __funnelshift_r(sign_place[ib], 0u, bd.y);
+        append_bits(hi, lo, gap);
+        append_bits(hi, lo, b);
+        const uint32_t len = (gap & 31u) + (b & 31u);
+        const uint32_t incl = warp_incl_scan(len);
+        const uint32_t end = bits + incl;
+        bits += __shfl_sync(0xffffffffu, incl, 31);
+        if (bits > window_bits) {                           // the window is sized for the most bits there can be; checked all the same
+            if (lane == 0) latch_status(ws, kErrInternal);
+            bits = window_bits;
+            return;
+        }
+        or_bits_ending(window, end, hi, lo);
+        return;
+    }
+
+    // ---- any symbols: the tokens of kStr elements form a string of at most 64 bits ----
+    constexpr int kStr = LEVELSET == kLevelsUniform ? 2 : 4;
+    uint32_t hi[8 / kStr], lo[8 / kStr], len[8 / kStr], total = 0;
+#pragma unroll
+    for (int g = 0; g < 8 / kStr; ++g) {
+        hi[g] = lo[g] = len[g] = 0;
+#pragma unroll
+        for (int j = 0; j < kStr; ++j) {
+            const int k = g * kStr + j;
+            if (kExp) {
+                const uint32_t up = (__float_as_uint(fmaxf(fminf(y[k], top), 1.0f)) + (0x007FFFFFu - 0x3F000000u) - (r[k] >> 9)) >> 23;
+                idx[k] = (nz >> (7 - k)) & 1u ? up : 0u;
+            }
+            const int pos = (int)(8u * lane) + k;
+            uint32_t gap = 0;
+            if (idx[k]) {
+                gap = lut[pos - prev - 1];
+                prev = pos;
+            }
+            const uint32_t w = index_word[idx[k]];
+            append_bits(hi[g], lo[g], gap);
+            append_bits(hi[g], lo[g], w | (__float_as_uint(x[k]) & 0x80000000u));
+            len[g] += (gap & 31u) + (w & 31u);
+        }
+        total += len[g];
+    }
+    const uint32_t incl = warp_incl_scan(total);
+    uint32_t end = bits + incl - total;
+    bits += __shfl_sync(0xffffffffu, incl, 31);
+    if (bits > window_bits) {
+        if (lane == 0) latch_status(ws, kErrInternal);
+        bits = window_bits;
+        return;
+    }
+#pragma unroll
+    for (int g = 0; g < 8 / kStr; ++g) {
+        end += len[g];
+        or_bits_ending(window, end, hi[g], lo[g]);
+    }
 }
 
 // ---------------------------------------------------------------------------
@@ -387,7 +559,9 @@ encode_kernel(const __grid_constant__ EncodeParams P) {
     extern __shared__ __align__(128) uint32_t smem[];
     __shared__ __align__(8) uint64_t s_full[kEncWarps];    // s_full[w] completes when warp w's part of a tile has landed
     __shared__ uint32_t s_lut[256];                        // ERC(N), N = 1..256: code left aligned | length
-    __shared__ uint32_t s_lut_signed[256];                 // exponential levels: sign bit + ERC(index) left aligned | length, by field
+    __shared__ uint32_t s_index[260];                      // level index: a bit for the sign, then its word, left aligned | length; 0: 0
+    __shared__ uint2 s_body[256];                          // EmitTables
+    __shared__ uint32_t s_sign[256];
     __shared__ double s_partial[32];                       // per sub-block (or per warp) sums of squares
     __shared__ uint32_t s_maxbits[32];                     // ... or max |x| bit patterns
     __shared__ float s_sb_inv[32], s_sb_norm[32];          // per sub-block of the current tile: 2^s / norm (0: not quantized), norm
@@ -416,6 +590,7 @@ encode_kernel(const __grid_constant__ EncodeParams P) {
     uint64_t* table = reinterpret_cast<uint64_t*>(P.out + G.header_words);
     uint32_t* payload = MODE == kModeErc ? P.out + G.header_words + 2 * (G.nblk + 1) : P.out + G.header_words;
     constexpr bool kSmall = LEVELSET != kLevelsUniform;     // level index <= 15: symbols travel as bytes
+    const bool one_bit = LEVELSET == kLevelsExp && (G.mode != kModeCoded || (P.level_code[0] >> 16) == 1u);   // index 1 is written as 0
     const float top = LEVELSET == kLevelsTable ? 1.0f : __uint_as_float((127u + G.s) << 23);   // the norm is divided into this
     const uint32_t c2 = (uint32_t)P.offset, c3 = (uint32_t)(P.offset >> 32);
     const bool narrow = G.bucket <= kBLK;
@@ -466,15 +641,20 @@ encode_kernel(const __grid_constant__ EncodeParams P) {
     if (tid < 256u) {
         const uint32_t e = c_erc_lut[tid], elen = e >> 16;  // at most 16 bits
         s_lut[tid] = ((e & 0xffffu) << (32u - elen)) | elen;
-        const uint32_t idx = tid & 0x7Fu;                   // field = sign << 7 | index: sign bit, then ERC(index)
+        if (MODE == kModeErc) {
+            s_body[tid] = g_emit_tables.body[tid];
+            s_sign[tid] = g_emit_tables.sign[tid];
+        }
+    }
+    if (MODE == kModeErc && tid < 257u) {
         uint32_t v = 0;
-        if (idx >= 1) {
+        if (tid >= 1u) {
             // the index's code word: ERC(index), or in the coded mode the word of the fitted code
             const bool coded = G.mode == kModeCoded;
-            const uint32_t l = coded ? (idx <= kMaxCodedS + 1u ? P.level_code[idx - 1u] : 0u) : c_erc_lut[idx - 1u], len = l >> 16;
-            v = ((((tid >> 7) << len) | (l & 0xffffu)) << (31u - len)) | (len + 1u);
+            const uint32_t l = coded ? (tid <= kMaxCodedS + 1u ? P.level_code[tid - 1u] : 0u) : c_erc_lut[tid - 1u], len = l >> 16;
+            v = ((l & 0xffffu) << (31u - len)) | (len + 1u);
         }
-        s_lut_signed[tid] = v;
+        s_index[tid] = v;
     }
     if (tid < 32u) s_sb_bi[tid] = tid / spb;
     if (tid < kMaxTableS + 2u) {
@@ -654,9 +834,11 @@ encode_kernel(const __grid_constant__ EncodeParams P) {
         }
         // the draws of the warp's first sub-block do not depend on the norms: they are made before the
         // barrier, where the warp would otherwise wait for the slowest one
-        const uint64_t ctr_warp = ((elem0 + wbase) >> 2) + lane;               // Philox counter of row 0's block
+        // A lane's eight elements of a sub-block: eight consecutive ones in the ERC mode, else four of either row.
+        constexpr uint32_t kNextBlock = MODE == kModeErc ? 1u : 32u;           // Philox counter of the second four
+        const uint64_t ctr_warp = ((elem0 + wbase) >> 2) + (MODE == kModeErc ? 2u : 1u) * lane;
         uint4 rn0 = philox4x32_10((uint32_t)ctr_warp, (uint32_t)(ctr_warp >> 32), c2, c3, P.round_keys);
-        uint4 rn1 = philox4x32_10((uint32_t)(ctr_warp + 32u), (uint32_t)((ctr_warp + 32u) >> 32), c2, c3, P.round_keys);
+        uint4 rn1 = philox4x32_10((uint32_t)(ctr_warp + kNextBlock), (uint32_t)((ctr_warp + kNextBlock) >> 32), c2, c3, P.round_keys);
         // ---- whichever warp gets here last turns the partial sums into norms, once for the whole CTA ----
         {
             uint32_t last = 0;
@@ -736,7 +918,7 @@ encode_kernel(const __grid_constant__ EncodeParams P) {
         uint32_t* const window = windows + ((it & 1u) * kEncWarps + warp) * P.window_words;   // this warp's token string
         // ---- quantize (Definition 1) and emit, one sub-block (two 128-element rows) at a time ----
         uint32_t bits = 0;                                  // ERC: bits in this warp's window so far
-        uint32_t cum = 0;                                   // ERC: nonzero symbols so far (warp uniform)
+        uint32_t cum = 0;                                   // ERC: nonzero symbols of this lane so far
         // fixed-width mode: where a sub-block's 8 * width words go and how many of them exist
         uint32_t* fx_rec = nullptr;
         uint32_t fx_sb = 0, fx_words = 0;                   // sub-block within its record, valid field words of the record
@@ -778,7 +960,14 @@ encode_kernel(const __grid_constant__ EncodeParams P) {
                 fx_valid = min(sbw, fx_words - fx_sb * sbw);
             }
 
-            if (inv != 0.0f) {
+            if (MODE == kModeErc && inv != 0.0f) {
+                const float4* const mine = reinterpret_cast<const float4*>(data + wbase + q * kSB) + 2u * lane;
+                const float4 x0 = mine[0], x1 = mine[1];
+                const float x[8] = {x0.x, x0.y, x0.z, x0.w, x1.x, x1.y, x1.z, x1.w};
+                const uint32_t r[8] = {rn0.x, rn0.y, rn0.z, rn0.w, rn1.x, rn1.y, rn1.z, rn1.w};
+                emit_sub_block<LEVELSET>(x, r, inv, top, G.s, one_bit, s_levels, s_invw, s_lut, s_index, s_body, s_sign, window,
+                                         32u * (P.window_words - 2u), lane, P.ws, bits, cum);
+            } else if (inv != 0.0f) {
                 const float4 x0 = rows[32 * (2 * q)], x1 = rows[32 * (2 * q + 1)];
                 __syncwarp();                               // the sub-block's bytes are in registers: their place is scratch now
                 const uint4 r0 = rn0, r1 = rn1;
@@ -815,95 +1004,7 @@ encode_kernel(const __grid_constant__ EncodeParams P) {
                     f1 = syms1 | (tops1 & nz1);
                 }
 
-                if (MODE == kModeErc) {
-                    // ---- keep the nonzero symbols, in element order: a lane's rank = nonzeros of row 0 in lower
-                    // lanes (+ all of row 0 and those of row 1 in lower lanes, for its row-1 elements) ----
-                    uint32_t cnt0, cnt1;
-                    if (kSmall) {
-                        cnt0 = __popc(nz0);
-                        cnt1 = __popc(nz1);
-                    } else {
-                        cnt0 = (qa[0] != 0) + (qa[1] != 0) + (qa[2] != 0) + (qa[3] != 0);
-                        cnt1 = (qa[4] != 0) + (qa[5] != 0) + (qa[6] != 0) + (qa[7] != 0);
-                    }
-                    const uint32_t packed = cnt0 | (cnt1 << 16);
-                    const uint32_t incl = warp_incl_scan(packed);
-                    const uint32_t totals = __shfl_sync(0xffffffffu, incl, 31);
-                    const uint32_t tot0 = totals & 0xffffu;
-                    const uint32_t ntok = tot0 + (totals >> 16);
-                    uint32_t at0 = (incl & 0xffffu) - cnt0, at1 = tot0 + (incl >> 16) - cnt1;
-                    uint32_t* list32 = reinterpret_cast<uint32_t*>(data + wbase + q * kSB);   // over the sub-block's own bytes
-                    uint16_t* list16 = reinterpret_cast<uint16_t*>(list32);
-                    if (kSmall) {
-                        // 16-bit entries position | field << 8, two at a time by byte permutation
-                        const uint32_t pb0 = (lane * 4u) * 0x01010101u + 0x03020100u;      // the four positions of row 0, one per byte
-                        const uint32_t pb1 = pb0 + 0x80808080u;                            // ... of row 1
-                        const uint32_t a01 = __byte_perm(pb0, f0, 0x5140), a23 = __byte_perm(pb0, f0, 0x7362);
-                        const uint32_t b01 = __byte_perm(pb1, f1, 0x5140), b23 = __byte_perm(pb1, f1, 0x7362);
-                        if (qa[0]) list16[at0++] = (uint16_t)a01;
-                        if (qa[1]) list16[at0++] = (uint16_t)(a01 >> 16);
-                        if (qa[2]) list16[at0++] = (uint16_t)a23;
-                        if (qa[3]) list16[at0++] = (uint16_t)(a23 >> 16);
-                        if (qa[4]) list16[at1++] = (uint16_t)b01;
-                        if (qa[5]) list16[at1++] = (uint16_t)(b01 >> 16);
-                        if (qa[6]) list16[at1++] = (uint16_t)b23;
-                        if (qa[7]) list16[at1++] = (uint16_t)(b23 >> 16);
-                    } else {
-                        // 32-bit entries position | field << 10, field = index | sign << 15
-#pragma unroll
-                        for (int c = 0; c < 4; ++c) {
-                            if (qa[c]) list32[at0++] = (lane * 4u + c) | ((qa[c] | ((xb[c] >> 16) & 0x8000u)) << 10);
-                        }
-#pragma unroll
-                        for (int c = 4; c < 8; ++c) {
-                            if (qa[c]) list32[at1++] = (128u + lane * 4u + (c - 4)) | ((qa[c] | ((xb[c] >> 16) & 0x8000u)) << 10);
-                        }
-                    }
-                    __syncwarp();
-                    // ---- tokens ERC(gap) sign ERC(index), 32 per step, appended to the warp's window ----
-                    int carry_pos = -1;                         // position of the last nonzero so far: the run starts at t_0 = 0
-                    for (uint32_t t0 = 0; t0 < ntok; t0 += 32) {
-                        const bool valid = t0 + lane < ntok;
-                        uint32_t e = 0;
-                        if (valid) e = kSmall ? (uint32_t)list16[t0 + lane] : list32[t0 + lane];
-                        const int pos = (int)(e & (kSmall ? 255u : 1023u));
-                        const uint32_t field = e >> (kSmall ? 8 : 10);
-                        int prev = __shfl_up_sync(0xffffffffu, pos, 1);
-                        if (lane == 0) prev = carry_pos;
-                        uint32_t gl = 0;                        // stays 0 in lanes without a token: no bits, no length
-                        if (valid) gl = s_lut[(pos - prev - 1) & 255];
-                        uint32_t tlen, tokA, lenA, tokB = 0, lenB = 0;
-                        if (kSmall) {
-                            // both codes left aligned with their length in the low bits: the token is the gap code
-                            // followed by sign and index code, i.e. the second shifted right by the first's length
-                            const uint32_t ll = s_lut_signed[field & 255u];
-                            lenA = (gl & 31u) + (ll & 31u);
-                            tokA = (gl & ~31u) | ((ll & ~31u) >> (gl & 31u));     // <= 16 + 8 bits, left aligned
-                            tlen = lenA;
-                        } else {
-                            const uint32_t ll = s_lut[((field & S::kMask) - 1u) & 255u];
-                            lenA = gl & 31u;
-                            tokA = gl & ~31u;
-                            lenB = valid ? (ll & 31u) + 1u : 0u;                  // sign + ERC(index) <= 17 bits
-                            tokB = valid ? ((field >> S::kBits) << 31) | ((ll & ~31u) >> 1) : 0u;
-                            tlen = lenA + lenB;
-                        }
-                        const uint32_t incl_bits = warp_incl_scan(tlen);
-                        const uint32_t step_bits = __shfl_sync(0xffffffffu, incl_bits, 31);
-                        // the window is sized for the most bits the warp's elements can produce; checked all the same
-                        if (bits + step_bits > 32u * (P.window_words - 2u)) {
-                            if (lane == 0) latch_status(P.ws, kErrInternal);
-                            break;
-                        }
-                        const uint32_t off = bits + incl_bits - tlen;     // bit of the window where my token starts
-                        or_bits_left(window, off, tokA);
-                        if (!kSmall) or_bits_left(window, off + lenA, tokB);
-                        bits += step_bits;
-                        carry_pos = __shfl_sync(0xffffffffu, pos, min(ntok - t0, 32u) - 1u);
-                    }
-                    cum += ntok;
-                    __syncwarp();
-                } else {
+                {
                     // ---- fixed-width fields (sign bit, then the level index), MSB first ----
                     const uint32_t wbits = G.width;
                     if (kSmall && wbits == 4u) {
@@ -954,7 +1055,7 @@ encode_kernel(const __grid_constant__ EncodeParams P) {
                 meta->sb_src[sbq] = start_bits;
             }
             if (q < 3u) {                                   // the draws of the next sub-block
-                const uint64_t ctr0 = ctr_warp + 64u * (q + 1u), ctr1 = ctr0 + 32u;
+                const uint64_t ctr0 = ctr_warp + 64u * (q + 1u), ctr1 = ctr0 + kNextBlock;
                 rn0 = philox4x32_10((uint32_t)ctr0, (uint32_t)(ctr0 >> 32), c2, c3, P.round_keys);
                 rn1 = philox4x32_10((uint32_t)ctr1, (uint32_t)(ctr1 >> 32), c2, c3, P.round_keys);
             }
@@ -965,6 +1066,7 @@ encode_kernel(const __grid_constant__ EncodeParams P) {
         __syncwarp();
         if (lane == 0) start_copy(it + 1u);
         if (MODE == kModeErc) {
+            cum = __reduce_add_sync(0xffffffffu, cum);
             if (lane == 0) {
                 meta->wnnz[warp] = cum;
                 if (warp == 0) {
