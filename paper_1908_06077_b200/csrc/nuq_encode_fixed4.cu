@@ -29,17 +29,17 @@ __device__ __forceinline__ uint32_t quantize8_fixed4(const float4& a, const floa
                                                      const uint4& rb) {
     const float x[8] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
     const uint32_t r[8] = {ra.x, ra.y, ra.z, ra.w, rb.x, rb.y, rb.z, rb.w};
-    uint32_t word = 0;
+    uint32_t nz = 0, neg = 0;
+    float y[8], most = 0.0f;
 #pragma unroll
     for (int k = 0; k < 8; ++k) {
-        const float y = fminf(__fmul_rn(fabsf(x[k]), inv), top);
-        // see quantize_exp: the round-up is the carry into the exponent field; below the lowest level an exact comparison
-        const uint32_t hi = (__float_as_uint(fmaxf(y, 1.0f)) + (0x007FFFFFu - 0x3F000000u) - (r[k] >> 9)) >> 23;
-        const bool up = __uint2float_rn(r[k] >> 8) < __fmul_rn(y, 16777216.0f);
-        const uint32_t field = hi | ((__float_as_uint(x[k]) >> 28) & 8u);      // a zero symbol carries no sign
-        word = (word << 4) | (up ? field : 0u);
+        y[k] = __fmul_rn(fabsf(x[k]), inv);
+        zero_test(y[k], x[k], r[k], 0x10000000u >> (4 * k), nz, neg);
+        most = fmaxf(most, y[k]);
     }
-    return word;
+    const uint32_t high = __ballot_sync(0xffffffffu, most >= 1.0f);
+    if (high) add_high_levels(y, r, top, high, nz);
+    return nz | (neg << 3);                                 // a zero symbol carries no sign
 }
 
 // COARSE: the bucket is a multiple of 1024 elements, so a warp's four sub-blocks share one bucket.
@@ -250,7 +250,7 @@ __global__ void __launch_bounds__(kEncThreads, kEncMinBlocks) encode_fixed4_kern
         if (COARSE && sbq0 < nsb_tile) locate(sbq0);
         const float inv_coarse = s_sb_inv[sbq0];
 
-#pragma unroll
+#pragma unroll COARSE ? 4 : 1
         for (uint32_t q = 0; q < 4; ++q) {
             const uint32_t sbq = sbq0 + q;
             if (sbq >= nsb_tile) break;
