@@ -189,14 +189,23 @@ __device__ __forceinline__ void append_bits(uint32_t& hi, uint32_t& lo, uint32_t
     lo = __funnelshift_l(v, lo, v);
 }
 
-// ORs the right-aligned bit string hi:lo into the MSB-first bit string `dst`, so that it ends before bit `end`.
-__device__ __forceinline__ void or_bits_ending(uint32_t* dst, uint32_t end, uint32_t hi, uint32_t lo) {
+// ORs the right-aligned bit string hi:lo into the MSB-first bit string at shared-memory address `dst`, so that it ends
+// before bit `end`.  Words that get nothing are not touched (they need not exist).
+__device__ __forceinline__ void or_bits_ending(uint32_t dst, uint32_t end, uint32_t hi, uint32_t lo) {
     const uint32_t sh = 0u - end;
     const uint32_t w0 = __funnelshift_l(0u, lo, sh), w1 = __funnelshift_l(lo, hi, sh), w2 = __funnelshift_l(hi, 0u, sh);
-    uint32_t* const w = dst + (int32_t)(end - 1u >> 5);
-    if (w0) atomicOr(w, w0);
-    if (w1) atomicOr(w - 1, w1);
-    if (w2) atomicOr(w - 2, w2);
+    asm volatile(
+        "{\n\t.reg .pred p, q, r;\n\tsetp.ne.u32 p, %1, 0;\n\tsetp.ne.u32 q, %2, 0;\n\tsetp.ne.u32 r, %3, 0;\n\t"
+        "@p red.shared.or.b32 [%0], %1;\n\t@q red.shared.or.b32 [%0 + -4], %2;\n\t@r red.shared.or.b32 [%0 + -8], %3;\n\t}"
+        ::"r"(dst + (((end - 1u) >> 5) << 2)), "r"(w0), "r"(w1), "r"(w2) : "memory");
+}
+
+// An entry of a table in shared memory, 0 unless `take`.
+__device__ __forceinline__ uint32_t entry_if(bool take, const uint32_t* table, uint32_t i) {
+    uint32_t v;
+    asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.u32 p, %1, 0;\n\tmov.b32 %0, 0;\n\t@p ld.shared.u32 %0, [%2];\n\t}"
+                 : "=r"(v) : "r"(take ? 1u : 0u), "r"(smem_u32(table + i)));
+    return v;
 }
 
 // One sub-block in the ERC and coded modes: quantizes (Definition 1) a lane's eight consecutive elements `x` with the
@@ -208,28 +217,32 @@ __device__ __forceinline__ void or_bits_ending(uint32_t* dst, uint32_t end, uint
 // are nonzero.  A lane's first gap reaches back to the last nonzero element of the nearest lane below that has one.
 // Where no element of the sub-block reaches the lowest level (most of them, for large buckets), every nonzero symbol
 // is 1 and a lane's bits follow from its eight-bit mask by table: one look-up for the tokens, two for their signs.
+// Where a few lanes have such an element they put their tokens together one by one while the others wait.
 template <uint32_t LEVELSET>
 __device__ __forceinline__ void emit_sub_block(const float (&x)[8], const uint32_t (&r)[8], float inv, float top, uint32_t s, bool one_bit,
                                                const float* levels, const float* invw, const uint32_t* lut, const uint32_t* index_word,
-                                               const uint2* body, const uint32_t* sign_place, uint32_t* window, uint32_t window_bits,
+                                               const uint2* body, const uint32_t* sign_place, uint32_t window, uint32_t window_bits,
                                                uint32_t lane, Workspace* ws, uint32_t& bits, uint32_t& nnz) {
     constexpr bool kExp = LEVELSET == kLevelsExp;
-    uint32_t nz = 0, sg = 0;                                // masks of the nonzero and the negative elements, the first in bit 7
+    uint32_t nz = 0, neg = 0;                               // masks of the nonzero and the negative nonzero elements, the first in bit 7
     uint32_t idx[8];
     float y[8];
-    bool all_one = false;                                   // every nonzero symbol of the warp's sub-block is 1
+    uint32_t high = 0, extra = 0;                           // lanes with an element at or above the lowest level; their indices less one
+    bool few = false;                                       // all other nonzero symbols of the warp's sub-block are 1
     if (kExp) {
         float most = 0.0f;
 #pragma unroll
         for (int k = 0; k < 8; ++k) {
-            // see quantize_exp: nonzero iff m < y 2^24, m the upper 24 bits of the draw (the difference is exact in its sign)
             y[k] = __fmul_rn(fabsf(x[k]), inv);
-            const float d = __fmaf_rn(-16777216.0f, y[k], __uint2float_rn(r[k] >> 8));
-            nz = __funnelshift_l(__float_as_uint(d), nz, 1);
-            sg = __funnelshift_l(__float_as_uint(x[k]), sg, 1);
+            zero_test(y[k], x[k], r[k], 0x80u >> k, nz, neg);
             most = fmaxf(most, y[k]);
         }
-        all_one = !__any_sync(0xffffffffu, most >= 1.0f) && one_bit;
+        high = __ballot_sync(0xffffffffu, most >= 1.0f);
+        few = one_bit && __popc(high) <= 6;
+        if (few && high) {
+            add_high_levels(y, r, top, high, extra);
+            few = !__any_sync(0xffffffffu, extra != 0u && __popc(nz) > 4);   // (such a lane's tokens might not fit 64 bits)
+        }
     } else {
 #pragma unroll
         for (int k = 0; k < 8; ++k) {
@@ -245,15 +258,28 @@ __device__ __forceinline__ void emit_sub_block(const float (&x)[8], const uint32
     int prev = (int)__shfl_sync(0xffffffffu, 8u * lane + last, 31 - __clz((int)(below | 1u)));
     if (below == 0u) prev = -1;
 
-    if (kExp && all_one) {
-        const uint32_t neg = sg & nz;
+    if (kExp && few) {
         const uint32_t ia = (nz >> 4) | (neg & 0xF0u), ib = (nz & 15u) | ((neg & 15u) << 4);
-        uint32_t gap = 0, hi = 0, lo = 0;
-        if (nz) gap = lut[8u * lane + first - (uint32_t)prev - 1u];
+        uint32_t gap = entry_if(nz != 0u, lut, 8u * lane + first - (uint32_t)prev - 1u), hi = 0, lo = 0;
         const uint32_t b = bd.x | sign_place[ia] | __funnelshift_r(sign_place[ib], 0u, bd.y);
         append_bits(hi, lo, gap);
         append_bits(hi, lo, b);
-        const uint32_t len = (gap & 31u) + (b & 31u);
+        uint32_t len = (gap & 31u) + (b & 31u);
+        if (high != 0u && extra != 0u) {                    // a few lanes, one token after the other
+            hi = lo = len = 0;
+            uint32_t m = nz << 24;
+            do {
+                const uint32_t k = (uint32_t)__clz((int)m);
+                m &= ~(0x80000000u >> k);
+                const int pos = (int)(8u * lane + k);
+                gap = lut[pos - prev - 1];
+                const uint32_t w = index_word[1u + ((extra >> (28u - 4u * k)) & 15u)];
+                append_bits(hi, lo, gap);
+                append_bits(hi, lo, w | ((neg << (24u + k)) & 0x80000000u));
+                len += (gap & 31u) + (w & 31u);
+                prev = pos;
+            } while (m);
+        }
         const uint32_t incl = warp_incl_scan(len);
         const uint32_t end = bits + incl;
         bits += __shfl_sync(0xffffffffu, incl, 31);
@@ -280,11 +306,8 @@ __device__ __forceinline__ void emit_sub_block(const float (&x)[8], const uint32
                 idx[k] = (nz >> (7 - k)) & 1u ? up : 0u;
             }
             const int pos = (int)(8u * lane) + k;
-            uint32_t gap = 0;
-            if (idx[k]) {
-                gap = lut[pos - prev - 1];
-                prev = pos;
-            }
+            const uint32_t gap = entry_if(idx[k] != 0u, lut, (uint32_t)(pos - prev - 1));
+            prev = idx[k] != 0u ? pos : prev;
             const uint32_t w = index_word[idx[k]];
             append_bits(hi[g], lo[g], gap);
             append_bits(hi[g], lo[g], w | (__float_as_uint(x[k]) & 0x80000000u));
@@ -581,7 +604,8 @@ encode_kernel(const __grid_constant__ EncodeParams P) {
 
     using S = Sym<LEVELSET>;
     const Geometry& G = P.geo;
-    const uint32_t tid = threadIdx.x, lane = tid & 31u, warp = tid >> 5;
+    const uint32_t tid = threadIdx.x, lane = tid & 31u;
+    const uint32_t warp = __shfl_sync(0xffffffffu, tid >> 5, 0);      // (the same in all lanes, and known to be)
     float* const data = reinterpret_cast<float*>(smem);                         // kBLK floats: the tile
     uint32_t* const images = smem + kBLK;                                       // [2][stage_words]: staged tile records
     uint32_t* const windows = images + 2u * P.stage_words;                      // [2][kEncWarps][window_words]: token strings
@@ -765,7 +789,7 @@ encode_kernel(const __grid_constant__ EncodeParams P) {
             break;
         }
         const uint64_t elem0 = ti.elem0;
-        const uint32_t tile_len = ti.tile_len, nsb_tile = ti.nsb;
+        const uint32_t tile_len = __shfl_sync(0xffffffffu, ti.tile_len, 0), nsb_tile = (tile_len + kSB - 1u) / kSB;
 
         // ---- the warp's part of the tile: wait for the bulk copy, fetch the ragged end, zero the rest ----
         {
@@ -786,49 +810,66 @@ encode_kernel(const __grid_constant__ EncodeParams P) {
         // of 2^-24 relative each, of random sign), everything beyond that in fp64: the norm stays within a
         // few 1e-8 of the exactly rounded one.  Linf: max |x|, exact. ----
         if (P.norms_in == nullptr) {
-            double acc = 0.0;
-            uint32_t mx = 0;
+            if (G.norm_kind == kNormL2) {
+                float p8[4];
 #pragma unroll
-            for (int q = 0; q < 4; ++q) {
-                const float4 x = rows[32 * (2 * q)], y = rows[32 * (2 * q + 1)];
-                if (G.norm_kind == kNormL2) {
+                for (int q = 0; q < 4; ++q) {
+                    const float4 x = rows[32 * (2 * q)], y = rows[32 * (2 * q + 1)];
                     float a = __fmul_rn(x.x, x.x), b = __fmul_rn(x.y, x.y);
                     a = __fmaf_rn(x.z, x.z, a); b = __fmaf_rn(x.w, x.w, b);
                     a = __fmaf_rn(y.x, y.x, a); b = __fmaf_rn(y.y, y.y, b);
                     a = __fmaf_rn(y.z, y.z, a); b = __fmaf_rn(y.w, y.w, b);
-                    const float p8 = a + b;
-                    // squares that leave the fp32 range (tiny or huge coordinates, NaN): the warp adds this
-                    // sub-block up in fp64 instead
-                    const bool out_of_range = !(p8 >= 0x1p-60f && p8 < 0x1p120f);
-                    if (__any_sync(0xffffffffu, out_of_range)) {
+                    p8[q] = a + b;
+                }
+                // squares that leave the fp32 range (tiny or huge coordinates, NaN): the warp adds that sub-block up in
+                // fp64 instead
+                auto out_of_range = [](float p) { return !(p >= 0x1p-60f && p < 0x1p120f); };
+                double e8[4];
+#pragma unroll
+                for (int q = 0; q < 4; ++q) e8[q] = (double)p8[q];
+                if (__any_sync(0xffffffffu, out_of_range(p8[0]) || out_of_range(p8[1]) || out_of_range(p8[2]) || out_of_range(p8[3]))) {
+#pragma unroll 1
+                    for (int q = 0; q < 4; ++q) {
+                        const float p = q == 0 ? p8[0] : q == 1 ? p8[1] : q == 2 ? p8[2] : p8[3];
+                        if (!__any_sync(0xffffffffu, out_of_range(p))) continue;
+                        const float4 x = rows[32 * (2 * q)], y = rows[32 * (2 * q + 1)];
                         double e = 0.0;
                         e = fma((double)x.x, (double)x.x, e); e = fma((double)x.y, (double)x.y, e);
                         e = fma((double)x.z, (double)x.z, e); e = fma((double)x.w, (double)x.w, e);
                         e = fma((double)y.x, (double)y.x, e); e = fma((double)y.y, (double)y.y, e);
                         e = fma((double)y.z, (double)y.z, e); e = fma((double)y.w, (double)y.w, e);
-                        acc += e;
-                    } else {
-                        acc += (double)p8;
+                        if (q == 0) e8[0] = e; else if (q == 1) e8[1] = e; else if (q == 2) e8[2] = e; else e8[3] = e;
                     }
-                } else {                                    // on the bit patterns: NaN sorts above inf
+                }
+                auto warp_sum = [&](double acc) {
+#pragma unroll
+                    for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+                    return acc;
+                };
+                if (coarse) {                               // one partial per warp, or one per sub-block
+                    const double acc = warp_sum(((e8[0] + e8[1]) + e8[2]) + e8[3]);
+                    if (lane == 0) s_partial[warp * 4 + 3] = acc;
+                } else {
+#pragma unroll
+                    for (int q = 0; q < 4; ++q) {
+                        const double acc = warp_sum(e8[q]);
+                        if (lane == 0) s_partial[warp * 4 + q] = acc;
+                    }
+                }
+            } else {
+                uint32_t mx = 0;
+#pragma unroll
+                for (int q = 0; q < 4; ++q) {               // on the bit patterns: NaN sorts above inf
+                    const float4 x = rows[32 * (2 * q)], y = rows[32 * (2 * q + 1)];
                     mx = max(max(mx, __float_as_uint(fabsf(x.x))), __float_as_uint(fabsf(x.y)));
                     mx = max(max(mx, __float_as_uint(fabsf(x.z))), __float_as_uint(fabsf(x.w)));
                     mx = max(max(mx, __float_as_uint(fabsf(y.x))), __float_as_uint(fabsf(y.y)));
                     mx = max(max(mx, __float_as_uint(fabsf(y.z))), __float_as_uint(fabsf(y.w)));
-                }
-                if (!coarse || q == 3) {                    // one partial per sub-block, or one per warp
-                    if (G.norm_kind == kNormL2) {
-#pragma unroll
-                        for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-                    } else {
+                    if (!coarse || q == 3) {
                         mx = __reduce_max_sync(0xffffffffu, mx);
+                        if (lane == 0) s_maxbits[warp * 4 + q] = mx;
+                        mx = 0;
                     }
-                    if (lane == 0) {
-                        s_partial[warp * 4 + q] = acc;
-                        s_maxbits[warp * 4 + q] = mx;
-                    }
-                    acc = 0.0;
-                    mx = 0;
                 }
             }
         }
@@ -919,20 +960,15 @@ encode_kernel(const __grid_constant__ EncodeParams P) {
         // ---- quantize (Definition 1) and emit, one sub-block (two 128-element rows) at a time ----
         uint32_t bits = 0;                                  // ERC: bits in this warp's window so far
         uint32_t cum = 0;                                   // ERC: nonzero symbols of this lane so far
+        uint32_t string_start = 0;                          // ERC: lane q: where the string of the warp's sub-block q starts in its window
         // fixed-width mode: where a sub-block's 8 * width words go and how many of them exist
         uint32_t* fx_rec = nullptr;
         uint32_t fx_sb = 0, fx_words = 0;                   // sub-block within its record, valid field words of the record
 #pragma unroll 1
         for (uint32_t q = 0; q < 4; ++q) {
             const uint32_t sbq = warp * 4u + q;
-            const uint32_t start_bits = bits;
-            if (sbq >= nsb_tile) {
-                if (MODE == kModeErc && lane == 0) {
-                    meta->sb_bits[sbq] = 0;
-                    meta->sb_src[sbq] = bits;
-                }
-                continue;
-            }
+            if (MODE == kModeErc && lane >= q) string_start = bits;
+            if (sbq >= nsb_tile) continue;
             const float inv = s_sb_inv[sbq];
 
             uint32_t* fx_dst = nullptr;
@@ -960,14 +996,15 @@ encode_kernel(const __grid_constant__ EncodeParams P) {
                 fx_valid = min(sbw, fx_words - fx_sb * sbw);
             }
 
-            if (MODE == kModeErc && inv != 0.0f) {
+            const bool quantized = __any_sync(0xffffffffu, inv != 0.0f);   // (a vote: the branch is known to be uniform)
+            if (MODE == kModeErc && quantized) {
                 const float4* const mine = reinterpret_cast<const float4*>(data + wbase + q * kSB) + 2u * lane;
                 const float4 x0 = mine[0], x1 = mine[1];
                 const float x[8] = {x0.x, x0.y, x0.z, x0.w, x1.x, x1.y, x1.z, x1.w};
                 const uint32_t r[8] = {rn0.x, rn0.y, rn0.z, rn0.w, rn1.x, rn1.y, rn1.z, rn1.w};
-                emit_sub_block<LEVELSET>(x, r, inv, top, G.s, one_bit, s_levels, s_invw, s_lut, s_index, s_body, s_sign, window,
+                emit_sub_block<LEVELSET>(x, r, inv, top, G.s, one_bit, s_levels, s_invw, s_lut, s_index, s_body, s_sign, smem_u32(window),
                                          32u * (P.window_words - 2u), lane, P.ws, bits, cum);
-            } else if (inv != 0.0f) {
+            } else if (quantized) {
                 const float4 x0 = rows[32 * (2 * q)], x1 = rows[32 * (2 * q + 1)];
                 __syncwarp();                               // the sub-block's bytes are in registers: their place is scratch now
                 const uint4 r0 = rn0, r1 = rn1;
@@ -1050,10 +1087,6 @@ encode_kernel(const __grid_constant__ EncodeParams P) {
             } else if (MODE == kModeFixed) {
                 for (uint32_t i = lane; i < fx_valid; i += 32) fx_dst[i] = 0;      // a bucket that is not quantized: all fields zero
             }
-            if (MODE == kModeErc && lane == 0) {
-                meta->sb_bits[sbq] = bits - start_bits;
-                meta->sb_src[sbq] = start_bits;
-            }
             if (q < 3u) {                                   // the draws of the next sub-block
                 const uint64_t ctr0 = ctr_warp + 64u * (q + 1u), ctr1 = ctr0 + kNextBlock;
                 rn0 = philox4x32_10((uint32_t)ctr0, (uint32_t)(ctr0 >> 32), c2, c3, P.round_keys);
@@ -1067,6 +1100,11 @@ encode_kernel(const __grid_constant__ EncodeParams P) {
         if (lane == 0) start_copy(it + 1u);
         if (MODE == kModeErc) {
             cum = __reduce_add_sync(0xffffffffu, cum);
+            const uint32_t next_start = __shfl_down_sync(0xffffffffu, string_start, 1);
+            if (lane < 4u) {                                // lane q: sub-block q of the warp
+                meta->sb_bits[warp * 4u + lane] = (lane < 3u ? next_start : bits) - string_start;
+                meta->sb_src[warp * 4u + lane] = string_start;
+            }
             if (lane == 0) {
                 meta->wnnz[warp] = cum;
                 if (warp == 0) {
