@@ -206,7 +206,24 @@ struct EncodePlan {
     uint32_t want_grid;      // CTAs that give every SM its full share
 };
 
-static EncodePlan plan_encode(EncodeParams& P, int sms, uint32_t flags) {
+// What the runtime says about an encoder's occupancy depends on the kernel and its shared memory only; asking takes longer
+// than the rest of a call's host work, so the answers are kept (guarded by g_mu; a few dozen entries at most, one per
+// combination of level set, mode, bucket kind, number of levels and cluster size in use).
+static int occupancy(const EncodeParams& P, int dev, bool clusters) {
+    static std::map<uint64_t, int> known;
+    const Geometry& G = P.geo;
+    const uint64_t key = (uint64_t)encode_smem_bytes(P) | (uint64_t)G.levelset << 32 | (uint64_t)G.mode << 34 |
+                         (uint64_t)(fixed4_applies(G) ? 1 : 0) << 36 | (uint64_t)(G.bucket % (kBLK / kEncWarps) == 0 ? 1 : 0) << 37 |
+                         (uint64_t)(clusters ? P.cluster : 0) << 38 | (uint64_t)(uint32_t)dev << 44;
+    const auto it = known.find(key);
+    if (it != known.end()) return it->second;
+    const int n = clusters ? encode_max_clusters(P) : encode_blocks_per_sm(P);
+    if (n > 0) known[key] = n;
+    return n;
+}
+
+static EncodePlan plan_encode(EncodeParams& P, int dev, uint32_t flags) {
+    const int sms = device_sms(dev);
     const Geometry& G = P.geo;
     const bool norms_are_ours = (flags & NUQ_TEST_NORMS) == 0;
     EncodePlan pl;
@@ -225,7 +242,7 @@ static EncodePlan plan_encode(EncodeParams& P, int sms, uint32_t flags) {
                                                              : (warp_elems % G.bucket == 0 ? warp_elems / G.bucket : warp_elems / G.bucket + 1u);
         P.window_words = (token_bits_bound(G, warp_elems, warp_buckets, norms_are_ours) + 31u) / 32u + 4u;
     }
-    int best = encode_blocks_per_sm(P);                     // resident CTAs per SM: what shared memory and registers allow
+    int best = occupancy(P, dev, false);                    // resident CTAs per SM: what shared memory and registers allow
     if (best > kEncMaxBlocks) best = kEncMaxBlocks;
     const int per_sm = best < 1 ? 1 : best;
     const uint64_t cap = (uint64_t)sms * (uint64_t)per_sm;
@@ -237,7 +254,7 @@ static EncodePlan plan_encode(EncodeParams& P, int sms, uint32_t flags) {
     P.overlap = 0;
     if (G.bucket > kBLK && norms_are_ours && !fixed4_applies(G)) {
         P.cluster = G.blk_per_bucket;
-        int clusters = encode_max_clusters(P);
+        int clusters = occupancy(P, dev, true);
         const int cap_clusters = sms * per_sm / (int)P.cluster;
         if (clusters > cap_clusters) clusters = cap_clusters;
         if (clusters >= 1) {
@@ -487,7 +504,7 @@ nuq_status nuq_encode(const float* g, uint64_t d, uint32_t bucket, uint32_t s, u
     if (!encode_args_ok(g, d, bucket, s, norm_kind, out, out_bits, &G)) return NUQ_ERR_INVALID_ARG;
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess) return NUQ_ERR_CUDA;
-    const EncodePlan pl = plan_encode(P, device_sms(dev), norm_kind);
+    const EncodePlan pl = plan_encode(P, dev, norm_kind);
     P.grid = pl.want_grid;
     Workspace* ws = nullptr;
     nuq_status st = get_workspace(stream, pl.state_bytes + pl.norms_bytes, &ws, &dev);
@@ -505,7 +522,7 @@ nuq_status nuq_encode_static(const float* g, uint64_t d, uint32_t bucket, uint32
     if (!encode_args_ok(g, d, bucket, s, norm_kind, out, out_bits, &G)) return NUQ_ERR_INVALID_ARG;
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess) return NUQ_ERR_CUDA;
-    const EncodePlan pl = plan_encode(P, device_sms(dev), norm_kind);
+    const EncodePlan pl = plan_encode(P, dev, norm_kind);
     if (pl.state_bytes + pl.norms_bytes > kStaticScratchBytes) return NUQ_ERR_CAPACITY;   // vector too long for the array
     P.grid = pl.want_grid;
     auto it = g_static_ws.find(dev);

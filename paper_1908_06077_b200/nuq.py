@@ -81,12 +81,16 @@ _lib = _load()
 LIBRARY_PATH = _build.LIB
 
 
+_current_raw_stream, _current_device = torch._C._cuda_getCurrentRawStream, torch._C._cuda_getDevice
+
+
 def _stream(stream):
+    """A cudaStream_t as an integer: the current torch stream of the current device unless one is given."""
     if stream is None:
-        return C.c_void_p(torch.cuda.current_stream().cuda_stream)
+        return _current_raw_stream(_current_device())
     if isinstance(stream, torch.cuda.Stream):
-        return C.c_void_p(stream.cuda_stream)
-    return C.c_void_p(int(stream))
+        return stream.cuda_stream
+    return int(stream)
 
 
 def version() -> str:
@@ -111,8 +115,8 @@ def level_histogram(g: torch.Tensor, bucket, s, norm_kind=0, seed=0, offset=0, h
     assert g.is_cuda and g.dtype == torch.float32 and g.is_contiguous()
     if hist is None:
         hist = torch.empty(s + 2, dtype=torch.int64, device=g.device)
-    rc = _lib.nuq_level_histogram(C.c_void_p(g.data_ptr()), g.numel(), bucket, s, norm_kind, seed, offset,
-                                  C.c_void_p(hist.data_ptr()), _stream(stream))
+    rc = _lib.nuq_level_histogram(g.data_ptr(), g.numel(), bucket, s, norm_kind, seed, offset,
+                                  hist.data_ptr(), _stream(stream))
     if rc != NUQ_OK:
         raise NuqError("nuq_level_histogram", rc)
     return hist
@@ -141,7 +145,7 @@ def set_level_code(lengths):
 
 def set_test_norms(norms: torch.Tensor | None):
     """norms: CUDA float32 tensor of ceil(d/bucket) bucket norms (kept by reference), or None."""
-    rc = _lib.nuq_set_test_norms(C.c_void_p(norms.data_ptr()) if norms is not None else None)
+    rc = _lib.nuq_set_test_norms(norms.data_ptr() if norms is not None else None)
     if rc != NUQ_OK:
         raise NuqError("nuq_set_test_norms", rc)
 
@@ -158,8 +162,8 @@ def encode(g: torch.Tensor, bucket, s, norm_kind=0, seed=0, offset=0, out=None, 
         out = torch.empty(nbytes // 4, dtype=torch.int32, device=g.device)
     if out_bits is None:
         out_bits = torch.empty(1, dtype=torch.int64, device=g.device)
-    rc = _lib.nuq_encode(C.c_void_p(g.data_ptr()), d, bucket, s, norm_kind, seed, offset, C.c_void_p(out.data_ptr()),
-                         C.c_void_p(out_bits.data_ptr()), _stream(stream))
+    rc = _lib.nuq_encode(g.data_ptr(), d, bucket, s, norm_kind, seed, offset, out.data_ptr(),
+                         out_bits.data_ptr(), _stream(stream))
     if rc != NUQ_OK:
         raise NuqError("nuq_encode", rc)
     return out, out_bits
@@ -172,19 +176,31 @@ def encode_static(g: torch.Tensor, bucket, s, norm_kind=0, seed=0, offset=0, *, 
     allocated here either.  Raises NuqError(ERR_CAPACITY) when d is too long for that array.
     Calls that could overlap on the GPU must be serialised by the caller."""
     assert g.is_cuda and g.dtype == torch.float32 and g.is_contiguous()
-    rc = _lib.nuq_encode_static(C.c_void_p(g.data_ptr()), g.numel(), bucket, s, norm_kind, seed, offset,
-                                C.c_void_p(out.data_ptr()), C.c_void_p(out_bits.data_ptr()), _stream(stream))
+    rc = _lib.nuq_encode_static(g.data_ptr(), g.numel(), bucket, s, norm_kind, seed, offset,
+                                out.data_ptr(), out_bits.data_ptr(), _stream(stream))
     if rc != NUQ_OK:
         raise NuqError("nuq_encode_static", rc)
     return out, out_bits
+
+
+_pointer_arrays = {}
+
+
+def _pointers(streams):
+    """the containers' addresses as a C array (copied by the call it is handed to)"""
+    n = len(streams)
+    array = _pointer_arrays.get(n)
+    if array is None:
+        array = _pointer_arrays[n] = C.c_void_p * n
+    return array(*[t.data_ptr() for t in streams])
 
 
 def decode_accumulate(streams, d, bucket, s, acc=None, stream=None):
     """acc <- sum_k DECODE(streams[k]); acc is overwritten."""
     if acc is None:
         acc = torch.empty(d, dtype=torch.float32, device=streams[0].device)
-    ptrs = (C.c_void_p * len(streams))(*[C.c_void_p(t.data_ptr()) for t in streams])
-    rc = _lib.nuq_decode_accumulate(ptrs, len(streams), d, bucket, s, C.c_void_p(acc.data_ptr()), _stream(stream))
+    ptrs = _pointers(streams)
+    rc = _lib.nuq_decode_accumulate(ptrs, len(streams), d, bucket, s, acc.data_ptr(), _stream(stream))
     if rc != NUQ_OK:
         raise NuqError("nuq_decode_accumulate", rc)
     return acc
@@ -192,10 +208,10 @@ def decode_accumulate(streams, d, bucket, s, acc=None, stream=None):
 
 def decode_update(streams, d, bucket, s, w, yl=None, alpha=1.0, mu=0.0, l=0.0, acc=None, stream=None):
     """w <- w - (alpha / K) sum_k DECODE(streams[k]), or the momentum rule with yl when mu != 0; in place."""
-    ptrs = (C.c_void_p * len(streams))(*[C.c_void_p(t.data_ptr()) for t in streams])
-    rc = _lib.nuq_decode_update(ptrs, len(streams), d, bucket, s, C.c_void_p(acc.data_ptr() if acc is not None else None),
-                                C.c_void_p(w.data_ptr()), C.c_void_p(yl.data_ptr() if yl is not None else None),
-                                C.c_float(alpha), C.c_float(mu), C.c_float(l), _stream(stream))
+    ptrs = _pointers(streams)
+    rc = _lib.nuq_decode_update(ptrs, len(streams), d, bucket, s, acc.data_ptr() if acc is not None else None,
+                                w.data_ptr(), yl.data_ptr() if yl is not None else None,
+                                alpha, mu, l, _stream(stream))
     if rc != NUQ_OK:
         raise NuqError("nuq_decode_update", rc)
     return w
@@ -207,7 +223,7 @@ def last_status(stream=None) -> int:
 
 def stream_info(out: torch.Tensor, stream=None) -> dict:
     info = _Info()
-    rc = _lib.nuq_stream_info(C.c_void_p(out.data_ptr()), C.byref(info), _stream(stream))
+    rc = _lib.nuq_stream_info(out.data_ptr(), C.byref(info), _stream(stream))
     if rc != NUQ_OK:
         raise NuqError("nuq_stream_info", rc)
     return {k: int(getattr(info, k)) for k, _ in _Info._fields_}
