@@ -662,6 +662,7 @@ encode_kernel(const __grid_constant__ EncodeParams P) {
     };
 
     let_next_kernel_start(P);
+    if (warp < (uint32_t)kEncWarps && lane == 0) prefetch_first_tile(P, warp);
     if (tid < 256u) {
         const uint32_t e = c_erc_lut[tid], elen = e >> 16;  // at most 16 bits
         s_lut[tid] = ((e & 0xffffu) << (32u - elen)) | elen;
@@ -687,7 +688,7 @@ encode_kernel(const __grid_constant__ EncodeParams P) {
     }
     if (MODE == kModeErc)
         for (uint32_t i = tid; i < 2u * P.stage_words + 2u * kEncWarps * P.window_words; i += blockDim.x) images[i] = 0;
-    wait_for_previous_kernel(P);                            // nothing above reads or writes global memory
+    wait_for_previous_kernel(P);                            // nothing above reads or writes global memory (tables apart, which never change)
     if (tid == 0) {
         for (int w = 0; w < kEncWarps; ++w) mbar_init(&s_full[w], 1);
         s_nnz = 0;
