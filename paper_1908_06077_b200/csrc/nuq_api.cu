@@ -197,7 +197,7 @@ using namespace nuq;
 // Mode of the containers this process has encoded, by device and address (see enqueue_encode): a hint
 // for the decoder's choice of kernels, which check it against the containers' headers on the device.
 // Guarded by g_mu.
-static std::map<std::pair<int, const void*>, uint32_t> g_container_mode;
+static std::map<std::pair<int, const void*>, uint32_t> g_container_mode;   // mode | level set << 8
 
 // What one encode call needs from its workspace and from shared memory.
 struct EncodePlan {
@@ -329,7 +329,7 @@ static nuq_status enqueue_encode(EncodeParams& P, const EncodePlan& pl, const fl
     // remember the mode of the container at this address: a hint for the decoder's choice of kernels,
     // checked against the header on the device
     if (g_container_mode.size() > 4096) g_container_mode.clear();
-    g_container_mode[std::make_pair(dev, static_cast<const void*>(out))] = G.mode;
+    g_container_mode[std::make_pair(dev, static_cast<const void*>(out))] = G.mode | G.levelset << 8;
     return NUQ_OK;
 }
 
@@ -569,9 +569,13 @@ static nuq_status enqueue_decode(const void* const* streams, uint32_t K, uint64_
     }
     P.unit_subs = 0;                                    // (chosen at the launch)
     P.after_fixed = w ? 0u : 1u;                        // all streams believed to be in the fixed-width mode? (sums only)
+    P.likely_table = kTabErc;
     for (uint32_t k = 0; k < K; ++k) {
         auto it = g_container_mode.find(std::make_pair(dev, streams[k]));
-        if (it == g_container_mode.end() || it->second != kModeFixed) P.after_fixed = 0;
+        const uint32_t mode = it == g_container_mode.end() ? kModeErc : it->second & 0xffu;
+        if (mode != kModeFixed) P.after_fixed = 0;
+        if (mode == kModeCoded) P.likely_table = kTabCoded;
+        else if (k == 0 && it != g_container_mode.end() && it->second >> 8 == kLevelsUniform) P.likely_table = kTabUniform;
     }
     P.acc = acc;
     P.w = w;
@@ -589,7 +593,7 @@ static nuq_status enqueue_decode(const void* const* streams, uint32_t K, uint64_
     WsEntry& entry = g_ws[std::make_pair(dev, stream)];
     if (P.after_fixed && ++entry.dec_epoch == 0) entry.dec_epoch = 2;       // never 0, parity kept
     P.epoch = entry.dec_epoch;
-    P.pad = 0;
+    P.let_next = 0;                                     // (chosen at the launch, like unit_subs)
     if (launch_decode(P, device_sms(dev), stream) != cudaSuccess) return NUQ_ERR_CUDA;
     return NUQ_OK;
 }

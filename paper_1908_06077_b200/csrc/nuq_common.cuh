@@ -88,14 +88,18 @@ struct EncodeParams {
     uint32_t overlap;        // launched so that its CTAs are set up while the kernel before it in the stream ends
 };
 
+// Token tables of the chain decoder: ERC level indices as exponential or as uniform levels, gaps alone, a fitted level code.
+enum : uint32_t { kTabErc = 0, kTabGaps = 1, kTabCoded = 2, kTabUniform = 3 };
+
 struct DecodeParams {
     Geometry geo;
     const uint32_t* streams[kMaxK];
     uint32_t K;
     uint32_t unit_subs;      // token streams: sub-blocks a warp decodes at a time
+    uint32_t likely_table;   // the token table the call most likely needs (kTabErc, kTabUniform), or kTabCoded: none to prepare
     uint32_t after_fixed;    // the fixed-width kernel runs first; the general kernel returns if it did the work
     uint32_t epoch;          // number of this decode call on its workspace (never 0)
-    uint32_t pad;
+    uint32_t let_next;       // token streams: the kernel behind may be launched early
     // the aggregation step fused into the decoder (w == nullptr: none): see step_value in nuq_decode.cu
     float* w;                // parameters, updated in place
     float* yl;               // the momentum rule's y^l, updated in place (not touched when mu == 0)

@@ -63,8 +63,7 @@ __device__ __forceinline__ uint32_t uniform_symbol(uint32_t index, uint32_t nega
     return (negative ? 0u - index : index) << kSymShift;
 }
 
-// Tables as kept in device memory: the symbol is the level index (1 .. 255), bit 31 of the entry the sign.
-enum : uint32_t { kTabErc = 0, kTabGaps = 1, kTabCoded = 2, kTabUniform = 3 };
+// Tables as kept in device memory (kTabErc and kTabGaps): the symbol is the level index (1 .. 255), bit 31 of the entry the sign.
 __device__ uint32_t g_token_tables[2][kTokEntries];
 
 // ERC^-1 of the nbits-bit prefix idx from bit `pos` on (Algorithm 2, decoding): false when the code does not end within it.
@@ -134,7 +133,7 @@ __device__ __forceinline__ bool erc_in_window(uint32_t win, uint32_t* at, uint32
 // A stream with coded level indices brings its own code: the level index and the word's length (<< 8) by the
 // next 7 bits, 0 where no word starts (possible only with an incomplete code).
 __device__ __forceinline__ uint32_t coded_entry(const StreamHead& hd, uint32_t s, uint32_t prefix) {
-    const uint32_t w0 = __ldg(hd.hdr + hd.hwords - 2u), w1 = __ldg(hd.hdr + hd.hwords - 1u);   // the lengths, one byte each
+    const uint32_t w0 = *(hd.hdr + hd.hwords - 2u), w1 = *(hd.hdr + hd.hwords - 1u);   // the lengths, one byte each
     auto len_of = [&](uint32_t j) { return ((j < 4u ? w0 : w1) >> (8u * (j & 3u))) & 0xffu; };
     for (uint32_t j = 0; j <= s; ++j) {
         // canonical words: level indices by (length, index), the first word all zeros, each next one the
@@ -331,8 +330,8 @@ __device__ __noinline__ bool four_fields(const Geometry& G, const StreamHead& hd
     const uint64_t blen = G.d - b * G.bucket < G.bucket ? G.d - b * G.bucket : G.bucket;
     const uint32_t last = (uint32_t)((blen * wd + 31u) / 32u) - 1u, bit = in_bucket * wd, wi = bit >> 5;
     const uint32_t* const rec = hd.hdr + hd.hwords + b * rec_words;
-    const float norm = __uint_as_float(__ldg(rec));
-    const uint32_t x0 = __ldg(rec + 1u + min(wi, last)), x1 = __ldg(rec + 1u + min(wi + 1u, last)), x2 = __ldg(rec + 1u + min(wi + 2u, last));
+    const float norm = __uint_as_float(rec[0]);
+    const uint32_t x0 = rec[1u + min(wi, last)], x1 = rec[1u + min(wi + 1u, last)], x2 = rec[1u + min(wi + 2u, last)];
     const uint64_t win = ((uint64_t)__funnelshift_l(x1, x0, bit) << 32) | __funnelshift_l(x2, x1, bit);   // 64 bits from the first field on
     float v[4];
     bool ok = true;
@@ -488,10 +487,6 @@ template <class Sym>
 __global__ void __launch_bounds__(32 * kChainMaxWarps, 1) decode_chains_kernel(const __grid_constant__ DecodeParams P) {
     extern __shared__ __align__(128) unsigned char dsm[];
     __shared__ uint32_t s_kind, s_alike;
-    // Behind the fixed-width kernel this one is launched with programmatic stream serialization: its launch is
-    // worked off while that kernel still runs, and it waits here until that kernel's writes are visible.
-    if (P.after_fixed) asm volatile("griddepcontrol.wait;" ::: "memory");
-    if (P.after_fixed && *reinterpret_cast<volatile uint32_t*>(&P.ws->dec_done_epoch) == P.epoch) return;   // the fixed-width kernel did it all
     const Geometry& G = P.geo;
     const uint32_t K = P.K, tid = threadIdx.x, lane = tid & 31u, warp = tid >> 5;
     uint32_t* const table = reinterpret_cast<uint32_t*>(dsm);
@@ -501,59 +496,12 @@ __global__ void __launch_bounds__(32 * kChainMaxWarps, 1) decode_chains_kernel(c
     const uint32_t norms = rows + 32u * Row<Sym>::kPitch;   // one per lane's chain
     const uint32_t copy = norms + 128u + lane * (4u * kChunkWords);   // this lane's words of its chain
 
-    // ---- headers against the call's arguments, once per stream; then the table that serves all the token streams ----
-    for (uint32_t k = tid; k < K; k += blockDim.x) {
-        heads[k] = read_head(G, P.streams[k]);
-        if (!heads[k].ok) latch_status(P.ws, kErrBadStream);
-    }
     auto clear_rows = [&] {
         for (uint32_t i = 16u * lane; i < 32u * Row<Sym>::kPitch; i += 512u)
             asm volatile("st.shared.v4.u32 [%0], {%1, %1, %1, %1};" ::"r"(rows + i), "r"(0u) : "memory");
     };
-    clear_rows();
-    __syncthreads();
-    if (tid == 0) {
-        bool coded = false, erc = false, uniform = false, other = false, same_code = true, odd = false;
-        uint32_t w0 = 0, w1 = 0;
-        for (uint32_t k = 0; k < K; ++k) {
-            odd = odd || !heads[k].ok || heads[k].mode == kModeFixed || heads[k].levelset == kLevelsTable;
-            if (!heads[k].ok || heads[k].mode == kModeFixed) continue;
-            if (heads[k].levelset == kLevelsUniform) uniform = true; else other = true;
-            if (heads[k].mode == kModeCoded) {
-                const uint32_t a = __ldg(heads[k].hdr + heads[k].hwords - 2u), b = __ldg(heads[k].hdr + heads[k].hwords - 1u);
-                same_code = same_code && (!coded || (a == w0 && b == w1));
-                w0 = a; w1 = b;
-                coded = true;
-            } else {
-                erc = true;
-            }
-        }
-        s_kind = coded ? (erc || !same_code ? kTabGaps : kTabCoded) : uniform ? (other ? kTabGaps : kTabUniform) : kTabErc;
-        s_alike = odd || (uniform && other) ? 2u : uniform ? 1u : 0u;
-    }
-    __syncthreads();
-    const uint32_t kind = s_kind, all_alike = s_alike;
-    for (uint32_t k = 0; k < K; ++k) {
-        const StreamHead& hd = heads[k];
-        if (!hd.ok || hd.mode == kModeFixed) continue;
-        uint16_t* const code = reinterpret_cast<uint16_t*>(stream_tabs + k * kStreamTabBytes);
-        if (kind == kTabGaps || hd.mode == kModeCoded) {    // level index by the next 7 bits
-            for (uint32_t i = tid; i < (1u << kMaxCodedS); i += blockDim.x) {
-                uint32_t c = 0, at = 0, index = 0;
-                if (hd.mode == kModeCoded) c = coded_entry(hd, G.s, i);
-                else if (erc_in_window(i << (32u - kMaxCodedS) | 0x01ffffffu, &at, &index) && at <= kMaxCodedS && index < hd.nlev) c = index | (at << 8);
-                code[i] = (uint16_t)c;
-            }
-        }
-        if (hd.levelset == kLevelsTable && tid <= G.s)
-            reinterpret_cast<float*>(stream_tabs + k * kStreamTabBytes + 256u)[tid] =
-                tid < G.s ? __uint_as_float(__ldg(hd.hdr + kHeaderWords + tid)) : 1.0f;
-    }
-    if (kind == kTabCoded) __syncthreads();
-    {
-        uint32_t first = 0;                                 // a token stream (all have the same code in the coded mode)
-        while (first + 1u < K && (!heads[first].ok || heads[first].mode == kModeFixed)) ++first;
-        const uint16_t* const code = reinterpret_cast<const uint16_t*>(stream_tabs + first * kStreamTabBytes);
+    // The token table for streams of kind `kind` (`code`: their level code, kTabCoded only).
+    auto build_table = [&](uint32_t kind, const uint16_t* code) {
         const uint4* src = reinterpret_cast<const uint4*>(g_token_tables[kind == kTabErc || kind == kTabUniform ? kTabErc : kTabGaps]);
         const uint32_t top = kind == kTabUniform ? 1u << G.s : G.s + 1u;
         auto entry = [&](uint32_t e, uint32_t i) {
@@ -580,8 +528,81 @@ __global__ void __launch_bounds__(32 * kChainMaxWarps, 1) decode_chains_kernel(c
             e.w = entry(e.w, 4u * i + 3u);
             reinterpret_cast<uint4*>(table)[i] = e;
         }
+    };
+
+    // The kernel is launched with programmatic stream serialization: its CTAs take the SMs as the kernel in front leaves
+    // them, build the table that the call is likely to need and clear their rows, and wait here until that kernel has ended.
+    // Nothing before the wait touches memory that another kernel writes.  The kernel behind is let in early only by calls
+    // that give every warp several units: a small encode call let in early finds room only where CTAs of this kernel have
+    // left and is packed onto a few SMs, four CTAs each (a step of 10^6 elements, K = 3: 66 -> 74 us).
+    if (P.let_next) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    if (P.after_fixed) {                                    // the fixed-width kernel in front has done it all, as a rule
+        asm volatile("griddepcontrol.wait;" ::: "memory");
+        if (*reinterpret_cast<volatile uint32_t*>(&P.ws->dec_done_epoch) == P.epoch) return;
+    }
+    if (P.likely_table != kTabCoded) build_table(P.likely_table, nullptr);
+    clear_rows();
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+
+    // ---- headers against the call's arguments, once per stream; then what kind of table serves all the token streams ----
+    for (uint32_t k = tid; k < K; k += blockDim.x) {
+        heads[k] = read_head(G, P.streams[k]);
+        if (!heads[k].ok) latch_status(P.ws, kErrBadStream);
     }
     __syncthreads();
+    if (warp == 0) {
+        bool coded = false, erc = false, uniform = false, other = false, odd = false, same_code = true;
+        uint32_t first0 = 0, first1 = 0;                    // the code lengths of the first coded stream
+        for (uint32_t k0 = 0; k0 < K; k0 += 32u) {
+            const uint32_t k = k0 + lane;
+            const bool tokens = k < K && heads[k].ok && heads[k].mode != kModeFixed, in_code = tokens && heads[k].mode == kModeCoded;
+            uint32_t w0 = 0, w1 = 0;
+            if (in_code) {
+                w0 = heads[k].hdr[heads[k].hwords - 2u];
+                w1 = heads[k].hdr[heads[k].hwords - 1u];
+            }
+            const uint32_t with_code = __ballot_sync(0xffffffffu, in_code);
+            if (with_code && !coded) {
+                first0 = __shfl_sync(0xffffffffu, w0, __ffs((int)with_code) - 1);
+                first1 = __shfl_sync(0xffffffffu, w1, __ffs((int)with_code) - 1);
+                coded = true;
+            }
+            same_code = same_code && !__any_sync(0xffffffffu, in_code && (w0 != first0 || w1 != first1));
+            erc = erc || __any_sync(0xffffffffu, tokens && !in_code);
+            uniform = uniform || __any_sync(0xffffffffu, tokens && heads[k].levelset == kLevelsUniform);
+            other = other || __any_sync(0xffffffffu, tokens && heads[k].levelset != kLevelsUniform);
+            odd = odd || __any_sync(0xffffffffu, k < K && (!tokens || heads[k].levelset == kLevelsTable));
+        }
+        if (lane == 0) {
+            s_kind = coded ? (erc || !same_code ? kTabGaps : kTabCoded) : uniform ? (other ? kTabGaps : kTabUniform) : kTabErc;
+            s_alike = odd || (uniform && other) ? 2u : uniform ? 1u : 0u;
+        }
+    }
+    __syncthreads();
+    const uint32_t kind = s_kind, all_alike = s_alike;
+    if (kind != P.likely_table || kind == kTabGaps || kind == kTabCoded || all_alike == 2u) {
+        uint32_t first = K;                                 // the first token stream (all have the same code in the coded mode)
+        for (uint32_t k = 0; k < K; ++k) {
+            const StreamHead& hd = heads[k];
+            if (!hd.ok || hd.mode == kModeFixed) continue;
+            uint16_t* const code = reinterpret_cast<uint16_t*>(stream_tabs + k * kStreamTabBytes);
+            if (kind == kTabGaps || (kind == kTabCoded && first == K)) {   // level index by the next 7 bits
+                for (uint32_t i = tid; i < (1u << kMaxCodedS); i += blockDim.x) {
+                    uint32_t c = 0, at = 0, index = 0;
+                    if (hd.mode == kModeCoded) c = coded_entry(hd, G.s, i);
+                    else if (erc_in_window(i << (32u - kMaxCodedS) | 0x01ffffffu, &at, &index) && at <= kMaxCodedS && index < hd.nlev) c = index | (at << 8);
+                    code[i] = (uint16_t)c;
+                }
+            }
+            if (hd.levelset == kLevelsTable && tid <= G.s)
+                reinterpret_cast<float*>(stream_tabs + k * kStreamTabBytes + 256u)[tid] =
+                    tid < G.s ? __uint_as_float(hd.hdr[kHeaderWords + tid]) : 1.0f;
+            if (first == K) first = k;
+        }
+        if (kind == kTabCoded) __syncthreads();
+        if (kind != P.likely_table || kind == kTabCoded) build_table(kind, reinterpret_cast<const uint16_t*>(stream_tabs + (first == K ? 0u : first) * kStreamTabBytes));
+        __syncthreads();
+    }
     // from here on warps run alone
 
     const uint32_t tab = smem_u32(table);
@@ -602,8 +623,8 @@ __global__ void __launch_bounds__(32 * kChainMaxWarps, 1) decode_chains_kernel(c
         const uint32_t k = g0 + lj;
         if (unit < nunits && sub < nsub && k < K && lj * S + lq < 32u && heads[k].ok && heads[k].mode != kModeFixed) {
             const uint64_t* at = reinterpret_cast<const uint64_t*>(heads[k].hdr + heads[k].hwords) + (uint32_t)sub / spb;
-            o.from = __ldg(at);
-            o.to = __ldg(at + 1);
+            o.from = at[0];
+            o.to = at[1];
         }
         return o;
     };
@@ -629,13 +650,13 @@ __global__ void __launch_bounds__(32 * kChainMaxWarps, 1) decode_chains_kernel(c
                 const uint64_t rec = head + (o.from >> 5);
                 const uint32_t* const lens = hd.hdr + rec + 1u;
                 uint32_t start = 0;
-                const uint32_t last = sbi >> 1, pair = __ldg(lens + last);
+                const uint32_t last = sbi >> 1, pair = lens[last];
 #pragma unroll 4
                 for (uint32_t w = 0; w < last; ++w) {
-                    const uint32_t v = __ldg(lens + w);
+                    const uint32_t v = lens[w];
                     start += (v & 0xffffu) + (v >> 16);
                 }
-                ch.norm = __uint_as_float(__ldg(lens - 1));
+                ch.norm = __uint_as_float(lens[-1]);
                 if (sbi & 1u) start += pair & 0xffffu;
                 const uint32_t len = sbi & 1u ? pair >> 16 : pair & 0xffffu;
                 ch.good = start + len <= 32u * ((uint32_t)words - head_words);
@@ -779,6 +800,7 @@ static cudaError_t launch_chains(const DecodeParams& P, int sms, cudaStream_t st
     const uint64_t share = (nsub + (uint64_t)sms * warps - 1u) / ((uint64_t)sms * warps);
     if (share < Q.unit_subs) Q.unit_subs = (uint32_t)share;
     const uint64_t units = (nsub + Q.unit_subs - 1u) / Q.unit_subs;
+    Q.let_next = units > 2u * (uint64_t)sms * warps ? 1u : 0u;
     cudaLaunchConfig_t cfg = cudaLaunchConfig_t{};
     cudaLaunchAttribute attr[1];
     cfg.gridDim = dim3((unsigned)(units < (uint64_t)sms ? units : (uint64_t)sms));
@@ -786,12 +808,9 @@ static cudaError_t launch_chains(const DecodeParams& P, int sms, cudaStream_t st
     cfg.dynamicSmemBytes = fixed + warps * Row<Sym>::kWarpBytes;
     cfg.stream = stream;
     cfg.attrs = attr;
-    cfg.numAttrs = 0;
-    if (P.after_fixed) {
-        attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-        attr[0].val.programmaticStreamSerializationAllowed = 1;
-        cfg.numAttrs = 1;
-    }
+    cfg.numAttrs = 1;
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
     return cudaLaunchKernelEx(&cfg, decode_chains_kernel<Sym>, Q);
 }
 

@@ -11,7 +11,7 @@ __device__ __forceinline__ float level_times_norm(float norm, uint32_t levelset,
     float level;
     if (levelset == kLevelsExp) level = __uint_as_float((126u + sym - s) << 23);
     else if (levelset == kLevelsUniform) level = (float)sym * __uint_as_float((127u - s) << 23);
-    else level = sym <= s ? __uint_as_float(__ldg(hdr + kHeaderWords + sym - 1u)) : 1.0f;
+    else level = sym <= s ? __uint_as_float(hdr[kHeaderWords + sym - 1u]) : 1.0f;
     return __fmul_rn(norm, level);
 }
 
@@ -77,13 +77,13 @@ struct StreamHead {
 
 // A container's header checked against the call's arguments.
 __device__ __forceinline__ StreamHead read_head(const Geometry& G, const uint32_t* hdr) {
-    const uint32_t flags = __ldg(hdr + 6);
+    const uint32_t flags = hdr[6];
     const uint32_t levelset = (flags >> 8) & 0xffu, mode = (flags >> 16) & 0xffu;
-    const uint64_t hd = (uint64_t)__ldg(hdr + 2) | ((uint64_t)__ldg(hdr + 3) << 32);
-    const uint64_t hnblk = (uint64_t)__ldg(hdr + 8) | ((uint64_t)__ldg(hdr + 9) << 32);
-    const uint64_t cbits = (uint64_t)__ldg(hdr + 10) | ((uint64_t)__ldg(hdr + 11) << 32);
-    bool ok = __ldg(hdr) == kMagic && __ldg(hdr + 1) == kVersion && hd == G.d && __ldg(hdr + 4) == G.bucket &&
-              __ldg(hdr + 5) == G.s && __ldg(hdr + 7) == kSB && levelset <= 2u && mode <= 2u &&
+    const uint64_t hd = (uint64_t)hdr[2] | ((uint64_t)hdr[3] << 32);
+    const uint64_t hnblk = (uint64_t)hdr[8] | ((uint64_t)hdr[9] << 32);
+    const uint64_t cbits = (uint64_t)hdr[10] | ((uint64_t)hdr[11] << 32);
+    bool ok = hdr[0] == kMagic && hdr[1] == kVersion && hd == G.d && hdr[4] == G.bucket &&
+              hdr[5] == G.s && hdr[7] == kSB && levelset <= 2u && mode <= 2u &&
               (flags & 0xffu) <= 1u && !(levelset == kLevelsUniform && G.s > 8u) && (cbits & 31u) == 0;
     const uint32_t nlev = levelset == kLevelsUniform ? (1u << G.s) + 1u : G.s + 2u;
     const uint32_t hwords = kHeaderWords + (levelset == kLevelsTable ? ((G.s + 1u) & ~1u) : 0u) + (mode == kModeCoded ? 2u : 0u);
@@ -91,7 +91,7 @@ __device__ __forceinline__ StreamHead read_head(const Geometry& G, const uint32_
         ok = levelset != kLevelsUniform && G.s <= kMaxCodedS;
         uint32_t kraft = 0;
         for (uint32_t j = 0; ok && j <= G.s; ++j) {
-            const uint32_t len = (__ldg(hdr + hwords - 2u + (j >> 2)) >> (8u * (j & 3u))) & 0xffu;
+            const uint32_t len = (hdr[hwords - 2u + (j >> 2)] >> (8u * (j & 3u))) & 0xffu;
             ok = len >= 1u && len <= kMaxCodedS;
             kraft += ok ? 1u << (kMaxCodedS - len) : 0u;
         }
@@ -100,7 +100,7 @@ __device__ __forceinline__ StreamHead read_head(const Geometry& G, const uint32_
     if (ok && levelset == kLevelsTable) {                   // the levels must increase strictly inside (0, 1)
         float below = 0.0f;
         for (uint32_t j = 0; j < G.s; ++j) {
-            const float l = __uint_as_float(__ldg(hdr + kHeaderWords + j));
+            const float l = __uint_as_float(hdr[kHeaderWords + j]);
             ok = ok && below < l;
             below = l;
         }
