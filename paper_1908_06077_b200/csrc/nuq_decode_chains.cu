@@ -706,6 +706,12 @@ __global__ void __launch_bounds__(32 * kChainMaxWarps, 1) decode_chains_kernel(c
         advance(unit2, group2);
         const Offsets next2 = load_offsets(unit2, 32u * group2);
         const uint32_t g0 = 32u * group, gcount = min(K - g0, 32u);
+        if (P.w != nullptr && group == 0u) {                // the parameters the add pass will read and write
+            const uint64_t first = unit * S * kSB, left = G.d - first;
+            const uint32_t bytes = 4u * ((left < S * kSB ? (uint32_t)left : S * kSB) & ~3u);
+            if (bytes && lane < (P.mu != 0.0f ? 2u : 1u))
+                asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"((lane == 0u ? P.w : P.yl) + first), "r"(bytes) : "memory");
+        }
         asm volatile("cp.async.wait_group 0;" ::: "memory");
 
         // ================= walk =================
