@@ -546,15 +546,12 @@ __device__ void lay_out_tile(const EncodeParams& P, TileMeta& m, Pending& pd, ui
     __syncwarp();
 }
 
-// Second half: find the place of the staged tile (its predecessors announced their sizes when they were
-// laid out, so the walk rarely waits), copy the image to the stream, clear the image.
-__device__ void flush_pending(const EncodeParams& P, Pending& pd, CtaTotals& tot, uint32_t* stg, uint64_t* tile_state,
-                              uint64_t* group_state, uint64_t* table, uint32_t* payload, uint32_t lane) {
+// Second half: copy the image of a staged tile to its place `off` in the stream, clear the image.
+__device__ void flush_pending(const EncodeParams& P, Pending& pd, CtaTotals& tot, uint32_t* stg, uint64_t off, bool failed,
+                              uint64_t* table, uint32_t* payload, uint32_t lane) {
     const Geometry& G = P.geo;
     const uint64_t tile = pd.tile;
     const uint32_t words = pd.words;
-    bool failed;
-    const uint64_t off = tile_lookback(P, tile_state, group_state, tile, words, &failed);
     for (uint32_t i = lane; i < words; i += 32) {
         if (!failed) payload[off + i] = stg[i];
         stg[i] = 0;
@@ -731,9 +728,13 @@ encode_kernel(const __grid_constant__ EncodeParams P) {
                 pair_arrive<kBarLayout>(p);
             }
             if (k >= 1) {
+                // the tile's place (its predecessors announced their sizes when they were laid out, so the walk rarely
+                // waits), while the workers move the last of its strings
+                Pending& pd = s_pend[p ^ 1u];
+                bool failed;
+                const uint64_t off = tile_lookback(P, tile_state, group_state, pd.tile, pd.words, &failed);
                 pair_sync<kBarMerged>(p ^ 1u);              // the strings of tile k - 1 are in its image
-                flush_pending(P, s_pend[p ^ 1u], s_tot, images + (p ^ 1u) * P.stage_words, tile_state, group_state, table,
-                              payload, lane);
+                flush_pending(P, pd, s_tot, images + (p ^ 1u) * P.stage_words, off, failed, table, payload, lane);
             }
             if (!have) break;
         }
