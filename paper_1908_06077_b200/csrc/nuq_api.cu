@@ -214,6 +214,7 @@ static int occupancy(const EncodeParams& P, int dev, bool clusters) {
     const Geometry& G = P.geo;
     const uint64_t key = (uint64_t)encode_smem_bytes(P) | (uint64_t)G.levelset << 32 | (uint64_t)G.mode << 34 |
                          (uint64_t)(fixed4_applies(G) ? 1 : 0) << 36 | (uint64_t)(G.bucket % (kBLK / kEncWarps) == 0 ? 1 : 0) << 37 |
+                         (uint64_t)(P.warps >> 3) << 42 |
                          (uint64_t)(clusters ? P.cluster : 0) << 38 | (uint64_t)(uint32_t)dev << 44;
     const auto it = known.find(key);
     if (it != known.end()) return it->second;
@@ -233,11 +234,15 @@ static EncodePlan plan_encode(EncodeParams& P, int dev, uint32_t flags) {
     P.patience = (flags & NUQ_TEST_SHORT_PATIENCE) ? 2u : 1u << 16;
     P.window_words = 0;
     P.stage_words = 0;
+    // A call that gives an SM two tiles at most (a tile's latency counts there, not the SM's throughput): twice the warps
+    // per tile.  65536 elements 11.0 -> 10.0 us, 10^6 elements 16.4 -> 12.7 us; from three tiles per SM on 8 warps are
+    // faster.  (Not in clusters, and the fixed-width encoders have no such variant.)
+    P.warps = G.mode != kModeFixed && G.bucket <= kBLK && G.ntiles <= 2u * (uint64_t)sms ? kEncMaxWarps : kEncWarps;
     if (G.mode != kModeFixed) {
         P.stage_words = (stage_words_for(G, norms_are_ours) + 3u) & ~3u;
-        // a warp's 1024 elements lie in at most this many buckets
-        const uint32_t warp_elems = kBLK / kEncWarps;
-        // (tiles start at bucket boundaries and a warp's part at a multiple of 1024 elements)
+        // a warp's elements lie in at most this many buckets
+        const uint32_t warp_elems = kBLK / P.warps;
+        // (tiles start at bucket boundaries and a warp's part at a multiple of its size)
         const uint32_t warp_buckets = G.bucket >= warp_elems ? (G.bucket % warp_elems == 0 ? 1u : 2u)
                                                              : (warp_elems % G.bucket == 0 ? warp_elems / G.bucket : warp_elems / G.bucket + 1u);
         P.window_words = (token_bits_bound(G, warp_elems, warp_buckets, norms_are_ours) + 31u) / 32u + 4u;
@@ -481,7 +486,7 @@ nuq_status nuq_level_histogram(const float* g, uint64_t d, uint32_t bucket, uint
         P.round_keys[2 * r] = (uint32_t)seed + r * 0x9E3779B9u;
         P.round_keys[2 * r + 1] = (uint32_t)(seed >> 32) + r * 0xBB67AE85u;
     }
-    P.stage_words = P.window_words = P.patience = P.grid = P.cluster = P.overlap = 0;
+    P.stage_words = P.window_words = P.patience = P.grid = P.cluster = P.overlap = P.warps = 0;
     if (cudaMemsetAsync(hist, 0, 8 * (s + 2), stream) != cudaSuccess) return NUQ_ERR_CUDA;
     if (launch_level_histogram(P, hist, device_sms(dev), stream) != cudaSuccess) return NUQ_ERR_CUDA;
     return NUQ_OK;

@@ -446,15 +446,13 @@ struct Sym {
     static constexpr uint32_t kMask = (1u << kBits) - 1u;
 };
 
-constexpr uint32_t kWarpElems = kBLK / kEncWarps;   // 1024 elements of a tile per warp (4 sub-blocks)
-
-// Named CTA barriers.  The 8 worker warps meet at kBarWork once per tile.  In the ERC mode the workers and the writer warp pass
+// Named CTA barriers.  The worker warps meet at kBarWork once per tile.  In the ERC mode the workers and the writer warp pass
 // a tile k from hand to hand through three barriers with index k & 1:
 //   kBarDone    the workers arrive when their strings of tile k are complete, the writer waits;
 //   kBarLayout  the writer arrives when it has laid the tile out, the workers wait (a tile later);
 //   kBarMerged  the workers arrive when they have moved their strings into the image, the writer waits.
 constexpr uint32_t kBarWork = 1, kBarDone = 2, kBarLayout = 4, kBarMerged = 6;
-constexpr uint32_t kEncAllThreads = kEncThreads + 32;      // ERC mode: workers + the writer warp
+__host__ __device__ constexpr uint32_t all_threads(uint32_t warps) { return 32u * (warps + 1u); }   // ERC mode: workers + the writer warp
 template <uint32_t ID, uint32_t COUNT>
 __device__ __forceinline__ void bar_sync() {
     asm volatile("bar.sync %0, %1;" ::"n"(ID), "n"(COUNT) : "memory");
@@ -465,15 +463,15 @@ __device__ __forceinline__ void bar_arrive() {
     asm volatile("bar.arrive %0, %1;" ::"n"(ID), "n"(COUNT) : "memory");
 }
 // the barrier BASE + p of tile parity p; immediate barrier numbers, so that the kernel claims only those it uses
-template <uint32_t BASE>
+template <uint32_t BASE, uint32_t COUNT>
 __device__ __forceinline__ void pair_sync(uint32_t p) {
-    if (p == 0) bar_sync<BASE, kEncAllThreads>();
-    else bar_sync<BASE + 1, kEncAllThreads>();
+    if (p == 0) bar_sync<BASE, COUNT>();
+    else bar_sync<BASE + 1, COUNT>();
 }
-template <uint32_t BASE>
+template <uint32_t BASE, uint32_t COUNT>
 __device__ __forceinline__ void pair_arrive(uint32_t p) {
-    if (p == 0) bar_arrive<BASE, kEncAllThreads>();
-    else bar_arrive<BASE + 1, kEncAllThreads>();
+    if (p == 0) bar_arrive<BASE, COUNT>();
+    else bar_arrive<BASE + 1, COUNT>();
 }
 
 // What the workers and the writer tell one another about a tile (ERC mode).
@@ -484,7 +482,7 @@ struct TileMeta {
     uint32_t sb_src[32];                                   // ... and where they start in the owning warp's window
     uint32_t blk_norm[32];                                 // norm word of each coding block of the tile
     uint32_t bitoff[32];                                   // written by the writer: where each sub-block's string goes in the image
-    uint32_t wnnz[kEncWarps];                              // nonzero symbols each warp produced
+    uint32_t wnnz[kEncMaxWarps];                           // nonzero symbols each warp produced
 };
 
 // A tile whose records are staged in shared memory and whose place in the stream is not
@@ -505,7 +503,7 @@ struct CtaTotals {
 // sub-block lengths (lane = sub-block), the block heads written into the (zeroed) image, the tile's
 // size announced to the tiles behind it, and what the second half needs noted in `pd`.
 __device__ void lay_out_tile(const EncodeParams& P, TileMeta& m, Pending& pd, uint32_t* stg, uint64_t* tile_state,
-                             uint64_t* group_state, uint32_t lane) {
+                             uint64_t* group_state, uint32_t warps, uint32_t lane) {
     const Geometry& G = P.geo;
     const bool narrow = G.bucket <= kBLK;
     const uint32_t spb = narrow ? G.sb_per_block : 32u;
@@ -534,7 +532,7 @@ __device__ void lay_out_tile(const EncodeParams& P, TileMeta& m, Pending& pd, ui
     if (lane < nsb && ((lane - sb0) & 1u) == 0)
         stg[blk_off + 1u + (lane - sb0) / 2u] = v | ((lane + 1u <= sb_last ? nv : 0u) << 16);
     pd.blk_wordoff[lane] = __shfl_sync(0xffffffffu, wexcl, (lane * spb) & 31u);
-    uint32_t nnz = lane < (uint32_t)kEncWarps ? m.wnnz[lane] : 0u;
+    uint32_t nnz = lane < warps ? m.wnnz[lane] : 0u;
     nnz = __reduce_add_sync(0xffffffffu, nnz);
     if (lane == 0) {
         pd.tile = m.tile;
@@ -573,11 +571,13 @@ __device__ void flush_pending(const EncodeParams& P, Pending& pd, CtaTotals& tot
 }
 
 // CLUSTERS: the call's buckets are wider than a tile and each is encoded by a thread-block cluster (see below).
-template <uint32_t LEVELSET, uint32_t MODE, bool CLUSTERS>
-__global__ void __launch_bounds__(MODE == kModeErc ? kEncAllThreads : kEncThreads, kEncMinBlocks)
+// W: worker warps, 8 as a rule.  Calls that give an SM two tiles at most take 16 (half the sub-blocks per warp): there a
+// tile's own latency is what counts.
+template <uint32_t LEVELSET, uint32_t MODE, bool CLUSTERS, uint32_t W>
+__global__ void __launch_bounds__(MODE == kModeErc ? all_threads(W) : 32u * W, W == 8u ? kEncMinBlocks : 2)
 encode_kernel(const __grid_constant__ EncodeParams P) {
     extern __shared__ __align__(128) uint32_t smem[];
-    __shared__ __align__(8) uint64_t s_full[kEncWarps];    // s_full[w] completes when warp w's part of a tile has landed
+    __shared__ __align__(8) uint64_t s_full[W];            // s_full[w] completes when warp w's part of a tile has landed
     __shared__ uint32_t s_lut[256];                        // ERC(N), N = 1..256: code left aligned | length
     __shared__ uint32_t s_index[260];                      // level index: a bit for the sign, then its word, left aligned | length; 0: 0
     __shared__ uint2 s_body[256];                          // EmitTables
@@ -600,12 +600,13 @@ encode_kernel(const __grid_constant__ EncodeParams P) {
     __shared__ unsigned long long s_bucket[4];             // buckets of the iterations to come, handed out by the cluster's first CTA
 
     using S = Sym<LEVELSET>;
+    constexpr uint32_t kAll = all_threads(W), kWarpElems = kBLK / W, kQ = kWarpElems / kSB;   // elements and sub-blocks of a tile per warp
     const Geometry& G = P.geo;
     const uint32_t tid = threadIdx.x, lane = tid & 31u;
     const uint32_t warp = __shfl_sync(0xffffffffu, tid >> 5, 0);      // (the same in all lanes, and known to be)
     float* const data = reinterpret_cast<float*>(smem);                         // kBLK floats: the tile
     uint32_t* const images = smem + kBLK;                                       // [2][stage_words]: staged tile records
-    uint32_t* const windows = images + 2u * P.stage_words;                      // [2][kEncWarps][window_words]: token strings
+    uint32_t* const windows = images + 2u * P.stage_words;                      // [2][W][window_words]: token strings
     uint64_t* tile_state = reinterpret_cast<uint64_t*>(P.ws + 1);
     uint64_t* group_state = tile_state + G.ntiles;
     uint64_t* table = reinterpret_cast<uint64_t*>(P.out + G.header_words);
@@ -615,7 +616,7 @@ encode_kernel(const __grid_constant__ EncodeParams P) {
     const float top = LEVELSET == kLevelsTable ? 1.0f : __uint_as_float((127u + G.s) << 23);   // the norm is divided into this
     const uint32_t c2 = (uint32_t)P.offset, c3 = (uint32_t)(P.offset >> 32);
     const bool narrow = G.bucket <= kBLK;
-    const bool coarse = G.bucket % kWarpElems == 0;         // a warp's four sub-blocks always share one bucket
+    const bool coarse = G.bucket % kWarpElems == 0;         // a warp's sub-blocks always share one bucket
     const uint32_t spb = narrow ? G.sb_per_block : 32u;     // sub-blocks per coding block
 
     // Clusters: a bucket wider than a tile is encoded by a cluster of as many CTAs as it has tiles, CTA r
@@ -659,7 +660,7 @@ encode_kernel(const __grid_constant__ EncodeParams P) {
     };
 
     let_next_kernel_start(P);
-    if (warp < (uint32_t)kEncWarps && lane == 0) prefetch_first_tile(P, warp);
+    if (warp < W && lane == 0) prefetch_first_tile(P, wbase, kWarpElems);
     if (tid < 256u) {
         const uint32_t e = c_erc_lut[tid], elen = e >> 16;  // at most 16 bits
         s_lut[tid] = ((e & 0xffffu) << (32u - elen)) | elen;
@@ -684,10 +685,10 @@ encode_kernel(const __grid_constant__ EncodeParams P) {
         s_invw[tid] = P.inv_width[tid];
     }
     if (MODE == kModeErc)
-        for (uint32_t i = tid; i < 2u * P.stage_words + 2u * kEncWarps * P.window_words; i += blockDim.x) images[i] = 0;
+        for (uint32_t i = tid; i < 2u * P.stage_words + 2u * W * P.window_words; i += blockDim.x) images[i] = 0;
     wait_for_previous_kernel(P);                            // nothing above reads or writes global memory (tables apart, which never change)
     if (tid == 0) {
-        for (int w = 0; w < kEncWarps; ++w) mbar_init(&s_full[w], 1);
+        for (uint32_t w = 0; w < W; ++w) mbar_init(&s_full[w], 1);
         s_nnz = 0;
         s_arrived = 0;
         s_tot.nnz = 0;
@@ -712,20 +713,20 @@ encode_kernel(const __grid_constant__ EncodeParams P) {
         if (tid == 0) take_ticket(0);
         __syncthreads();
     }
-    if (warp < (uint32_t)kEncWarps && lane == 0) start_copy(0);
+    if (warp < W && lane == 0) start_copy(0);
     if (tid == 0) take_ticket(1);                           // its round trip runs while the first bytes arrive
 
-    const bool writer = MODE == kModeErc && warp == (uint32_t)kEncWarps;
+    const bool writer = MODE == kModeErc && warp == W;
     if (writer) {
         // ---- the writer warp: lays out every tile the workers have encoded, and a tile later, when they
         // have moved their strings into the image, finds the tile's place in the stream and copies it out
         for (uint32_t k = 0;; ++k) {
             const uint32_t p = k & 1u;
-            pair_sync<kBarDone>(p);                         // the workers' strings of tile k are complete (or there is no tile k)
+            pair_sync<kBarDone, kAll>(p);                         // the workers' strings of tile k are complete (or there is no tile k)
             const bool have = k < *reinterpret_cast<volatile uint32_t*>(&s_tot.stop);
             if (have) {
-                lay_out_tile(P, s_meta[p], s_pend[p], images + p * P.stage_words, tile_state, group_state, lane);
-                pair_arrive<kBarLayout>(p);
+                lay_out_tile(P, s_meta[p], s_pend[p], images + p * P.stage_words, tile_state, group_state, W, lane);
+                pair_arrive<kBarLayout, kAll>(p);
             }
             if (k >= 1) {
                 // the tile's place (its predecessors announced their sizes when they were laid out, so the walk rarely
@@ -733,7 +734,7 @@ encode_kernel(const __grid_constant__ EncodeParams P) {
                 Pending& pd = s_pend[p ^ 1u];
                 bool failed;
                 const uint64_t off = tile_lookback(P, tile_state, group_state, pd.tile, pd.words, &failed);
-                pair_sync<kBarMerged>(p ^ 1u);              // the strings of tile k - 1 are in its image
+                pair_sync<kBarMerged, kAll>(p ^ 1u);              // the strings of tile k - 1 are in its image
                 flush_pending(P, pd, s_tot, images + (p ^ 1u) * P.stage_words, off, failed, table, payload, lane);
             }
             if (!have) break;
@@ -744,15 +745,15 @@ encode_kernel(const __grid_constant__ EncodeParams P) {
     // the image once the writer has laid the tile out ----
     auto merge_tile = [&](uint32_t k, uint32_t bits) {
         const uint32_t p = k & 1u;
-        pair_sync<kBarLayout>(p);
+        pair_sync<kBarLayout, kAll>(p);
         const TileMeta& m = s_meta[p];
         uint32_t* stg = images + p * P.stage_words;
-        uint32_t* win = windows + (p * kEncWarps + warp) * P.window_words;
+        uint32_t* win = windows + (p * W + warp) * P.window_words;
 #pragma unroll 1
-        for (uint32_t q = 0; q < 4; q += coarse ? 4u : 1u) {
+        for (uint32_t q = 0; q < kQ; q += coarse ? kQ : 1u) {
             // the strings of sub-blocks of one block follow one another in the window and in the
-            // tile alike, so a warp whose four sub-blocks share a block moves them in one piece
-            const uint32_t sbq = warp * 4u + q;
+            // tile alike, so a warp whose sub-blocks share a block moves them in one piece
+            const uint32_t sbq = warp * kQ + q;
             if (sbq >= m.nsb) break;
             const uint32_t len = coarse ? bits : m.sb_bits[sbq], src = coarse ? 0u : m.sb_src[sbq];
             const uint32_t dst = m.bitoff[sbq];
@@ -772,7 +773,7 @@ encode_kernel(const __grid_constant__ EncodeParams P) {
         __syncwarp();
         for (uint32_t i = lane; i < (bits + 31u) / 32u + 2u; i += 32) win[i] = 0;   // ready for tile k + 2
         __syncwarp();
-        pair_arrive<kBarMerged>(p);                        // the writer may take the tile
+        pair_arrive<kBarMerged, kAll>(p);                        // the writer may take the tile
     };
 
     uint32_t it = 0;
@@ -813,9 +814,9 @@ encode_kernel(const __grid_constant__ EncodeParams P) {
         // few 1e-8 of the exactly rounded one.  Linf: max |x|, exact. ----
         if (P.norms_in == nullptr) {
             if (G.norm_kind == kNormL2) {
-                float p8[4];
+                float p8[kQ];
 #pragma unroll
-                for (int q = 0; q < 4; ++q) {
+                for (uint32_t q = 0; q < kQ; ++q) {
                     const float4 x = rows[32 * (2 * q)], y = rows[32 * (2 * q + 1)];
                     float a = __fmul_rn(x.x, x.x), b = __fmul_rn(x.y, x.y);
                     a = __fmaf_rn(x.z, x.z, a); b = __fmaf_rn(x.w, x.w, b);
@@ -826,13 +827,19 @@ encode_kernel(const __grid_constant__ EncodeParams P) {
                 // squares that leave the fp32 range (tiny or huge coordinates, NaN): the warp adds that sub-block up in
                 // fp64 instead
                 auto out_of_range = [](float p) { return !(p >= 0x1p-60f && p < 0x1p120f); };
-                double e8[4];
+                double e8[kQ];
+                bool out = false;
 #pragma unroll
-                for (int q = 0; q < 4; ++q) e8[q] = (double)p8[q];
-                if (__any_sync(0xffffffffu, out_of_range(p8[0]) || out_of_range(p8[1]) || out_of_range(p8[2]) || out_of_range(p8[3]))) {
+                for (uint32_t q = 0; q < kQ; ++q) {
+                    e8[q] = (double)p8[q];
+                    out = out || out_of_range(p8[q]);
+                }
+                if (__any_sync(0xffffffffu, out)) {
 #pragma unroll 1
-                    for (int q = 0; q < 4; ++q) {
-                        const float p = q == 0 ? p8[0] : q == 1 ? p8[1] : q == 2 ? p8[2] : p8[3];
+                    for (uint32_t q = 0; q < kQ; ++q) {
+                        float p = p8[0];
+#pragma unroll
+                        for (uint32_t k = 1; k < kQ; ++k) p = q == k ? p8[k] : p;
                         if (!__any_sync(0xffffffffu, out_of_range(p))) continue;
                         const float4 x = rows[32 * (2 * q)], y = rows[32 * (2 * q + 1)];
                         double e = 0.0;
@@ -840,7 +847,8 @@ encode_kernel(const __grid_constant__ EncodeParams P) {
                         e = fma((double)x.z, (double)x.z, e); e = fma((double)x.w, (double)x.w, e);
                         e = fma((double)y.x, (double)y.x, e); e = fma((double)y.y, (double)y.y, e);
                         e = fma((double)y.z, (double)y.z, e); e = fma((double)y.w, (double)y.w, e);
-                        if (q == 0) e8[0] = e; else if (q == 1) e8[1] = e; else if (q == 2) e8[2] = e; else e8[3] = e;
+#pragma unroll
+                        for (uint32_t k = 0; k < kQ; ++k) e8[k] = q == k ? e : e8[k];
                     }
                 }
                 auto warp_sum = [&](double acc) {
@@ -849,27 +857,30 @@ encode_kernel(const __grid_constant__ EncodeParams P) {
                     return acc;
                 };
                 if (coarse) {                               // one partial per warp, or one per sub-block
-                    const double acc = warp_sum(((e8[0] + e8[1]) + e8[2]) + e8[3]);
-                    if (lane == 0) s_partial[warp * 4 + 3] = acc;
+                    double acc = e8[0];
+#pragma unroll
+                    for (uint32_t q = 1; q < kQ; ++q) acc += e8[q];
+                    acc = warp_sum(acc);
+                    if (lane == 0) s_partial[warp * kQ + kQ - 1u] = acc;
                 } else {
 #pragma unroll
-                    for (int q = 0; q < 4; ++q) {
+                    for (uint32_t q = 0; q < kQ; ++q) {
                         const double acc = warp_sum(e8[q]);
-                        if (lane == 0) s_partial[warp * 4 + q] = acc;
+                        if (lane == 0) s_partial[warp * kQ + q] = acc;
                     }
                 }
             } else {
                 uint32_t mx = 0;
 #pragma unroll
-                for (int q = 0; q < 4; ++q) {               // on the bit patterns: NaN sorts above inf
+                for (uint32_t q = 0; q < kQ; ++q) {         // on the bit patterns: NaN sorts above inf
                     const float4 x = rows[32 * (2 * q)], y = rows[32 * (2 * q + 1)];
                     mx = max(max(mx, __float_as_uint(fabsf(x.x))), __float_as_uint(fabsf(x.y)));
                     mx = max(max(mx, __float_as_uint(fabsf(x.z))), __float_as_uint(fabsf(x.w)));
                     mx = max(max(mx, __float_as_uint(fabsf(y.x))), __float_as_uint(fabsf(y.y)));
                     mx = max(max(mx, __float_as_uint(fabsf(y.z))), __float_as_uint(fabsf(y.w)));
-                    if (!coarse || q == 3) {
+                    if (!coarse || q == kQ - 1u) {
                         mx = __reduce_max_sync(0xffffffffu, mx);
-                        if (lane == 0) s_maxbits[warp * 4 + q] = mx;
+                        if (lane == 0) s_maxbits[warp * kQ + q] = mx;
                         mx = 0;
                     }
                 }
@@ -888,7 +899,7 @@ encode_kernel(const __grid_constant__ EncodeParams P) {
             __syncwarp();
             if (lane == 0) {
                 __threadfence_block();
-                last = (atomicAdd(&s_arrived, 1u) & (kEncWarps - 1u)) == kEncWarps - 1u;
+                last = (atomicAdd(&s_arrived, 1u) & (W - 1u)) == W - 1u;
             }
             if (__shfl_sync(0xffffffffu, last, 0)) {
                 __threadfence_block();
@@ -903,7 +914,7 @@ encode_kernel(const __grid_constant__ EncodeParams P) {
                     // maximum) to all of them, and all add the parts up in the same order
                     double a = 0.0;
                     uint32_t mxb = 0;
-                    for (uint32_t j = 3u; j < 32u; j += 4u) {       // one partial per warp
+                    for (uint32_t j = kQ - 1u; j < 32u; j += kQ) {       // one partial per warp
                         a += s_partial[j];
                         mxb = max(mxb, s_maxbits[j]);
                     }
@@ -928,12 +939,12 @@ encode_kernel(const __grid_constant__ EncodeParams P) {
                     }
                 } else if (G.norm_kind == kNormL2) {
                     double a = 0.0;
-                    if (coarse) for (uint32_t j = sb0 + 3u; j < sb0 + spb; j += 4u) a += s_partial[j];     // one partial per warp
+                    if (coarse) for (uint32_t j = sb0 + kQ - 1u; j < sb0 + spb; j += kQ) a += s_partial[j];     // one partial per warp
                     else for (uint32_t j = sb0; j < sb0 + spb; ++j) a += s_partial[j];
                     norm = (float)sqrt(a);
                 } else {
                     uint32_t mxb = 0;
-                    if (coarse) for (uint32_t j = sb0 + 3u; j < sb0 + spb; j += 4u) mxb = max(mxb, s_maxbits[j]);
+                    if (coarse) for (uint32_t j = sb0 + kQ - 1u; j < sb0 + spb; j += kQ) mxb = max(mxb, s_maxbits[j]);
                     else for (uint32_t j = sb0; j < sb0 + spb; ++j) mxb = max(mxb, s_maxbits[j]);
                     norm = __uint_as_float(mxb);
                 }
@@ -951,14 +962,14 @@ encode_kernel(const __grid_constant__ EncodeParams P) {
                 if (MODE == kModeErc && lane == sb0 && lane < nsb_tile) s_meta[it & 1u].blk_norm[bi] = __float_as_uint(norm);
             }
         }
-        bar_sync<kBarWork, kEncThreads>();                    // the one barrier of a tile: norms visible,
+        bar_sync<kBarWork, 32u * W>();                        // the one barrier of a tile: norms visible,
                                                             // and every warp is done with the previous tile
         // the ticket of the tile after the next is taken now: its round trip ends long before anyone looks
         if (tid == 0) take_ticket(it + 2u);
         if (cl > 1u && tid == 0 && crank == 0) hand_out_bucket(it + 3u);   // seen by the others after the next exchange of norms
 
         TileMeta* const meta = &s_meta[it & 1u];
-        uint32_t* const window = windows + ((it & 1u) * kEncWarps + warp) * P.window_words;   // this warp's token string
+        uint32_t* const window = windows + ((it & 1u) * W + warp) * P.window_words;   // this warp's token string
         // ---- quantize (Definition 1) and emit, one sub-block (two 128-element rows) at a time ----
         uint32_t bits = 0;                                  // ERC: bits in this warp's window so far
         uint32_t cum = 0;                                   // ERC: nonzero symbols of this lane so far
@@ -967,8 +978,8 @@ encode_kernel(const __grid_constant__ EncodeParams P) {
         uint32_t* fx_rec = nullptr;
         uint32_t fx_sb = 0, fx_words = 0;                   // sub-block within its record, valid field words of the record
 #pragma unroll 1
-        for (uint32_t q = 0; q < 4; ++q) {
-            const uint32_t sbq = warp * 4u + q;
+        for (uint32_t q = 0; q < kQ; ++q) {
+            const uint32_t sbq = warp * kQ + q;
             if (MODE == kModeErc && lane >= q) string_start = bits;
             if (sbq >= nsb_tile) continue;
             const float inv = s_sb_inv[sbq];
@@ -1089,7 +1100,7 @@ encode_kernel(const __grid_constant__ EncodeParams P) {
             } else if (MODE == kModeFixed) {
                 for (uint32_t i = lane; i < fx_valid; i += 32) fx_dst[i] = 0;      // a bucket that is not quantized: all fields zero
             }
-            if (q < 3u) {                                   // the draws of the next sub-block
+            if (q + 1u < kQ) {                              // the draws of the next sub-block
                 const uint64_t ctr0 = ctr_warp + 64u * (q + 1u), ctr1 = ctr0 + kNextBlock;
                 rn0 = philox4x32_10((uint32_t)ctr0, (uint32_t)(ctr0 >> 32), c2, c3, P.round_keys);
                 rn1 = philox4x32_10((uint32_t)ctr1, (uint32_t)(ctr1 >> 32), c2, c3, P.round_keys);
@@ -1103,9 +1114,9 @@ encode_kernel(const __grid_constant__ EncodeParams P) {
         if (MODE == kModeErc) {
             cum = __reduce_add_sync(0xffffffffu, cum);
             const uint32_t next_start = __shfl_down_sync(0xffffffffu, string_start, 1);
-            if (lane < 4u) {                                // lane q: sub-block q of the warp
-                meta->sb_bits[warp * 4u + lane] = (lane < 3u ? next_start : bits) - string_start;
-                meta->sb_src[warp * 4u + lane] = string_start;
+            if (lane < kQ) {                                // lane q: sub-block q of the warp
+                meta->sb_bits[warp * kQ + lane] = (lane < kQ - 1u ? next_start : bits) - string_start;
+                meta->sb_src[warp * kQ + lane] = string_start;
             }
             if (lane == 0) {
                 meta->wnnz[warp] = cum;
@@ -1115,7 +1126,7 @@ encode_kernel(const __grid_constant__ EncodeParams P) {
                 }
             }
             __syncwarp();
-            pair_arrive<kBarDone>(it & 1u);                 // the writer may lay the tile out
+            pair_arrive<kBarDone, kAll>(it & 1u);                 // the writer may lay the tile out
             if (it > 0) merge_tile(it - 1u, prev_bits);     // the tile before it has been laid out long ago
             prev_bits = bits;
         }
@@ -1125,7 +1136,7 @@ encode_kernel(const __grid_constant__ EncodeParams P) {
         // ---- the workers ran `it` iterations: tell the writer that no further tile comes, and move the
         // last tile's strings into its image ----
         if (tid == 0) s_tot.stop = it;
-        pair_arrive<kBarDone>(it & 1u);
+        pair_arrive<kBarDone, kAll>(it & 1u);
         if (it > 0) merge_tile(it - 1u, prev_bits);
     }
     if (MODE == kModeFixed) {
@@ -1263,7 +1274,7 @@ cudaError_t launch_level_histogram(const EncodeParams& P, uint64_t* hist, int sm
 size_t encode_smem_bytes(const EncodeParams& P) {
     if (fixed4_applies(P.geo)) return 0;                    // that kernel's tile buffer is static
     size_t words = kBLK;
-    if (P.geo.mode != kModeFixed) words += 2u * (size_t)P.stage_words + 2u * (size_t)kEncWarps * P.window_words;
+    if (P.geo.mode != kModeFixed) words += 2u * (size_t)P.stage_words + 2u * (size_t)P.warps * P.window_words;
     return 4u * words;
 }
 
@@ -1273,21 +1284,27 @@ template <uint32_t L, uint32_t M>
 static cudaError_t prepare_kernel() {
     static bool attr_set = false;
     if (attr_set) return cudaSuccess;
-    cudaError_t e = cudaFuncSetAttribute(encode_kernel<L, M, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kEncMaxDynSmem);
+    cudaError_t e = cudaFuncSetAttribute(encode_kernel<L, M, false, 8>, cudaFuncAttributeMaxDynamicSharedMemorySize, kEncMaxDynSmem);
     if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(encode_kernel<L, M, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kEncMaxDynSmem);
+        e = cudaFuncSetAttribute(encode_kernel<L, M, true, 8>, cudaFuncAttributeMaxDynamicSharedMemorySize, kEncMaxDynSmem);
+    if (M == kModeErc && e == cudaSuccess)
+        e = cudaFuncSetAttribute(encode_kernel<L, kModeErc, false, kEncMaxWarps>, cudaFuncAttributeMaxDynamicSharedMemorySize, kEncMaxDynSmem);
     if (e == cudaSuccess) attr_set = true;
     return e;
 }
+
+template <uint32_t M>
+static int threads_of(const EncodeParams& P) { return M == kModeErc ? (int)all_threads(P.warps) : 32 * (int)P.warps; }
 
 template <uint32_t L, uint32_t M>
 static int blocks_per_sm(const EncodeParams& P) {
     if (prepare_kernel<L, M>() != cudaSuccess) return 0;
     int n = 0;
-    const int threads = M == kModeErc ? (int)kEncAllThreads : kEncThreads;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, encode_kernel<L, M, false>, threads, encode_smem_bytes(P)) != cudaSuccess)
-        return 0;
-    return n;
+    const size_t smem = encode_smem_bytes(P);
+    const cudaError_t e = M == kModeErc && P.warps == (uint32_t)kEncMaxWarps
+        ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, encode_kernel<L, kModeErc, false, kEncMaxWarps>, threads_of<M>(P), smem)
+        : cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, encode_kernel<L, M, false, 8>, threads_of<M>(P), smem);
+    return e == cudaSuccess ? n : 0;
 }
 
 int encode_blocks_per_sm(const EncodeParams& P) {
@@ -1310,7 +1327,7 @@ template <uint32_t M>
 static void fill_launch(EncodeLaunch* L, const EncodeParams& P, unsigned grid, cudaStream_t stream) {
     L->cfg = cudaLaunchConfig_t{};
     L->cfg.gridDim = dim3(grid);
-    L->cfg.blockDim = dim3(M == kModeErc ? kEncAllThreads : (uint32_t)kEncThreads);
+    L->cfg.blockDim = dim3((unsigned)threads_of<M>(P));
     L->cfg.dynamicSmemBytes = encode_smem_bytes(P);
     L->cfg.stream = stream;
     L->cfg.attrs = L->attr;
@@ -1337,8 +1354,10 @@ static cudaError_t launch_one(const EncodeParams& P, cudaStream_t stream) {
     if (smem > (size_t)kEncMaxDynSmem || P.grid == 0 || (P.cluster > 1u && P.grid % P.cluster != 0)) return cudaErrorInvalidValue;
     EncodeLaunch cfg;
     fill_launch<M>(&cfg, P, P.grid, stream);
-    if (P.cluster > 1u) return cudaLaunchKernelEx(&cfg.cfg, encode_kernel<L, M, true>, P);
-    return cudaLaunchKernelEx(&cfg.cfg, encode_kernel<L, M, false>, P);
+    if (P.cluster > 1u) return cudaLaunchKernelEx(&cfg.cfg, encode_kernel<L, M, true, 8>, P);
+    if (M == kModeErc && P.warps == (uint32_t)kEncMaxWarps)
+        return cudaLaunchKernelEx(&cfg.cfg, encode_kernel<L, kModeErc, false, kEncMaxWarps>, P);
+    return cudaLaunchKernelEx(&cfg.cfg, encode_kernel<L, M, false, 8>, P);
 }
 
 // clusters of P.cluster CTAs the device holds at once (0 on error)
@@ -1348,7 +1367,7 @@ static int max_clusters(const EncodeParams& P) {
     EncodeLaunch cfg;
     fill_launch<M>(&cfg, P, P.cluster, nullptr);
     int n = 0;
-    if (cudaOccupancyMaxActiveClusters(&n, encode_kernel<L, M, true>, &cfg.cfg) != cudaSuccess) {
+    if (cudaOccupancyMaxActiveClusters(&n, encode_kernel<L, M, true, 8>, &cfg.cfg) != cudaSuccess) {
         cudaGetLastError();
         return 0;
     }

@@ -173,16 +173,16 @@ __device__ __forceinline__ void describe_tile(const Geometry& G, unsigned long l
 __device__ __forceinline__ void let_next_kernel_start(const EncodeParams& P) {
     if (P.overlap) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }
-// The bytes of the tile a CTA is likely to get first (that of its own number) are asked into the L2 ahead of the wait, while
+// The warp's bytes (`elems` elements from `first` on) of the tile a CTA is likely to get first (that of its own number) are asked into the L2 ahead of the wait, while
 // the kernel in front drains: all CTAs together would otherwise start with 19 MB from HBM at once.  A prefetch changes
 // nothing that anyone can see: the L2 is where all writes meet, so what is copied to shared memory later is what
 // the kernel in front has written.
-__device__ __forceinline__ void prefetch_first_tile(const EncodeParams& P, uint32_t warp) {
+__device__ __forceinline__ void prefetch_first_tile(const EncodeParams& P, uint32_t first, uint32_t elems) {
     const Geometry& G = P.geo;
     if (!P.overlap || blockIdx.x >= G.ntiles) return;
-    const uint64_t at = (uint64_t)blockIdx.x * G.tile_elems + warp * (kBLK / kEncWarps);
-    if (at + kBLK / kEncWarps <= G.d)
-        asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(P.g + at), "r"((uint32_t)(4u * kBLK / kEncWarps)) : "memory");
+    const uint64_t at = (uint64_t)blockIdx.x * G.tile_elems + first;
+    if (at + elems <= G.d)
+        asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(P.g + at), "r"(4u * elems) : "memory");
 }
 __device__ __forceinline__ void wait_for_previous_kernel(const EncodeParams& P) {
     if (P.overlap) asm volatile("griddepcontrol.wait;" ::: "memory");

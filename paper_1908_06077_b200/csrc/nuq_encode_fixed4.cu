@@ -80,7 +80,7 @@ __global__ void __launch_bounds__(kEncThreads, kEncMinBlocks) encode_fixed4_kern
     };
 
     let_next_kernel_start(P);
-    if (lane == 0) prefetch_first_tile(P, warp);
+    if (lane == 0) prefetch_first_tile(P, wbase, kFx4WarpElems);
     wait_for_previous_kernel(P);                            // (this kernel has next to no set-up to do meanwhile)
     if (tid == 0) {
         for (int w = 0; w < kEncWarps; ++w) mbar_init(&s_full[w], 1);
