@@ -1,6 +1,6 @@
 // C ABI of the library (see include/nuq.h): argument validation, geometry,
 // per-stream workspace, kernel launches.  No torch types, no CPU fallback: every
-// step of the path runs in the kernels of nuq_encode.cu / nuq_decode.cu.
+// step of the path runs in the kernels of nuq_encode.cu / nuq_decode_chains.cu.
 #include <map>
 #include <mutex>
 #include <set>
@@ -26,7 +26,6 @@ struct WsEntry {
     // (0: none).  The allocation is zeroed and every encode kernel leaves its scan state zeroed, but the bucket
     // norms of a wide-bucket call or of a histogram call stay behind, at a place that depends on that call's size.
     size_t dirty_to = 0;
-    uint32_t dec_epoch = 0;  // fixed-width decode calls made on this workspace (see DecodeParams::epoch)
 };
 
 // One mutex guards the host-side bookkeeping below (maps, tables); it is held for the microseconds a
@@ -573,13 +572,11 @@ static nuq_status enqueue_decode(const void* const* streams, uint32_t K, uint64_
         g_token_tables_ready.insert(dev);
     }
     P.unit_subs = 0;                                    // (chosen at the launch)
-    P.after_fixed = w ? 0u : 1u;                        // all streams believed to be in the fixed-width mode? (sums only)
     P.likely_table = kTabErc;
     for (uint32_t k = 0; k < K; ++k) {
         auto it = g_container_mode.find(std::make_pair(dev, streams[k]));
         const uint32_t mode = it == g_container_mode.end() ? kModeErc : it->second & 0xffu;
-        if (mode != kModeFixed) P.after_fixed = 0;
-        if (mode == kModeCoded) P.likely_table = kTabCoded;
+        if (mode != kModeErc) P.likely_table = kTabCoded;
         else if (k == 0 && it != g_container_mode.end() && it->second >> 8 == kLevelsUniform) P.likely_table = kTabUniform;
     }
     P.acc = acc;
@@ -588,16 +585,11 @@ static nuq_status enqueue_decode(const void* const* streams, uint32_t K, uint64_
     P.step_c = w ? (float)((double)alpha / (double)K) : 0.0f;          // one rounding each
     P.step_lc = w ? (float)((double)l * (double)alpha / (double)K) : 0.0f;
     P.mu = w ? mu : 0.0f;
-    P.pad2 = 0;
+    P.minus_zero = -0.0f;
     Workspace* ws = nullptr;
     nuq_status st = get_workspace(stream, sizeof(Workspace), &ws, &dev);
     if (st != NUQ_OK) return st;
     P.ws = ws;
-    // The ticket counter a fixed-width decode call uses has been zeroed by the one before it (or by the allocation, or
-    // by an encode call, which leaves both zeroed): such calls take the two counters in turn and each zeroes the other one.
-    WsEntry& entry = g_ws[std::make_pair(dev, stream)];
-    if (P.after_fixed && ++entry.dec_epoch == 0) entry.dec_epoch = 2;       // never 0, parity kept
-    P.epoch = entry.dec_epoch;
     P.let_next = 0;                                     // (chosen at the launch, like unit_subs)
     if (launch_decode(P, device_sms(dev), stream) != cudaSuccess) return NUQ_ERR_CUDA;
     return NUQ_OK;

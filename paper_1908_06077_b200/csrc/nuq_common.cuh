@@ -37,14 +37,13 @@ constexpr uint64_t kTileValueMask = (1ull << 62) - 1;
 // per-stream scratch owned by the library
 struct Workspace {
     int status;             // latched kernel status; survives calls until nuq_last_status reads it
-    uint32_t dec_done_epoch; // decoder: the call (DecodeParams::epoch) whose fixed-width kernel did all the work
+    int pad;
     // everything below is cleared at the start of every encode call
     uint64_t ticket;        // next tile to hand out
     uint64_t done;          // CTAs that have finished (they take no further ticket)
     uint64_t code_bits;     // token bits of the whole call
     uint64_t nnz;           // nonzero symbols of the whole call
     uint64_t total_words;   // payload words of the whole call
-    uint64_t dec_ticket[2]; // decoder: next unit to hand out; a call uses the counter of its epoch's parity and zeroes the other one
     // followed by: uint64_t tile_state[ntiles], group_state[ceil(ntiles / 32)], then float norms[nb] for wide buckets
 };
 constexpr size_t kWorkspaceClearFrom = 8;
@@ -98,16 +97,14 @@ struct DecodeParams {
     const uint32_t* streams[kMaxK];
     uint32_t K;
     uint32_t unit_subs;      // token streams: sub-blocks a warp decodes at a time
-    uint32_t likely_table;   // the token table the call most likely needs (kTabErc, kTabUniform), or kTabCoded: none to prepare
-    uint32_t after_fixed;    // the fixed-width kernel runs first; the general kernel returns if it did the work
-    uint32_t epoch;          // number of this decode call on its workspace (never 0)
+    uint32_t likely_table;   // the token table the call most likely needs (kTabErc, kTabUniform), or kTabCoded: none to prepare (a level code of the streams' own, or no tokens)
     uint32_t let_next;       // token streams: the kernel behind may be launched early
-    // the aggregation step fused into the decoder (w == nullptr: none): see step_value in nuq_decode.cu
+    // the aggregation step fused into the decoder (w == nullptr: none): see step_value in nuq_decode_common.cuh
     float* w;                // parameters, updated in place
     float* yl;               // the momentum rule's y^l, updated in place (not touched when mu == 0)
     float step_c, step_lc;   // alpha / K and l alpha / K
     float mu;
-    uint32_t pad2;
+    float minus_zero;        // -0.0f, which the compiler must not know (see product2 in nuq_decode_common.cuh)
     float* acc;
     Workspace* ws;
 };

@@ -32,6 +32,7 @@
 // are on their way during the walk.  16 warps fit an SM (12 KB each: rows, chain copies).
 #include "nuq_async.cuh"
 #include "nuq_decode_common.cuh"
+#include "nuq_decode_fields.cuh"
 #include "nuq_launch.h"
 
 namespace nuq {
@@ -41,7 +42,8 @@ constexpr uint32_t kTokEntries = 1u << kTokBits;
 constexpr uint32_t kChainMaxWarps = 16;                 // warps per CTA, one CTA per SM
 constexpr uint32_t kChunkWords = 28;                    // words of its chain a lane holds at a time
 constexpr uint32_t kChunkSlack = 3;                     // of these, words it needs behind the chain's last one
-constexpr uint32_t kStreamTabBytes = 256 + 64;          // per stream: level code by 7-bit prefix, level table
+constexpr uint32_t kCodeBytes = 256;                    // per stream: level code by 7-bit prefix, or level by symbol
+constexpr uint32_t kLevelBytes = 64;                    // per stream: level table
 constexpr size_t kChainSmem = 227u * 1024u - 512u;      // (512 bytes: static)
 
 // A row of symbols: 256 positions and a place for what a malformed chain would write behind them.  Rows of
@@ -50,6 +52,7 @@ template <class Sym>
 struct Row {
     static constexpr uint32_t kPitch = kSB * sizeof(Sym) + 4u;
     static constexpr uint32_t kWarpBytes = 32u * kPitch + 128u + 32u * 4u * kChunkWords;   // rows, norms, chain copies
+    static_assert(kWarpBytes >= field_warp_bytes(5) && kWarpBytes >= field_warp_bytes(10), "fixed-width streams use the same memory");
 };
 
 // Token table entries.  Bits 0-4: bits consumed (0: not resolved here); bits 8-15: gap; bits 22-31: symbol, signed
@@ -264,32 +267,6 @@ __device__ __noinline__ uint32_t walk_rare(uint32_t copy, uint32_t from, uint32_
     return walk_body<Sym, LONG, GAPS>(copy, from, bits, tab, row, row_end, hd, code, s, good);
 }
 
-__device__ __forceinline__ uint64_t pack2(float a, float b) {
-    uint64_t r;
-    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
-    return r;
-}
-__device__ __forceinline__ float2 unpack2(uint64_t v) {
-    float2 r;
-    asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(v));
-    return r;
-}
-// two fp32 operations at once, each rounded like the single one
-__device__ __forceinline__ uint64_t fma2(uint64_t a, uint64_t b, uint64_t c) {
-    uint64_t r;
-    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
-    return r;
-}
-__device__ __forceinline__ uint64_t mul2(uint64_t a, uint64_t b) {
-    uint64_t r;
-    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
-    return r;
-}
-__device__ __forceinline__ uint64_t add2(uint64_t a, uint64_t b) {
-    uint64_t r;
-    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
-    return r;
-}
 // two fp16 numbers given by their upper bytes, in the upper bytes of the halves
 __device__ __forceinline__ uint64_t halves(uint32_t h) {
     uint64_t r;
@@ -297,64 +274,34 @@ __device__ __forceinline__ uint64_t halves(uint32_t h) {
     return r;
 }
 
-// Four symbols of one stream as level values: a pair each.
-template <class Sym, bool UNIFORM>
-__device__ __forceinline__ void four_levels(uint32_t row, uint32_t s, uint64_t* v01, uint64_t* v23) {
-    if (!UNIFORM) {
-        const uint32_t x = lds_u32(row), y = sizeof(Sym) == 1 ? x : lds_u32(row + 4u);
-        *v01 = halves(sizeof(Sym) == 1 ? __byte_perm(x, 0u, 0x1404) : __byte_perm(x, 0u, 0x2404));
-        *v23 = halves(sizeof(Sym) == 1 ? __byte_perm(x, 0u, 0x3424) : __byte_perm(y, 0u, 0x2404));
-        return;
-    }
-    const float step = __uint_as_float((127u - s) << 23);   // k 2^-s is exact
-    float k[4];
-    if (sizeof(Sym) == 1) {
-        const uint32_t x = lds_u32(row);
-#pragma unroll
-        for (int i = 0; i < 4; ++i) k[i] = (float)(int8_t)(x >> (8 * i));
-    } else {
-        const uint32_t x = lds_u32(row), y = lds_u32(row + 4u);
-        k[0] = (float)(int16_t)x; k[1] = (float)(int16_t)(x >> 16);
-        k[2] = (float)(int16_t)y; k[3] = (float)(int16_t)(y >> 16);
-    }
-    *v01 = mul2(pack2(k[0], k[1]), pack2(step, step));
-    *v23 = mul2(pack2(k[2], k[3]), pack2(step, step));
+// Four symbols of one stream: powers of two (exponential levels, by way of fp16) ...
+template <class Sym>
+__device__ __forceinline__ void four_powers(uint32_t row, uint64_t* v01, uint64_t* v23) {
+    const uint32_t x = lds_u32(row), y = sizeof(Sym) == 1 ? x : lds_u32(row + 4u);
+    *v01 = halves(sizeof(Sym) == 1 ? __byte_perm(x, 0u, 0x1404) : __byte_perm(x, 0u, 0x2404));
+    *v23 = halves(sizeof(Sym) == 1 ? __byte_perm(x, 0u, 0x3424) : __byte_perm(y, 0u, 0x2404));
 }
-
-// Four fields of a fixed-width stream, elements e .. e + 3 of the vector (e a multiple of 4), as values.  Returns
-// false when a symbol does not exist.
-__device__ __noinline__ bool four_fields(const Geometry& G, const StreamHead& hd, uint64_t e, float4* out) {
-    const uint32_t wd = hd.width, smask = (1u << (wd - 1u)) - 1u;
-    const uint64_t b = e / G.bucket;
-    const uint32_t in_bucket = (uint32_t)(e - b * G.bucket), rec_words = 1u + (G.bucket * wd + 31u) / 32u;
-    const uint64_t blen = G.d - b * G.bucket < G.bucket ? G.d - b * G.bucket : G.bucket;
-    const uint32_t last = (uint32_t)((blen * wd + 31u) / 32u) - 1u, bit = in_bucket * wd, wi = bit >> 5;
-    const uint32_t* const rec = hd.hdr + hd.hwords + b * rec_words;
-    const float norm = __uint_as_float(rec[0]);
-    const uint32_t x0 = rec[1u + min(wi, last)], x1 = rec[1u + min(wi + 1u, last)], x2 = rec[1u + min(wi + 2u, last)];
-    const uint64_t win = ((uint64_t)__funnelshift_l(x1, x0, bit) << 32) | __funnelshift_l(x2, x1, bit);   // 64 bits from the first field on
-    float v[4];
-    bool ok = true;
-#pragma unroll
-    for (uint32_t c = 0; c < 4; ++c) {
-        const uint32_t field = (uint32_t)(win >> (64u - (c + 1u) * wd)) & ((1u << wd) - 1u), sym = field & smask;
-        v[c] = 0.0f;
-        if (sym == 0u || e + c >= G.d) continue;
-        if (sym >= hd.nlev) ok = false;
-        else v[c] = level_times_norm(norm, hd.levelset, G.s, sym, hd.hdr);
-        if (field >> (wd - 1u)) v[c] = -v[c];
-    }
-    *out = make_float4(v[0], v[1], v[2], v[3]);
-    return ok;
+// ... or signed level indices (uniform levels), put into the mantissa of 2^23: converting integers takes four times as long.
+template <class Sym>
+__device__ __forceinline__ void four_indices(uint32_t row, uint64_t* v01, uint64_t* v23) {
+    constexpr bool kBytes = sizeof(Sym) == 1;
+    const uint32_t flip = kBytes ? 0x80808080u : 0x80008000u, top = 0x4B000000u;
+    const float bias = -(8388608.0f + (kBytes ? 128.0f : 32768.0f));
+    const uint32_t x = lds_u32(row) ^ flip, y = kBytes ? x : lds_u32(row + 4u) ^ flip;
+    const float m0 = __uint_as_float(__byte_perm(x, top, kBytes ? 0x7650 : 0x7610)), m1 = __uint_as_float(__byte_perm(x, top, kBytes ? 0x7651 : 0x7632)),
+                m2 = __uint_as_float(__byte_perm(y, top, kBytes ? 0x7652 : 0x7610)), m3 = __uint_as_float(__byte_perm(y, top, kBytes ? 0x7653 : 0x7632));
+    *v01 = add2(pack2(m0, m1), pack2(bias, bias));
+    *v23 = add2(pack2(m2, m3), pack2(bias, bias));
 }
 
 // The add pass of a unit.
 struct AddPass {
     const StreamHead* heads;           // of the group's streams
-    const unsigned char* stream_tabs;
+    const unsigned char* levels;       // their level tables, kLevelBytes each ...
+    uint32_t by_symbol;                // ... and levels by symbol (alike == 3), kCodeBytes each: shared-memory address, a multiple of 256
     uint32_t rows, norms;              // shared-memory addresses
     uint32_t S, streams;
-    uint32_t alike;                    // all streams are tokens of exponential (0) or uniform (1) levels; else 2
+    uint32_t alike;                    // all streams are tokens of exponential (0), uniform (1) or table (3) levels; else 2
     bool exact;                        // norm times a power of two is exact for all the unit's norms
     bool last, carried;                // the last group of streams; sums of earlier groups are in `carry`
 };
@@ -372,6 +319,8 @@ __device__ __forceinline__ void add_block(const DecodeParams& P, const AddPass& 
         for (int i = 0; i < 4; ++i) sum[i] = carry[i];
     }
     uint32_t nrm = A.norms + 4u * q0, at = A.rows + q0 * Row<Sym>::kPitch + 4u * lane * (uint32_t)sizeof(Sym);
+    const uint64_t minus_zero = pack2(P.minus_zero, P.minus_zero);
+    const float step = __uint_as_float((127u - s) << 23);   // 2^-s
     auto add_rows = [&](auto value) {
 #pragma unroll
         for (int b = 0; b < NB; ++b) {
@@ -383,15 +332,16 @@ __device__ __forceinline__ void add_block(const DecodeParams& P, const AddPass& 
     };
     auto add_exp = [&](uint32_t row, float nm, uint64_t& s01, uint64_t& s23) {
         uint64_t a, b;
-        four_levels<Sym, false>(row, s, &a, &b);
+        four_powers<Sym>(row, &a, &b);
         s01 = fma2(a, pack2(nm, nm), s01);
         s23 = fma2(b, pack2(nm, nm), s23);
     };
     auto add_uniform = [&](uint32_t row, float nm, uint64_t& s01, uint64_t& s23) {
         uint64_t a, b;
-        four_levels<Sym, true>(row, s, &a, &b);
-        s01 = add2(s01, mul2(a, pack2(nm, nm)));
-        s23 = add2(s23, mul2(b, pack2(nm, nm)));
+        four_indices<Sym>(row, &a, &b);
+        const float n = nm * step;                          // exact, like k 2^-s: either way one rounding of k nm 2^-s
+        s01 = add2(s01, product2(a, pack2(n, n), minus_zero));
+        s23 = add2(s23, product2(b, pack2(n, n), minus_zero));
     };
     if (A.alike == 0u) {
 #pragma unroll 4 / NB
@@ -399,6 +349,19 @@ __device__ __forceinline__ void add_block(const DecodeParams& P, const AddPass& 
     } else if (A.alike == 1u) {
 #pragma unroll 4 / NB
         for (uint32_t j = 0; j < A.streams; ++j, nrm += 4u * A.S, at += A.S * Row<Sym>::kPitch) add_rows(add_uniform);
+    } else if (A.alike == 3u) {
+        uint32_t by_symbol = A.by_symbol;
+#pragma unroll 4 / NB
+        for (uint32_t j = 0; j < A.streams; ++j, nrm += 4u * A.S, at += A.S * Row<Sym>::kPitch, by_symbol += kCodeBytes) {
+            add_rows([&](uint32_t row, float nm, uint64_t& s01, uint64_t& s23) {
+                const uint32_t x = lds_u32(row), y = sizeof(Sym) == 1 ? x : lds_u32(row + 4u);
+                // a symbol's lower byte is the offset of its level
+                const float l0 = field_level(__byte_perm(x, by_symbol, 0x7650)), l1 = field_level(__byte_perm(x, by_symbol, sizeof(Sym) == 1 ? 0x7651 : 0x7652)),
+                            l2 = field_level(__byte_perm(y, by_symbol, sizeof(Sym) == 1 ? 0x7652 : 0x7650)), l3 = field_level(__byte_perm(y, by_symbol, sizeof(Sym) == 1 ? 0x7653 : 0x7652));
+                s01 = add2(s01, product2(pack2(l0, l1), pack2(nm, nm), minus_zero));
+                s23 = add2(s23, product2(pack2(l2, l3), pack2(nm, nm), minus_zero));
+            });
+        }
     } else {
 #pragma unroll 1
         for (uint32_t j = 0; j < A.streams; ++j, nrm += 4u * A.S, at += A.S * Row<Sym>::kPitch) {
@@ -417,7 +380,7 @@ __device__ __forceinline__ void add_block(const DecodeParams& P, const AddPass& 
                 }
                 if (!ok) latch_status(P.ws, kErrBadStream);
             } else {
-                const float* const lv = reinterpret_cast<const float*>(A.stream_tabs + j * kStreamTabBytes + 256u);
+                const float* const lv = reinterpret_cast<const float*>(A.levels + j * kLevelBytes);
                 add_rows([&](uint32_t row, float nm, uint64_t& s01, uint64_t& s23) {
                     float v[4];
 #pragma unroll
@@ -480,18 +443,41 @@ __device__ __forceinline__ void add_block(const DecodeParams& P, const AddPass& 
 
 // Shared memory: the token table, the streams' tables and heads, then per warp its rows, norms and chain copies.
 __host__ __device__ inline size_t chain_fixed_bytes(uint32_t K) {
-    return (4u * kTokEntries + (size_t)K * (kStreamTabBytes + sizeof(StreamHead)) + 15u) & ~(size_t)15u;
+    // (256: the codes start at a multiple of 256)
+    return (4u * kTokEntries + 256u + (size_t)K * (kCodeBytes + kLevelBytes + sizeof(StreamHead)) + 15u) & ~(size_t)15u;
+}
+
+// All streams in the fixed-width mode.  (16-bit symbols: s = 7 or 8, hence fields of 5 bits, or of 9 and 10 with uniform levels.)
+template <class Sym>
+__device__ __forceinline__ void fields_of_width(const DecodeParams& P, const StreamHead* heads, uint32_t tables, uint32_t mine, uint32_t width) {
+    if (heads[0].levelset == kLevelsExp) {
+        if (width == 5u) return decode_fields<5, true>(P, heads, tables, mine);
+        if (sizeof(Sym) == 1 && width == 4u) return decode_fields<4, true>(P, heads, tables, mine);
+        if (sizeof(Sym) == 1 && width == 3u) return decode_fields<3, true>(P, heads, tables, mine);
+    }
+    if (width == 5u) return decode_fields<5, false>(P, heads, tables, mine);
+    if (sizeof(Sym) == 1) {
+        if (width == 3u) return decode_fields<3, false>(P, heads, tables, mine);
+        if (width == 4u) return decode_fields<4, false>(P, heads, tables, mine);
+        if (width == 6u) return decode_fields<6, false>(P, heads, tables, mine);
+        if (width == 7u) return decode_fields<7, false>(P, heads, tables, mine);
+        if (width == 8u) return decode_fields<8, false>(P, heads, tables, mine);
+    } else {
+        if (width == 9u) return decode_fields<9, false>(P, heads, tables, mine);
+        if (width == 10u) return decode_fields<10, false>(P, heads, tables, mine);
+    }
 }
 
 template <class Sym>
 __global__ void __launch_bounds__(32 * kChainMaxWarps, 1) decode_chains_kernel(const __grid_constant__ DecodeParams P) {
     extern __shared__ __align__(128) unsigned char dsm[];
-    __shared__ uint32_t s_kind, s_alike;
+    __shared__ uint32_t s_kind, s_alike, s_fields;
     const Geometry& G = P.geo;
     const uint32_t K = P.K, tid = threadIdx.x, lane = tid & 31u, warp = tid >> 5;
     uint32_t* const table = reinterpret_cast<uint32_t*>(dsm);
-    unsigned char* const stream_tabs = dsm + 4u * kTokEntries;
-    StreamHead* const heads = reinterpret_cast<StreamHead*>(stream_tabs + K * kStreamTabBytes);
+    unsigned char* const codes = dsm + 4u * kTokEntries + (0u - smem_u32(dsm) & 255u);
+    unsigned char* const levels = codes + K * kCodeBytes;
+    StreamHead* const heads = reinterpret_cast<StreamHead*>(levels + K * kLevelBytes);
     const uint32_t rows = smem_u32(dsm) + (uint32_t)chain_fixed_bytes(K) + warp * Row<Sym>::kWarpBytes;
     const uint32_t norms = rows + 32u * Row<Sym>::kPitch;   // one per lane's chain
     const uint32_t copy = norms + 128u + lane * (4u * kChunkWords);   // this lane's words of its chain
@@ -536,10 +522,6 @@ __global__ void __launch_bounds__(32 * kChainMaxWarps, 1) decode_chains_kernel(c
     // that give every warp several units: a small encode call let in early finds room only where CTAs of this kernel have
     // left and is packed onto a few SMs, four CTAs each (a step of 10^6 elements, K = 3: 66 -> 74 us).
     if (P.let_next) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-    if (P.after_fixed) {                                    // the fixed-width kernel in front has done it all, as a rule
-        asm volatile("griddepcontrol.wait;" ::: "memory");
-        if (*reinterpret_cast<volatile uint32_t*>(&P.ws->dec_done_epoch) == P.epoch) return;
-    }
     if (P.likely_table != kTabCoded) build_table(P.likely_table, nullptr);
     clear_rows();
     asm volatile("griddepcontrol.wait;" ::: "memory");
@@ -551,7 +533,7 @@ __global__ void __launch_bounds__(32 * kChainMaxWarps, 1) decode_chains_kernel(c
     }
     __syncthreads();
     if (warp == 0) {
-        bool coded = false, erc = false, uniform = false, other = false, odd = false, same_code = true;
+        bool coded = false, erc = false, uniform = false, other = false, tabled = false, odd = false, same_code = true, fields = true;
         uint32_t first0 = 0, first1 = 0;                    // the code lengths of the first coded stream
         for (uint32_t k0 = 0; k0 < K; k0 += 32u) {
             const uint32_t k = k0 + lane;
@@ -571,21 +553,31 @@ __global__ void __launch_bounds__(32 * kChainMaxWarps, 1) decode_chains_kernel(c
             erc = erc || __any_sync(0xffffffffu, tokens && !in_code);
             uniform = uniform || __any_sync(0xffffffffu, tokens && heads[k].levelset == kLevelsUniform);
             other = other || __any_sync(0xffffffffu, tokens && heads[k].levelset != kLevelsUniform);
-            odd = odd || __any_sync(0xffffffffu, k < K && (!tokens || heads[k].levelset == kLevelsTable));
+            tabled = tabled || __any_sync(0xffffffffu, tokens && heads[k].levelset == kLevelsTable);
+            odd = odd || __any_sync(0xffffffffu, k < K && (!tokens || heads[k].levelset != heads[0].levelset));
+            fields = fields && __all_sync(0xffffffffu, k >= K || (heads[k].ok && heads[k].mode == kModeFixed && heads[k].levelset == heads[0].levelset));
         }
         if (lane == 0) {
             s_kind = coded ? (erc || !same_code ? kTabGaps : kTabCoded) : uniform ? (other ? kTabGaps : kTabUniform) : kTabErc;
-            s_alike = odd || (uniform && other) ? 2u : uniform ? 1u : 0u;
+            s_alike = odd ? 2u : uniform ? 1u : tabled ? 3u : 0u;
+            s_fields = fields ? heads[0].width : 0u;
         }
     }
     __syncthreads();
-    const uint32_t kind = s_kind, all_alike = s_alike;
-    if (kind != P.likely_table || kind == kTabGaps || kind == kTabCoded || all_alike == 2u) {
+    if (s_fields != 0u) {                                   // no tokens at all
+        const uint32_t tables = (smem_u32(dsm) + 4095u) & ~4095u;               // where the token table would be
+        build_field_tables(G, heads, K, dsm + (tables - smem_u32(dsm)));
+        __syncthreads();
+        fields_of_width<Sym>(P, heads, tables, rows, s_fields);
+        return;
+    }
+    const uint32_t kind = s_kind, all_alike = s_alike == 3u && s_kind == kTabGaps ? 2u : s_alike;
+    if (kind != P.likely_table || kind == kTabGaps || kind == kTabCoded || all_alike >= 2u) {
         uint32_t first = K;                                 // the first token stream (all have the same code in the coded mode)
         for (uint32_t k = 0; k < K; ++k) {
             const StreamHead& hd = heads[k];
             if (!hd.ok || hd.mode == kModeFixed) continue;
-            uint16_t* const code = reinterpret_cast<uint16_t*>(stream_tabs + k * kStreamTabBytes);
+            uint16_t* const code = reinterpret_cast<uint16_t*>(codes + k * kCodeBytes);
             if (kind == kTabGaps || (kind == kTabCoded && first == K)) {   // level index by the next 7 bits
                 for (uint32_t i = tid; i < (1u << kMaxCodedS); i += blockDim.x) {
                     uint32_t c = 0, at = 0, index = 0;
@@ -595,13 +587,21 @@ __global__ void __launch_bounds__(32 * kChainMaxWarps, 1) decode_chains_kernel(c
                 }
             }
             if (hd.levelset == kLevelsTable && tid <= G.s)
-                reinterpret_cast<float*>(stream_tabs + k * kStreamTabBytes + 256u)[tid] =
+                reinterpret_cast<float*>(levels + k * kLevelBytes)[tid] =
                     tid < G.s ? __uint_as_float(hd.hdr[kHeaderWords + tid]) : 1.0f;
             if (first == K) first = k;
         }
         if (kind == kTabCoded) __syncthreads();
-        if (kind != P.likely_table || kind == kTabCoded) build_table(kind, reinterpret_cast<const uint16_t*>(stream_tabs + (first == K ? 0u : first) * kStreamTabBytes));
+        if (kind != P.likely_table || kind == kTabCoded) build_table(kind, reinterpret_cast<const uint16_t*>(codes + (first == K ? 0u : first) * kCodeBytes));
         __syncthreads();
+        if (all_alike == 3u) {                              // levels by symbol, sign included (the codes are no longer needed)
+            for (uint32_t i = tid; i < 64u * K; i += blockDim.x) {
+                const uint32_t k = i >> 6, index = (i & 31u) + G.s - 14u;
+                const float l = index >= 1u && index <= G.s + 1u ? reinterpret_cast<const float*>(levels + k * kLevelBytes)[index - 1u] : 0.0f;
+                reinterpret_cast<float*>(codes + k * kCodeBytes)[i & 63u] = i & 32u ? -l : l;
+            }
+            __syncthreads();
+        }
     }
     // from here on warps run alone
 
@@ -716,7 +716,7 @@ __global__ void __launch_bounds__(32 * kChainMaxWarps, 1) decode_chains_kernel(c
 
         // ================= walk =================
         const StreamHead& my_head = heads[g0 + min(lj, gcount - 1u)];
-        const uint16_t* const my_code = reinterpret_cast<const uint16_t*>(stream_tabs + (g0 + min(lj, gcount - 1u)) * kStreamTabBytes);
+        const uint16_t* const my_code = reinterpret_cast<const uint16_t*>(codes + (g0 + min(lj, gcount - 1u)) * kCodeBytes);
         const uint32_t row0 = rows + lane * Row<Sym>::kPitch - (uint32_t)sizeof(Sym), row_end = row0 + (kSB + 1u) * (uint32_t)sizeof(Sym);
         uint32_t row = row0;
         bool good = ch.good;
@@ -769,7 +769,7 @@ __global__ void __launch_bounds__(32 * kChainMaxWarps, 1) decode_chains_kernel(c
         start_copy(after);
 
         // ================= add =================
-        const AddPass ap = {heads + g0, stream_tabs + g0 * kStreamTabBytes, rows, norms, S, gcount, exact ? all_alike : 2u,
+        const AddPass ap = {heads + g0, levels + g0 * kLevelBytes, smem_u32(codes) + g0 * kCodeBytes, rows, norms, S, gcount, exact ? all_alike : 2u,
                             exact, group + 1u == ngroups, group != 0u};
         const uint64_t e0 = unit * S * kSB + 4u * lane;
         uint32_t q0 = 0;
@@ -820,7 +820,7 @@ static cudaError_t launch_chains(const DecodeParams& P, int sms, cudaStream_t st
     return cudaLaunchKernelEx(&cfg, decode_chains_kernel<Sym>, Q);
 }
 
-cudaError_t launch_decode_chains(const DecodeParams& P, int sms, cudaStream_t stream) {
+cudaError_t launch_decode(const DecodeParams& P, int sms, cudaStream_t stream) {
     // With s = 7 or 8 the streams may have uniform levels, whose indices up to 256 do not fit a byte with their sign.
     return P.geo.s == 7u || P.geo.s == 8u ? launch_chains<int16_t>(P, sms, stream) : launch_chains<int8_t>(P, sms, stream);
 }

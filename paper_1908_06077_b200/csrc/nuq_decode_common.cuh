@@ -122,4 +122,30 @@ __device__ __forceinline__ StreamHead read_head(const Geometry& G, const uint32_
     return h;
 }
 
+__device__ __forceinline__ uint64_t pack2(float a, float b) {
+    uint64_t r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
+    return r;
+}
+__device__ __forceinline__ float2 unpack2(uint64_t v) {
+    float2 r;
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(v));
+    return r;
+}
+// two fp32 operations at once, each rounded like the single one
+__device__ __forceinline__ uint64_t fma2(uint64_t a, uint64_t b, uint64_t c) {
+    uint64_t r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+    return r;
+}
+// A rounded product that is added to something afterwards.  Not mul.rn.f32x2: the assembler was seen to put that and an
+// add.rn.f32x2 together into one fused operation, with one rounding instead of two, in spite of the rounding modifiers.
+// A fused operation that adds -0 changes no product, and it cannot be fused again as long as the -0 is not known to be one.
+__device__ __forceinline__ uint64_t product2(uint64_t a, uint64_t b, uint64_t minus_zero) { return fma2(a, b, minus_zero); }
+__device__ __forceinline__ uint64_t add2(uint64_t a, uint64_t b) {
+    uint64_t r;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+
 }  // namespace nuq

@@ -1,0 +1,334 @@
+// DECODE + aggregate of calls whose streams are all in the fixed-width mode with the same field width and kind of levels:
+// no chains to walk, a part of the decode kernel of nuq_decode_chains.cu that its warps enter when the headers say so.
+//
+// A warp takes units of up to four 256-element sub-blocks; a lane has eight consecutive elements of each, one word of
+// every stream when fields have 4 bits.  A field, its sign bit included, is looked up in a table of level values in shared
+// memory, multiplied by the bucket's norm and added in stream order: an element of a stream is one extraction, one look-up
+// and one fused multiply-add.  No value depends on a unit, so nothing is built per
+// unit and warps never meet.  An item, that is the fields of a unit in up to eight streams, is brought into the warp's
+// shared memory by one bulk copy per stream, two items ahead, so that no address is computed per word and the bytes in
+// flight do not depend on registers.
+// 25.6 x 10^6 elements, K = 8 (200 MB, 31 us at the memory's rate): 4-bit fields 55 us, other widths and small buckets 60
+// to 90 us (a kernel of one thread per 32 elements: 104 to 117 us, level tables 547 us); 65536 elements 6.6 us (in front of
+// the token kernel: 12 us).  What bounds it is the look-ups (one shared-memory word per element and stream, a wavefront
+// per 32 of them) and, with four warps per scheduler, what the warps wait for.
+#pragma once
+#include <type_traits>
+
+#include "nuq_async.cuh"
+#include "nuq_decode_common.cuh"
+
+namespace nuq {
+
+constexpr uint32_t kFieldStreams = 8;                       // streams of an item
+// words of a stream that hold a lane's eight fields (8 W bits from a byte boundary on)
+__host__ __device__ constexpr uint32_t field_words(uint32_t w) { return w == 4u ? 1u : w == 7u || w > 8u ? 3u : 2u; }
+// sub-blocks of a unit: two items fit the warp's shared memory
+__host__ __device__ constexpr uint32_t field_slots(uint32_t w) { return w <= 5u ? 4u : 2u; }
+// bytes of an item's part of a stream: the fields, norms between them, and what 16-byte alignment adds
+__host__ __device__ constexpr uint32_t field_pitch(uint32_t w) { return 4u * ((field_slots(w) * (8u * w + 1u) + 6u + 3u) & ~3u); }
+// a warp's shared memory: two items with their norms, two mbarriers
+__host__ __device__ constexpr uint32_t field_warp_bytes(uint32_t w) { return 2u * kFieldStreams * field_pitch(w) + 256u + 16u; }
+
+// Bytes between the tables of two streams (level-table streams have one each).
+__host__ __device__ constexpr uint32_t field_table_stride(uint32_t w) { return w <= 6u ? 256u : 4u << w; }
+
+// The level values by field; a symbol that does not exist stands for NaN, which the sums keep (and are checked for).
+__device__ __forceinline__ void build_field_tables(const Geometry& G, const StreamHead* heads, uint32_t K, unsigned char* tables) {
+    const uint32_t w = heads[0].width, stride = field_table_stride(w), n = heads[0].levelset == kLevelsTable ? K : 1u;
+    for (uint32_t i = threadIdx.x; i < n << w; i += blockDim.x) {
+        const uint32_t k = i >> w, f = i & ((1u << w) - 1u), sym = f & ((1u << (w - 1u)) - 1u);
+        float v = sym == 0u ? 0.0f : sym < heads[k].nlev ? level_times_norm(1.0f, heads[k].levelset, G.s, sym, heads[k].hdr)
+                                                         : __uint_as_float(0x7FC00000u);
+        if (f >> (w - 1u)) v = -v;
+        *reinterpret_cast<float*>(tables + k * stride + 4u * f) = v;
+    }
+}
+
+__device__ __forceinline__ uint32_t field_word(uint32_t addr) {
+    uint32_t v;
+    asm volatile("ld.shared.u32 %0, [%1];" : "=r"(v) : "r"(addr));
+    return v;
+}
+// A table entry (tables do not change any more)
+__device__ __forceinline__ float field_level(uint32_t addr) {
+    float v;
+    asm("ld.shared.f32 %0, [%1];" : "=f"(v) : "r"(addr));
+    return v;
+}
+
+// The levels of a lane's eight fields.  `tab` is a multiple of 256 and of the table's size, so that it can be put together
+// with a field's offset instead of added to it.
+template <uint32_t W>
+__device__ __forceinline__ void eight_levels(const uint32_t (&x)[field_words(W)], uint32_t shift, uint32_t tab, float (&l)[8]) {
+    if (W == 4u) {
+        // the fields times four, four to a register: elements 0 2 4 6 and 1 3 5 7 from the top byte
+        const uint32_t a = (x[0] >> 2) & 0x3C3C3C3Cu, c = (x[0] << 2) & 0x3C3C3C3Cu;
+        l[0] = field_level(__byte_perm(a, tab, 0x7653)); l[1] = field_level(__byte_perm(c, tab, 0x7653));
+        l[2] = field_level(__byte_perm(a, tab, 0x7652)); l[3] = field_level(__byte_perm(c, tab, 0x7652));
+        l[4] = field_level(__byte_perm(a, tab, 0x7651)); l[5] = field_level(__byte_perm(c, tab, 0x7651));
+        l[6] = field_level(__byte_perm(a, tab, 0x7650)); l[7] = field_level(__byte_perm(c, tab, 0x7650));
+        return;
+    }
+    constexpr uint32_t kWords = field_words(W);
+    uint32_t y[4] = {0, 0, 0, 0};                           // the fields from bit 31 of y[0] on
+#pragma unroll
+    for (uint32_t i = 0; i < kWords; ++i) y[i] = __funnelshift_l(i + 1u < kWords ? x[i + 1u < kWords ? i + 1u : i] : 0u, x[i], shift);
+#pragma unroll
+    for (uint32_t i = 0; i < 8; ++i) {
+        const uint32_t bit = i * W, at = bit >> 5, end = (bit & 31u) + W;          // in y[at], and in y[at + 1] if end > 32
+        const uint32_t t = end <= 30u ? y[at] >> (30u - end) : end <= 32u ? y[at] << (end - 30u) : __funnelshift_r(y[at + 1u], y[at], 62u - end);
+        l[i] = field_level((t & (((1u << W) - 1u) << 2)) | tab);
+    }
+}
+
+// Four fields of a fixed-width stream, elements e .. e + 3 of the vector (e a multiple of 4), as values.  Returns
+// false when a symbol does not exist.
+__device__ __noinline__ bool four_fields(const Geometry& G, const StreamHead& hd, uint64_t e, float4* out) {
+    const uint32_t wd = hd.width, smask = (1u << (wd - 1u)) - 1u;
+    const uint64_t b = e / G.bucket;
+    const uint32_t in_bucket = (uint32_t)(e - b * G.bucket), rec_words = 1u + (G.bucket * wd + 31u) / 32u;
+    const uint64_t blen = G.d - b * G.bucket < G.bucket ? G.d - b * G.bucket : G.bucket;
+    const uint32_t last = (uint32_t)((blen * wd + 31u) / 32u) - 1u, bit = in_bucket * wd, wi = bit >> 5;
+    const uint32_t* const rec = hd.hdr + hd.hwords + b * rec_words;
+    const float norm = __uint_as_float(rec[0]);
+    const uint32_t x0 = rec[1u + min(wi, last)], x1 = rec[1u + min(wi + 1u, last)], x2 = rec[1u + min(wi + 2u, last)];
+    const uint64_t win = ((uint64_t)__funnelshift_l(x1, x0, bit) << 32) | __funnelshift_l(x2, x1, bit);   // 64 bits from the first field on
+    float v[4];
+    bool ok = true;
+#pragma unroll
+    for (uint32_t c = 0; c < 4; ++c) {
+        const uint32_t field = (uint32_t)(win >> (64u - (c + 1u) * wd)) & ((1u << wd) - 1u), sym = field & smask;
+        v[c] = 0.0f;
+        if (sym == 0u || e + c >= G.d) continue;
+        if (sym >= hd.nlev) ok = false;
+        else v[c] = level_times_norm(norm, hd.levelset, G.s, sym, hd.hdr);
+        if (field >> (wd - 1u)) v[c] = -v[c];
+    }
+    *out = make_float4(v[0], v[1], v[2], v[3]);
+    return ok;
+}
+
+// adds eight fields of one stream from element e on to the sums, by the slow way
+__device__ __forceinline__ bool add_eight_slowly(const Geometry& G, const StreamHead& hd, uint64_t e, float (&sum)[8]) {
+    bool ok = true;
+#pragma unroll
+    for (uint32_t h = 0; h < 2; ++h) {
+        if (e + 4u * h >= G.d) continue;
+        float4 v;
+        ok = four_fields(G, hd, e + 4u * h, &v) && ok;
+        sum[4 * h] += v.x; sum[4 * h + 1] += v.y; sum[4 * h + 2] += v.z; sum[4 * h + 3] += v.w;
+    }
+    return ok;
+}
+
+// eight values to a multiple of 32 bytes: a whole sector per lane and instruction
+__device__ __forceinline__ void store8(float* dst, const float (&v)[8]) {
+    asm volatile("st.global.v8.f32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(dst), "f"(v[0]), "f"(v[1]), "f"(v[2]), "f"(v[3]),
+                 "f"(v[4]), "f"(v[5]), "f"(v[6]), "f"(v[7])
+                 : "memory");
+}
+
+// EXACT: powers of two, whose product with a norm of ordinary size is exact, so that one fused operation gives the sum
+// that two would; else product and sum are rounded one after the other.  Other norms (tiny ones; not finite ones, where an
+// element without a symbol has no product) take the slow way.
+// `mine`: the warp's shared memory (a multiple of 16).
+template <uint32_t W, bool EXACT>
+__device__ __forceinline__ void decode_fields(const DecodeParams& P, const StreamHead* heads, uint32_t tables, uint32_t mine) {
+    constexpr uint32_t kWords = field_words(W), kSlots = field_slots(W), kPitch = field_pitch(W), kItem = kFieldStreams * kPitch;
+    const Geometry& G = P.geo;
+    const uint32_t lane = lane_id(), K = P.K, spb = G.bucket / kSB, rec_words = 1u + G.bucket * W / 32u, hwords = heads[0].hwords;
+    const uint32_t tab_stride = heads[0].levelset == kLevelsTable ? field_table_stride(W) : 0u;
+    const uint32_t nsub = (uint32_t)((G.d + kSB - 1u) / kSB), nwarps = gridDim.x * (blockDim.x >> 5);
+    const uint32_t S = min(max(nsub / nwarps, 1u), kSlots);                    // (a small call: one sub-block for every warp first)
+    const uint32_t nunits = (nsub + S - 1u) / S;
+    const uint32_t shift = W == 4u ? 0u : 8u * ((W * lane) & 3u);
+    const uint32_t norms = mine + 2u * kItem, full = norms + 256u;
+
+    struct Item {
+        uint32_t unit, k0, b, in;                           // first stream; the first sub-block: the in-th of bucket b
+    };
+    const uint32_t stride_b = nwarps * S / spb, stride_in = nwarps * S - stride_b * spb;
+    auto behind = [&](Item it) {
+        it.k0 += kFieldStreams;
+        if (it.k0 >= K) {
+            it.k0 = 0;
+            it.unit += nwarps;
+            it.b += stride_b;
+            it.in += stride_in;
+            if (it.in >= spb) {
+                it.in -= spb;
+                it.b += 1u;
+            }
+        }
+        return it;
+    };
+    auto norms_before = [&](const Item& it, uint32_t q) {   // bucket boundaries between the first sub-block and the q-th behind it
+        return (it.in + q >= spb ? 1u : 0u) + (it.in + q >= 2u * spb ? 1u : 0u) + (it.in + q >= 3u * spb ? 1u : 0u);
+    };
+    // starts the copies of an item: lane q * 8 + j the norm of slot q in stream j, lane j the fields of stream j
+    auto start_copy = [&](const Item& it, uint32_t stage) {
+        if (it.unit < nunits) {
+            const uint32_t sub = it.unit * S, slots = min(S, nsub - sub), count = min(K - it.k0, kFieldStreams);
+            const uint64_t rec = hwords + (uint64_t)it.b * rec_words;
+            const uint32_t q = lane / kFieldStreams, j = lane % kFieldStreams;
+            if (q < slots && j < count)
+                asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(norms + 128u * stage + 4u * lane), "l"(heads[it.k0 + j].hdr + rec + norms_before(it, q) * rec_words) : "memory");
+            // where the fields start in every container, in words, and how many there are (with the norms between them)
+            const uint64_t first = rec + 1u + it.in * (8u * W), from = first & ~(uint64_t)3u;
+            const uint32_t words = (uint32_t)(first - from) + slots * 8u * W + norms_before(it, slots - 1u);
+            const uint32_t dst = mine + stage * kItem, bar = full + 8u * stage;
+            if (lane < kFieldStreams) {
+                if (lane < count) {
+                    const StreamHead& hd = heads[it.k0 + lane];
+                    uint32_t n = (words + 3u) & ~3u;
+                    if (hd.cwords - from < n) {             // the container ends here: its last words one by one
+                        const uint32_t have = (uint32_t)(hd.cwords - from);
+                        n = have & ~3u;
+                        for (uint32_t i = n; i < have; ++i)
+                            asm volatile("st.shared.u32 [%0], %1;" ::"r"(dst + lane * kPitch + 4u * i), "r"(hd.hdr[from + i]) : "memory");
+                    }
+                    if (n != 0u) bulk_load(dst + lane * kPitch, hd.hdr + from, 4u * n, bar);
+                    else mbar_arrive(bar);
+                } else {
+                    mbar_arrive(bar);
+                }
+            }
+        }
+        asm volatile("cp.async.commit_group;" ::: "memory");
+    };
+
+    if (lane == 0) {
+        mbar_init(full, kFieldStreams);
+        mbar_init(full + 8u, kFieldStreams);
+    }
+    __syncwarp();
+    bool ok = true, in_time = true;
+    Item cur;
+    cur.unit = (threadIdx.x >> 5) * gridDim.x + blockIdx.x;
+    cur.k0 = 0;
+    cur.b = cur.unit * S / spb;
+    cur.in = cur.unit * S - cur.b * spb;
+    Item next = behind(cur);
+    start_copy(cur, 0);
+    start_copy(next, 1);
+    const bool wide = (reinterpret_cast<uintptr_t>(P.acc) & 31u) == 0;
+    float sum[kSlots][8];
+    auto clear = [&] {
+#pragma unroll
+        for (uint32_t i = 0; i < 8u * kSlots; ++i) sum[i / 8u][i % 8u] = 0.0f;
+    };
+    clear();
+    for (uint32_t n = 0; cur.unit < nunits; ++n) {
+        const uint32_t sub = cur.unit * S, slots = min(S, nsub - sub), count = min(K - cur.k0, kFieldStreams);
+        const uint64_t e0 = (uint64_t)sub * kSB + 8u * lane;
+        const Item after = behind(next);
+        if (P.w != nullptr && cur.k0 == 0u && (uint64_t)(sub + slots) * kSB <= G.d && lane < (P.mu != 0.0f ? 2u : 1u))   // the parameters, for later
+            asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"((lane == 0u ? P.w : P.yl) + (uint64_t)sub * kSB), "r"(4u * kSB * slots) : "memory");
+
+        const uint32_t stage = n & 1u;
+        asm volatile("cp.async.wait_group 1;" ::: "memory");
+        const float norm = lane / kFieldStreams < slots && lane % kFieldStreams < count ? __uint_as_float(field_word(norms + 128u * stage + 4u * lane)) : 0.0f;
+        const bool fine = EXACT ? norm == 0.0f || (norm >= 0x1p-100f && norm < 0x1p126f) : fabsf(norm) <= 3.4028234e38f;
+        const bool all_fine = __all_sync(0xffffffffu, fine);
+        __syncwarp();                                       // the other lanes' norms are there
+        in_time = mbar_wait(full + 8u * stage, (n >> 1) & 1u) && in_time;
+        if (all_fine) {
+            // where the lane's fields of each slot start
+            const uint32_t first = mine + stage * kItem + 4u * ((hwords + cur.b * rec_words + 1u + cur.in * (8u * W)) & 3u) + (W * lane & ~3u);
+            auto add_item = [&](auto whole) {               // whole: all slots, within one bucket
+                uint32_t at = first, nrm = norms + 128u * stage, tab = tables + cur.k0 * tab_stride;
+#pragma unroll 1
+                for (uint32_t j = 0; j < count; ++j) {
+#pragma unroll
+                    for (uint32_t q = 0; q < kSlots; ++q) {
+                        if (!decltype(whole)::value && q >= slots) break;
+                        const uint32_t from = decltype(whole)::value ? at : at + 4u * norms_before(cur, q);
+                        uint32_t x[kWords];
+                        float l[8];
+#pragma unroll
+                        for (uint32_t i = 0; i < kWords; ++i) x[i] = field_word(from + 32u * W * q + 4u * i);
+                        const float nm = __uint_as_float(field_word(nrm + 4u * kFieldStreams * q));
+                        eight_levels<W>(x, shift, tab, l);
+#pragma unroll
+                        for (int i = 0; i < 8; ++i) sum[q][i] = EXACT ? __fmaf_rn(l[i], nm, sum[q][i]) : __fadd_rn(sum[q][i], __fmul_rn(l[i], nm));
+                    }
+                    at += kPitch;
+                    nrm += 4u;
+                    tab += tab_stride;
+                }
+            };
+            if (slots == kSlots && cur.in + kSlots <= spb) add_item(std::true_type());
+            else add_item(std::false_type());
+        } else {
+            for (uint32_t j = 0; j < count; ++j) {
+#pragma unroll
+                for (uint32_t q = 0; q < kSlots; ++q)
+                    if (q < slots) ok = add_eight_slowly(G, heads[cur.k0 + j], e0 + kSB * q, sum[q]) && ok;
+            }
+        }
+        __syncwarp();                                       // the item's words and norms have been read
+        start_copy(after, stage);
+        if (cur.k0 + kFieldStreams >= K) {                  // the sums are complete
+            float check = 0.0f;                             // NaN when a sum is not finite
+#pragma unroll
+            for (uint32_t i = 0; i < 8u * kSlots; ++i) check = __fmaf_rn(sum[i / 8u][i % 8u], 0.0f, check);
+            if (!(check == 0.0f)) {                     // a symbol that does not exist?
+                for (uint32_t q = 0; q < slots; ++q) {
+                    for (uint32_t k = 0; k < K; ++k) {
+                        float none[8] = {};
+                        ok = add_eight_slowly(G, heads[k], e0 + kSB * q, none) && ok;
+                    }
+                }
+            }
+            auto value = [&](uint32_t q, uint32_t h) {
+                return make_float4(sum[q][4u * h], sum[q][4u * h + 1u], sum[q][4u * h + 2u], sum[q][4u * h + 3u]);
+            };
+            if (e0 - 8u * lane + kSB * slots > G.d) {       // the vector's end
+#pragma unroll
+                for (uint32_t i = 0; i < 2u * kSlots; ++i) {
+                    const uint64_t e = e0 + kSB * (i / 2u) + 4u * (i & 1u);
+                    if (i / 2u >= slots || e >= G.d) continue;
+                    if (e + 4u <= G.d) finish4(P, e, value(i / 2u, i & 1u));
+                    else finish_part(P, e, value(i / 2u, i & 1u), (uint32_t)(G.d - e));
+                }
+            } else if (P.w == nullptr) {
+#pragma unroll
+                for (uint32_t q = 0; q < kSlots; ++q) {
+                    if (q >= slots) break;
+                    float* const dst = P.acc + e0 + kSB * q;
+                    if (wide) {
+                        store8(dst, sum[q]);
+                    } else {
+                        *reinterpret_cast<float4*>(dst) = value(q, 0u);
+                        *reinterpret_cast<float4*>(dst + 4) = value(q, 1u);
+                    }
+                }
+            } else {
+#pragma unroll
+                for (uint32_t i0 = 0; i0 < 2u * kSlots; i0 += 4u) {            // the loads of two slots are on their way together
+                    float4 w[4], yl[4];
+#pragma unroll
+                    for (uint32_t i = 0; i < 4; ++i) {
+                        const uint64_t e = e0 + kSB * ((i0 + i) / 2u) + 4u * (i & 1u);
+                        w[i] = yl[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+                        if ((i0 + i) / 2u < slots) {
+                            w[i] = *reinterpret_cast<const float4*>(P.w + e);
+                            if (P.mu != 0.0f) yl[i] = *reinterpret_cast<const float4*>(P.yl + e);
+                        }
+                    }
+#pragma unroll
+                    for (uint32_t i = 0; i < 4; ++i)
+                        if ((i0 + i) / 2u < slots) step4(P, e0 + kSB * ((i0 + i) / 2u) + 4u * (i & 1u), value((i0 + i) / 2u, i & 1u), w[i], yl[i]);
+                }
+            }
+            clear();
+        }
+        cur = next;
+        next = after;
+    }
+    if (__any_sync(0xffffffffu, !ok) && lane == 0) latch_status(P.ws, kErrBadStream);
+    if (__any_sync(0xffffffffu, !in_time) && lane == 0) latch_status(P.ws, kErrTimeout);
+}
+
+}  // namespace nuq

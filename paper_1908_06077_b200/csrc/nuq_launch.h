@@ -20,7 +20,6 @@ int fixed4_blocks_per_sm(const EncodeParams& P);
 cudaError_t launch_encode_fixed4(const EncodeParams& P, cudaStream_t stream);
 cudaError_t launch_level_histogram(const EncodeParams& P, uint64_t* hist, int sms, cudaStream_t stream);   // hist: s + 2 zeroed counters
 cudaError_t upload_token_tables();                    // the chain decoder's tables, into the current device's memory
-cudaError_t launch_decode_chains(const DecodeParams& P, int sms, cudaStream_t stream);
 cudaError_t launch_decode(const DecodeParams& P, int sms, cudaStream_t stream);
 
 }  // namespace nuq
