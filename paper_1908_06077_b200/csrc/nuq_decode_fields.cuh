@@ -187,6 +187,8 @@ __device__ __forceinline__ void decode_fields(const DecodeParams& P, const Strea
                         n = have & ~3u;
                         for (uint32_t i = n; i < have; ++i)
                             asm volatile("st.shared.u32 [%0], %1;" ::"r"(dst + lane * kPitch + 4u * i), "r"(hd.hdr[from + i]) : "memory");
+                        for (uint32_t i = have; i < words; ++i)                 // and no symbols behind them
+                            asm volatile("st.shared.u32 [%0], %1;" ::"r"(dst + lane * kPitch + 4u * i), "r"(0u) : "memory");
                     }
                     if (n != 0u) bulk_load(dst + lane * kPitch, hd.hdr + from, 4u * n, bar);
                     else mbar_arrive(bar);
