@@ -87,6 +87,7 @@ struct EncodeParams {
     uint32_t grid;           // CTAs to launch
     uint32_t cluster;        // CTAs per thread-block cluster: the blocks of one wide bucket (0: no clusters)
     uint32_t overlap;        // launched so that its CTAs are set up while the kernel before it in the stream ends
+    uint32_t let_next;       // the kernel behind it may be launched while this one runs
 };
 
 // Token tables of the chain decoder: ERC level indices as exponential or as uniform levels, gaps alone, a fitted level code.

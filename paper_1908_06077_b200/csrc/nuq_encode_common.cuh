@@ -164,17 +164,17 @@ __device__ __forceinline__ void describe_tile(const Geometry& G, unsigned long l
     ti.nsb = (ti.tile_len + kSB - 1) / kSB;
 }
 
-// Kernels that follow one another in a stream (programmatic dependent launch).  An encode kernel says at once,
+// Kernels that follow one another in a stream (programmatic dependent launch).  An encode kernel says (P.let_next) at once,
 // as each CTA starts, that the kernel behind it may be launched: that kernel's CTAs then take the SM slots as
 // this one's leave them and do their set-up (tables in shared memory, barriers) while the last CTAs here still
 // work.  A kernel launched that way must not touch global memory before the kernel in front of it has ended
 // and its writes are visible: every thread waits for that ahead of its first access (the input may have been
 // written by that very kernel).  Without the launch attribute both instructions do nothing.
 __device__ __forceinline__ void let_next_kernel_start(const EncodeParams& P) {
-    if (P.overlap) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    if (P.let_next) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }
-// The warp's bytes (`elems` elements from `first` on) of the tile a CTA is likely to get first (that of its own number) are asked into the L2 ahead of the wait, while
-// the kernel in front drains: all CTAs together would otherwise start with 19 MB from HBM at once.  A prefetch changes
+// The warp's bytes (`elems` elements from `first` on) of the tile a CTA is likely to get first (that of its own number)
+// are asked into the L2 ahead of the wait, while the kernel in front drains: all CTAs together would otherwise start with 19 MB from HBM at once.  A prefetch changes
 // nothing that anyone can see: the L2 is where all writes meet, so what is copied to shared memory later is what
 // the kernel in front has written.
 __device__ __forceinline__ void prefetch_first_tile(const EncodeParams& P, uint32_t first, uint32_t elems) {
