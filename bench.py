@@ -384,11 +384,10 @@ class Workload:
     def launches_per_step(self):
         # my kernels only: one encode kernel per worker (two for buckets wider than a tile in the 4-bit
         # fixed-width mode: the norms come first; otherwise a cluster adds the norm up inside the encode
-        # kernel), one decode kernel (two when all streams are fixed-width: that path's own kernel, then
-        # the general one, which returns at once)
+        # kernel), one decode kernel
         fixed = (self.flags >> 16) & 0xff == 1
         wide = self.bucket > 8192
-        return self.K * (2 if wide and fixed else 1) + (2 if fixed else 1)
+        return self.K * (2 if wide and fixed else 1) + 1
 
 
 def summarize(ms):
@@ -520,7 +519,7 @@ def run_gpu(args):
             "decode_us_per_call": {k: 1e3 * v for k, v in summarize(dec_ms).items()},
             "roofline": roofline_entry(ENCODE_KERNEL.get(args.workload, "encode_kernel"), enc_bytes, enc_launch_ms, peak, peak_kind,
                                        ENCODE_TRAFFIC_BYTES.get(args.workload) if full else None),
-            "roofline_decode": roofline_entry(DECODE_KERNEL.get(args.workload, "decode_kernel"), dec_bytes, t_dec, peak, peak_kind,
+            "roofline_decode": roofline_entry("decode_chains_kernel", dec_bytes, t_dec, peak, peak_kind,
                                               DECODE_TRAFFIC_BYTES.get(args.workload) if full else None),
             "gpu_launches": steps * w.launches_per_step(),
             "clocks": clocks,
@@ -577,7 +576,6 @@ ENCODE_TRAFFIC_BYTES = {"c3": 102_306_816 + 3_938_560, "c3-fixed": 102_282_752 +
 DECODE_TRAFFIC_BYTES = {"c3": 24_617_728 + 44_184_320, "c3-fixed": 102_410_752 + 57_455_872}
 # the kernel that does the work of a call, where it is not the general one
 ENCODE_KERNEL = {"c3-fixed": "encode_fixed4_kernel"}
-DECODE_KERNEL = {"c3-fixed": "decode_fixed_kernel"}
 
 
 def main():

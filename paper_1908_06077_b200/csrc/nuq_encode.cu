@@ -5,27 +5,33 @@
 // A persistent CTA takes tiles of up to 8192 consecutive elements (whole buckets, or
 // one 8192-element coding block of a wider bucket) by ticket.  The tile's bytes are
 // brought into shared memory by bulk asynchronous copies (TMA, completion on an
-// mbarrier), one per warp: eight worker warps own 1024 elements (four 256-element
-// coding sub-blocks) of the tile each, and a warp starts the copy of its part of the
-// next tile as soon as it is done with its part of this one.  Per tile a worker
+// mbarrier), one per warp: the worker warps (eight, or sixteen in small calls) own an equal
+// part of the tile's 256-element coding sub-blocks each, and a warp starts the copy of its
+// part of the next tile as soon as it is done with its part of this one.  Per tile a worker
 //   1. adds up the squares of its elements per sub-block (eight per lane in fp32,
 //      everything beyond that in fp64); whichever warp is done last turns the partial
 //      sums into the tile's bucket norms, once for the whole CTA, before the only CTA
 //      barrier of the tile;
-//   2. per sub-block: quantizes 8 elements per lane (two Philox blocks), compacts the
-//      nonzero symbols into a dense list (one warp scan of per-lane counts; the list
-//      lies over the sub-block's own, already consumed, input bytes) and turns the list
-//      into tokens ERC(gap) sign ERC(index), 32 per step, appended to the warp's own
-//      bit window (two windows per warp, used in turn);
+//   2. per sub-block: quantizes 8 consecutive elements per lane (two Philox blocks) and
+//      turns them into the lane's own token string.  Where all symbols are 0 or 1 (nearly
+//      always) the string comes from a table by the mask of the nonzero ones, except the
+//      first token's gap, which depends on the lanes before; a few higher symbols are put
+//      in one at a time, many take a general path.  One warp scan of the strings' lengths
+//      gives their places in the warp's own bit window (two windows per warp, used in
+//      turn), and two shared-memory reductions per lane write them there.  25.6 x 10^6
+//      elements, s = 4: 68.6 us; compacting the nonzero symbols into a list first, 32
+//      tokens per step, took 83.
 //   3. (ERC mode) shifts its strings of the PREVIOUS tile to their place in a staged
 //      image of that tile, which has been laid out in the meantime.
-// In the ERC mode a ninth warp, the writer, does everything that concerns a tile as a
+// In the ERC mode one more warp, the writer, does everything that concerns a tile as a
 // whole: the scan over its 32 sub-block lengths (the layout of its records), the block
-// heads, the announcement of its size to the tiles behind it and, once the workers have
-// moved their strings, the tile's place in the stream (two-level decoupled look-back
-// over tile and group sizes, every wait bounded), the copy of the image to the stream
-// and the block offsets.  Workers and writer meet through named barriers on which one
-// side only arrives, so the workers never wait for other CTAs.
+// heads, the announcement of its size to the tiles behind it, the tile's place in the
+// stream (two-level decoupled look-back over tile and group sizes, every wait bounded),
+// which it looks for while the workers move their strings, and, once they have, the copy
+// of the image to the stream and the block offsets.  Workers and writer meet through named
+// barriers on which one side only arrives, so the workers never wait for other CTAs.
+// What bounds it: instruction issue (Philox's wide multiplications take two slots each),
+// and in small calls the latency of the first loads, of one tile and of the end.
 // In the fixed-width mode there is no writer: a lane packs the fields of its eight
 // elements, two lanes exchange halves, and every lane stores one finished word (4-bit
 // fields of the exponential level set have a leaner kernel of their own, nuq_encode_fixed4.cu).
