@@ -1,0 +1,114 @@
+"""Edges of the kernels' ranges, against the oracle: streams from 1 to 64 and the units that follow from them, empty and
+full sub-blocks, gaps and tokens too long for the decoder's table, chains longer than a lane's copy of them, fields of every
+width, norms whose products are not exact, and the encoders' sizes at which another variant takes over."""
+import numpy as np
+import pytest
+
+import oracle as O
+from gpu_util import gpu_decode, gpu_encode, require_cuda
+
+pytestmark = pytest.mark.gpu
+
+
+def _vector(kind, d, seed):
+    rng = np.random.default_rng(seed)
+    g = rng.standard_normal(d).astype(np.float32)
+    if kind == "sparse":                        # gaps of 128 and more
+        g[rng.random(d) > 0.004] = 0.0
+    elif kind == "ends":                        # a sub-block's last element alone: gap 256
+        keep = np.arange(d) % 256 == 255
+        g[~keep] = 0.0
+    elif kind == "dense":                       # nearly all symbols high, all tokens long
+        g = (np.sign(g) * rng.uniform(0.5, 1.0, d)).astype(np.float32)
+    elif kind == "mixed":                       # empty, sparse and dense sub-blocks side by side
+        g *= np.repeat(np.float32([0.0, 1e-3, 0.05, 1.0]), 256)[np.arange(d) % 1024]
+    elif kind == "tiny":                        # norm times level is not a normal number
+        g *= np.float32(1e-38)
+    return g
+
+
+def _container(kind, d, bucket, s, nk, ls, mode, seed):
+    return O.encode(_vector(kind, d, seed), bucket, s, O.make_flags(nk, ls, mode), seed=seed, offset=seed)[0]
+
+
+def _same_sums(streams, d, bucket, s):
+    rc, want = O.decode_accumulate(streams, d, bucket, s)
+    assert rc == 0
+    assert np.array_equal(gpu_decode(streams, d, bucket, s).view(np.uint32), want.view(np.uint32))
+
+
+@pytest.mark.parametrize("K", [1, 2, 3, 5, 6, 7, 12, 16, 31, 32, 33, 64])
+@pytest.mark.parametrize("mode", [O.MODE_ERC, O.MODE_FIXED])
+def test_sums_for_every_shape_of_a_unit(K, mode):
+    kinds = ["normal", "sparse", "mixed", "dense", "ends"]
+    for d, bucket in ((200, 256), (70003, 1024)):
+        _same_sums([_container(kinds[k % 5], d, bucket, 4, O.NORM_L2, O.LEVELS_EXP, mode, k) for k in range(K)], d, bucket, 4)
+
+
+@pytest.mark.parametrize("kind", ["normal", "sparse", "ends", "dense", "mixed", "tiny"])
+@pytest.mark.parametrize("d,bucket,s,nk,ls", [
+    (30001, 512, 2, O.NORM_LINF, O.LEVELS_EXP), (30001, 8192, 6, O.NORM_LINF, O.LEVELS_EXP),
+    (30001, 1024, 14, O.NORM_LINF, O.LEVELS_EXP), (30001, 768, 5, O.NORM_L2, O.LEVELS_UNIFORM),
+    (30001, 8192, 6, O.NORM_LINF, O.LEVELS_UNIFORM), (30001, 512, 7, O.NORM_LINF, O.LEVELS_UNIFORM),
+    (30001, 1024, 8, O.NORM_LINF, O.LEVELS_UNIFORM), (30001, 1024, 8, O.NORM_LINF, O.LEVELS_EXP)])
+def test_sums_of_long_tokens_and_chains(kind, d, bucket, s, nk, ls):
+    for mode in (O.MODE_ERC, O.MODE_FIXED):
+        _same_sums([_container(kind, d, bucket, s, nk, ls, mode, k) for k in range(3)], d, bucket, s)
+
+
+@pytest.mark.parametrize("ls,s", [(O.LEVELS_EXP, s) for s in (1, 2, 3, 6, 7, 14)] + [(O.LEVELS_UNIFORM, s) for s in range(1, 9)])
+@pytest.mark.parametrize("bucket", [256, 768, 2048])
+def test_fields_of_every_width(ls, s, bucket):
+    for d in (256, 1023, 8 * bucket + 5, 148 * 16 * 256 + 77):      # the last: more than one sub-block for every warp
+        K = 2 if d > 100000 else 9
+        _same_sums([_container("normal", d, bucket, s, O.NORM_LINF, ls, O.MODE_FIXED, k) for k in range(K)], d, bucket, s)
+
+
+def test_sums_of_streams_with_different_codes_and_level_sets():
+    d, bucket, s = 20001, 1024, 4
+    streams = []
+    for k, weights in enumerate(([9, 5, 3, 2, 1], [1, 1, 1, 1, 1], [1, 2, 4, 8, 16])):
+        O.set_level_code(O.huffman_lengths(weights))
+        streams.append(_container("dense" if k else "sparse", d, bucket, s, O.NORM_LINF, O.LEVELS_EXP, O.MODE_CODED, k))
+    _same_sums(streams[1:2] * 3, d, bucket, s)
+    _same_sums(streams, d, bucket, s)
+    for ls, mode in ((O.LEVELS_EXP, O.MODE_ERC), (O.LEVELS_UNIFORM, O.MODE_ERC), (O.LEVELS_UNIFORM, O.MODE_FIXED)):
+        streams.append(_container("mixed", d, bucket, s, O.NORM_LINF, ls, mode, 7))
+    _same_sums(streams, d, bucket, s)
+    O.set_levels(np.array([0.1, 0.2, 0.5, 0.8], np.float32))
+    tables = [_container(kind, d, bucket, s, O.NORM_LINF, O.LEVELS_TABLE, O.MODE_ERC, 8) for kind in ("dense", "tiny")]
+    _same_sums(tables, d, bucket, s)
+    _same_sums(streams + tables, d, bucket, s)
+
+
+def test_missing_symbols_and_values_that_are_not_finite_in_fixed_width_streams():
+    require_cuda()
+    d, bucket, s = 5000, 1024, 3                                    # 5 levels in 3 bits: 5, 6 and 7 do not exist
+    good = _container("normal", d, bucket, s, O.NORM_LINF, O.LEVELS_EXP, O.MODE_FIXED, 1)
+    bad = good.copy()
+    bad[16 + 1 + 3] |= np.uint32(0x70000000)
+    gpu_decode([good, bad], d, bucket, s, expect_status=-3)
+    for norm in (np.inf, np.float32(3e38)):                         # infinite, or a sum that overflows: no error
+        big = good.copy()
+        big[16] = np.float32(norm).view(np.uint32)
+        rc, want = O.decode_accumulate([big] * 3, d, bucket, s)
+        got = gpu_decode([big] * 3, d, bucket, s)
+        assert rc == 0 and np.array_equal(got, want, equal_nan=True)
+
+
+@pytest.mark.parametrize("kind", ["normal", "sparse", "dense", "mixed"])
+@pytest.mark.parametrize("d,bucket,s,ls", [
+    (1, 256, 4, O.LEVELS_EXP), (8191, 8192, 4, O.LEVELS_EXP), (40000, 512, 6, O.LEVELS_EXP), (40000, 768, 5, O.LEVELS_UNIFORM),
+    (2 * 148 * 8192, 8192, 4, O.LEVELS_EXP), (2 * 148 * 8192 + 1, 8192, 4, O.LEVELS_EXP)])      # two tiles per SM, one more
+def test_containers_at_the_encoders_edges(kind, d, bucket, s, ls):
+    g = _vector(kind, d, 3)
+    for mode in (O.MODE_ERC, O.MODE_FIXED) + ((O.MODE_CODED,) if ls == O.LEVELS_EXP else ()):
+        if mode == O.MODE_CODED:
+            lengths = list(O.huffman_lengths(list(range(1, s + 2))))  # high levels get the short words
+            O.set_level_code(lengths)
+            require_cuda()[1].set_level_code(lengths)
+        flags = O.make_flags(O.NORM_LINF, ls, mode)
+        norms = O.bucket_norms(g, bucket, O.NORM_LINF)
+        want, want_bits = O.encode(g, bucket, s, flags, seed=5, offset=9, norms=norms)
+        got, got_bits = gpu_encode(g, bucket, s, flags, seed=5, offset=9, norms=norms)
+        assert got_bits == want_bits and np.array_equal(got, want)
