@@ -1295,6 +1295,8 @@ static cudaError_t prepare_kernel() {
         e = cudaFuncSetAttribute(encode_kernel<L, M, true, 8>, cudaFuncAttributeMaxDynamicSharedMemorySize, kEncMaxDynSmem);
     if (M == kModeErc && e == cudaSuccess)
         e = cudaFuncSetAttribute(encode_kernel<L, kModeErc, false, kEncMaxWarps>, cudaFuncAttributeMaxDynamicSharedMemorySize, kEncMaxDynSmem);
+    if (M == kModeErc && e == cudaSuccess)
+        e = cudaFuncSetAttribute(encode_kernel<L, kModeErc, true, kEncMaxWarps>, cudaFuncAttributeMaxDynamicSharedMemorySize, kEncMaxDynSmem);
     if (e == cudaSuccess) attr_set = true;
     return e;
 }
@@ -1360,9 +1362,10 @@ static cudaError_t launch_one(const EncodeParams& P, cudaStream_t stream) {
     if (smem > (size_t)kEncMaxDynSmem || P.grid == 0 || (P.cluster > 1u && P.grid % P.cluster != 0)) return cudaErrorInvalidValue;
     EncodeLaunch cfg;
     fill_launch<M>(&cfg, P, P.grid, stream);
-    if (P.cluster > 1u) return cudaLaunchKernelEx(&cfg.cfg, encode_kernel<L, M, true, 8>, P);
     if (M == kModeErc && P.warps == (uint32_t)kEncMaxWarps)
-        return cudaLaunchKernelEx(&cfg.cfg, encode_kernel<L, kModeErc, false, kEncMaxWarps>, P);
+        return P.cluster > 1u ? cudaLaunchKernelEx(&cfg.cfg, encode_kernel<L, kModeErc, true, kEncMaxWarps>, P)
+                              : cudaLaunchKernelEx(&cfg.cfg, encode_kernel<L, kModeErc, false, kEncMaxWarps>, P);
+    if (P.cluster > 1u) return cudaLaunchKernelEx(&cfg.cfg, encode_kernel<L, M, true, 8>, P);
     return cudaLaunchKernelEx(&cfg.cfg, encode_kernel<L, M, false, 8>, P);
 }
 
@@ -1373,7 +1376,10 @@ static int max_clusters(const EncodeParams& P) {
     EncodeLaunch cfg;
     fill_launch<M>(&cfg, P, P.cluster, nullptr);
     int n = 0;
-    if (cudaOccupancyMaxActiveClusters(&n, encode_kernel<L, M, true, 8>, &cfg.cfg) != cudaSuccess) {
+    const cudaError_t e = M == kModeErc && P.warps == (uint32_t)kEncMaxWarps
+        ? cudaOccupancyMaxActiveClusters(&n, encode_kernel<L, kModeErc, true, kEncMaxWarps>, &cfg.cfg)
+        : cudaOccupancyMaxActiveClusters(&n, encode_kernel<L, M, true, 8>, &cfg.cfg);
+    if (e != cudaSuccess) {
         cudaGetLastError();
         return 0;
     }

@@ -99,6 +99,7 @@ def test_missing_symbols_and_values_that_are_not_finite_in_fixed_width_streams()
 @pytest.mark.parametrize("kind", ["normal", "sparse", "dense", "mixed"])
 @pytest.mark.parametrize("d,bucket,s,ls", [
     (1, 256, 4, O.LEVELS_EXP), (8191, 8192, 4, O.LEVELS_EXP), (40000, 512, 6, O.LEVELS_EXP), (40000, 768, 5, O.LEVELS_UNIFORM),
+    (65536, 65536, 4, O.LEVELS_EXP), (3 * 16384 + 9000, 16384, 4, O.LEVELS_EXP),      # one cluster, several
     (2 * 148 * 8192, 8192, 4, O.LEVELS_EXP), (2 * 148 * 8192 + 1, 8192, 4, O.LEVELS_EXP)])      # two tiles per SM, one more
 def test_containers_at_the_encoders_edges(kind, d, bucket, s, ls):
     g = _vector(kind, d, 3)
@@ -112,3 +113,5 @@ def test_containers_at_the_encoders_edges(kind, d, bucket, s, ls):
         want, want_bits = O.encode(g, bucket, s, flags, seed=5, offset=9, norms=norms)
         got, got_bits = gpu_encode(g, bucket, s, flags, seed=5, offset=9, norms=norms)
         assert got_bits == want_bits and np.array_equal(got, want)
+        free, free_bits = gpu_encode(g, bucket, s, flags, seed=5, offset=9)       # (largest magnitudes are exact: the same norms)
+        assert free_bits == want_bits and np.array_equal(free, want)
