@@ -121,9 +121,8 @@ typedef struct nuq_info {
  * kernel has ended, so the order of the stream holds for g, out, out_bits.
  * Once the stream's workspace exists (after a first call of at least this
  * size on the stream), encode calls may be captured into a CUDA graph and
- * replayed: the kernels leave the workspace as they found it.  Decode calls
- * may not: their hand-out counter alternates with the number of the call,
- * which a replay does not advance.
+ * replayed: the kernels leave the workspace as they found it.  (Decode calls keep
+ * nothing in the workspace but a latched error.)
  */
 nuq_status nuq_encode(const float* g, uint64_t d, uint32_t bucket, uint32_t s, uint32_t norm_kind, uint64_t seed,
                       uint64_t offset, void* out, uint64_t* out_bits, void* stream);
