@@ -8,7 +8,7 @@
 // unit and warps never meet.  An item, that is the fields of a unit in up to eight streams, is brought into the warp's
 // shared memory by one bulk copy per stream, two items ahead, so that no address is computed per word and the bytes in
 // flight do not depend on registers.
-// 25.6 x 10^6 elements, K = 8 (200 MB, 31 us at the memory's rate): 4-bit fields 55 us, other widths and small buckets 60
+// 25.6 x 10^6 elements, K = 8 (200 MB, 31 us at the memory's rate): 4-bit fields 52 us, other widths and small buckets 60
 // to 90 us (a kernel of one thread per 32 elements: 104 to 117 us, level tables 547 us); 65536 elements 6.6 us (in front of
 // the token kernel: 12 us).  What bounds it is the look-ups (one shared-memory word per element and stream, a wavefront
 // per 32 of them) and, with four warps per scheduler, what the warps wait for.
@@ -118,6 +118,19 @@ __device__ __forceinline__ bool add_eight_slowly(const Geometry& G, const Stream
         float4 v;
         ok = four_fields(G, hd, e + 4u * h, &v) && ok;
         sum[4 * h] += v.x; sum[4 * h + 1] += v.y; sum[4 * h + 2] += v.z; sum[4 * h + 3] += v.w;
+    }
+    return ok;
+}
+
+// Whether all symbols of a lane's elements exist (e0 + 256 q + 0 .. 7 in all streams).  A call, so that its code is out of the
+// way of the loop: four warps per scheduler wait for instructions as much as for data (56.0 -> 52.3 us).
+__device__ __noinline__ bool fields_exist(const Geometry& G, const StreamHead* heads, uint32_t K, uint64_t e0, uint32_t slots) {
+    bool ok = true;
+    for (uint32_t q = 0; q < slots; ++q) {
+        for (uint32_t k = 0; k < K; ++k) {
+            float none[8] = {};
+            ok = add_eight_slowly(G, heads[k], e0 + kSB * q, none) && ok;
+        }
     }
     return ok;
 }
@@ -276,12 +289,7 @@ __device__ __forceinline__ void decode_fields(const DecodeParams& P, const Strea
 #pragma unroll
             for (uint32_t i = 0; i < 8u * kSlots; ++i) check = __fmaf_rn(sum[i / 8u][i % 8u], 0.0f, check);
             if (!(check == 0.0f)) {                     // a symbol that does not exist?
-                for (uint32_t q = 0; q < slots; ++q) {
-                    for (uint32_t k = 0; k < K; ++k) {
-                        float none[8] = {};
-                        ok = add_eight_slowly(G, heads[k], e0 + kSB * q, none) && ok;
-                    }
-                }
+                ok = fields_exist(G, heads, K, e0, slots) && ok;
             }
             auto value = [&](uint32_t q, uint32_t h) {
                 return make_float4(sum[q][4u * h], sum[q][4u * h + 1u], sum[q][4u * h + 2u], sum[q][4u * h + 3u]);
