@@ -99,7 +99,9 @@ cudaError_t upload_token_tables() {
         else if (pos > 1u)
             tab[kTabErc][i] = (pos - 1u) | ((gap - 1u) << kGapShift);
     }
-    return cudaMemcpyToSymbol(g_token_tables, tab, sizeof(tab));
+    const cudaError_t e = cudaMemcpyToSymbol(g_token_tables, tab, sizeof(tab));
+    // (the copy goes by the default stream, whose end kernels of a non-blocking stream do not wait for)
+    return e == cudaSuccess ? cudaStreamSynchronize(nullptr) : e;
 }
 
 __device__ __forceinline__ void copy_async16(uint32_t dst, const void* src) {

@@ -110,8 +110,10 @@ cudaError_t upload_erc_lut() {
     static EmitTables emit;
     build_erc_lut(lut);
     build_emit_tables(lut, &emit);
-    const cudaError_t e = cudaMemcpyToSymbol(g_emit_tables, &emit, sizeof(emit));
-    return e == cudaSuccess ? cudaMemcpyToSymbol(c_erc_lut, lut, sizeof(lut)) : e;
+    cudaError_t e = cudaMemcpyToSymbol(g_emit_tables, &emit, sizeof(emit));
+    if (e == cudaSuccess) e = cudaMemcpyToSymbol(c_erc_lut, lut, sizeof(lut));
+    // (the copies go by the default stream, whose end kernels of a non-blocking stream do not wait for)
+    return e == cudaSuccess ? cudaStreamSynchronize(nullptr) : e;
 }
 
 // Uniform levels k / 2^s:  p = y - floor(y).

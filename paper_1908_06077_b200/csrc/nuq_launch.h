@@ -8,7 +8,7 @@
 namespace nuq {
 
 void build_erc_lut(uint32_t* lut256);                 // ERC(N), N = 1..256: code | len << 16
-cudaError_t upload_erc_lut();                         // into the current device's constant memory
+cudaError_t upload_erc_lut();                         // the encoder's tables, into the current device's memory; returns when they are there
 cudaError_t launch_bucket_norms(const float* g, uint64_t d, uint32_t bucket, uint32_t norm_kind, float* norms,
                                 uint64_t nb, cudaStream_t stream);
 size_t encode_smem_bytes(const EncodeParams& P);      // dynamic shared memory of one encoder CTA
@@ -19,7 +19,7 @@ bool fixed4_applies(const Geometry& G);               // the call is served by t
 int fixed4_blocks_per_sm(const EncodeParams& P);
 cudaError_t launch_encode_fixed4(const EncodeParams& P, cudaStream_t stream);
 cudaError_t launch_level_histogram(const EncodeParams& P, uint64_t* hist, int sms, cudaStream_t stream);   // hist: s + 2 zeroed counters
-cudaError_t upload_token_tables();                    // the chain decoder's tables, into the current device's memory
+cudaError_t upload_token_tables();                    // the chain decoder's tables, likewise
 cudaError_t launch_decode(const DecodeParams& P, int sms, cudaStream_t stream);
 
 }  // namespace nuq

@@ -1,0 +1,46 @@
+"""What the library's host code asks of the CUDA runtime, and in which order: the library's own objects linked with a runtime
+that runs nothing (fake_cudart.cpp).  No GPU is needed."""
+import ctypes as C
+import os
+import subprocess
+
+import pytest
+
+from paper_1908_06077_b200 import build as cuda_build
+
+HERE = os.path.dirname(os.path.abspath(__file__))
+STREAM = 0x10                                               # a stream of the caller's own; the fake never looks at it
+ERC, FIXED = 0, 1 << 16
+
+
+@pytest.fixture()
+def lib(tmp_path):
+    if not all(os.path.exists(o) for o in cuda_build.OBJECTS):
+        cuda_build.build(force=True)
+    path = str(tmp_path / "libnuq_host.so")                 # another file, so another instance of the library, for every test
+    subprocess.run(["g++", "-std=c++17", "-O1", "-shared", "-fPIC", "-I/usr/local/cuda/include", "-Wl,-Bsymbolic", "-o", path,
+                    os.path.join(HERE, "fake_cudart.cpp")] + cuda_build.OBJECTS, check=True)
+    lib = C.CDLL(path)
+    lib.nuq_encode.argtypes = [C.c_void_p, C.c_uint64, C.c_uint32, C.c_uint32, C.c_uint32, C.c_uint64, C.c_uint64, C.c_void_p, C.c_void_p, C.c_void_p]
+    lib.nuq_decode_accumulate.argtypes = [C.POINTER(C.c_void_p), C.c_uint32, C.c_uint64, C.c_uint32, C.c_uint32, C.c_void_p, C.c_void_p]
+    lib.fake_events.restype = C.c_char_p
+    return lib
+
+
+def _encode(lib, d=100000, bucket=1024, s=4, kind=ERC, stream=STREAM):
+    return lib.nuq_encode(0x1000, d, bucket, s, kind, 1, 0, 0x2000, None, stream)
+
+
+def _decode(lib, d=100000, bucket=1024, s=4, stream=STREAM):
+    return lib.nuq_decode_accumulate((C.c_void_p * 1)(0x2000), 1, d, bucket, s, 0x3000, stream)
+
+
+def _launches(lib):
+    return [e for e in lib.fake_events().decode().splitlines() if e.startswith("launch")]
+
+
+@pytest.mark.parametrize("call", [_encode, _decode])
+def test_the_first_call_waits_for_the_tables_it_uploads(lib, call):
+    """the upload runs on the default stream, which a non-blocking stream's kernels do not wait for"""
+    assert call(lib) == 0 and call(lib) == 0
+    assert len(_launches(lib)) == 2 and all(e.endswith("unordered 0") for e in _launches(lib))
