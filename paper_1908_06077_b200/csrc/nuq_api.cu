@@ -622,13 +622,14 @@ nuq_status nuq_last_status(void* stream_) {
     auto it = g_ws.find(std::make_pair(dev, stream));
     if (it != g_ws.end() && it->second.ptr) {
         if (cudaMemcpy(&status, &it->second.ptr->status, sizeof(int), cudaMemcpyDeviceToHost) != cudaSuccess) return NUQ_ERR_CUDA;
-        if (status != 0 && cudaMemset(&it->second.ptr->status, 0, sizeof(int)) != cudaSuccess) return NUQ_ERR_CUDA;
+        // (cleared in the stream itself: its next kernels do not wait for the default stream)
+        if (status != 0 && cudaMemsetAsync(&it->second.ptr->status, 0, sizeof(int), stream) != cudaSuccess) return NUQ_ERR_CUDA;
     }
     auto st = g_static_ws.find(dev);               // kernels of nuq_encode_static latch into the static scratch
     if (st != g_static_ws.end()) {
         int s2 = 0;
         if (cudaMemcpy(&s2, &st->second->status, sizeof(int), cudaMemcpyDeviceToHost) != cudaSuccess) return NUQ_ERR_CUDA;
-        if (s2 != 0 && cudaMemset(&st->second->status, 0, sizeof(int)) != cudaSuccess) return NUQ_ERR_CUDA;
+        if (s2 != 0 && cudaMemsetAsync(&st->second->status, 0, sizeof(int), stream) != cudaSuccess) return NUQ_ERR_CUDA;
         if (s2 < status) status = s2;
     }
     return status;

@@ -12,9 +12,10 @@
 namespace {
 std::map<const void*, std::string> names;                   // host stub -> device name
 std::map<std::pair<int, const void*>, size_t> smem_allowed; // (device, kernel), as cudaFuncSetAttribute left it
-std::set<std::pair<int, const void*>> in_flight;            // (device, symbol): copies that the host has not waited for
+std::set<std::pair<int, const void*>> in_flight;            // (device, target): work on the default stream that the host has not waited for
 int device = 0, capturing = 0;
 std::string events;
+void* last_alloc = nullptr;
 
 void note(const std::string& s) { events += s + "\n"; }
 
@@ -41,6 +42,7 @@ extern "C" {
 // for the test
 void fake_reset() { events.clear(); capturing = 0; }
 void fake_capture(int on) { capturing = on; }
+void* fake_last_alloc() { return last_alloc; }
 const char* fake_events() { return events.c_str(); }
 
 // registration, called when the library is loaded
@@ -69,13 +71,17 @@ cudaError_t cudaOccupancyMaxActiveClusters(int* n, const void*, const cudaLaunch
 
 cudaError_t cudaMalloc(void** p, size_t n) {
     const cudaError_t e = refused_in_capture("cudaMalloc");
-    if (e == cudaSuccess) *p = std::calloc(1, n);
+    if (e == cudaSuccess) *p = last_alloc = std::calloc(1, n);
     return e;
 }
 cudaError_t cudaFree(void* p) { std::free(p); return cudaSuccess; }
 cudaError_t cudaMemcpy(void* d, const void* s, size_t n, cudaMemcpyKind) { std::memcpy(d, s, n); return cudaSuccess; }
 cudaError_t cudaMemcpyAsync(void* d, const void* s, size_t n, cudaMemcpyKind, cudaStream_t) { std::memcpy(d, s, n); return cudaSuccess; }
-cudaError_t cudaMemset(void* d, int v, size_t n) { std::memset(d, v, n); return cudaSuccess; }
+cudaError_t cudaMemset(void* d, int v, size_t n) {           // returns before the device has done it
+    std::memset(d, v, n);
+    in_flight.insert({device, d});
+    return cudaSuccess;
+}
 cudaError_t cudaMemsetAsync(void* d, int v, size_t n, cudaStream_t) { std::memset(d, v, n); return cudaSuccess; }
 cudaError_t cudaGetSymbolAddress(void** p, const void*) { static char array[1 << 20]; *p = array; return cudaSuccess; }
 // from pageable memory: returns when the source has been staged, not when the device has the bytes

@@ -23,7 +23,9 @@ def lib(tmp_path):
     lib = C.CDLL(path)
     lib.nuq_encode.argtypes = [C.c_void_p, C.c_uint64, C.c_uint32, C.c_uint32, C.c_uint32, C.c_uint64, C.c_uint64, C.c_void_p, C.c_void_p, C.c_void_p]
     lib.nuq_decode_accumulate.argtypes = [C.POINTER(C.c_void_p), C.c_uint32, C.c_uint64, C.c_uint32, C.c_uint32, C.c_void_p, C.c_void_p]
+    lib.nuq_last_status.argtypes = [C.c_void_p]
     lib.fake_events.restype = C.c_char_p
+    lib.fake_last_alloc.restype = C.c_void_p
     return lib
 
 
@@ -44,3 +46,13 @@ def test_the_first_call_waits_for_the_tables_it_uploads(lib, call):
     """the upload runs on the default stream, which a non-blocking stream's kernels do not wait for"""
     assert call(lib) == 0 and call(lib) == 0
     assert len(_launches(lib)) == 2 and all(e.endswith("unordered 0") for e in _launches(lib))
+
+
+def test_a_status_is_cleared_in_its_own_stream(lib):
+    """a clearing pass on the default stream could wipe out what the next kernel of a non-blocking stream latches"""
+    assert _decode(lib) == 0
+    status = C.cast(lib.fake_last_alloc(), C.POINTER(C.c_int))      # the workspace begins with it
+    status[0] = -3
+    assert lib.nuq_last_status(STREAM) == -3 and lib.nuq_last_status(STREAM) == 0
+    assert _decode(lib) == 0
+    assert all(e.endswith("unordered 0") for e in _launches(lib))
