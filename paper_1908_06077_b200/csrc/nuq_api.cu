@@ -630,7 +630,7 @@ nuq_status nuq_last_status(void* stream_) {
         int s2 = 0;
         if (cudaMemcpy(&s2, &st->second->status, sizeof(int), cudaMemcpyDeviceToHost) != cudaSuccess) return NUQ_ERR_CUDA;
         if (s2 != 0 && cudaMemsetAsync(&st->second->status, 0, sizeof(int), stream) != cudaSuccess) return NUQ_ERR_CUDA;
-        if (s2 < status) status = s2;
+        if (s2 < 0 ? s2 < status : status == 0) status = s2;    // (a warning only where there is no error)
     }
     return status;
 }

@@ -83,7 +83,7 @@ cudaError_t cudaMemset(void* d, int v, size_t n) {           // returns before t
     return cudaSuccess;
 }
 cudaError_t cudaMemsetAsync(void* d, int v, size_t n, cudaStream_t) { std::memset(d, v, n); return cudaSuccess; }
-cudaError_t cudaGetSymbolAddress(void** p, const void*) { static char array[1 << 20]; *p = array; return cudaSuccess; }
+cudaError_t cudaGetSymbolAddress(void** p, const void*) { static char array[1 << 20]; *p = last_alloc = array; return cudaSuccess; }
 // from pageable memory: returns when the source has been staged, not when the device has the bytes
 cudaError_t cudaMemcpyToSymbol(const void* symbol, const void*, size_t, size_t, cudaMemcpyKind) {
     const cudaError_t e = refused_in_capture("cudaMemcpyToSymbol");

@@ -2,6 +2,7 @@
 that runs nothing (fake_cudart.cpp).  No GPU is needed."""
 import ctypes as C
 import os
+import shutil
 import subprocess
 
 import pytest
@@ -13,15 +14,21 @@ STREAM = 0x10                                               # a stream of the ca
 ERC, FIXED = 0, 1 << 16
 
 
-@pytest.fixture()
-def lib(tmp_path):
+@pytest.fixture(scope="module")
+def built(tmp_path_factory):
     if not all(os.path.exists(o) for o in cuda_build.OBJECTS):
         cuda_build.build(force=True)
-    path = str(tmp_path / "libnuq_host.so")                 # another file, so another instance of the library, for every test
+    path = str(tmp_path_factory.mktemp("host") / "libnuq_host.so")
     subprocess.run(["g++", "-std=c++17", "-O1", "-shared", "-fPIC", "-I/usr/local/cuda/include", "-Wl,-Bsymbolic", "-o", path,
                     os.path.join(HERE, "fake_cudart.cpp")] + cuda_build.OBJECTS, check=True)
-    lib = C.CDLL(path)
+    return path
+
+
+@pytest.fixture()
+def lib(built, tmp_path):
+    lib = C.CDLL(shutil.copy(built, tmp_path))              # another file, so another instance of the library, for every test
     lib.nuq_encode.argtypes = [C.c_void_p, C.c_uint64, C.c_uint32, C.c_uint32, C.c_uint32, C.c_uint64, C.c_uint64, C.c_void_p, C.c_void_p, C.c_void_p]
+    lib.nuq_encode_static.argtypes = lib.nuq_encode.argtypes
     lib.nuq_decode_accumulate.argtypes = [C.POINTER(C.c_void_p), C.c_uint32, C.c_uint64, C.c_uint32, C.c_uint32, C.c_void_p, C.c_void_p]
     lib.nuq_last_status.argtypes = [C.c_void_p]
     lib.fake_events.restype = C.c_char_p
@@ -56,3 +63,13 @@ def test_a_status_is_cleared_in_its_own_stream(lib):
     assert lib.nuq_last_status(STREAM) == -3 and lib.nuq_last_status(STREAM) == 0
     assert _decode(lib) == 0
     assert all(e.endswith("unordered 0") for e in _launches(lib))
+
+
+@pytest.mark.parametrize("own,static,want", [(0, 1, 1), (1, 0, 1), (1, 1, 1), (-3, 1, -3), (1, -5, -5), (-3, -5, -5), (0, 0, 0)])
+def test_the_static_array_s_status_is_joined_with_the_stream_s(lib, own, static, want):
+    """the most negative one wins, a warning shows where there is no error"""
+    assert _decode(lib) == 0
+    C.cast(lib.fake_last_alloc(), C.POINTER(C.c_int))[0] = own
+    assert lib.nuq_encode_static(0x1000, 100000, 1024, 4, ERC, 1, 0, 0x2000, None, STREAM) == 0
+    C.cast(lib.fake_last_alloc(), C.POINTER(C.c_int))[0] = static
+    assert lib.nuq_last_status(STREAM) == want and lib.nuq_last_status(STREAM) == 0
