@@ -119,10 +119,18 @@ typedef struct nuq_info {
  * The kernel is launched so that its blocks may be set up while the kernel
  * before it in the stream ends; it reads and writes memory only after that
  * kernel has ended, so the order of the stream holds for g, out, out_bits.
- * Once the stream's workspace exists (after a first call of at least this
- * size on the stream), encode calls may be captured into a CUDA graph and
- * replayed: the kernels leave the workspace as they found it.  (Decode calls keep
- * nothing in the workspace but a latched error.)
+ * CUDA graphs: encode and decode calls (nuq_decode_accumulate, nuq_decode_update)
+ * may be captured and replayed.  Arguments, level table and level code are those
+ * of the capture; data are those in the buffers at the replay.  The encode
+ * kernels leave the workspace as they found it, the decode kernels keep nothing
+ * there but a latched error.  What a capture does not allow has to be done by a
+ * call before it: the first encode call and the first decode call on a device
+ * upload tables, and on a stream that has no workspace yet, or one too small for
+ * the call, either kind of call allocates.  So make an encode call of at least the
+ * captured size, and a decode call, on the stream first; without them the captured
+ * call returns NUQ_ERR_CUDA (and the capture may be invalid).  A graph holds the
+ * workspace's address: it must not be replayed once a larger call on the stream
+ * has made the workspace grow, or after nuq_shutdown.
  */
 nuq_status nuq_encode(const float* g, uint64_t d, uint32_t bucket, uint32_t s, uint32_t norm_kind, uint64_t seed,
                       uint64_t offset, void* out, uint64_t* out_bits, void* stream);

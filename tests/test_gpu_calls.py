@@ -1,4 +1,4 @@
-"""How calls stand among other work: the first ones of a process, on streams of their own."""
+"""How calls stand among other work: the first ones of a process, on streams of their own; whole steps captured into graphs."""
 import os
 import subprocess
 import sys
@@ -50,3 +50,60 @@ def test_first_calls_of_a_process_on_a_stream_of_its_own(decode_first):
     root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
     done = subprocess.run([sys.executable, "-c", FIRST_CALLS.format(root=root, decode_first=decode_first)], capture_output=True, text=True, timeout=300)
     assert done.returncode == 0, done.stderr[-2000:]
+
+
+@pytest.mark.parametrize("mode", [O.MODE_ERC, O.MODE_FIXED, O.MODE_CODED])
+@pytest.mark.parametrize("update", [False, True])
+def test_a_step_replayed_from_a_cuda_graph(mode, update):
+    """The encode calls of three workers and the decode behind them, captured once and replayed on changing gradients: every
+    replay gives what the same calls give outside the graph.  A level code that is set later does not reach the graph."""
+    torch, nuq = require_cuda()
+    K, d, bucket, s = 3, 400001, 1024, 4
+    flags = O.make_flags(O.NORM_L2, O.LEVELS_EXP, mode)
+    code = [1, 2, 3, 4, 4]
+    nuq.set_level_code(code)
+    gen = torch.Generator(device="cuda").manual_seed(5)
+    src = [torch.randn(d, generator=gen, device="cuda") for _ in range(5)]
+    words = nuq.encode_bound(d, bucket, s, flags) // 4
+
+    class Step:
+        def __init__(self):
+            self.gs = [torch.zeros(d, device="cuda") for _ in range(K)]
+            self.outs = [torch.zeros(words, dtype=torch.int32, device="cuda") for _ in range(K)]
+            self.bits = [torch.zeros(1, dtype=torch.int64, device="cuda") for _ in range(K)]
+            self.acc, self.w, self.yl = torch.zeros(d, device="cuda"), torch.ones(d, device="cuda"), torch.ones(d, device="cuda")
+
+        def enqueue(self, stream):
+            for k in range(K):
+                nuq.encode(self.gs[k], bucket, s, flags, seed=k + 1, out=self.outs[k], out_bits=self.bits[k], stream=stream)
+            if update:
+                nuq.decode_update(self.outs, d, bucket, s, self.w, self.yl, 0.1, 0.9, 1.0, acc=self.acc, stream=stream)
+            else:
+                nuq.decode_accumulate(self.outs, d, bucket, s, acc=self.acc, stream=stream)
+
+    side, captured, plain = torch.cuda.Stream(), Step(), Step()
+    with torch.cuda.stream(side):                            # first use of the stream: workspace and tables
+        captured.enqueue(side)
+    torch.cuda.synchronize()
+    captured.w.fill_(1.0)
+    captured.yl.fill_(1.0)
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph, stream=side):
+        captured.enqueue(side)
+    for rnd in range(3):
+        for st in (captured, plain):
+            for k in range(K):
+                st.gs[k].copy_(src[(k + rnd) % 5])
+        nuq.set_level_code([4, 4, 3, 2, 1])
+        torch.cuda.synchronize()
+        graph.replay()
+        torch.cuda.synchronize()
+        assert nuq.last_status(side) == 0
+        nuq.set_level_code(code)
+        plain.enqueue(None)
+        torch.cuda.synchronize()
+        assert nuq.last_status() == 0
+        for name in ("acc", "w", "yl"):
+            assert torch.equal(getattr(captured, name), getattr(plain, name)), (rnd, name)
+        for a, b, n in zip(captured.outs, plain.outs, plain.bits):
+            assert torch.equal(a[: int(n.item()) // 32], b[: int(n.item()) // 32])

@@ -73,3 +73,15 @@ def test_the_static_array_s_status_is_joined_with_the_stream_s(lib, own, static,
     assert lib.nuq_encode_static(0x1000, 100000, 1024, 4, ERC, 1, 0, 0x2000, None, STREAM) == 0
     C.cast(lib.fake_last_alloc(), C.POINTER(C.c_int))[0] = static
     assert lib.nuq_last_status(STREAM) == want and lib.nuq_last_status(STREAM) == 0
+
+
+@pytest.mark.parametrize("call", [_encode, _decode])
+def test_a_first_call_is_refused_inside_a_capture_and_works_behind_it(lib, call):
+    """tables and workspace come from calls that a capture does not allow; later calls ask for neither"""
+    lib.fake_capture(1)
+    assert call(lib) == -4 and not _launches(lib)
+    lib.fake_capture(0)
+    assert call(lib) == 0
+    lib.fake_reset()
+    lib.fake_capture(1)
+    assert call(lib) == 0 and "refused" not in lib.fake_events().decode()
