@@ -22,10 +22,14 @@ static __device__ __align__(256) unsigned char g_static_scratch[kStaticScratchBy
 struct WsEntry {
     Workspace* ptr = nullptr;
     size_t bytes = 0;
-    // Bytes from the start that may hold something else than zeros where an encode call keeps its scan state
-    // (0: none).  The allocation is zeroed and every encode kernel leaves its scan state zeroed, but the bucket
-    // norms of a wide-bucket call or of a histogram call stay behind, at a place that depends on that call's size.
-    size_t dirty_to = 0;
+    // Something else than zeros may lie where an encode call keeps its scan state.  The allocation is zeroed and every
+    // encode kernel leaves its scan state zeroed, so that is the case only after a launch that failed.
+    bool dirty = false;
+    // Bucket norms that are taken in a pass of their own (wide buckets with 4-bit fields, histograms): an allocation of its
+    // own, so that no call (nor a replay of a captured one, of which the host knows nothing) leaves them where another
+    // call's scan state lies.
+    float* norms = nullptr;
+    size_t norms_bytes = 0;
 };
 
 // One mutex guards the host-side bookkeeping below (maps, tables); it is held for the microseconds a
@@ -179,12 +183,29 @@ nuq_status get_workspace(cudaStream_t stream, size_t bytes, Workspace** out, int
         if (cudaMemsetAsync(p, 0, want, stream) != cudaSuccess) return NUQ_ERR_CUDA;
         e.ptr = static_cast<Workspace*>(p);
         e.bytes = want;
-        e.dirty_to = 0;
+        e.dirty = false;
         if (carried && (cudaMemcpyAsync(&e.ptr->status, &carried, sizeof(int), cudaMemcpyHostToDevice, stream) != cudaSuccess ||
                         cudaStreamSynchronize(stream) != cudaSuccess))
             return NUQ_ERR_CUDA;
     }
     *out = e.ptr;
+    return NUQ_OK;
+}
+
+// Room for `bytes` of bucket norms behind the workspace of (current device, stream).  Growing synchronises the stream.
+nuq_status get_norms(cudaStream_t stream, size_t bytes, WsEntry& e) {
+    if (e.norms_bytes >= bytes) return NUQ_OK;
+    if (e.norms) {
+        if (cudaStreamSynchronize(stream) != cudaSuccess) return NUQ_ERR_CUDA;
+        cudaFree(e.norms);
+        e.norms = nullptr;
+        e.norms_bytes = 0;
+    }
+    const size_t want = bytes + bytes / 2;
+    void* p = nullptr;
+    if (cudaMalloc(&p, want) != cudaSuccess) { cudaGetLastError(); return NUQ_ERR_CUDA; }
+    e.norms = static_cast<float*>(p);
+    e.norms_bytes = want;
     return NUQ_OK;
 }
 
@@ -201,7 +222,7 @@ static std::map<std::pair<int, const void*>, uint32_t> g_container_mode;   // mo
 // What one encode call needs from its workspace and from shared memory.
 struct EncodePlan {
     size_t state_bytes;      // control block + one look-back word per tile and per group of 32 tiles
-    size_t norms_bytes;      // bucket norms for buckets wider than a tile
+    size_t norms_bytes;      // bucket norms that a pass of its own takes (0: none)
     uint32_t want_grid;      // CTAs that give every SM its full share
 };
 
@@ -272,10 +293,10 @@ static EncodePlan plan_encode(EncodeParams& P, int dev, uint32_t flags) {
     return pl;
 }
 
-// Shared tail of the two encode entry points: clears the call's scan state in `ws` and
-// enqueues the kernels.  `ws` must hold pl.state_bytes + pl.norms_bytes.
+// Shared tail of the two encode entry points: clears the call's scan state in `ws` where needed and
+// enqueues the kernels.  `ws` must hold pl.state_bytes, `norms` (if any) pl.norms_bytes.
 static nuq_status enqueue_encode(EncodeParams& P, const EncodePlan& pl, const float* g, uint32_t norm_kind,
-                                 uint64_t seed, uint64_t offset, void* out, uint64_t* out_bits, Workspace* ws,
+                                 uint64_t seed, uint64_t offset, void* out, uint64_t* out_bits, Workspace* ws, float* norms,
                                  WsEntry* entry, int dev, cudaStream_t stream) {
     Geometry& G = P.geo;
     const bool test_norms = (norm_kind & NUQ_TEST_NORMS) != 0;
@@ -284,16 +305,14 @@ static nuq_status enqueue_encode(EncodeParams& P, const EncodePlan& pl, const fl
         g_lut_ready.insert(dev);
     }
     // The encode kernel leaves its scan state zeroed when it ends, so a clearing pass is needed only where
-    // that cannot be relied on: entry == nullptr (the shared static array: always), or something was left
-    // behind in the workspace (then all of that is cleared, not only what this call will use: a later, longer
-    // call keeps scan state further up).
-    if (entry == nullptr || entry->dirty_to > kWorkspaceClearFrom) {
-        size_t upto = pl.state_bytes;
-        if (entry && entry->dirty_to > upto) upto = entry->dirty_to < entry->bytes ? entry->dirty_to : entry->bytes;
+    // that cannot be relied on: entry == nullptr (the shared static array: always), or a launch failed (then all of
+    // the workspace is cleared, not only what this call will use: a later, longer call keeps scan state further up).
+    if (entry == nullptr || entry->dirty) {
+        const size_t upto = entry ? entry->bytes : pl.state_bytes;
         if (cudaMemsetAsync(reinterpret_cast<char*>(ws) + kWorkspaceClearFrom, 0, upto - kWorkspaceClearFrom, stream) !=
             cudaSuccess)
             return NUQ_ERR_CUDA;
-        if (entry) entry->dirty_to = 0;
+        if (entry) entry->dirty = false;
     }
 
     P.g = g;
@@ -301,7 +320,6 @@ static nuq_status enqueue_encode(EncodeParams& P, const EncodePlan& pl, const fl
     if (test_norms) {
         P.norms_in = g_test_norms[dev];
     } else if (pl.norms_bytes) {
-        float* norms = reinterpret_cast<float*>(reinterpret_cast<char*>(ws) + pl.state_bytes);
         if (launch_bucket_norms(g, G.d, G.bucket, G.norm_kind, norms, G.nb, stream) != cudaSuccess) return NUQ_ERR_CUDA;
         P.norms_in = norms;
     }
@@ -328,11 +346,8 @@ static nuq_status enqueue_encode(EncodeParams& P, const EncodePlan& pl, const fl
         P.round_keys[2 * r] = (uint32_t)seed + r * 0x9E3779B9u;
         P.round_keys[2 * r + 1] = (uint32_t)(seed >> 32) + r * 0xBB67AE85u;
     }
-    // the bucket norms of a wide-bucket call lie behind its scan state, where a later call with more tiles
-    // keeps scan state: the next call has to clear first
-    if (pl.norms_bytes && entry && !test_norms) entry->dirty_to = pl.state_bytes + pl.norms_bytes;
     if (launch_encode(P, stream) != cudaSuccess) {
-        if (entry) entry->dirty_to = entry->bytes;          // whatever state the failed launch left
+        if (entry) entry->dirty = true;                     // whatever state the failed launch left
         return NUQ_ERR_CUDA;
     }
     // remember the mode of the container at this address: a hint for the decoder's choice of kernels,
@@ -470,13 +485,12 @@ nuq_status nuq_level_histogram(const float* g, uint64_t d, uint32_t bucket, uint
         P.norms_in = g_test_norms[dev];
     } else {
         Workspace* ws = nullptr;
-        nuq_status st = get_workspace(stream, sizeof(Workspace) + 4 * G.nb, &ws, &dev);
+        WsEntry& e = g_ws[std::make_pair(dev, stream)];
+        nuq_status st = get_workspace(stream, sizeof(Workspace), &ws, &dev);
+        if (st == NUQ_OK) st = get_norms(stream, 4 * G.nb, e);
         if (st != NUQ_OK) return st;
-        WsEntry& e = g_ws[std::make_pair(dev, stream)];     // the norms lie where an encode call keeps its scan state
-        if (e.dirty_to < sizeof(Workspace) + 4 * G.nb) e.dirty_to = sizeof(Workspace) + 4 * G.nb;
-        float* norms = reinterpret_cast<float*>(reinterpret_cast<char*>(ws) + sizeof(Workspace));
-        if (launch_bucket_norms(g, G.d, G.bucket, G.norm_kind, norms, G.nb, stream) != cudaSuccess) return NUQ_ERR_CUDA;
-        P.norms_in = norms;
+        if (launch_bucket_norms(g, G.d, G.bucket, G.norm_kind, e.norms, G.nb, stream) != cudaSuccess) return NUQ_ERR_CUDA;
+        P.norms_in = e.norms;
     }
     P.out = nullptr; P.out_bits = nullptr; P.ws = nullptr;
     P.seed = seed;
@@ -516,10 +530,11 @@ nuq_status nuq_encode(const float* g, uint64_t d, uint32_t bucket, uint32_t s, u
     const EncodePlan pl = plan_encode(P, dev, norm_kind);
     P.grid = pl.want_grid;
     Workspace* ws = nullptr;
-    nuq_status st = get_workspace(stream, pl.state_bytes + pl.norms_bytes, &ws, &dev);
+    WsEntry& e = g_ws[std::make_pair(dev, stream)];
+    nuq_status st = get_workspace(stream, pl.state_bytes, &ws, &dev);
+    if (st == NUQ_OK && pl.norms_bytes && !(norm_kind & NUQ_TEST_NORMS)) st = get_norms(stream, pl.norms_bytes, e);
     if (st != NUQ_OK) return st;
-    return enqueue_encode(P, pl, g, norm_kind, seed, offset, out, out_bits, ws, &g_ws[std::make_pair(dev, stream)],
-                          dev, stream);
+    return enqueue_encode(P, pl, g, norm_kind, seed, offset, out, out_bits, ws, e.norms, &e, dev, stream);
 }
 
 nuq_status nuq_encode_static(const float* g, uint64_t d, uint32_t bucket, uint32_t s, uint32_t norm_kind,
@@ -545,7 +560,8 @@ nuq_status nuq_encode_static(const float* g, uint64_t d, uint32_t bucket, uint32
         it = g_static_ws.emplace(dev, static_cast<Workspace*>(p)).first;
     }
     // the array is shared by every stream of the device: it is cleared before every call
-    return enqueue_encode(P, pl, g, norm_kind, seed, offset, out, out_bits, it->second, nullptr, dev, stream);
+    float* const norms = reinterpret_cast<float*>(reinterpret_cast<char*>(it->second) + pl.state_bytes);
+    return enqueue_encode(P, pl, g, norm_kind, seed, offset, out, out_bits, it->second, norms, nullptr, dev, stream);
 }
 
 // Shared by the two decode entry points.  `w` == nullptr: the sums only.
@@ -660,10 +676,9 @@ void nuq_shutdown(void) {
     int cur = 0;
     cudaGetDevice(&cur);
     for (auto& kv : g_ws) {
-        if (kv.second.ptr) {
-            cudaSetDevice(kv.first.first);
-            cudaFree(kv.second.ptr);
-        }
+        cudaSetDevice(kv.first.first);
+        cudaFree(kv.second.ptr);
+        cudaFree(kv.second.norms);
     }
     g_ws.clear();
     cudaSetDevice(cur);

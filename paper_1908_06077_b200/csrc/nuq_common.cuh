@@ -38,13 +38,13 @@ constexpr uint64_t kTileValueMask = (1ull << 62) - 1;
 struct Workspace {
     int status;             // latched kernel status; survives calls until nuq_last_status reads it
     int pad;
-    // everything below is cleared at the start of every encode call
+    // everything below is zero between calls: an encode kernel leaves it so when it ends
     uint64_t ticket;        // next tile to hand out
     uint64_t done;          // CTAs that have finished (they take no further ticket)
     uint64_t code_bits;     // token bits of the whole call
     uint64_t nnz;           // nonzero symbols of the whole call
     uint64_t total_words;   // payload words of the whole call
-    // followed by: uint64_t tile_state[ntiles], group_state[ceil(ntiles / 32)], then float norms[nb] for wide buckets
+    // followed by: uint64_t tile_state[ntiles], group_state[ceil(ntiles / 32)]
 };
 constexpr size_t kWorkspaceClearFrom = 8;
 

@@ -8,6 +8,7 @@
 #include <set>
 #include <string>
 #include <utility>
+#include <vector>
 
 namespace {
 std::map<const void*, std::string> names;                   // host stub -> device name
@@ -16,6 +17,7 @@ std::set<std::pair<int, const void*>> in_flight;            // (device, target):
 int device = 0, capturing = 0;
 std::string events;
 void* last_alloc = nullptr;
+std::vector<std::pair<char*, size_t>> allocations;
 
 void note(const std::string& s) { events += s + "\n"; }
 
@@ -71,7 +73,10 @@ cudaError_t cudaOccupancyMaxActiveClusters(int* n, const void*, const cudaLaunch
 
 cudaError_t cudaMalloc(void** p, size_t n) {
     const cudaError_t e = refused_in_capture("cudaMalloc");
-    if (e == cudaSuccess) *p = last_alloc = std::calloc(1, n);
+    if (e == cudaSuccess) {
+        *p = last_alloc = std::calloc(1, n);
+        allocations.push_back({static_cast<char*>(*p), n});
+    }
     return e;
 }
 cudaError_t cudaFree(void* p) { std::free(p); return cudaSuccess; }
@@ -97,6 +102,14 @@ cudaError_t cudaStreamSynchronize(cudaStream_t stream) {
     return e;
 }
 
-cudaError_t cudaLaunchKernel(const void* f, dim3, dim3, void**, size_t smem, cudaStream_t stream) { return launch(f, smem, stream); }
+cudaError_t cudaLaunchKernel(const void* f, dim3, dim3, void** args, size_t smem, cudaStream_t stream) {
+    if (names[f].find("bucket_norm_kernel") != std::string::npos) {     // where the norms go: which allocation, which byte of it
+        const char* norms = *static_cast<char**>(args[4]);
+        for (size_t i = 0; i < allocations.size(); ++i)
+            if (norms >= allocations[i].first && norms < allocations[i].first + allocations[i].second)
+                note("norms in allocation " + std::to_string(i) + " of " + std::to_string(allocations.size()));
+    }
+    return launch(f, smem, stream);
+}
 cudaError_t cudaLaunchKernelExC(const cudaLaunchConfig_t* c, const void* f, void**) { return launch(f, c->dynamicSmemBytes, c->stream); }
 }

@@ -107,3 +107,29 @@ def test_a_step_replayed_from_a_cuda_graph(mode, update):
             assert torch.equal(getattr(captured, name), getattr(plain, name)), (rnd, name)
         for a, b, n in zip(captured.outs, plain.outs, plain.bits):
             assert torch.equal(a[: int(n.item()) // 32], b[: int(n.item()) // 32])
+
+
+def test_a_replay_between_calls_that_take_norms_apart():
+    """A captured encode call is replayed after calls on its stream that keep bucket norms (4-bit fields in wide buckets, a
+    histogram), which the graph knows nothing of: they leave its scan state alone."""
+    torch, nuq = require_cuda()
+    d, bucket, s = 3_000_001, 1024, 4
+    g = torch.randn(d, generator=torch.Generator(device="cuda").manual_seed(6), device="cuda")
+    want, bits = nuq.encode(g, bucket, s, 0, seed=2)
+    n = int(bits.item()) // 32
+    out, wide = torch.zeros_like(want), torch.zeros(nuq.encode_bound(d, 65536, s, nuq.MODE_FIXED) // 4, dtype=torch.int32, device="cuda")
+    side, hist = torch.cuda.Stream(), torch.zeros(s + 2, dtype=torch.int64, device="cuda")
+    side.wait_stream(torch.cuda.current_stream())
+    with torch.cuda.stream(side):
+        nuq.encode(g, bucket, s, 0, seed=2, out=out, out_bits=bits)
+        torch.cuda.synchronize()
+        graph = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(graph, stream=side):
+            nuq.encode(g, bucket, s, 0, seed=2, out=out, out_bits=bits)
+        for _ in range(3):
+            nuq.encode(g, 65536, s, nuq.MODE_FIXED, seed=1, out=wide)
+            nuq.level_histogram(g, 256, s, hist=hist)
+            out.zero_()
+            graph.replay()
+            assert nuq.last_status() == 0
+            assert torch.equal(out[:n], want[:n])

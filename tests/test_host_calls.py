@@ -30,6 +30,7 @@ def lib(built, tmp_path):
     lib.nuq_encode.argtypes = [C.c_void_p, C.c_uint64, C.c_uint32, C.c_uint32, C.c_uint32, C.c_uint64, C.c_uint64, C.c_void_p, C.c_void_p, C.c_void_p]
     lib.nuq_encode_static.argtypes = lib.nuq_encode.argtypes
     lib.nuq_decode_accumulate.argtypes = [C.POINTER(C.c_void_p), C.c_uint32, C.c_uint64, C.c_uint32, C.c_uint32, C.c_void_p, C.c_void_p]
+    lib.nuq_level_histogram.argtypes = [C.c_void_p, C.c_uint64, C.c_uint32, C.c_uint32, C.c_uint32, C.c_uint64, C.c_uint64, C.c_void_p, C.c_void_p]
     lib.nuq_last_status.argtypes = [C.c_void_p]
     lib.fake_events.restype = C.c_char_p
     lib.fake_last_alloc.restype = C.c_void_p
@@ -85,3 +86,13 @@ def test_a_first_call_is_refused_inside_a_capture_and_works_behind_it(lib, call)
     lib.fake_reset()
     lib.fake_capture(1)
     assert call(lib) == 0 and "refused" not in lib.fake_events().decode()
+
+
+def test_norms_never_lie_where_an_encode_call_keeps_its_scan_state(lib):
+    """a replay of a captured call would leave them there, and the host would not know that the next call has to clear"""
+    hist = (C.c_uint64 * 8)()
+    assert _encode(lib, d=1 << 20, bucket=65536, kind=FIXED) == 0                       # wide buckets with 4-bit fields
+    assert lib.nuq_level_histogram(0x1000, 1 << 20, 256, 4, 0, 1, 0, C.addressof(hist), STREAM) == 0
+    assert _encode(lib, d=1 << 20, bucket=65536, kind=FIXED) == 0
+    where = [e for e in lib.fake_events().decode().splitlines() if e.startswith("norms")]
+    assert len(where) == 3 and not any("allocation 0" in e for e in where)              # (0 is the workspace)
