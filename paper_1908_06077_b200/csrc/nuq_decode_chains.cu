@@ -791,12 +791,9 @@ __global__ void __launch_bounds__(32 * kChainMaxWarps, 1) decode_chains_kernel(c
 
 template <class Sym>
 static cudaError_t launch_chains(const DecodeParams& P, int sms, cudaStream_t stream) {
-    static bool attr_set = false;
-    if (!attr_set) {
-        const cudaError_t e = cudaFuncSetAttribute(decode_chains_kernel<Sym>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kChainSmem);
-        if (e != cudaSuccess) return e;
-        attr_set = true;
-    }
+    static OncePerDevice prepared;
+    const cudaError_t e = prepared([] { return cudaFuncSetAttribute(decode_chains_kernel<Sym>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kChainSmem); });
+    if (e != cudaSuccess) return e;
     const size_t fixed = chain_fixed_bytes(P.K);
     size_t warps = (kChainSmem - fixed) / Row<Sym>::kWarpBytes;
     if (warps > kChainMaxWarps) warps = kChainMaxWarps;

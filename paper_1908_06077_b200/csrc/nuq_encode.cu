@@ -1290,17 +1290,15 @@ constexpr int kEncMaxDynSmem = 112 * 1024;
 
 template <uint32_t L, uint32_t M>
 static cudaError_t prepare_kernel() {
-    static bool attr_set = false;
-    if (attr_set) return cudaSuccess;
-    cudaError_t e = cudaFuncSetAttribute(encode_kernel<L, M, false, 8>, cudaFuncAttributeMaxDynamicSharedMemorySize, kEncMaxDynSmem);
-    if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(encode_kernel<L, M, true, 8>, cudaFuncAttributeMaxDynamicSharedMemorySize, kEncMaxDynSmem);
-    if (M == kModeErc && e == cudaSuccess)
-        e = cudaFuncSetAttribute(encode_kernel<L, kModeErc, false, kEncMaxWarps>, cudaFuncAttributeMaxDynamicSharedMemorySize, kEncMaxDynSmem);
-    if (M == kModeErc && e == cudaSuccess)
-        e = cudaFuncSetAttribute(encode_kernel<L, kModeErc, true, kEncMaxWarps>, cudaFuncAttributeMaxDynamicSharedMemorySize, kEncMaxDynSmem);
-    if (e == cudaSuccess) attr_set = true;
-    return e;
+    static OncePerDevice prepared;
+    return prepared([] {
+        constexpr cudaFuncAttribute kSmem = cudaFuncAttributeMaxDynamicSharedMemorySize;
+        cudaError_t e = cudaFuncSetAttribute(encode_kernel<L, M, false, 8>, kSmem, kEncMaxDynSmem);
+        if (e == cudaSuccess) e = cudaFuncSetAttribute(encode_kernel<L, M, true, 8>, kSmem, kEncMaxDynSmem);
+        if (M == kModeErc && e == cudaSuccess) e = cudaFuncSetAttribute(encode_kernel<L, kModeErc, false, kEncMaxWarps>, kSmem, kEncMaxDynSmem);
+        if (M == kModeErc && e == cudaSuccess) e = cudaFuncSetAttribute(encode_kernel<L, kModeErc, true, kEncMaxWarps>, kSmem, kEncMaxDynSmem);
+        return e;
+    });
 }
 
 template <uint32_t M>

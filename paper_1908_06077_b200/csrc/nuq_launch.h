@@ -3,9 +3,28 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <set>
+
 #include "nuq_common.cuh"
 
 namespace nuq {
+
+// Runs what has to be done once per device (a kernel's attributes are kept per device) before the first launch there.
+// Its callers hold the library's mutex.
+class OncePerDevice {
+    std::set<int> done_;
+
+public:
+    template <class F>
+    cudaError_t operator()(F&& prepare) {
+        int dev = 0;
+        cudaError_t e = cudaGetDevice(&dev);
+        if (e != cudaSuccess || done_.count(dev)) return e;
+        e = prepare();
+        if (e == cudaSuccess) done_.insert(dev);
+        return e;
+    }
+};
 
 void build_erc_lut(uint32_t* lut256);                 // ERC(N), N = 1..256: code | len << 16
 cudaError_t upload_erc_lut();                         // the encoder's tables, into the current device's memory; returns when they are there

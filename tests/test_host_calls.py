@@ -96,3 +96,16 @@ def test_norms_never_lie_where_an_encode_call_keeps_its_scan_state(lib):
     assert _encode(lib, d=1 << 20, bucket=65536, kind=FIXED) == 0
     where = [e for e in lib.fake_events().decode().splitlines() if e.startswith("norms")]
     assert len(where) == 3 and not any("allocation 0" in e for e in where)              # (0 is the workspace)
+
+
+@pytest.mark.parametrize("kind", [ERC, FIXED, 2 << 16, 1 << 8])
+@pytest.mark.parametrize("bucket", [512, 65536])
+def test_every_device_is_told_how_much_shared_memory_the_kernels_take(lib, kind, bucket):
+    """the runtime keeps that per device"""
+    lengths = (C.c_uint8 * 6)(1, 2, 3, 4, 5, 5)
+    assert lib.nuq_set_level_code(lengths, 5) == 0
+    for device in (0, 1, 0, 2):
+        lib.cudaSetDevice(device)
+        for d in (100000, 10000000):
+            assert _encode(lib, d=d, bucket=bucket, s=5, kind=kind) == 0 and _decode(lib, d=d, bucket=bucket, s=5) == 0
+            assert _decode(lib, d=d, bucket=bucket, s=7) == 0                           # (16-bit symbols)
