@@ -304,7 +304,6 @@ struct AddPass {
     uint32_t rows, norms;              // shared-memory addresses
     uint32_t S, streams;
     uint32_t alike;                    // all streams are tokens of exponential (0), uniform (1) or table (3) levels; else 2
-    bool exact;                        // norm times a power of two is exact for all the unit's norms
     bool last, carried;                // the last group of streams; sums of earlier groups are in `carry`
 };
 
@@ -772,7 +771,7 @@ __global__ void __launch_bounds__(32 * kChainMaxWarps, 1) decode_chains_kernel(c
 
         // ================= add =================
         const AddPass ap = {heads + g0, levels + g0 * kLevelBytes, smem_u32(codes) + g0 * kCodeBytes, rows, norms, S, gcount, exact ? all_alike : 2u,
-                            exact, group + 1u == ngroups, group != 0u};
+                            group + 1u == ngroups, group != 0u};
         const uint64_t e0 = unit * S * kSB + 4u * lane;
         uint32_t q0 = 0;
 #pragma unroll 1

@@ -151,23 +151,6 @@ __device__ __forceinline__ void or_bits(uint32_t* dst, uint32_t bitpos, uint64_t
     if (w2) atomicOr(dst + w + 2, w2);
 }
 
-// OR `nbits` (0..32) right-aligned bits of `value` into the MSB-first bit string `dst` at `bitpos`.
-// Two words are touched unconditionally (a zero is OR-ed when there is nothing to add).
-__device__ __forceinline__ void or_bits32(uint32_t* dst, uint32_t bitpos, uint32_t value, uint32_t nbits) {
-    const uint32_t a = nbits ? value << (32u - nbits) : 0u;
-    const uint32_t w = bitpos >> 5, sh = bitpos & 31u;
-    atomicOr(dst + w, a >> sh);
-    atomicOr(dst + w + 1, __funnelshift_r(0u, a, sh));
-}
-
-// OR the left-aligned bits of `a` (zero beyond its last bit) into the MSB-first bit string `dst` at
-// `bitpos`.  Two words are touched unconditionally (a zero is OR-ed when there is nothing to add).
-__device__ __forceinline__ void or_bits_left(uint32_t* dst, uint32_t bitpos, uint32_t a) {
-    const uint32_t w = bitpos >> 5, sh = bitpos & 31u;
-    atomicOr(dst + w, a >> sh);
-    atomicOr(dst + w + 1, __funnelshift_r(0u, a, sh));
-}
-
 // 32 bits of the MSB-first bit string `src` starting at bit `sbit` (>= -31); bits before
 // the string read as garbage and must be masked by the caller.
 __device__ __forceinline__ uint32_t bits_at(const uint32_t* src, int sbit) {
