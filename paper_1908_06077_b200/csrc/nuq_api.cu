@@ -593,19 +593,29 @@ static nuq_status enqueue_decode(const void* const* streams, uint32_t K, uint64_
         g_token_tables_ready.insert(dev);
     }
     P.unit_subs = 0;                                    // (chosen at the launch)
-    P.likely_table = kTabErc;
+    uint32_t fixed = 0, tokens = 0;                     // streams of each mode, as far as is known
+    P.likely_levels = kLevelsExp;
+    bool alike = true;
     for (uint32_t k = 0; k < K; ++k) {
-        auto it = g_container_mode.find(std::make_pair(dev, streams[k]));
+        const auto it = g_container_mode.find(std::make_pair(dev, streams[k]));
         const uint32_t mode = it == g_container_mode.end() ? kModeErc : it->second & 0xffu;
-        if (mode != kModeErc) P.likely_table = kTabCoded;
-        else if (k == 0 && it != g_container_mode.end() && it->second >> 8 == kLevelsUniform) P.likely_table = kTabUniform;
+        const uint32_t levels = it == g_container_mode.end() ? kLevelsExp : it->second >> 8;
+        fixed += mode == kModeFixed;
+        tokens += mode == kModeErc;
+        if (k == 0) P.likely_levels = levels;
+        alike = alike && levels == P.likely_levels;
     }
-    P.acc = acc;
-    P.w = w;
-    P.yl = w && mu != 0.0f ? yl : nullptr;
-    P.step_c = w ? (float)((double)alpha / (double)K) : 0.0f;          // one rounding each
-    P.step_lc = w ? (float)((double)l * (double)alpha / (double)K) : 0.0f;
-    P.mu = w ? mu : 0.0f;
+    // (what is known of an address may be out of date, also in s: tables are only prepared for level sets that exist)
+    const bool exists = P.likely_levels != kLevelsUniform || s <= 8u;
+    P.likely_table = kTabCoded;
+    if (exists && fixed == K && alike) P.likely_table = kTabFields;
+    else if (exists && tokens == K) P.likely_table = P.likely_levels == kLevelsUniform ? kTabUniform : kTabErc;
+    P.sum.acc = acc;
+    P.sum.w = w;
+    P.sum.yl = w && mu != 0.0f ? yl : nullptr;
+    P.sum.step_c = w ? (float)((double)alpha / (double)K) : 0.0f;          // one rounding each
+    P.sum.step_lc = w ? (float)((double)l * (double)alpha / (double)K) : 0.0f;
+    P.sum.mu = w ? mu : 0.0f;
     P.minus_zero = -0.0f;
     Workspace* ws = nullptr;
     nuq_status st = get_workspace(stream, sizeof(Workspace), &ws, &dev);

@@ -90,23 +90,30 @@ struct EncodeParams {
     uint32_t let_next;       // the kernel behind it may be launched while this one runs
 };
 
-// Token tables of the chain decoder: ERC level indices as exponential or as uniform levels, gaps alone, a fitted level code.
-enum : uint32_t { kTabErc = 0, kTabGaps = 1, kTabCoded = 2, kTabUniform = 3 };
+// Token tables of the chain decoder: ERC level indices as exponential or as uniform levels, gaps alone, a fitted level code;
+// fixed-width fields: no token table.
+enum : uint32_t { kTabErc = 0, kTabGaps = 1, kTabCoded = 2, kTabUniform = 3, kTabFields = 4 };
 
-struct DecodeParams {
-    Geometry geo;
-    const uint32_t* streams[kMaxK];
-    uint32_t K;
-    uint32_t unit_subs;      // token streams: sub-blocks a warp decodes at a time
-    uint32_t likely_table;   // the token table the call most likely needs (kTabErc, kTabUniform), or kTabCoded: none to prepare (a level code of the streams' own, or no tokens)
-    uint32_t let_next;       // token streams: the kernel behind may be launched early
-    // the aggregation step fused into the decoder (w == nullptr: none): see step_value in nuq_decode_common.cuh
+// What becomes of a finished sum: see step_value in nuq_decode_common.cuh.
+struct SumParams {
+    float* acc;              // where it is stored (may be nullptr when there are parameters)
+    // the aggregation step fused into the decoder (w == nullptr: none)
     float* w;                // parameters, updated in place
     float* yl;               // the momentum rule's y^l, updated in place (not touched when mu == 0)
     float step_c, step_lc;   // alpha / K and l alpha / K
     float mu;
+};
+
+struct DecodeParams {
+    Geometry geo;
+    SumParams sum;
+    const uint32_t* streams[kMaxK];
+    uint32_t K;
+    uint32_t unit_subs;      // token streams: sub-blocks a warp decodes at a time
+    uint32_t likely_table;   // the table the call most likely needs (kTabErc, kTabUniform, kTabFields), or kTabCoded: none to prepare (a level code of the streams' own, or streams of several kinds)
+    uint32_t likely_levels;  // ... and the level set of its fields (kTabFields)
+    uint32_t let_next;       // token streams: the kernel behind may be launched early
     float minus_zero;        // -0.0f, which the compiler must not know (see product2 in nuq_decode_common.cuh)
-    float* acc;
     Workspace* ws;
 };
 

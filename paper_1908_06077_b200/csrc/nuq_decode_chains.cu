@@ -30,6 +30,8 @@
 //
 // The copy of the next unit's chains runs during the add pass, the block offsets of the one after that
 // are on their way during the walk.  16 warps fit an SM (12 KB each: rows, chain copies).
+#include <map>
+
 #include "nuq_async.cuh"
 #include "nuq_decode_common.cuh"
 #include "nuq_decode_fields.cuh"
@@ -308,14 +310,14 @@ struct AddPass {
 };
 
 // NB sub-blocks from sub-block q0 of the unit on; e: the lane's first element, 128 more for each half of a sub-block.
-template <class Sym, int NB>
+template <class Sym, int NB, bool MANY>
 __device__ __forceinline__ void add_block(const DecodeParams& P, const AddPass& A, uint32_t q0, uint64_t e, uint64_t (&carry)[4]) {
     const Geometry& G = P.geo;
     const uint32_t lane = lane_id(), s = G.s;
     uint64_t sum[4 * NB];                                   // two halves of each, four elements in two pairs
 #pragma unroll
     for (int i = 0; i < 4 * NB; ++i) sum[i] = 0;
-    if (NB == 1 && A.carried) {
+    if (MANY && NB == 1 && A.carried) {
 #pragma unroll
         for (int i = 0; i < 4; ++i) sum[i] = carry[i];
     }
@@ -405,7 +407,7 @@ __device__ __forceinline__ void add_block(const DecodeParams& P, const AddPass& 
             }
         }
     }
-    if (NB == 1 && !A.last) {
+    if (MANY && NB == 1 && !A.last) {
 #pragma unroll
         for (int i = 0; i < 4; ++i) carry[i] = sum[i];
         return;
@@ -415,9 +417,9 @@ __device__ __forceinline__ void add_block(const DecodeParams& P, const AddPass& 
         return make_float4(a.x, a.y, b.x, b.y);
     };
     if (e + 128u * (2 * NB - 1) + 4u <= G.d) {
-        if (P.w == nullptr) {
+        if (P.sum.w == nullptr) {
 #pragma unroll
-            for (int h = 0; h < 2 * NB; ++h) *reinterpret_cast<float4*>(P.acc + e + 128 * h) = value(h);
+            for (int h = 0; h < 2 * NB; ++h) *reinterpret_cast<float4*>(P.sum.acc + e + 128 * h) = value(h);
         } else {
             constexpr int kAtOnce = NB == 1 ? 2 : 4;        // the loads of four steps are on their way together
 #pragma unroll
@@ -425,19 +427,19 @@ __device__ __forceinline__ void add_block(const DecodeParams& P, const AddPass& 
                 float4 w[kAtOnce], yl[kAtOnce];
 #pragma unroll
                 for (int h = 0; h < kAtOnce; ++h) {
-                    w[h] = *reinterpret_cast<const float4*>(P.w + e + 128 * (h0 + h));
-                    yl[h] = P.mu != 0.0f ? *reinterpret_cast<const float4*>(P.yl + e + 128 * (h0 + h)) : make_float4(0.f, 0.f, 0.f, 0.f);
+                    w[h] = *reinterpret_cast<const float4*>(P.sum.w + e + 128 * (h0 + h));
+                    yl[h] = P.sum.mu != 0.0f ? *reinterpret_cast<const float4*>(P.sum.yl + e + 128 * (h0 + h)) : make_float4(0.f, 0.f, 0.f, 0.f);
                 }
 #pragma unroll
-                for (int h = 0; h < kAtOnce; ++h) step4(P, e + 128 * (h0 + h), value(h0 + h), w[h], yl[h]);
+                for (int h = 0; h < kAtOnce; ++h) step4(P.sum, e + 128 * (h0 + h), value(h0 + h), w[h], yl[h]);
             }
         }
     } else {                                                // the end of the vector
 #pragma unroll
         for (int h = 0; h < 2 * NB; ++h) {
             const uint64_t at_h = e + 128u * h;
-            if (at_h + 4u <= G.d) finish4(P, at_h, value(h));
-            else if (at_h < G.d) finish_part(P, at_h, value(h), (uint32_t)(G.d - at_h));
+            if (at_h + 4u <= G.d) finish4(P.sum, at_h, value(h));
+            else if (at_h < G.d) finish_part(P.sum, at_h, value(h), (uint32_t)(G.d - at_h));
         }
     }
 }
@@ -448,38 +450,59 @@ __host__ __device__ inline size_t chain_fixed_bytes(uint32_t K) {
     return (4u * kTokEntries + 256u + (size_t)K * (kCodeBytes + kLevelBytes + sizeof(StreamHead)) + 15u) & ~(size_t)15u;
 }
 
+// Where things lie in it.
+template <class Sym>
+struct Layout {
+    unsigned char* codes;
+    unsigned char* levels;
+    StreamHead* heads;
+    unsigned char* field_tables;                            // fixed-width streams: where the token table would be, a multiple of 4096
+    uint32_t rows;                                          // the warp's own
+    __device__ __forceinline__ Layout(unsigned char* dsm, uint32_t K) {
+        const uint32_t base = smem_u32(dsm);
+        codes = dsm + 4u * kTokEntries + (0u - base & 255u);
+        levels = codes + K * kCodeBytes;
+        heads = reinterpret_cast<StreamHead*>(levels + K * kLevelBytes);
+        field_tables = dsm + ((base + 4095u & ~4095u) - base);
+        rows = base + (uint32_t)chain_fixed_bytes(K) + (threadIdx.x >> 5) * Row<Sym>::kWarpBytes;
+    }
+};
+
 // All streams in the fixed-width mode.  (16-bit symbols: s = 7 or 8, hence fields of 5 bits, or of 9 and 10 with uniform levels.)
 template <class Sym>
-__device__ __forceinline__ void fields_of_width(const DecodeParams& P, const StreamHead* heads, uint32_t tables, uint32_t mine, uint32_t width) {
+__device__ __forceinline__ void fields_of_width(const DecodeParams& P, const StreamHead* heads, unsigned char* tables, uint32_t mine, uint32_t width) {
     if (heads[0].levelset == kLevelsExp) {
-        if (width == 5u) return decode_fields<5, true>(P, heads, tables, mine);
-        if (sizeof(Sym) == 1 && width == 4u) return decode_fields<4, true>(P, heads, tables, mine);
-        if (sizeof(Sym) == 1 && width == 3u) return decode_fields<3, true>(P, heads, tables, mine);
+        if (width == 5u) return decode_fields_call<5, true>(P, heads, tables, false, mine);
+        if (sizeof(Sym) == 1 && width == 4u) return decode_fields_call<4, true>(P, heads, tables, false, mine);
+        if (sizeof(Sym) == 1 && width == 3u) return decode_fields_call<3, true>(P, heads, tables, false, mine);
     }
-    if (width == 5u) return decode_fields<5, false>(P, heads, tables, mine);
+    if (width == 5u) return decode_fields_call<5, false>(P, heads, tables, false, mine);
     if (sizeof(Sym) == 1) {
-        if (width == 3u) return decode_fields<3, false>(P, heads, tables, mine);
-        if (width == 4u) return decode_fields<4, false>(P, heads, tables, mine);
-        if (width == 6u) return decode_fields<6, false>(P, heads, tables, mine);
-        if (width == 7u) return decode_fields<7, false>(P, heads, tables, mine);
-        if (width == 8u) return decode_fields<8, false>(P, heads, tables, mine);
+        if (width == 3u) return decode_fields_call<3, false>(P, heads, tables, false, mine);
+        if (width == 4u) return decode_fields_call<4, false>(P, heads, tables, false, mine);
+        if (width == 6u) return decode_fields_call<6, false>(P, heads, tables, false, mine);
+        if (width == 7u) return decode_fields_call<7, false>(P, heads, tables, false, mine);
+        if (width == 8u) return decode_fields_call<8, false>(P, heads, tables, false, mine);
     } else {
-        if (width == 9u) return decode_fields<9, false>(P, heads, tables, mine);
-        if (width == 10u) return decode_fields<10, false>(P, heads, tables, mine);
+        if (width == 9u) return decode_fields_call<9, false>(P, heads, tables, false, mine);
+        if (width == 10u) return decode_fields_call<10, false>(P, heads, tables, false, mine);
     }
 }
 
-template <class Sym>
-__global__ void __launch_bounds__(32 * kChainMaxWarps, 1) decode_chains_kernel(const __grid_constant__ DecodeParams P) {
+// Streams of any kind.  MANY: more than 32 of them, in groups (the sums of a unit are kept in registers from group to group:
+// an instance of its own, since these and the counters of groups cost the common one 2 % of its time in the walk).
+// CALLED: from the kernel for fixed-width streams, where those the call was made for are not; fields are then added one by one.
+template <class Sym, bool MANY, bool CALLED>
+__device__ __forceinline__ void decode_streams(const DecodeParams& P) {
     extern __shared__ __align__(128) unsigned char dsm[];
     __shared__ uint32_t s_kind, s_alike, s_fields;
     const Geometry& G = P.geo;
     const uint32_t K = P.K, tid = threadIdx.x, lane = tid & 31u, warp = tid >> 5;
     uint32_t* const table = reinterpret_cast<uint32_t*>(dsm);
-    unsigned char* const codes = dsm + 4u * kTokEntries + (0u - smem_u32(dsm) & 255u);
-    unsigned char* const levels = codes + K * kCodeBytes;
-    StreamHead* const heads = reinterpret_cast<StreamHead*>(levels + K * kLevelBytes);
-    const uint32_t rows = smem_u32(dsm) + (uint32_t)chain_fixed_bytes(K) + warp * Row<Sym>::kWarpBytes;
+    const Layout<Sym> at(dsm, K);
+    unsigned char *const codes = at.codes, *const levels = at.levels;
+    StreamHead* const heads = at.heads;
+    const uint32_t rows = at.rows;
     const uint32_t norms = rows + 32u * Row<Sym>::kPitch;   // one per lane's chain
     const uint32_t copy = norms + 128u + lane * (4u * kChunkWords);   // this lane's words of its chain
 
@@ -522,56 +545,64 @@ __global__ void __launch_bounds__(32 * kChainMaxWarps, 1) decode_chains_kernel(c
     // Nothing before the wait touches memory that another kernel writes.  The kernel behind is let in early only by calls
     // that give every warp several units: a small encode call let in early finds room only where CTAs of this kernel have
     // left and is packed onto a few SMs, four CTAs each (a step of 10^6 elements, K = 3: 66 -> 74 us).
-    if (P.let_next) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-    if (P.likely_table != kTabCoded) build_table(P.likely_table, nullptr);
-    clear_rows();
-    asm volatile("griddepcontrol.wait;" ::: "memory");
+    if (!CALLED) {
+        if (P.let_next) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+        if (P.likely_table == kTabErc || P.likely_table == kTabUniform) build_table(P.likely_table, nullptr);
+        clear_rows();
+        asm volatile("griddepcontrol.wait;" ::: "memory");
+    }
 
     // ---- headers against the call's arguments, once per stream; then what kind of table serves all the token streams ----
-    for (uint32_t k = tid; k < K; k += blockDim.x) {
-        heads[k] = read_head(G, P.streams[k]);
-        if (!heads[k].ok) latch_status(P.ws, kErrBadStream);
-    }
-    __syncthreads();
     if (warp == 0) {
-        bool coded = false, erc = false, uniform = false, other = false, tabled = false, odd = false, same_code = true, fields = true;
+        enum : uint32_t { kCoded = 1, kErc = 2, kUniform = 4, kOther = 8, kTabled = 16, kOdd = 32, kNotFields = 64, kSeveralCodes = 128 };
+        uint32_t found = 0;                                 // of these, among the streams
         uint32_t first0 = 0, first1 = 0;                    // the code lengths of the first coded stream
+        uint32_t levels0 = 0, width0 = 0;                   // of the first stream
         for (uint32_t k0 = 0; k0 < K; k0 += 32u) {
             const uint32_t k = k0 + lane;
-            const bool tokens = k < K && heads[k].ok && heads[k].mode != kModeFixed, in_code = tokens && heads[k].mode == kModeCoded;
-            uint32_t w0 = 0, w1 = 0;
-            if (in_code) {
-                w0 = heads[k].hdr[heads[k].hwords - 2u];
-                w1 = heads[k].hdr[heads[k].hwords - 1u];
+            StreamHead hd = {};
+            if (k < K) {
+                heads[k] = hd = read_head(G, P.streams[k]);
+                if (!hd.ok) latch_status(P.ws, kErrBadStream);
             }
-            const uint32_t with_code = __ballot_sync(0xffffffffu, in_code);
-            if (with_code && !coded) {
-                first0 = __shfl_sync(0xffffffffu, w0, __ffs((int)with_code) - 1);
-                first1 = __shfl_sync(0xffffffffu, w1, __ffs((int)with_code) - 1);
-                coded = true;
+            if (k0 == 0u) {
+                levels0 = __shfl_sync(0xffffffffu, hd.levelset, 0);
+                width0 = __shfl_sync(0xffffffffu, hd.width, 0);
             }
-            same_code = same_code && !__any_sync(0xffffffffu, in_code && (w0 != first0 || w1 != first1));
-            erc = erc || __any_sync(0xffffffffu, tokens && !in_code);
-            uniform = uniform || __any_sync(0xffffffffu, tokens && heads[k].levelset == kLevelsUniform);
-            other = other || __any_sync(0xffffffffu, tokens && heads[k].levelset != kLevelsUniform);
-            tabled = tabled || __any_sync(0xffffffffu, tokens && heads[k].levelset == kLevelsTable);
-            odd = odd || __any_sync(0xffffffffu, k < K && (!tokens || heads[k].levelset != heads[0].levelset));
-            fields = fields && __all_sync(0xffffffffu, k >= K || (heads[k].ok && heads[k].mode == kModeFixed && heads[k].levelset == heads[0].levelset));
+            const bool tokens = hd.ok && hd.mode != kModeFixed, in_code = tokens && hd.mode == kModeCoded;
+            uint32_t mine = 0;
+            if (tokens) mine = (in_code ? kCoded : kErc) | (hd.levelset == kLevelsUniform ? kUniform : kOther) | (hd.levelset == kLevelsTable ? kTabled : 0u);
+            if (k < K && (!tokens || hd.levelset != levels0)) mine |= kOdd;
+            if (k < K && !(hd.ok && hd.mode == kModeFixed && hd.levelset == levels0)) mine |= kNotFields;
+            const uint32_t had = found;
+            found |= __reduce_or_sync(0xffffffffu, mine);
+            if (found & kCoded) {
+                uint32_t w0 = 0, w1 = 0;
+                if (in_code) {
+                    w0 = hd.hdr[hd.hwords - 2u];
+                    w1 = hd.hdr[hd.hwords - 1u];
+                }
+                if (!(had & kCoded)) {
+                    const int first = __ffs((int)__ballot_sync(0xffffffffu, in_code)) - 1;
+                    first0 = __shfl_sync(0xffffffffu, w0, first);
+                    first1 = __shfl_sync(0xffffffffu, w1, first);
+                }
+                if (__any_sync(0xffffffffu, in_code && (w0 != first0 || w1 != first1))) found |= kSeveralCodes;
+            }
         }
         if (lane == 0) {
-            s_kind = coded ? (erc || !same_code ? kTabGaps : kTabCoded) : uniform ? (other ? kTabGaps : kTabUniform) : kTabErc;
-            s_alike = odd ? 2u : uniform ? 1u : tabled ? 3u : 0u;
-            s_fields = fields ? heads[0].width : 0u;
+            s_kind = found & kCoded ? (found & (kErc | kSeveralCodes) ? kTabGaps : kTabCoded)
+                     : found & kUniform ? (found & kOther ? kTabGaps : kTabUniform) : kTabErc;
+            s_alike = found & kOdd ? 2u : found & kUniform ? 1u : found & kTabled ? 3u : 0u;
+            s_fields = found & kNotFields ? 0u : width0;
         }
     }
     __syncthreads();
-    if (s_fields != 0u) {                                   // no tokens at all
-        const uint32_t tables = (smem_u32(dsm) + 4095u) & ~4095u;               // where the token table would be
-        build_field_tables(G, heads, K, dsm + (tables - smem_u32(dsm)));
-        __syncthreads();
-        fields_of_width<Sym>(P, heads, tables, rows, s_fields);
+    if (!CALLED && s_fields != 0u) {                        // no tokens at all
+        fields_of_width<Sym>(P, heads, at.field_tables, rows, s_fields);
         return;
     }
+    if (CALLED) clear_rows();
     const uint32_t kind = s_kind, all_alike = s_alike == 3u && s_kind == kTabGaps ? 2u : s_alike;
     if (kind != P.likely_table || kind == kTabGaps || kind == kTabCoded || all_alike >= 2u) {
         uint32_t first = K;                                 // the first token stream (all have the same code in the coded mode)
@@ -608,42 +639,39 @@ __global__ void __launch_bounds__(32 * kChainMaxWarps, 1) decode_chains_kernel(c
 
     const uint32_t tab = smem_u32(table);
     const uint32_t S = P.unit_subs;                         // sub-blocks of a unit
-    const uint64_t nsub = (G.d + kSB - 1u) / kSB, nunits = (nsub + S - 1u) / S, stride = (uint64_t)gridDim.x * (blockDim.x >> 5);
+    const uint32_t nsub = (uint32_t)((G.d + kSB - 1u) / kSB), nunits = (uint32_t)(((uint64_t)nsub + S - 1u) / S), stride = gridDim.x * (blockDim.x >> 5);
     const uint32_t spb = G.bucket <= kBLK ? G.sb_per_block : 32u;   // sub-blocks of a coding block
     const uint32_t lj = lane / S, lq = lane - lj * S;
-    const uint32_t ngroups = (K + 31u) / 32u;               // of up to 32 streams (S = 1 when there are several)
+    const uint32_t ngroups = MANY ? (K + 31u) / 32u : 1u;   // of up to 32 streams (S = 1 when there are several)
 
     // An item is a unit of a group of streams.  The block offsets of an item's chains ...
     struct Offsets {
         uint64_t from, to;
     };
-    auto load_offsets = [&](uint64_t unit, uint32_t g0) {
+    auto load_offsets = [&](uint32_t unit, uint32_t g0) {
         Offsets o;
         o.from = o.to = 0;
-        const uint64_t sub = unit * S + lq;
-        const uint32_t k = g0 + lj;
+        const uint32_t sub = unit * S + lq, k = g0 + lj;    // (below 2^32 for units that exist: there are fewer sub-blocks)
         if (unit < nunits && sub < nsub && k < K && lj * S + lq < 32u && heads[k].ok && heads[k].mode != kModeFixed) {
-            const uint64_t* at = reinterpret_cast<const uint64_t*>(heads[k].hdr + heads[k].hwords) + (uint32_t)sub / spb;
+            const uint64_t* at = reinterpret_cast<const uint64_t*>(heads[k].hdr + heads[k].hwords) + sub / spb;
             o.from = at[0];
             o.to = at[1];
         }
         return o;
     };
     // ... and, from them, where this lane's chain lies: the lengths of the sub-blocks before it in its block
-    auto describe = [&](uint64_t unit, uint32_t g0, const Offsets& o) {
+    auto describe = [&](uint32_t unit, uint32_t g0, const Offsets& o) {
         Chain ch;
         ch.src = nullptr;
         ch.left = 0;
         ch.bit = ch.len = 0;
         ch.norm = 0.0f;
         ch.good = true;
-        const uint64_t sub = unit * S + lq;
-        const uint32_t k = g0 + lj;
+        const uint32_t sub = unit * S + lq, k = g0 + lj;
         if (unit < nunits && sub < nsub && k < K && heads[k].ok && heads[k].mode != kModeFixed) {
             const StreamHead& hd = heads[k];
-            const uint32_t blk = (uint32_t)sub / spb, sbi = (uint32_t)sub - blk * spb;
-            const uint64_t in_blk = nsub - (uint64_t)blk * spb;
-            const uint32_t nsb_blk = in_blk < spb ? (uint32_t)in_blk : spb, head_words = 1u + (nsb_blk + 1u) / 2u;
+            const uint32_t blk = sub / spb, sbi = sub - blk * spb;
+            const uint32_t nsb_blk = min(nsub - blk * spb, spb), head_words = 1u + (nsb_blk + 1u) / 2u;
             const uint64_t head = hd.hwords + 2 * (G.nblk + 1), words = (o.to - o.from) >> 5;
             ch.good = ((o.from | o.to) & 31u) == 0 && o.from < o.to && (o.to >> 5) <= hd.cwords - head &&
                       words >= head_words && words <= (1u << 20);
@@ -688,13 +716,12 @@ __global__ void __launch_bounds__(32 * kChainMaxWarps, 1) decode_chains_kernel(c
     // the whole of the lane's chain is in its copy, with room for the ones behind it
     auto fits = [&](const Chain& ch) { return (ch.bit + ch.len + 31u) / 32u + kChunkSlack <= kChunkWords; };
 
-    uint64_t unit = (uint64_t)warp * gridDim.x + blockIdx.x, unit1 = unit;
+    uint32_t unit = warp * gridDim.x + blockIdx.x, unit1 = unit;
     uint32_t group = 0, group1 = 0;
-    auto advance = [&](uint64_t& u, uint32_t& g) {
-        if (++g == ngroups) {
-            g = 0;
-            u += stride;
-        }
+    auto advance = [&](uint32_t& u, uint32_t& g) {          // (behind the last unit u stays there: nunits + stride may pass 2^32)
+        if (MANY && ++g != ngroups) return;
+        g = 0;
+        u = u < nunits && nunits - u > stride ? u + stride : nunits;
     };
     Chain ch = describe(unit, 0, load_offsets(unit, 0));
     start_copy(ch);
@@ -702,16 +729,15 @@ __global__ void __launch_bounds__(32 * kChainMaxWarps, 1) decode_chains_kernel(c
     Offsets next = load_offsets(unit1, 32u * group1);
     uint64_t carry[4] = {0, 0, 0, 0};                       // sums of the groups of streams before this one (S = 1)
     while (unit < nunits) {
-        uint64_t unit2 = unit1;
-        uint32_t group2 = group1;
+        uint32_t unit2 = unit1, group2 = group1;
         advance(unit2, group2);
         const Offsets next2 = load_offsets(unit2, 32u * group2);
         const uint32_t g0 = 32u * group, gcount = min(K - g0, 32u);
-        if (P.w != nullptr && group == 0u) {                // the parameters the add pass will read and write
-            const uint64_t first = unit * S * kSB, left = G.d - first;
+        if (P.sum.w != nullptr && group == 0u) {                // the parameters the add pass will read and write
+            const uint64_t first = (uint64_t)(unit * S) * kSB, left = G.d - first;
             const uint32_t bytes = 4u * ((left < S * kSB ? (uint32_t)left : S * kSB) & ~3u);
-            if (bytes && lane < (P.mu != 0.0f ? 2u : 1u))
-                asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"((lane == 0u ? P.w : P.yl) + first), "r"(bytes) : "memory");
+            if (bytes && lane < (P.sum.mu != 0.0f ? 2u : 1u))
+                asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"((lane == 0u ? P.sum.w : P.sum.yl) + first), "r"(bytes) : "memory");
         }
         asm volatile("cp.async.wait_group 0;" ::: "memory");
 
@@ -771,13 +797,13 @@ __global__ void __launch_bounds__(32 * kChainMaxWarps, 1) decode_chains_kernel(c
 
         // ================= add =================
         const AddPass ap = {heads + g0, levels + g0 * kLevelBytes, smem_u32(codes) + g0 * kCodeBytes, rows, norms, S, gcount, exact ? all_alike : 2u,
-                            group + 1u == ngroups, group != 0u};
-        const uint64_t e0 = unit * S * kSB + 4u * lane;
+                            !MANY || group + 1u == ngroups, MANY && group != 0u};
+        const uint64_t e0 = (uint64_t)(unit * S) * kSB + 4u * lane;
         uint32_t q0 = 0;
 #pragma unroll 1
-        for (; q0 + 4u <= S; q0 += 4u) add_block<Sym, 4>(P, ap, q0, e0 + 256u * q0, carry);
+        for (; q0 + 4u <= S; q0 += 4u) add_block<Sym, 4, MANY>(P, ap, q0, e0 + 256u * q0, carry);
 #pragma unroll 1
-        for (; q0 < S; ++q0) add_block<Sym, 1>(P, ap, q0, e0 + 256u * q0, carry);
+        for (; q0 < S; ++q0) add_block<Sym, 1, MANY>(P, ap, q0, e0 + 256u * q0, carry);
         __syncwarp();
         clear_rows();
         __syncwarp();
@@ -788,10 +814,69 @@ __global__ void __launch_bounds__(32 * kChainMaxWarps, 1) decode_chains_kernel(c
     }
 }
 
+template <class Sym, bool MANY>
+__global__ void __launch_bounds__(32 * kChainMaxWarps, 1) decode_chains_kernel(const __grid_constant__ DecodeParams P) {
+    decode_streams<Sym, MANY, false>(P);
+}
+
+template <class Sym>
+__device__ __noinline__ void decode_streams_call(const DecodeParams& P) {
+    decode_streams<Sym, true, true>(P);
+}
+
+// Calls whose streams are likely all in the fixed-width mode, with fields of W bits of one level set: a kernel of its own for
+// each, so that neither its registers nor its code are shared with the walks of token streams.  25.6 x 10^6 elements, K = 8, 4
+// bits, in one kernel with the walks: 67.6 us behind eight encode calls (where the code has to be fetched), 53.6 us repeated;
+// here 56 and 52 us.  Of that, headers are read 1.4 us behind the wait (the table stands ready then), the first bytes are there
+// after 4 us and the code of an item, its sums and its copies has been fetched after 2 more.
+template <uint32_t W, bool EXACT>
+__global__ void __launch_bounds__(32 * kChainMaxWarps, 1) decode_fields_kernel(const __grid_constant__ DecodeParams P) {
+    extern __shared__ __align__(128) unsigned char dsm[];
+    __shared__ uint32_t s_likely;
+    const uint32_t K = P.K, lane = lane_id();
+    const bool wide_symbols = P.geo.s == 7u || P.geo.s == 8u;
+    const Layout<int8_t> at(dsm, K);
+    if (P.let_next) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    const bool tables_ready = P.likely_levels != kLevelsTable;
+    if (tables_ready) build_field_tables(P.geo, P.likely_levels, nullptr, 1u, at.field_tables);
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    if (threadIdx.x < 32u) {
+        bool likely = true;
+        for (uint32_t k = lane; k < K; k += 32u) {
+            const StreamHead hd = read_head(P.geo, P.streams[k]);
+            at.heads[k] = hd;
+            likely = likely && hd.ok && hd.mode == kModeFixed && hd.levelset == P.likely_levels;
+        }
+        likely = __all_sync(0xffffffffu, likely);
+        if (lane == 0) s_likely = likely;
+    }
+    __syncthreads();
+    if (s_likely) {
+        const uint32_t mine = wide_symbols ? Layout<int16_t>(dsm, K).rows : at.rows;
+        decode_fields<W, EXACT, true>(P, at.heads, at.field_tables, tables_ready, mine);
+    } else if (wide_symbols) {                              // another kind of streams after all
+        decode_streams_call<int16_t>(P);
+    } else {
+        decode_streams_call<int8_t>(P);
+    }
+}
+
+using DecodeKernel = void (*)(DecodeParams);
+// (level tables and exponential levels: s + 2 of them; uniform levels: 2^s + 1, s <= 8)
+static DecodeKernel fields_kernel(uint32_t s, uint32_t levelset) {
+    if (levelset == kLevelsExp) return s <= 2u ? decode_fields_kernel<3, true> : s <= 6u ? decode_fields_kernel<4, true> : decode_fields_kernel<5, true>;
+    const uint32_t width = levelset == kLevelsUniform ? s + 2u : s <= 2u ? 3u : s <= 6u ? 4u : 5u;
+    static const DecodeKernel by_width[] = {decode_fields_kernel<3, false>, decode_fields_kernel<4, false>, decode_fields_kernel<5, false>, decode_fields_kernel<6, false>,
+                                            decode_fields_kernel<7, false>, decode_fields_kernel<8, false>, decode_fields_kernel<9, false>, decode_fields_kernel<10, false>};
+    return by_width[width - 3u];
+}
+
 template <class Sym>
 static cudaError_t launch_chains(const DecodeParams& P, int sms, cudaStream_t stream) {
-    static OncePerDevice prepared;
-    const cudaError_t e = prepared([] { return cudaFuncSetAttribute(decode_chains_kernel<Sym>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kChainSmem); });
+    const DecodeKernel kernel = P.likely_table == kTabFields ? fields_kernel(P.geo.s, P.likely_levels)
+                                : P.K > 32u ? decode_chains_kernel<Sym, true> : decode_chains_kernel<Sym, false>;
+    static std::map<DecodeKernel, OncePerDevice> prepared;
+    const cudaError_t e = prepared[kernel]([=] { return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kChainSmem); });
     if (e != cudaSuccess) return e;
     const size_t fixed = chain_fixed_bytes(P.K);
     size_t warps = (kChainSmem - fixed) / Row<Sym>::kWarpBytes;
@@ -815,7 +900,7 @@ static cudaError_t launch_chains(const DecodeParams& P, int sms, cudaStream_t st
     cfg.numAttrs = 1;
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
-    return cudaLaunchKernelEx(&cfg, decode_chains_kernel<Sym>, Q);
+    return cudaLaunchKernelEx(&cfg, kernel, Q);
 }
 
 cudaError_t launch_decode(const DecodeParams& P, int sms, cudaStream_t stream) {

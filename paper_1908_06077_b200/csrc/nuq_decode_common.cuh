@@ -23,7 +23,7 @@ __device__ __forceinline__ float level_times_norm(float norm, uint32_t levelset,
 // (Sec. 4, "NUQSGD with momentum"; mu = 0 is Algorithm 1's own line and leaves y^l alone).  fp32, each line
 // one fused multiply-add.
 // ---------------------------------------------------------------------------
-__device__ __forceinline__ float step_value(const DecodeParams& P, float w, float G, float* yl) {
+__device__ __forceinline__ float step_value(const SumParams& P, float w, float G, float* yl) {
     const float y = __fmaf_rn(-P.step_c, G, w);
     if (P.mu == 0.0f) return y;
     const float yl_next = __fmaf_rn(-P.step_lc, G, w);
@@ -32,7 +32,7 @@ __device__ __forceinline__ float step_value(const DecodeParams& P, float w, floa
     return w_next;
 }
 // element e (a multiple of 4) and the three behind it, with the parameters and y^l as they were
-__device__ __forceinline__ void step4(const DecodeParams& P, uint64_t e, float4 G, float4 w, float4 yl) {
+__device__ __forceinline__ void step4(const SumParams& P, uint64_t e, float4 G, float4 w, float4 yl) {
     if (P.acc) *reinterpret_cast<float4*>(P.acc + e) = G;
     w.x = step_value(P, w.x, G.x, &yl.x);
     w.y = step_value(P, w.y, G.y, &yl.y);
@@ -41,7 +41,7 @@ __device__ __forceinline__ void step4(const DecodeParams& P, uint64_t e, float4 
     *reinterpret_cast<float4*>(P.w + e) = w;
     if (P.mu != 0.0f) *reinterpret_cast<float4*>(P.yl + e) = yl;
 }
-__device__ __forceinline__ void finish4(const DecodeParams& P, uint64_t e, float4 G) {
+__device__ __forceinline__ void finish4(const SumParams& P, uint64_t e, float4 G) {
     if (!P.w) {
         *reinterpret_cast<float4*>(P.acc + e) = G;
         return;
@@ -51,7 +51,7 @@ __device__ __forceinline__ void finish4(const DecodeParams& P, uint64_t e, float
     if (P.mu != 0.0f) yl = *reinterpret_cast<const float4*>(P.yl + e);
     step4(P, e, G, w, yl);
 }
-__device__ __forceinline__ void finish1(const DecodeParams& P, uint64_t e, float G) {
+__device__ __forceinline__ void finish1(const SumParams& P, uint64_t e, float G) {
     if (P.acc) P.acc[e] = G;
     if (P.w) {
         float yl = P.mu != 0.0f ? P.yl[e] : 0.0f;
@@ -61,7 +61,7 @@ __device__ __forceinline__ void finish1(const DecodeParams& P, uint64_t e, float
 }
 
 // the first n < 4 elements from e on
-__device__ __forceinline__ void finish_part(const DecodeParams& P, uint64_t e, float4 G, uint32_t n) {
+__device__ __forceinline__ void finish_part(const SumParams& P, uint64_t e, float4 G, uint32_t n) {
     if (n > 0u) finish1(P, e, G.x);
     if (n > 1u) finish1(P, e + 1, G.y);
     if (n > 2u) finish1(P, e + 2, G.z);
@@ -75,17 +75,23 @@ struct StreamHead {
     uint32_t hwords;         // header words: 16, plus the level table of a level-table stream
 };
 
-// A container's header checked against the call's arguments.
+// Levels of a level set (zero included) and the bits of a fixed-width field: sign and level index.
+__device__ __forceinline__ uint32_t level_count(uint32_t levelset, uint32_t s) { return levelset == kLevelsUniform ? (1u << s) + 1u : s + 2u; }
+__device__ __forceinline__ uint32_t field_width(uint32_t nlev) { return 1u + (32u - __clz(nlev - 1u)); }
+
+// A container's header checked against the call's arguments.  Its words are loaded at once: the checks would otherwise
+// wait for one word after the other.
 __device__ __forceinline__ StreamHead read_head(const Geometry& G, const uint32_t* hdr) {
-    const uint32_t flags = hdr[6];
+    const uint4 a = *reinterpret_cast<const uint4*>(hdr), b = *reinterpret_cast<const uint4*>(hdr + 4), c = *reinterpret_cast<const uint4*>(hdr + 8);
+    const uint32_t flags = b.z;
     const uint32_t levelset = (flags >> 8) & 0xffu, mode = (flags >> 16) & 0xffu;
-    const uint64_t hd = (uint64_t)hdr[2] | ((uint64_t)hdr[3] << 32);
-    const uint64_t hnblk = (uint64_t)hdr[8] | ((uint64_t)hdr[9] << 32);
-    const uint64_t cbits = (uint64_t)hdr[10] | ((uint64_t)hdr[11] << 32);
-    bool ok = hdr[0] == kMagic && hdr[1] == kVersion && hd == G.d && hdr[4] == G.bucket &&
-              hdr[5] == G.s && hdr[7] == kSB && levelset <= 2u && mode <= 2u &&
+    const uint64_t hd = (uint64_t)a.z | ((uint64_t)a.w << 32);
+    const uint64_t hnblk = (uint64_t)c.x | ((uint64_t)c.y << 32);
+    const uint64_t cbits = (uint64_t)c.z | ((uint64_t)c.w << 32);
+    bool ok = a.x == kMagic && a.y == kVersion && hd == G.d && b.x == G.bucket &&
+              b.y == G.s && b.w == kSB && levelset <= 2u && mode <= 2u &&
               (flags & 0xffu) <= 1u && !(levelset == kLevelsUniform && G.s > 8u) && (cbits & 31u) == 0;
-    const uint32_t nlev = levelset == kLevelsUniform ? (1u << G.s) + 1u : G.s + 2u;
+    const uint32_t nlev = level_count(levelset, G.s);
     const uint32_t hwords = kHeaderWords + (levelset == kLevelsTable ? ((G.s + 1u) & ~1u) : 0u) + (mode == kModeCoded ? 2u : 0u);
     if (ok && mode == kModeCoded) {                         // the lengths must be those of a prefix code of at most 7 bits
         ok = levelset != kLevelsUniform && G.s <= kMaxCodedS;
@@ -106,7 +112,7 @@ __device__ __forceinline__ StreamHead read_head(const Geometry& G, const uint32_
         }
         ok = ok && below < 1.0f;
     }
-    const uint32_t width = 1u + (32u - __clz(nlev - 1u));                   // fixed mode: sign bit + ceil(log2(levels))
+    const uint32_t width = field_width(nlev);
     const uint64_t cwords = cbits >> 5;
     if (ok && mode != kModeFixed) {
         ok = hnblk == G.nblk && cwords > hwords + 2 * (G.nblk + 1);

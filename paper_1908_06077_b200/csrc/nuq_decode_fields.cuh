@@ -34,12 +34,13 @@ __host__ __device__ constexpr uint32_t field_warp_bytes(uint32_t w) { return 2u 
 __host__ __device__ constexpr uint32_t field_table_stride(uint32_t w) { return w <= 6u ? 256u : 4u << w; }
 
 // The level values by field; a symbol that does not exist stands for NaN, which the sums keep (and are checked for).
-__device__ __forceinline__ void build_field_tables(const Geometry& G, const StreamHead* heads, uint32_t K, unsigned char* tables) {
-    const uint32_t w = heads[0].width, stride = field_table_stride(w), n = heads[0].levelset == kLevelsTable ? K : 1u;
+// `heads`: of the n streams whose own levels they are (level tables).
+__device__ __noinline__ void build_field_tables(const Geometry& G, uint32_t levelset, const StreamHead* heads, uint32_t n, unsigned char* tables) {
+    const uint32_t nlev = level_count(levelset, G.s), w = field_width(nlev), stride = field_table_stride(w);
     for (uint32_t i = threadIdx.x; i < n << w; i += blockDim.x) {
         const uint32_t k = i >> w, f = i & ((1u << w) - 1u), sym = f & ((1u << (w - 1u)) - 1u);
-        float v = sym == 0u ? 0.0f : sym < heads[k].nlev ? level_times_norm(1.0f, heads[k].levelset, G.s, sym, heads[k].hdr)
-                                                         : __uint_as_float(0x7FC00000u);
+        float v = sym == 0u ? 0.0f : sym < nlev ? level_times_norm(1.0f, levelset, G.s, sym, levelset == kLevelsTable ? heads[k].hdr : nullptr)
+                                                : __uint_as_float(0x7FC00000u);
         if (f >> (w - 1u)) v = -v;
         *reinterpret_cast<float*>(tables + k * stride + 4u * f) = v;
     }
@@ -109,30 +110,56 @@ __device__ __noinline__ bool four_fields(const Geometry& G, const StreamHead& hd
     return ok;
 }
 
-// adds eight fields of one stream from element e on to the sums, by the slow way
-__device__ __forceinline__ bool add_eight_slowly(const Geometry& G, const StreamHead& hd, uint64_t e, float (&sum)[8]) {
+// The rare parts are calls that need nothing of the loop's registers: inlined, their code lay between that of the common
+// ones, and four warps per scheduler wait for instructions as much as for data (check_fields alone: 56.0 -> 52.3 us).
+
+// A lane's elements (e0 + 256 q + 0 .. 7) of a unit with norms that are not all of ordinary size, from the containers.
+__device__ __noinline__ void unit_slowly(const DecodeParams& P, const StreamHead* heads, uint64_t e0, uint32_t slots) {
     bool ok = true;
-#pragma unroll
-    for (uint32_t h = 0; h < 2; ++h) {
-        if (e + 4u * h >= G.d) continue;
-        float4 v;
-        ok = four_fields(G, hd, e + 4u * h, &v) && ok;
-        sum[4 * h] += v.x; sum[4 * h + 1] += v.y; sum[4 * h + 2] += v.z; sum[4 * h + 3] += v.w;
+#pragma unroll 1
+    for (uint32_t i = 0; i < 2u * slots; ++i) {
+        const uint64_t e = e0 + kSB * (i / 2u) + 4u * (i & 1u);
+        if (e >= P.geo.d) break;
+        float4 sum = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll 1
+        for (uint32_t k = 0; k < P.K; ++k) {
+            float4 v;
+            ok = four_fields(P.geo, heads[k], e, &v) && ok;
+            sum.x += v.x; sum.y += v.y; sum.z += v.z; sum.w += v.w;
+        }
+        if (e + 4u <= P.geo.d) finish4(P.sum, e, sum);
+        else finish_part(P.sum, e, sum, (uint32_t)(P.geo.d - e));
     }
-    return ok;
+    if (!ok) latch_status(P.ws, kErrBadStream);
 }
 
-// Whether all symbols of a lane's elements exist (e0 + 256 q + 0 .. 7 in all streams).  A call, so that its code is out of the
-// way of the loop: four warps per scheduler wait for instructions as much as for data (56.0 -> 52.3 us).
-__device__ __noinline__ bool fields_exist(const Geometry& G, const StreamHead* heads, uint32_t K, uint64_t e0, uint32_t slots) {
+// Looks for symbols that do not exist among a lane's elements.
+__device__ __noinline__ void check_fields(const DecodeParams& P, const StreamHead* heads, uint64_t e0, uint32_t slots) {
     bool ok = true;
-    for (uint32_t q = 0; q < slots; ++q) {
-        for (uint32_t k = 0; k < K; ++k) {
-            float none[8] = {};
-            ok = add_eight_slowly(G, heads[k], e0 + kSB * q, none) && ok;
+    for (uint32_t i = 0; i < 2u * slots; ++i) {
+        const uint64_t e = e0 + kSB * (i / 2u) + 4u * (i & 1u);
+        for (uint32_t k = 0; k < P.K && e < P.geo.d; ++k) {
+            float4 v;
+            ok = four_fields(P.geo, heads[k], e, &v) && ok;
         }
     }
-    return ok;
+    if (!ok) latch_status(P.ws, kErrBadStream);
+}
+
+// The sums of a unit that reaches behind the vector's end.
+template <uint32_t SLOTS>
+__device__ __forceinline__ void finish_end(const SumParams& P, uint64_t d, uint64_t e0, uint32_t slots, const float (&sum)[SLOTS][8]) {
+    float v[8u * SLOTS];                                    // (a copy that can be indexed)
+#pragma unroll
+    for (uint32_t i = 0; i < 8u * SLOTS; ++i) v[i] = sum[i / 8u][i % 8u];
+#pragma unroll 1
+    for (uint32_t i = 0; i < 2u * slots; ++i) {
+        const uint64_t e = e0 + kSB * (i / 2u) + 4u * (i & 1u);
+        if (e >= d) return;
+        const float4 G = make_float4(v[4u * i], v[4u * i + 1u], v[4u * i + 2u], v[4u * i + 3u]);
+        if (e + 4u <= d) finish4(P, e, G);
+        else finish_part(P, e, G, (uint32_t)(d - e));
+    }
 }
 
 // eight values to a multiple of 32 bytes: a whole sector per lane and instruction
@@ -145,18 +172,20 @@ __device__ __forceinline__ void store8(float* dst, const float (&v)[8]) {
 // EXACT: powers of two, whose product with a norm of ordinary size is exact, so that one fused operation gives the sum
 // that two would; else product and sum are rounded one after the other.  Other norms (tiny ones; not finite ones, where an
 // element without a symbol has no product) take the slow way.
-// `mine`: the warp's shared memory (a multiple of 16).
-template <uint32_t W, bool EXACT>
-__device__ __forceinline__ void decode_fields(const DecodeParams& P, const StreamHead* heads, uint32_t tables, uint32_t mine) {
+// WIDE: sums are stored 32 bytes at a time where acc is aligned for it.
+// `mine`: the warp's shared memory (a multiple of 16).  `tables_ready`: the table of levels has been built, and all threads
+// have met since.
+template <uint32_t W, bool EXACT, bool WIDE>
+__device__ __forceinline__ void decode_fields(const DecodeParams& P, const StreamHead* heads, unsigned char* table_memory, bool tables_ready, uint32_t mine) {
     constexpr uint32_t kWords = field_words(W), kSlots = field_slots(W), kPitch = field_pitch(W), kItem = kFieldStreams * kPitch;
     const Geometry& G = P.geo;
     const uint32_t lane = lane_id(), K = P.K, spb = G.bucket / kSB, rec_words = 1u + G.bucket * W / 32u, hwords = heads[0].hwords;
     const uint32_t tab_stride = heads[0].levelset == kLevelsTable ? field_table_stride(W) : 0u;
-    const uint32_t nsub = (uint32_t)((G.d + kSB - 1u) / kSB), nwarps = gridDim.x * (blockDim.x >> 5);
+    const uint32_t nsub = (uint32_t)((G.d + kSB - 1u) / kSB), nfull = (uint32_t)(G.d / kSB), nwarps = gridDim.x * (blockDim.x >> 5);
     const uint32_t S = min(max(nsub / nwarps, 1u), kSlots);                    // (a small call: one sub-block for every warp first)
     const uint32_t nunits = (nsub + S - 1u) / S;
     const uint32_t shift = W == 4u ? 0u : 8u * ((W * lane) & 3u);
-    const uint32_t norms = mine + 2u * kItem, full = norms + 256u;
+    const uint32_t norms = mine + 2u * kItem, full = norms + 256u, tables = smem_u32(table_memory);
 
     struct Item {
         uint32_t unit, k0, b, in;                           // first stream; the first sub-block: the in-th of bucket b
@@ -179,14 +208,14 @@ __device__ __forceinline__ void decode_fields(const DecodeParams& P, const Strea
     auto norms_before = [&](const Item& it, uint32_t q) {   // bucket boundaries between the first sub-block and the q-th behind it
         return (it.in + q >= spb ? 1u : 0u) + (it.in + q >= 2u * spb ? 1u : 0u) + (it.in + q >= 3u * spb ? 1u : 0u);
     };
-    // starts the copies of an item: lane q * 8 + j the norm of slot q in stream j, lane j the fields of stream j
+    // starts the copies of an item: lane j the fields of stream j, lane q * 8 + j the norm of slot q in stream j.  (No fence
+    // in front of the bulk copies: the words they overwrite have been read, and the one place that writes such words has
+    // its own.  A fence waits for the copies in flight.)
     auto start_copy = [&](const Item& it, uint32_t stage) {
         if (it.unit < nunits) {
             const uint32_t sub = it.unit * S, slots = min(S, nsub - sub), count = min(K - it.k0, kFieldStreams);
             const uint64_t rec = hwords + (uint64_t)it.b * rec_words;
             const uint32_t q = lane / kFieldStreams, j = lane % kFieldStreams;
-            if (q < slots && j < count)
-                asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(norms + 128u * stage + 4u * lane), "l"(heads[it.k0 + j].hdr + rec + norms_before(it, q) * rec_words) : "memory");
             // where the fields start in every container, in words, and how many there are (with the norms between them)
             const uint64_t first = rec + 1u + it.in * (8u * W), from = first & ~(uint64_t)3u;
             const uint32_t words = (uint32_t)(first - from) + slots * 8u * W + norms_before(it, slots - 1u);
@@ -195,20 +224,23 @@ __device__ __forceinline__ void decode_fields(const DecodeParams& P, const Strea
                 if (lane < count) {
                     const StreamHead& hd = heads[it.k0 + lane];
                     uint32_t n = (words + 3u) & ~3u;
-                    if (hd.cwords - from < n) {             // the container ends here: its last words one by one
+                    if (__builtin_expect(hd.cwords - from < n, 0)) {    // the container ends here: its last words one by one
                         const uint32_t have = (uint32_t)(hd.cwords - from);
                         n = have & ~3u;
                         for (uint32_t i = n; i < have; ++i)
                             asm volatile("st.shared.u32 [%0], %1;" ::"r"(dst + lane * kPitch + 4u * i), "r"(hd.hdr[from + i]) : "memory");
                         for (uint32_t i = have; i < words; ++i)                 // and no symbols behind them
                             asm volatile("st.shared.u32 [%0], %1;" ::"r"(dst + lane * kPitch + 4u * i), "r"(0u) : "memory");
+                        fence_async_proxy();                // (before a later item's copy to the same place)
                     }
-                    if (n != 0u) bulk_load(dst + lane * kPitch, hd.hdr + from, 4u * n, bar);
+                    if (n != 0u) bulk_load_unfenced(dst + lane * kPitch, hd.hdr + from, 4u * n, bar);
                     else mbar_arrive(bar);
                 } else {
                     mbar_arrive(bar);
                 }
             }
+            if (q < slots && j < count)
+                asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(norms + 128u * stage + 4u * lane), "l"(heads[it.k0 + j].hdr + rec + norms_before(it, q) * rec_words) : "memory");
         }
         asm volatile("cp.async.commit_group;" ::: "memory");
     };
@@ -217,96 +249,88 @@ __device__ __forceinline__ void decode_fields(const DecodeParams& P, const Strea
         mbar_init(full, kFieldStreams);
         mbar_init(full + 8u, kFieldStreams);
     }
+    fence_async_proxy();                                    // (rows may have been cleared here)
     __syncwarp();
-    bool ok = true, in_time = true;
-    Item cur;
-    cur.unit = (threadIdx.x >> 5) * gridDim.x + blockIdx.x;
-    cur.k0 = 0;
-    cur.b = cur.unit * S / spb;
-    cur.in = cur.unit * S - cur.b * spb;
-    Item next = behind(cur);
-    start_copy(cur, 0);
-    start_copy(next, 1);
-    const bool wide = (reinterpret_cast<uintptr_t>(P.acc) & 31u) == 0;
+    bool in_time = true;
+    Item cur = {}, next = {}, after;                        // item n is copied two rounds before it is added up
+    after.unit = (threadIdx.x >> 5) * gridDim.x + blockIdx.x;
+    after.k0 = 0;
+    after.b = after.unit * S / spb;
+    after.in = after.unit * S - after.b * spb;
+    const bool wide = WIDE && (reinterpret_cast<uintptr_t>(P.sum.acc) & 31u) == 0;
     float sum[kSlots][8];
+    bool ordinary = true;                                   // so far, all norms of the unit
     auto clear = [&] {
 #pragma unroll
         for (uint32_t i = 0; i < 8u * kSlots; ++i) sum[i / 8u][i % 8u] = 0.0f;
     };
     clear();
-    for (uint32_t n = 0; cur.unit < nunits; ++n) {
+    for (uint32_t n = 0; n < 2u || cur.unit < nunits; ++n) {
+        const uint32_t stage = n & 1u;
         const uint32_t sub = cur.unit * S, slots = min(S, nsub - sub), count = min(K - cur.k0, kFieldStreams);
         const uint64_t e0 = (uint64_t)sub * kSB + 8u * lane;
-        const Item after = behind(next);
-        if (P.w != nullptr && cur.k0 == 0u && (uint64_t)(sub + slots) * kSB <= G.d && lane < (P.mu != 0.0f ? 2u : 1u))   // the parameters, for later
-            asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"((lane == 0u ? P.w : P.yl) + (uint64_t)sub * kSB), "r"(4u * kSB * slots) : "memory");
-
-        const uint32_t stage = n & 1u;
-        asm volatile("cp.async.wait_group 1;" ::: "memory");
-        const float norm = lane / kFieldStreams < slots && lane % kFieldStreams < count ? __uint_as_float(field_word(norms + 128u * stage + 4u * lane)) : 0.0f;
-        const bool fine = EXACT ? norm == 0.0f || (norm >= 0x1p-100f && norm < 0x1p126f) : fabsf(norm) <= 3.4028234e38f;
-        const bool all_fine = __all_sync(0xffffffffu, fine);
-        __syncwarp();                                       // the other lanes' norms are there
-        in_time = mbar_wait(full + 8u * stage, (n >> 1) & 1u) && in_time;
-        if (all_fine) {
-            // where the lane's fields of each slot start
-            const uint32_t first = mine + stage * kItem + 4u * ((hwords + cur.b * rec_words + 1u + cur.in * (8u * W)) & 3u) + (W * lane & ~3u);
-            auto add_item = [&](auto whole) {               // whole: all slots, within one bucket
-                uint32_t at = first, nrm = norms + 128u * stage, tab = tables + cur.k0 * tab_stride;
+        if (n >= 2u) {
+            if (P.sum.w != nullptr && cur.k0 == 0u && sub + slots <= nfull && lane < (P.sum.mu != 0.0f ? 2u : 1u))   // the parameters, for later
+                asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"((lane == 0u ? P.sum.w : P.sum.yl) + (uint64_t)sub * kSB), "r"(4u * kSB * slots) : "memory");
+            asm volatile("cp.async.wait_group 1;" ::: "memory");
+            const float norm = lane / kFieldStreams < slots && lane % kFieldStreams < count ? __uint_as_float(field_word(norms + 128u * stage + 4u * lane)) : 0.0f;
+            const bool fine = EXACT ? norm == 0.0f || (norm >= 0x1p-100f && norm < 0x1p126f) : fabsf(norm) <= 3.4028234e38f;
+            const bool all_fine = __all_sync(0xffffffffu, fine);
+            __syncwarp();                                   // the other lanes' norms are there
+            in_time = mbar_wait(full + 8u * stage, ((n >> 1) & 1u) ^ 1u) && in_time;
+            ordinary = ordinary && all_fine;
+            if (__builtin_expect(ordinary, 1)) {
+                // where the lane's fields of each slot start
+                const uint32_t first = mine + stage * kItem + 4u * ((hwords + cur.b * rec_words + 1u + cur.in * (8u * W)) & 3u) + (W * lane & ~3u);
+                auto add_item = [&](auto whole) {           // whole: all slots, within one bucket
+                    uint32_t at = first, nrm = norms + 128u * stage, tab = tables + cur.k0 * tab_stride;
 #pragma unroll 1
-                for (uint32_t j = 0; j < count; ++j) {
+                    for (uint32_t j = 0; j < count; ++j) {
 #pragma unroll
-                    for (uint32_t q = 0; q < kSlots; ++q) {
-                        if (!decltype(whole)::value && q >= slots) break;
-                        const uint32_t from = decltype(whole)::value ? at : at + 4u * norms_before(cur, q);
-                        uint32_t x[kWords];
-                        float l[8];
+                        for (uint32_t q = 0; q < kSlots; ++q) {
+                            if (!decltype(whole)::value && q >= slots) break;
+                            const uint32_t from = decltype(whole)::value ? at : at + 4u * norms_before(cur, q);
+                            uint32_t x[kWords];
+                            float l[8];
 #pragma unroll
-                        for (uint32_t i = 0; i < kWords; ++i) x[i] = field_word(from + 32u * W * q + 4u * i);
-                        const float nm = __uint_as_float(field_word(nrm + 4u * kFieldStreams * q));
-                        eight_levels<W>(x, shift, tab, l);
+                            for (uint32_t i = 0; i < kWords; ++i) x[i] = field_word(from + 32u * W * q + 4u * i);
+                            const float nm = __uint_as_float(field_word(nrm + 4u * kFieldStreams * q));
+                            eight_levels<W>(x, shift, tab, l);
 #pragma unroll
-                        for (int i = 0; i < 8; ++i) sum[q][i] = EXACT ? __fmaf_rn(l[i], nm, sum[q][i]) : __fadd_rn(sum[q][i], __fmul_rn(l[i], nm));
+                            for (int i = 0; i < 8; ++i) sum[q][i] = EXACT ? __fmaf_rn(l[i], nm, sum[q][i]) : __fadd_rn(sum[q][i], __fmul_rn(l[i], nm));
+                        }
+                        at += kPitch;
+                        nrm += 4u;
+                        tab += tab_stride;
                     }
-                    at += kPitch;
-                    nrm += 4u;
-                    tab += tab_stride;
-                }
-            };
-            if (slots == kSlots && cur.in + kSlots <= spb) add_item(std::true_type());
-            else add_item(std::false_type());
-        } else {
-            for (uint32_t j = 0; j < count; ++j) {
-#pragma unroll
-                for (uint32_t q = 0; q < kSlots; ++q)
-                    if (q < slots) ok = add_eight_slowly(G, heads[cur.k0 + j], e0 + kSB * q, sum[q]) && ok;
+                };
+                if (slots == kSlots && cur.in + kSlots <= spb) add_item(std::true_type());
+                else add_item(std::false_type());
             }
+            __syncwarp();                                   // the item's words and norms have been read
         }
-        __syncwarp();                                       // the item's words and norms have been read
         start_copy(after, stage);
-        if (cur.k0 + kFieldStreams >= K) {                  // the sums are complete
+        if (n == 0u && !tables_ready) {                     // (every warp is here)
+            build_field_tables(G, heads[0].levelset, heads, heads[0].levelset == kLevelsTable ? K : 1u, table_memory);
+            __syncthreads();
+        }
+        if (n >= 2u && cur.k0 + kFieldStreams >= K) {       // the sums are complete
+            const SumParams out = P.sum;
             float check = 0.0f;                             // NaN when a sum is not finite
 #pragma unroll
             for (uint32_t i = 0; i < 8u * kSlots; ++i) check = __fmaf_rn(sum[i / 8u][i % 8u], 0.0f, check);
-            if (!(check == 0.0f)) {                     // a symbol that does not exist?
-                ok = fields_exist(G, heads, K, e0, slots) && ok;
-            }
             auto value = [&](uint32_t q, uint32_t h) {
                 return make_float4(sum[q][4u * h], sum[q][4u * h + 1u], sum[q][4u * h + 2u], sum[q][4u * h + 3u]);
             };
-            if (e0 - 8u * lane + kSB * slots > G.d) {       // the vector's end
-#pragma unroll
-                for (uint32_t i = 0; i < 2u * kSlots; ++i) {
-                    const uint64_t e = e0 + kSB * (i / 2u) + 4u * (i & 1u);
-                    if (i / 2u >= slots || e >= G.d) continue;
-                    if (e + 4u <= G.d) finish4(P, e, value(i / 2u, i & 1u));
-                    else finish_part(P, e, value(i / 2u, i & 1u), (uint32_t)(G.d - e));
-                }
-            } else if (P.w == nullptr) {
+            if (__builtin_expect(!ordinary, 0)) {
+                unit_slowly(P, heads, e0, slots);
+            } else if (__builtin_expect(sub + slots > nfull, 0)) {
+                finish_end<kSlots>(out, G.d, e0, slots, sum);
+            } else if (out.w == nullptr) {
 #pragma unroll
                 for (uint32_t q = 0; q < kSlots; ++q) {
                     if (q >= slots) break;
-                    float* const dst = P.acc + e0 + kSB * q;
+                    float* const dst = out.acc + e0 + kSB * q;
                     if (wide) {
                         store8(dst, sum[q]);
                     } else {
@@ -323,22 +347,32 @@ __device__ __forceinline__ void decode_fields(const DecodeParams& P, const Strea
                         const uint64_t e = e0 + kSB * ((i0 + i) / 2u) + 4u * (i & 1u);
                         w[i] = yl[i] = make_float4(0.f, 0.f, 0.f, 0.f);
                         if ((i0 + i) / 2u < slots) {
-                            w[i] = *reinterpret_cast<const float4*>(P.w + e);
-                            if (P.mu != 0.0f) yl[i] = *reinterpret_cast<const float4*>(P.yl + e);
+                            w[i] = *reinterpret_cast<const float4*>(out.w + e);
+                            if (out.mu != 0.0f) yl[i] = *reinterpret_cast<const float4*>(out.yl + e);
                         }
                     }
 #pragma unroll
                     for (uint32_t i = 0; i < 4; ++i)
-                        if ((i0 + i) / 2u < slots) step4(P, e0 + kSB * ((i0 + i) / 2u) + 4u * (i & 1u), value((i0 + i) / 2u, i & 1u), w[i], yl[i]);
+                        if ((i0 + i) / 2u < slots) step4(out, e0 + kSB * ((i0 + i) / 2u) + 4u * (i & 1u), value((i0 + i) / 2u, i & 1u), w[i], yl[i]);
                 }
             }
+            if (__builtin_expect(ordinary && !(check == 0.0f), 0)) check_fields(P, heads, e0, slots);   // a symbol that does not exist?
+            ordinary = true;
             clear();
         }
         cur = next;
         next = after;
+        after = behind(after);
     }
-    if (__any_sync(0xffffffffu, !ok) && lane == 0) latch_status(P.ws, kErrBadStream);
     if (__any_sync(0xffffffffu, !in_time) && lane == 0) latch_status(P.ws, kErrTimeout);
+}
+
+// The same as a function, for the kernel of token streams.  (Inlined there, fields and tokens share registers and the
+// instruction cache; as a function its parameters are memory.  Without the wide store: in a called function that more than
+// one kernel uses, nvcc 12.9 was seen to let it write its first element only in all kernels but one.)
+template <uint32_t W, bool EXACT>
+__device__ __noinline__ void decode_fields_call(const DecodeParams& P, const StreamHead* heads, unsigned char* table_memory, bool tables_ready, uint32_t mine) {
+    decode_fields<W, EXACT, false>(P, heads, table_memory, tables_ready, mine);
 }
 
 }  // namespace nuq

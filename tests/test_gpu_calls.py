@@ -133,3 +133,79 @@ def test_a_replay_between_calls_that_take_norms_apart():
             graph.replay()
             assert nuq.last_status() == 0
             assert torch.equal(out[:n], want[:n])
+
+
+KINDS = [(O.MODE_ERC, O.LEVELS_EXP, 4), (O.MODE_ERC, O.LEVELS_EXP, 14), (O.MODE_ERC, O.LEVELS_UNIFORM, 4), (O.MODE_ERC, O.LEVELS_UNIFORM, 8),
+         (O.MODE_ERC, O.LEVELS_TABLE, 14), (O.MODE_FIXED, O.LEVELS_EXP, 4), (O.MODE_FIXED, O.LEVELS_EXP, 14), (O.MODE_FIXED, O.LEVELS_UNIFORM, 4),
+         (O.MODE_FIXED, O.LEVELS_UNIFORM, 8), (O.MODE_FIXED, O.LEVELS_TABLE, 14), (O.MODE_CODED, O.LEVELS_EXP, 4)]
+
+
+@pytest.mark.parametrize("was", range(len(KINDS)))
+@pytest.mark.parametrize("K", [1, 3])
+def test_containers_that_lie_where_others_were_encoded(was, K):
+    """The library remembers what it encoded where, to choose the decoder's kernel and tables; what lies there now decides."""
+    torch, nuq = require_cuda()
+    d, bucket = 40001, 1024
+    rng = np.random.default_rng(7)
+    gs = [rng.standard_normal(d).astype(np.float32) for _ in range(K)]
+    words = max(nuq.encode_bound(d, bucket, s, O.make_flags(O.NORM_L2, ls, mode)) // 4 for mode, ls, s in KINDS)
+    outs = [torch.zeros(words, dtype=torch.int32, device="cuda") for _ in range(K)]
+    for mode, ls, s in KINDS:
+        for old, (omode, ols, os_) in enumerate([KINDS[was]] * K if K == 1 else [KINDS[was], KINDS[was], KINDS[(was + 1) % len(KINDS)]]):
+            if ols == O.LEVELS_TABLE:
+                nuq.set_level_table([0.7 ** (os_ + 1 - j) for j in range(1, os_ + 1)])
+            if omode == O.MODE_CODED:
+                nuq.set_level_code([1, 2, 3, 4, 4])
+            nuq.encode(torch.from_numpy(gs[0]).cuda(), bucket, os_, O.make_flags(O.NORM_L2, ols, omode), out=outs[old])
+        if ls == O.LEVELS_TABLE:
+            O.set_levels(np.float32([0.6 ** (s + 1 - j) for j in range(1, s + 1)]))
+        O.set_level_code([3, 3, 2, 2, 2])
+        streams = [O.encode(g, bucket, s, O.make_flags(O.NORM_LINF, ls, mode), seed=k, offset=0)[0] for k, g in enumerate(gs)]
+        for out, st in zip(outs, streams):
+            out[: st.size].copy_(torch.from_numpy(st.view(np.int32)))
+        rc, want = O.decode_accumulate(streams, d, bucket, s)
+        acc = nuq.decode_accumulate(outs, d, bucket, s)
+        assert rc == 0 and nuq.last_status() == 0
+        assert np.array_equal(acc.cpu().numpy().view(np.uint32), want.view(np.uint32)), (mode, ls, s)
+
+
+@pytest.mark.parametrize("ls,s", [(O.LEVELS_EXP, s) for s in (1, 2, 3, 6, 7, 8, 14)] + [(O.LEVELS_TABLE, s) for s in (2, 5, 8, 14)] +
+                         [(O.LEVELS_UNIFORM, s) for s in range(1, 9)])
+@pytest.mark.parametrize("bucket", [256, 2048])
+@pytest.mark.parametrize("known", [True, False])
+def test_fields_of_every_width_where_they_were_encoded_and_elsewhere(ls, s, bucket, known):
+    """Sums (into an acc of either alignment) and the fused step of fixed-width streams whose kind the library knows from their
+    addresses, and of those it does not know."""
+    torch, nuq = require_cuda()
+    if ls == O.LEVELS_TABLE:
+        levels = np.float32([0.7 ** (s + 1 - j) for j in range(1, s + 1)])
+        nuq.set_level_table(levels)
+        O.set_levels(levels)
+    flags = O.make_flags(O.NORM_LINF, ls, O.MODE_FIXED)
+    gen = torch.Generator(device="cuda").manual_seed(s)
+    for d, K in ((255, 2), (3 * 2048 + 11, 9), (148 * 16 * 256 + 77, 1), (4 * 148 * 16 * 256 + 4096, 2)):
+        gs = [torch.randn(d, generator=gen, device="cuda") for _ in range(K)]
+        outs, streams = [], []
+        for k, g in enumerate(gs):
+            out, bits = nuq.encode(g, bucket, s, flags, seed=k)
+            n = int(bits.item()) // 32
+            if not known:                                    # (nothing is ever encoded 16 bytes behind the start of a tensor here)
+                out = torch.cat([out.new_zeros(4), out])[4:]
+            outs.append(out)
+            streams.append(out.cpu().numpy().view(np.uint32)[:n].copy())
+        rc, want = O.decode_accumulate(streams, d, bucket, s)
+        assert rc == 0
+        want = torch.from_numpy(want).cuda()
+        for shift in (0, 4):                                 # 32-byte or only 16-byte aligned
+            buf = torch.full((d + 16,), float("nan"), device="cuda")
+            acc = buf[shift:shift + d]
+            nuq.decode_accumulate(outs, d, bucket, s, acc=acc)
+            assert nuq.last_status() == 0
+            assert torch.equal(acc.view(torch.int32), want.view(torch.int32)), (d, K, shift)
+            assert buf[:shift].isnan().all() and buf[shift + d:].isnan().all()
+        w, yl = torch.ones(d, device="cuda"), torch.ones(d, device="cuda")
+        nuq.decode_update(outs, d, bucket, s, w, yl, 0.25, 0.5, 1.0, acc=acc)
+        step = torch.tensor(0.25 / K, dtype=torch.float32, device="cuda").double()
+        y = (1.0 - step * want.double()).float()             # one fused operation: one rounding
+        assert nuq.last_status() == 0 and torch.equal(yl, y)
+        assert torch.equal(w, ((y - 1.0).double() * 0.5 + y.double()).float())
