@@ -469,23 +469,23 @@ struct Layout {
 };
 
 // All streams in the fixed-width mode.  (16-bit symbols: s = 7 or 8, hence fields of 5 bits, or of 9 and 10 with uniform levels.)
-template <class Sym>
+template <class Sym, bool MANY>
 __device__ __forceinline__ void fields_of_width(const DecodeParams& P, const StreamHead* heads, unsigned char* tables, uint32_t mine, uint32_t width) {
     if (heads[0].levelset == kLevelsExp) {
-        if (width == 5u) return decode_fields_call<5, true>(P, heads, tables, false, mine);
-        if (sizeof(Sym) == 1 && width == 4u) return decode_fields_call<4, true>(P, heads, tables, false, mine);
-        if (sizeof(Sym) == 1 && width == 3u) return decode_fields_call<3, true>(P, heads, tables, false, mine);
+        if (width == 5u) return decode_fields_call<5, true, Row<Sym>, std::integral_constant<bool, MANY>>(P, heads, tables, mine);
+        if (sizeof(Sym) == 1 && width == 4u) return decode_fields_call<4, true, Row<Sym>, std::integral_constant<bool, MANY>>(P, heads, tables, mine);
+        if (sizeof(Sym) == 1 && width == 3u) return decode_fields_call<3, true, Row<Sym>, std::integral_constant<bool, MANY>>(P, heads, tables, mine);
     }
-    if (width == 5u) return decode_fields_call<5, false>(P, heads, tables, false, mine);
+    if (width == 5u) return decode_fields_call<5, false, Row<Sym>, std::integral_constant<bool, MANY>>(P, heads, tables, mine);
     if (sizeof(Sym) == 1) {
-        if (width == 3u) return decode_fields_call<3, false>(P, heads, tables, false, mine);
-        if (width == 4u) return decode_fields_call<4, false>(P, heads, tables, false, mine);
-        if (width == 6u) return decode_fields_call<6, false>(P, heads, tables, false, mine);
-        if (width == 7u) return decode_fields_call<7, false>(P, heads, tables, false, mine);
-        if (width == 8u) return decode_fields_call<8, false>(P, heads, tables, false, mine);
+        if (width == 3u) return decode_fields_call<3, false, Row<Sym>, std::integral_constant<bool, MANY>>(P, heads, tables, mine);
+        if (width == 4u) return decode_fields_call<4, false, Row<Sym>, std::integral_constant<bool, MANY>>(P, heads, tables, mine);
+        if (width == 6u) return decode_fields_call<6, false, Row<Sym>, std::integral_constant<bool, MANY>>(P, heads, tables, mine);
+        if (width == 7u) return decode_fields_call<7, false, Row<Sym>, std::integral_constant<bool, MANY>>(P, heads, tables, mine);
+        if (width == 8u) return decode_fields_call<8, false, Row<Sym>, std::integral_constant<bool, MANY>>(P, heads, tables, mine);
     } else {
-        if (width == 9u) return decode_fields_call<9, false>(P, heads, tables, false, mine);
-        if (width == 10u) return decode_fields_call<10, false>(P, heads, tables, false, mine);
+        if (width == 9u) return decode_fields_call<9, false, Row<Sym>, std::integral_constant<bool, MANY>>(P, heads, tables, mine);
+        if (width == 10u) return decode_fields_call<10, false, Row<Sym>, std::integral_constant<bool, MANY>>(P, heads, tables, mine);
     }
 }
 
@@ -599,7 +599,7 @@ __device__ __forceinline__ void decode_streams(const DecodeParams& P) {
     }
     __syncthreads();
     if (!CALLED && s_fields != 0u) {                        // no tokens at all
-        fields_of_width<Sym>(P, heads, at.field_tables, rows, s_fields);
+        fields_of_width<Sym, MANY>(P, heads, at.field_tables, rows, s_fields);
         return;
     }
     if (CALLED) clear_rows();
@@ -827,8 +827,8 @@ __device__ __noinline__ void decode_streams_call(const DecodeParams& P) {
 // Calls whose streams are likely all in the fixed-width mode, with fields of W bits of one level set: a kernel of its own for
 // each, so that neither its registers nor its code are shared with the walks of token streams.  25.6 x 10^6 elements, K = 8, 4
 // bits, in one kernel with the walks: 67.6 us behind eight encode calls (where the code has to be fetched), 53.6 us repeated;
-// here 56 and 52 us.  Of that, headers are read 1.4 us behind the wait (the table stands ready then), the first bytes are there
-// after 4 us and the code of an item, its sums and its copies has been fetched after 2 more.
+// here 56 and 51 us; as a function called by the kernel for token streams, which is what containers that were not encoded here
+// take, 65.5 and 53 us.
 template <uint32_t W, bool EXACT>
 __global__ void __launch_bounds__(32 * kChainMaxWarps, 1) decode_fields_kernel(const __grid_constant__ DecodeParams P) {
     extern __shared__ __align__(128) unsigned char dsm[];
@@ -853,7 +853,7 @@ __global__ void __launch_bounds__(32 * kChainMaxWarps, 1) decode_fields_kernel(c
     __syncthreads();
     if (s_likely) {
         const uint32_t mine = wide_symbols ? Layout<int16_t>(dsm, K).rows : at.rows;
-        decode_fields<W, EXACT, true>(P, at.heads, at.field_tables, tables_ready, mine);
+        decode_fields<W, EXACT>(P, at.heads, at.field_tables, tables_ready, mine);
     } else if (wide_symbols) {                              // another kind of streams after all
         decode_streams_call<int16_t>(P);
     } else {

@@ -1,5 +1,5 @@
 // DECODE + aggregate of calls whose streams are all in the fixed-width mode with the same field width and kind of levels:
-// no chains to walk, a part of the decode kernel of nuq_decode_chains.cu that its warps enter when the headers say so.
+// no chains to walk.  The kernels for it, and the way here from the kernels for token streams, are in nuq_decode_chains.cu.
 //
 // A warp takes units of up to four 256-element sub-blocks; a lane has eight consecutive elements of each, one word of
 // every stream when fields have 4 bits.  A field, its sign bit included, is looked up in a table of level values in shared
@@ -7,11 +7,13 @@
 // and one fused multiply-add.  No value depends on a unit, so nothing is built per
 // unit and warps never meet.  An item, that is the fields of a unit in up to eight streams, is brought into the warp's
 // shared memory by one bulk copy per stream, two items ahead, so that no address is computed per word and the bytes in
-// flight do not depend on registers.
-// 25.6 x 10^6 elements, K = 8 (200 MB, 31 us at the memory's rate): 4-bit fields 52 us, other widths and small buckets 60
-// to 90 us (a kernel of one thread per 32 elements: 104 to 117 us, level tables 547 us); 65536 elements 6.6 us (in front of
-// the token kernel: 12 us).  What bounds it is the look-ups (one shared-memory word per element and stream, a wavefront
-// per 32 of them) and, with four warps per scheduler, what the warps wait for.
+// flight do not depend on registers.  The copies are started in one place of the loop, which begins two rounds early: their
+// code is there when the first item is.
+// 25.6 x 10^6 elements, K = 8 (200 MB with 4 bits, 31 us at the memory's rate): 4-bit fields 51 us repeated and 56 us behind
+// eight encode calls, level tables 57 us, 3 bits 56 us, 5 to 8 bits 72 to 85 us, 9 and 10 bits up to 107 us, buckets of 256 and 512
+// 62 to 67 us; 65536 elements 4.8 us.  (A kernel of one thread per 32 elements: 104 to 117 us, level tables 547 us.)  What bounds
+// it is the look-ups (one shared-memory word per element and stream, a wavefront per 32 of them) and, with four warps per
+// scheduler, what the warps wait for.
 #pragma once
 #include <type_traits>
 
@@ -172,10 +174,9 @@ __device__ __forceinline__ void store8(float* dst, const float (&v)[8]) {
 // EXACT: powers of two, whose product with a norm of ordinary size is exact, so that one fused operation gives the sum
 // that two would; else product and sum are rounded one after the other.  Other norms (tiny ones; not finite ones, where an
 // element without a symbol has no product) take the slow way.
-// WIDE: sums are stored 32 bytes at a time where acc is aligned for it.
 // `mine`: the warp's shared memory (a multiple of 16).  `tables_ready`: the table of levels has been built, and all threads
 // have met since.
-template <uint32_t W, bool EXACT, bool WIDE>
+template <uint32_t W, bool EXACT>
 __device__ __forceinline__ void decode_fields(const DecodeParams& P, const StreamHead* heads, unsigned char* table_memory, bool tables_ready, uint32_t mine) {
     constexpr uint32_t kWords = field_words(W), kSlots = field_slots(W), kPitch = field_pitch(W), kItem = kFieldStreams * kPitch;
     const Geometry& G = P.geo;
@@ -257,9 +258,10 @@ __device__ __forceinline__ void decode_fields(const DecodeParams& P, const Strea
     after.k0 = 0;
     after.b = after.unit * S / spb;
     after.in = after.unit * S - after.b * spb;
-    const bool wide = WIDE && (reinterpret_cast<uintptr_t>(P.sum.acc) & 31u) == 0;
+    const bool wide = (reinterpret_cast<uintptr_t>(P.sum.acc) & 31u) == 0;
     float sum[kSlots][8];
     bool ordinary = true;                                   // so far, all norms of the unit
+    const uint32_t params = P.sum.w == nullptr ? 0u : P.sum.mu != 0.0f ? 2u : 1u;        // vectors of parameters
     auto clear = [&] {
 #pragma unroll
         for (uint32_t i = 0; i < 8u * kSlots; ++i) sum[i / 8u][i % 8u] = 0.0f;
@@ -270,7 +272,7 @@ __device__ __forceinline__ void decode_fields(const DecodeParams& P, const Strea
         const uint32_t sub = cur.unit * S, slots = min(S, nsub - sub), count = min(K - cur.k0, kFieldStreams);
         const uint64_t e0 = (uint64_t)sub * kSB + 8u * lane;
         if (n >= 2u) {
-            if (P.sum.w != nullptr && cur.k0 == 0u && sub + slots <= nfull && lane < (P.sum.mu != 0.0f ? 2u : 1u))   // the parameters, for later
+            if (cur.k0 == 0u && sub + slots <= nfull && lane < params)    // the parameters, for later
                 asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"((lane == 0u ? P.sum.w : P.sum.yl) + (uint64_t)sub * kSB), "r"(4u * kSB * slots) : "memory");
             asm volatile("cp.async.wait_group 1;" ::: "memory");
             const float norm = lane / kFieldStreams < slots && lane % kFieldStreams < count ? __uint_as_float(field_word(norms + 128u * stage + 4u * lane)) : 0.0f;
@@ -367,12 +369,12 @@ __device__ __forceinline__ void decode_fields(const DecodeParams& P, const Strea
     if (__any_sync(0xffffffffu, !in_time) && lane == 0) latch_status(P.ws, kErrTimeout);
 }
 
-// The same as a function, for the kernel of token streams.  (Inlined there, fields and tokens share registers and the
-// instruction cache; as a function its parameters are memory.  Without the wide store: in a called function that more than
-// one kernel uses, nvcc 12.9 was seen to let it write its first element only in all kernels but one.)
-template <uint32_t W, bool EXACT>
-__device__ __noinline__ void decode_fields_call(const DecodeParams& P, const StreamHead* heads, unsigned char* table_memory, bool tables_ready, uint32_t mine) {
-    decode_fields<W, EXACT, false>(P, heads, table_memory, tables_ready, mine);
+// The same as a function, for the kernels of token streams: inlined there, fields and tokens share registers and the
+// instruction cache.  (Kernel: a function for each of them.  In one that several kernels called, nvcc 12.9 was seen to let the
+// wide store write its first element only, in all kernels but one.)
+template <uint32_t W, bool EXACT, class... Kernel>
+__device__ __noinline__ void decode_fields_call(const DecodeParams& P, const StreamHead* heads, unsigned char* table_memory, uint32_t mine) {
+    decode_fields<W, EXACT>(P, heads, table_memory, false, mine);
 }
 
 }  // namespace nuq
