@@ -115,3 +115,22 @@ def test_containers_at_the_encoders_edges(kind, d, bucket, s, ls):
         assert got_bits == want_bits and np.array_equal(got, want)
         free, free_bits = gpu_encode(g, bucket, s, flags, seed=5, offset=9)       # (largest magnitudes are exact: the same norms)
         assert free_bits == want_bits and np.array_equal(free, want)
+
+
+@pytest.mark.parametrize("mode", [O.MODE_ERC, O.MODE_FIXED])
+@pytest.mark.parametrize("ls,s,K", [(O.LEVELS_UNIFORM, 4, 3), (O.LEVELS_UNIFORM, 8, 3), (O.LEVELS_TABLE, 5, 3), (O.LEVELS_TABLE, 8, 2), (O.LEVELS_TABLE, 3, 40)])
+def test_products_are_rounded_before_they_are_added(ls, s, K, mode):
+    """norm times level is a product of its own (one rounding), the sum another: where the product is not exact, an operation
+    that rounds once for both gives other last bits.  (The packed multiply and add of two elements were once joined so.)"""
+    d, bucket = 60001, 1024
+    O.set_levels(np.float32([0.61 ** (s + 1 - j) for j in range(1, s + 1)]))
+    streams = [_container("normal", d, bucket, s, O.NORM_LINF, ls, mode, k) for k in range(K)]
+    joined = np.zeros(d, np.float32)
+    for st in streams:
+        rc, sign, sym, norms = O.decode_symbols(st, d, bucket, s)
+        level = np.float32([O.level_value(ls, s, j) for j in range(O.num_levels(ls, s))])[sym].astype(np.float64)
+        product = np.where(sign != 0, -1.0, 1.0) * level * np.repeat(norms, bucket)[:d].astype(np.float64)      # exact: 48 bits
+        joined = (joined.astype(np.float64) + product).astype(np.float32)
+    rc, want = O.decode_accumulate(streams, d, bucket, s)
+    assert rc == 0 and np.mean(joined != want) > 0.02               # the input tells the two apart
+    _same_sums(streams, d, bucket, s)
