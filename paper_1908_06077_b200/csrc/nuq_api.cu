@@ -233,7 +233,7 @@ static int occupancy(const EncodeParams& P, int dev, bool clusters) {
     static std::map<uint64_t, int> known;
     const Geometry& G = P.geo;
     const uint64_t key = (uint64_t)encode_smem_bytes(P) | (uint64_t)G.levelset << 32 | (uint64_t)G.mode << 34 |
-                         (uint64_t)(fixed4_applies(G) ? 1 : 0) << 36 | (uint64_t)(G.bucket % (kBLK / kEncWarps) == 0 ? 1 : 0) << 37 |
+                         (uint64_t)(fixed4_applies(G) ? 1u + fixed4_variant(G) : 0u) << 36 |
                          (uint64_t)(P.warps >> 3) << 42 |
                          (uint64_t)(clusters ? P.cluster : 0) << 38 | (uint64_t)(uint32_t)dev << 44;
     const auto it = known.find(key);

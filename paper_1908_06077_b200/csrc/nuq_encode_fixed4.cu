@@ -13,6 +13,8 @@
 //      one CTA barrier;
 //   2. per sub-block, a lane quantizes 8 consecutive elements (two Philox blocks), which are exactly one
 //      32-bit word of eight fields, and stores that word to its place: 128 contiguous bytes per warp.
+#include <type_traits>
+
 #include "nuq_encode_common.cuh"
 #include "nuq_launch.h"
 
@@ -24,9 +26,10 @@ bool fixed4_applies(const Geometry& G) {
     return G.mode == kModeFixed && G.levelset == kLevelsExp && G.width == 4u;
 }
 
-// Eight elements -> eight fields sign << 3 | index, first element in the top nibble.
+// Eight elements -> eight fields sign << 3 | index, first element in the top nibble.  `dense`: so many lanes have elements at or
+// above the lowest level that their index is better worked out for every element.
 __device__ __forceinline__ uint32_t quantize8_fixed4(const float4& a, const float4& b, float inv, float top, const uint4& ra,
-                                                     const uint4& rb) {
+                                                     const uint4& rb, bool* dense) {
     const float x[8] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
     const uint32_t r[8] = {ra.x, ra.y, ra.z, ra.w, rb.x, rb.y, rb.z, rb.w};
     uint32_t nz = 0, neg = 0;
@@ -39,11 +42,30 @@ __device__ __forceinline__ uint32_t quantize8_fixed4(const float4& a, const floa
     }
     const uint32_t high = __ballot_sync(0xffffffffu, most >= 1.0f);
     if (high) add_high_levels(y, r, top, high, nz);
+    *dense = __popc(high) > 6;
     return nz | (neg << 3);                                 // a zero symbol carries no sign
 }
 
-// COARSE: the bucket is a multiple of 1024 elements, so a warp's four sub-blocks share one bucket.
-template <bool COARSE>
+// The same fields, with the index worked out for every element.
+__device__ __forceinline__ uint32_t quantize8_dense(const float4& a, const float4& b, float inv, float top, const uint4& ra, const uint4& rb) {
+    const float x[8] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
+    const uint32_t r[8] = {ra.x, ra.y, ra.z, ra.w, rb.x, rb.y, rb.z, rb.w};
+    uint32_t word = 0;
+#pragma unroll
+    for (int k = 0; k < 8; ++k) {
+        const float y = fminf(__fmul_rn(fabsf(x[k]), inv), top);               // (see quantize_exp)
+        const uint32_t hi = (__float_as_uint(fmaxf(y, 1.0f)) + (0x007FFFFFu - 0x3F000000u) - (r[k] >> 9)) >> 23;
+        const bool up = __uint2float_rn(r[k] >> 8) < __fmul_rn(y, 16777216.0f);
+        word = (word << 4) | (up ? hi | ((__float_as_uint(x[k]) >> 28) & 8u) : 0u);
+    }
+    return word;
+}
+
+// COARSE: the bucket is a multiple of 1024 elements, so a warp's four sub-blocks share one bucket, and the first of them tells
+// how the others are quantized, in straight lines of code for either way (2^28 elements with dense symbols 475 -> 446 us, sparse
+// ones 398 -> 384; chosen at every sub-block 459 and 398).
+// DENSE: every sub-block the dense way (buckets of 256 and 512: 531 -> 515 us).
+template <bool COARSE, bool DENSE>
 __global__ void __launch_bounds__(kEncThreads, kEncMinBlocks) encode_fixed4_kernel(const __grid_constant__ EncodeParams P) {
     __shared__ __align__(128) float data[kBLK];            // the tile
     __shared__ __align__(8) uint64_t s_full[kEncWarps];    // s_full[w] completes when warp w's part of a tile has landed
@@ -250,11 +272,10 @@ __global__ void __launch_bounds__(kEncThreads, kEncMinBlocks) encode_fixed4_kern
         };
         if (COARSE && sbq0 < nsb_tile) locate(sbq0);
         const float inv_coarse = s_sb_inv[sbq0];
+        bool dense = false;
 
-#pragma unroll COARSE ? 4 : 1
-        for (uint32_t q = 0; q < 4; ++q) {
+        auto sub_block = [&](uint32_t q, auto densely) {
             const uint32_t sbq = sbq0 + q;
-            if (sbq >= nsb_tile) break;
             if (!COARSE) locate(sbq);
             else if (q) fx_sb += 1u;
             const float inv = COARSE ? inv_coarse : s_sb_inv[sbq];
@@ -262,7 +283,8 @@ __global__ void __launch_bounds__(kEncThreads, kEncMinBlocks) encode_fixed4_kern
             if (fx_sb == 0 && lane == 0) rec[0] = __float_as_uint(s_sb_norm[sbq]);
             uint32_t word = 0;                              // a bucket that is not quantized: all fields zero
             if (inv != 0.0f) {
-                word = quantize8_fixed4(rows[64 * q], rows[64 * q + 1], inv, top, rn0, rn1);
+                if (decltype(densely)::value) word = quantize8_dense(rows[64 * q], rows[64 * q + 1], inv, top, rn0, rn1);
+                else word = quantize8_fixed4(rows[64 * q], rows[64 * q + 1], inv, top, rn0, rn1, &dense);
                 // a field is nonzero iff its index is: adding 7 to the index carries into the field's top bit
                 my_nnz += __popc(((word & 0x77777777u) + 0x77777777u) & 0x88888888u);
             }
@@ -271,6 +293,25 @@ __global__ void __launch_bounds__(kEncThreads, kEncMinBlocks) encode_fixed4_kern
                 const uint64_t ctr = ctr_lane + 64u * (q + 1u);
                 rn0 = philox4x32_10((uint32_t)ctr, (uint32_t)(ctr >> 32), c2, c3, P.round_keys);
                 rn1 = philox4x32_10((uint32_t)(ctr + 1u), (uint32_t)((ctr + 1u) >> 32), c2, c3, P.round_keys);
+            }
+        };
+        const uint32_t mine = sbq0 < nsb_tile ? min(4u, nsb_tile - sbq0) : 0u;
+        if (COARSE) {
+            if (mine != 0u) sub_block(0u, std::false_type());
+            if (!dense) {
+#pragma unroll
+                for (uint32_t q = 1; q < 4; ++q)
+                    if (q < mine) sub_block(q, std::false_type());
+            } else {
+#pragma unroll
+                for (uint32_t q = 1; q < 4; ++q)
+                    if (q < mine) sub_block(q, std::true_type());
+            }
+        } else {
+#pragma unroll DENSE ? 4 : 1
+            for (uint32_t q = 0; q < 4; ++q) {
+                if (sbq0 + q >= nsb_tile) break;
+                sub_block(q, std::integral_constant<bool, DENSE>());
             }
         }
 
@@ -295,12 +336,24 @@ __global__ void __launch_bounds__(kEncThreads, kEncMinBlocks) encode_fixed4_kern
     }
 }
 
+// Which instance.  The dense one where a coordinate of ordinary size reaches the lowest level often: one of size norm /
+// sqrt(bucket) is 2^s / sqrt(bucket) times that level (2^28 normal values in buckets of 512: s = 4 531 -> 515 us, but s = 3, where
+// the bucket is 8 4^s, 512 -> 520).  Larger buckets that are not multiples of 1024 keep the test for zeros (768 elements: normal
+// values 558 -> 543 us with the dense one, outliers with the largest magnitude as norm 496 -> 508).
+uint32_t fixed4_variant(const Geometry& G) {
+    if (G.bucket % kFx4WarpElems == 0) return 1;
+    return G.bucket <= 512u && G.bucket < (8u << (2u * G.s)) ? 2 : 0;
+}
+
+using Fixed4Kernel = void (*)(EncodeParams);
+static Fixed4Kernel kernel_for(const Geometry& G) {
+    const uint32_t v = fixed4_variant(G);
+    return v == 1u ? encode_fixed4_kernel<true, false> : v == 2u ? encode_fixed4_kernel<false, true> : encode_fixed4_kernel<false, false>;
+}
+
 int fixed4_blocks_per_sm(const EncodeParams& P) {
     int n = 0;
-    const bool coarse = P.geo.bucket % kFx4WarpElems == 0;
-    const cudaError_t e = coarse ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, encode_fixed4_kernel<true>, kEncThreads, 0)
-                                 : cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, encode_fixed4_kernel<false>, kEncThreads, 0);
-    return e == cudaSuccess ? n : 0;
+    return cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, kernel_for(P.geo), kEncThreads, 0) == cudaSuccess ? n : 0;
 }
 
 cudaError_t launch_encode_fixed4(const EncodeParams& P, cudaStream_t stream) {
@@ -317,8 +370,7 @@ cudaError_t launch_encode_fixed4(const EncodeParams& P, cudaStream_t stream) {
         attr[0].val.programmaticStreamSerializationAllowed = 1;
         cfg.numAttrs = 1;
     }
-    if (P.geo.bucket % kFx4WarpElems == 0) return cudaLaunchKernelEx(&cfg, encode_fixed4_kernel<true>, P);
-    return cudaLaunchKernelEx(&cfg, encode_fixed4_kernel<false>, P);
+    return cudaLaunchKernelEx(&cfg, kernel_for(P.geo), P);
 }
 
 }  // namespace nuq

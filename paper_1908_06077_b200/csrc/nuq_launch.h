@@ -35,6 +35,7 @@ int encode_blocks_per_sm(const EncodeParams& P);      // encoder CTAs one SM hol
 int encode_max_clusters(const EncodeParams& P);       // clusters of P.cluster encoder CTAs the device holds at once (0 on error)
 cudaError_t launch_encode(const EncodeParams& P, cudaStream_t stream);
 bool fixed4_applies(const Geometry& G);               // the call is served by the 4-bit fixed-width encoder
+uint32_t fixed4_variant(const Geometry& G);           // which instance of it (0 to 2)
 int fixed4_blocks_per_sm(const EncodeParams& P);
 cudaError_t launch_encode_fixed4(const EncodeParams& P, cudaStream_t stream);
 cudaError_t launch_level_histogram(const EncodeParams& P, uint64_t* hist, int sms, cudaStream_t stream);   // hist: s + 2 zeroed counters

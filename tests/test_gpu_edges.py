@@ -134,3 +134,20 @@ def test_products_are_rounded_before_they_are_added(ls, s, K, mode):
     rc, want = O.decode_accumulate(streams, d, bucket, s)
     assert rc == 0 and np.mean(joined != want) > 0.02               # the input tells the two apart
     _same_sums(streams, d, bucket, s)
+
+
+@pytest.mark.parametrize("bucket", [256, 512, 768, 1024, 8192])
+@pytest.mark.parametrize("s", [3, 4, 6])
+def test_four_bit_containers_of_dense_and_sparse_symbols(bucket, s):
+    """The 4-bit encoder's ways to quantize: by instance (buckets) and, in buckets of 1024 and more, by what a warp's first
+    sub-block looks like; kinds change from sub-block to sub-block here, and the last tile ends inside a warp's part."""
+    d = 3 * 8192 + 1500
+    for kind in ("normal", "sparse", "dense", "mixed", "ends"):
+        for nk in (O.NORM_L2, O.NORM_LINF):
+            g = _vector(kind, d, s)
+            g[5000:9000] *= np.float32(40.0)
+            norms = O.bucket_norms(g, bucket, nk)
+            flags = O.make_flags(nk, O.LEVELS_EXP, O.MODE_FIXED)
+            want, want_bits = O.encode(g, bucket, s, flags, seed=5, offset=9, norms=norms)
+            got, got_bits = gpu_encode(g, bucket, s, flags, seed=5, offset=9, norms=norms)
+            assert got_bits == want_bits and np.array_equal(got, want), (kind, nk)
