@@ -351,7 +351,7 @@ class Workload:
         w = torch.zeros(self.d, device="cuda")
         yl = torch.zeros(self.d, device="cuda")
         alpha, mu, l = 0.1, 0.9, 1.0
-        acc = self.acc if self.K < 3 else None              # with one or two streams the library adds up in acc
+        acc = self.acc if self.K < 3 else None              # (required with one or two streams)
         fused, pair = [], []
         for it in range(reps + 2):
             ev = [torch.cuda.Event(enable_timing=True) for _ in range(4)]
@@ -519,7 +519,7 @@ def run_gpu(args):
             "decode_us_per_call": {k: 1e3 * v for k, v in summarize(dec_ms).items()},
             "roofline": roofline_entry(ENCODE_KERNEL.get(args.workload, "encode_kernel"), enc_bytes, enc_launch_ms, peak, peak_kind,
                                        ENCODE_TRAFFIC_BYTES.get(args.workload) if full else None),
-            "roofline_decode": roofline_entry("decode_chains_kernel", dec_bytes, t_dec, peak, peak_kind,
+            "roofline_decode": roofline_entry("decode_fields_kernel" if (flags >> 16) & 0xff == 1 else "decode_chains_kernel", dec_bytes, t_dec, peak, peak_kind,
                                               DECODE_TRAFFIC_BYTES.get(args.workload) if full else None),
             "gpu_launches": steps * w.launches_per_step(),
             "clocks": clocks,

@@ -164,7 +164,7 @@ nuq_status nuq_decode_accumulate(const void* const* streams, uint32_t K, uint64_
  *   streams, K, d, bucket, s   as for nuq_decode_accumulate
  *   acc      device, d floats, 16-byte aligned, or NULL.  If given it receives
  *            the sum as from nuq_decode_accumulate.  With K <= 2 it is REQUIRED
- *            (the library adds the streams up in it).
+ *            (a rule of the interface: NUQ_ERR_INVALID_ARG without it).
  *   w        device, d floats, 16-byte aligned: the parameters, updated in place
  *   yl       device, d floats, 16-byte aligned: y^l of the previous step on
  *            entry (the parameters themselves before the first step), y^l of

@@ -214,8 +214,8 @@ nuq_status get_norms(cudaStream_t stream, size_t bytes, WsEntry& e) {
 
 using namespace nuq;
 
-// Mode of the containers this process has encoded, by device and address (see enqueue_encode): a hint
-// for the decoder's choice of kernels, which check it against the containers' headers on the device.
+// Mode and level set of the containers this process has encoded, by device and address (see enqueue_encode): a hint
+// for the decoder's choice of kernels, which go by the containers' headers.
 // Guarded by g_mu.
 static std::map<std::pair<int, const void*>, uint32_t> g_container_mode;   // mode | level set << 8
 
@@ -350,8 +350,7 @@ static nuq_status enqueue_encode(EncodeParams& P, const EncodePlan& pl, const fl
         if (entry) entry->dirty = true;                     // whatever state the failed launch left
         return NUQ_ERR_CUDA;
     }
-    // remember the mode of the container at this address: a hint for the decoder's choice of kernels,
-    // checked against the header on the device
+    // what the container at this address is (a hint; the map is bounded)
     if (g_container_mode.size() > 4096) g_container_mode.clear();
     g_container_mode[std::make_pair(dev, static_cast<const void*>(out))] = G.mode | G.levelset << 8;
     return NUQ_OK;
@@ -571,7 +570,7 @@ static nuq_status enqueue_decode(const void* const* streams, uint32_t K, uint64_
     cudaStream_t stream = static_cast<cudaStream_t>(stream_);
     DecodeParams P;
     if (!streams || K < 1 || K > kMaxK) return NUQ_ERR_INVALID_ARG;
-    // with one or two streams the sums are added up in acc itself, so it is needed even when only w is wanted
+    // (with one or two streams acc has to be given: a rule of the interface, which the kernels have no need of)
     if (!acc && (!w || K < 3)) return NUQ_ERR_INVALID_ARG;
     if (w && mu != 0.0f && !yl) return NUQ_ERR_INVALID_ARG;
     if (w && !(alpha == alpha && mu >= 0.0f && mu < 1.0f && l >= 0.0f && l <= 1.0f)) return NUQ_ERR_INVALID_ARG;

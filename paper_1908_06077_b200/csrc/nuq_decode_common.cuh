@@ -144,8 +144,8 @@ __device__ __forceinline__ uint64_t fma2(uint64_t a, uint64_t b, uint64_t c) {
     asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
     return r;
 }
-// A rounded product that is added to something afterwards.  Not mul.rn.f32x2: the assembler was seen to put that and an
-// add.rn.f32x2 together into one fused operation, with one rounding instead of two, in spite of the rounding modifiers.
+// A rounded product that is added to something afterwards.  Not mul.rn.f32x2: with that and an add.rn.f32x2 behind it sums came
+// out as if product and sum had been rounded once, in spite of the rounding modifiers (they differ from the oracle's then).
 // A fused operation that adds -0 changes no product, and it cannot be fused again as long as the -0 is not known to be one.
 __device__ __forceinline__ uint64_t product2(uint64_t a, uint64_t b, uint64_t minus_zero) { return fma2(a, b, minus_zero); }
 __device__ __forceinline__ uint64_t add2(uint64_t a, uint64_t b) {
