@@ -21,8 +21,9 @@
 //           its last bit and for a gap one smaller, without a symbol, leaves an ordinary token of gap 1
 //           behind.  What the table cannot resolve at all (gaps from 128 on, long level codes) takes
 //           Algorithm 2's loop.
-//   window  64 bits hi:lo, at least 32 of them valid, shifted by the token's length; the next table
-//           index needs only the 13 top bits, which are valid before the window is refilled.
+//   window  64 bits hi:lo, shifted by the token's length and refilled to at least 32 valid bits every
+//           second step: a look-up needs the 13 top bits, so 32 last for two tokens.  (Refilled at every
+//           step the walk takes 3 of 18 instructions more: ResNet-50, K = 8 85.2 us, now 83.4.)
 //   end     every lane has its own copy of its chain (cp.async, 112 bytes at a time) and puts ones
 //           behind the chain's last bit: thirteen ones are no token, the table says "0 bits, no gap, no
 //           symbol", and the lane stands still until all others have ended too.  So a step has no
@@ -199,7 +200,7 @@ __device__ __forceinline__ uint32_t walk_body(uint32_t copy, uint32_t from, uint
     uint32_t next = w0 + (sh ? 12u : 8u);                   // where the word behind nxt lies
     // q counts the bits down to c; its low five bits are those of the number of valid bits in hi:lo
     const uint32_t c = (0u - sh - bits) & 31u;
-    uint32_t q = bits + c, e = 0, at = row;
+    uint32_t q = bits + c, q_was = q, e = 0, at = row;
     auto look_up = [&] {
         const uint32_t addr = tab + ((hi >> (32u - kTokBits)) << 2);
         if (LONG) asm("{\n\t.reg .pred p;\n\tsetp.gt.s32 p, %1, %2;\n\tmov.b32 %0, 0;\n\t@p ld.shared.u32 %0, [%3];\n\t}"
@@ -211,6 +212,14 @@ __device__ __forceinline__ uint32_t walk_body(uint32_t copy, uint32_t from, uint
             const uint32_t sym = hd.levelset == kLevelsUniform ? uniform_symbol(index, negative) : exp_symbol(index, negative, s);
             e = e != 0u && cw != 0u ? len | (e & (0xffu << kGapShift)) | sym : 0u;
         }
+    };
+    // brings the number of valid bits back to 32 at least, when it is below; fewer than 32 have been taken since it was done last
+    auto refill = [&] {
+        asm("{\n\t.reg .pred p;\n\t.reg .b32 t;\n\txor.b32 t, %4, %5;\n\tand.b32 t, t, 32;\n\tsetp.ne.u32 p, t, 0;\n\t"
+            "shf.r.wrap.b32 t, %2, 0, %4;\n\t@p or.b32 %0, %0, t;\n\t@p shf.r.wrap.b32 %1, 0, %2, %4;\n\t"
+            "@p ld.shared.u32 %2, [%3];\n\t@p add.u32 %3, %3, 4;\n\t}"
+            : "+r"(hi), "+r"(lo), "+r"(nxt), "+r"(next) : "r"(q), "r"(q_was));
+        q_was = q;
     };
     if (bits != 0u) {
         look_up();
@@ -225,21 +234,6 @@ __device__ __forceinline__ uint32_t walk_body(uint32_t copy, uint32_t from, uint
             }
 #pragma unroll
             for (int u = 0; u < 4; ++u) {
-                if (!GAPS && !LONG && sizeof(Sym) == 1) {
-                    asm volatile(
-                        "{\n\t.reg .pred p, r;\n\t.reg .b32 g, y, t, n;\n\t"
-                        "prmt.b32 g, %0, 0, 0x4441;\n\tadd.u32 %1, %1, g;\n\tmin.u32 %1, %1, %7;\n\t"
-                        "shr.u32 y, %0, 22;\n\tsetp.ne.u32 r, y, 0;\n\t@r st.shared.u8 [%1], y;\n\t"
-                        "shf.l.wrap.b32 %2, %3, %2, %0;\n\tshf.l.wrap.b32 %3, 0, %3, %0;\n\t"
-                        "and.b32 t, %0, 31;\n\tsub.u32 n, %6, t;\n\t"
-                        "shr.u32 g, %2, 19;\n\tshl.b32 g, g, 2;\n\tadd.u32 g, g, %8;\n\tld.shared.u32 %0, [g];\n\t"
-                        "xor.b32 t, n, %6;\n\tand.b32 t, t, 32;\n\tsetp.ne.u32 p, t, 0;\n\tmov.b32 %6, n;\n\t"
-                        "shf.r.wrap.b32 t, %4, 0, n;\n\t@p or.b32 %2, %2, t;\n\t@p shf.r.wrap.b32 %3, 0, %4, n;\n\t"
-                        "@p ld.shared.u32 %4, [%5];\n\t@p add.u32 %5, %5, 4;\n\t}"
-                        : "+r"(e), "+r"(at), "+r"(hi), "+r"(lo), "+r"(nxt), "+r"(next), "+r"(q)
-                        : "r"(row_end), "r"(tab) : "memory");
-                    continue;
-                }
                 at += __byte_perm(e, 0u, 0x4441) * (uint32_t)sizeof(Sym);
                 at = min(at, row_end);
                 // (no symbol: a part of a gap, or a lane that stands still)
@@ -247,16 +241,14 @@ __device__ __forceinline__ uint32_t walk_body(uint32_t copy, uint32_t from, uint
                     asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.u32 p, %1, 0;\n\t@p st.shared.u8 [%0], %1;\n\t}" ::"r"(at), "r"(e >> kSymShift) : "memory");
                 else
                     asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.u32 p, %1, 0;\n\t@p st.shared.u16 [%0], %1;\n\t}" ::"r"(at), "r"((int32_t)e >> kSymShift) : "memory");
-                const uint32_t q_was = q;
                 hi = __funnelshift_l(lo, hi, e);
                 lo = __funnelshift_l(0u, lo, e);
                 q -= e & kLenMask;
-                if (!GAPS) look_up();                       // (at least 13 valid bits are left)
-                asm("{\n\t.reg .pred p;\n\t.reg .b32 t;\n\txor.b32 t, %4, %5;\n\tand.b32 t, t, 32;\n\tsetp.ne.u32 p, t, 0;\n\t"
-                    "shf.r.wrap.b32 t, %2, 0, %4;\n\t@p or.b32 %0, %0, t;\n\t@p shf.r.wrap.b32 %1, 0, %2, %4;\n\t"
-                    "@p ld.shared.u32 %2, [%3];\n\t@p add.u32 %3, %3, 4;\n\t}"
-                    : "+r"(hi), "+r"(lo), "+r"(nxt), "+r"(next) : "r"(q), "r"(q_was));
-                if (GAPS) look_up();
+                // A look-up needs 13 valid bits, so of 32 two tokens can be taken (18 bits at most by a long one, 13 by an entry of the table).
+                // (With symbols of two bytes there are fewer warps and the look-ups' latency counts: each goes ahead of its refill.)
+                if (!GAPS && sizeof(Sym) == 2) look_up();
+                if (GAPS || sizeof(Sym) == 2 || (u & 1)) refill();
+                if (GAPS || sizeof(Sym) == 1) look_up();
             }
         }
     }
