@@ -15,14 +15,14 @@
 //
 // The walk is a chain of dependent steps.  What a step waits for is one table look-up and two shifts:
 //
-//   table   the next 13 bits of the chain give a whole token: the bits it takes, its gap and its symbol.
+//   table   the next 13 bits of the chain give a whole token, or two that fit: the bits, the gap and the symbols.
 //           A token that is longer than 13 bits is taken in two steps: the code of a gap ends with the
 //           bit 0, which is itself the code of gap 1, so an entry that stands for the gap's code without
 //           its last bit and for a gap one smaller, without a symbol, leaves an ordinary token of gap 1
 //           behind.  What the table cannot resolve at all (gaps from 128 on, long level codes) takes
 //           Algorithm 2's loop.
 //   window  64 bits hi:lo, shifted by the token's length and refilled to at least 32 valid bits every
-//           second step: a look-up needs the 13 top bits, so 32 last for two tokens.  (Refilled at every
+//           second step: a look-up needs the 13 top bits, so 32 last for two steps.  (Refilled at every
 //           step the walk takes 3 of 18 instructions more: ResNet-50, K = 8 85.2 us, now 83.4.)
 //   end     every lane has its own copy of its chain (cp.async, 112 bytes at a time) and puts ones
 //           behind the chain's last bit: thirteen ones are no token, the table says "0 bits, no gap, no
@@ -58,19 +58,29 @@ struct Row {
     static_assert(kWarpBytes >= field_warp_bytes(5) && kWarpBytes >= field_warp_bytes(10), "fixed-width streams use the same memory");
 };
 
-// Token table entries.  Bits 0-4: bits consumed (0: not resolved here); bits 8-15: gap; bits 22-31: symbol, signed
+// Token table entries.  Bits 0-4: bits consumed (0: not resolved here); bits 8-15: gap; on top, from Symbol::kShift on, the symbol, signed
 // (0: none, only a part of the gap).  Symbols: for exponential levels the upper byte of the level (with its sign) as
 // an fp16 number, 2^(j-1-s) being one without mantissa bits; for uniform levels the signed index.
-constexpr uint32_t kLenMask = 31u, kGapShift = 8u, kSymShift = 22u;
-__device__ __forceinline__ uint32_t exp_symbol(uint32_t index, uint32_t negative, uint32_t s) {
-    return ((negative ? 0x80u : 0u) | ((14u + index - s) << 2)) << kSymShift;
-}
-__device__ __forceinline__ uint32_t uniform_symbol(uint32_t index, uint32_t negative) {
-    return (negative ? 0u - index : index) << kSymShift;
-}
+// With symbols of one byte an entry may stand for two tokens (pairs): the gap is then that of both together, bits 5-7 are the
+// second one's (0: one token), bits 16-23 the first one's symbol.  Dense symbols take 5 bits a token and most look-ups give two;
+// sparse ones (8 bits and more) one in four, and gain next to nothing (K = 8 ResNet-50 containers: largest-magnitude norms with uniform
+// levels 193 -> 150 us, s = 4 in buckets of 512 149 -> 125, 8192 83.4 -> 81.1, s = 3 there 72.2 -> 72.6).
+constexpr uint32_t kLenMask = 31u, kGap2Shift = 5u, kMaxGap2 = 7u, kGapShift = 8u, kFirstShift = 16u;
+template <class Sym>
+constexpr bool kPairs = sizeof(Sym) == 1;
+template <class Sym>
+struct Symbol {
+    static constexpr uint32_t kShift = sizeof(Sym) == 1 ? 24u : 22u;
+    static __device__ __forceinline__ uint32_t exponential(uint32_t index, uint32_t negative, uint32_t s) {
+        return ((negative ? 0x80u : 0u) | ((14u + index - s) << 2)) << kShift;
+    }
+    static __device__ __forceinline__ uint32_t uniform(uint32_t index, uint32_t negative) { return (negative ? 0u - index : index) << kShift; }
+};
 
-// Tables as kept in device memory (kTabErc and kTabGaps): the symbol is the level index (1 .. 255), bit 31 of the entry the sign.
-__device__ uint32_t g_token_tables[2][kTokEntries];
+// Tables as kept in device memory: kTabErc and kTabGaps with one token to an entry, bits 22-30 the level index (1 .. 255), bit 31 its
+// sign; and ERC tokens in pairs, in the format above but for the symbols, which are level indices (1 .. 31: longer codes do not fit) with the sign in bit 7.
+constexpr uint32_t kTabPairs = 2u, kIndexShift = 22u;
+__device__ uint32_t g_token_tables[3][kTokEntries];
 
 // ERC^-1 of the nbits-bit prefix idx from bit `pos` on (Algorithm 2, decoding): false when the code does not end within it.
 static bool erc_of_prefix(uint32_t idx, uint32_t nbits, uint32_t* pos, uint32_t* value) {
@@ -90,7 +100,7 @@ static bool erc_of_prefix(uint32_t idx, uint32_t nbits, uint32_t* pos, uint32_t*
 }
 
 cudaError_t upload_token_tables() {
-    static uint32_t tab[2][kTokEntries];
+    static uint32_t tab[3][kTokEntries];
     for (uint32_t i = 0; i < kTokEntries; ++i) {
         uint32_t pos = 0, gap = 0;
         tab[kTabErc][i] = tab[kTabGaps][i] = 0;
@@ -98,9 +108,18 @@ cudaError_t upload_token_tables() {
         tab[kTabGaps][i] = pos | (gap << kGapShift);
         uint32_t at = pos + 1u, index = 0;                  // behind the sign bit
         if (at < kTokBits && erc_of_prefix(i, kTokBits, &at, &index) && index <= 255u)
-            tab[kTabErc][i] = at | (gap << kGapShift) | (index << kSymShift) | (((i >> (kTokBits - 1u - pos)) & 1u) << 31);
+            tab[kTabErc][i] = at | (gap << kGapShift) | (index << kIndexShift) | (((i >> (kTokBits - 1u - pos)) & 1u) << 31);
         else if (pos > 1u)
             tab[kTabErc][i] = (pos - 1u) | ((gap - 1u) << kGapShift);
+    }
+    for (uint32_t i = 0; i < kTokEntries; ++i) {
+        auto symbol = [](uint32_t e) { return (e >> kIndexShift & 0x1ffu) | (e >> 31) << 7; };
+        const uint32_t e = tab[kTabErc][i], then = tab[kTabErc][(i << (e & kLenMask)) & (kTokEntries - 1u)];
+        const uint32_t len = (e & kLenMask) + (then & kLenMask), gap2 = (then >> kGapShift) & 0xffu;
+        if (symbol(e) && symbol(then) && len <= kTokBits && gap2 <= kMaxGap2)
+            tab[kTabPairs][i] = len | gap2 << kGap2Shift | ((e & 0xff00u) + (gap2 << kGapShift)) | symbol(e) << kFirstShift | symbol(then) << 24;
+        else
+            tab[kTabPairs][i] = (e & 0xffffu) | symbol(e) << 24;
     }
     const cudaError_t e = cudaMemcpyToSymbol(g_token_tables, tab, sizeof(tab));
     // (the copy goes by the default stream, whose end kernels of a non-blocking stream do not wait for)
@@ -138,27 +157,32 @@ __device__ __forceinline__ bool erc_in_window(uint32_t win, uint32_t* at, uint32
     return false;
 }
 
-// A stream with coded level indices brings its own code: the level index and the word's length (<< 8) by the
-// next 7 bits, 0 where no word starts (possible only with an incomplete code).
-__device__ __forceinline__ uint32_t coded_entry(const StreamHead& hd, uint32_t s, uint32_t prefix) {
-    const uint32_t w0 = *(hd.hdr + hd.hwords - 2u), w1 = *(hd.hdr + hd.hwords - 1u);   // the lengths, one byte each
+// A stream with coded level indices brings its own code, w0 and w1: the words' lengths, one byte each.  Canonical words: level
+// indices by (length, index), the first word all zeros, each next one the previous plus one; so the word of index j (+ 1) counts, in
+// units of its own length, the words before it.  Returned with its length << 16.
+__device__ __forceinline__ uint32_t level_word(uint32_t w0, uint32_t w1, uint32_t s, uint32_t j) {
     auto len_of = [&](uint32_t j) { return ((j < 4u ? w0 : w1) >> (8u * (j & 3u))) & 0xffu; };
+    const uint32_t lj = len_of(j);
+    uint32_t word = 0;
+    for (uint32_t k = 0; k <= s; ++k) {
+        const uint32_t lk = len_of(k);
+        if (lk < lj || (lk == lj && k < j)) word += 1u << (lj - lk);
+    }
+    return word | lj << 16;
+}
+// The level index and its word's length (<< 8) by the next 7 bits, 0 where no word starts (possible only with an incomplete code).
+template <class WordOf>
+__device__ __forceinline__ uint32_t coded_entry(WordOf word_of, uint32_t s, uint32_t prefix) {
     for (uint32_t j = 0; j <= s; ++j) {
-        // canonical words: level indices by (length, index), the first word all zeros, each next one the
-        // previous plus one; so the word of j counts, in units of its own length, the words before it
-        const uint32_t lj = len_of(j);
-        uint32_t word = 0;
-        for (uint32_t k = 0; k <= s; ++k) {
-            const uint32_t lk = len_of(k);
-            if (lk < lj || (lk == lj && k < j)) word += 1u << (lj - lk);
-        }
-        if ((prefix >> (kMaxCodedS - lj)) == word) return (j + 1u) | (lj << 8);
+        const uint32_t w = word_of(j);
+        if ((prefix >> (kMaxCodedS - (w >> 16))) == (w & 0xffffu)) return (j + 1u) | (w >> 16 << 8);
     }
     return 0;
 }
 
 // A token the table does not resolve, by Algorithm 2's loop; a gap longer than 1 is taken on its own, as in the table.
 // Returns the entry the table would hold, 0 when the bits are no token.
+template <class Sym>
 __device__ __noinline__ uint32_t long_token(uint32_t win, const StreamHead& hd, const uint16_t* code, bool gaps_only, uint32_t s) {
     uint32_t at = 0, gap = 0, index = 0;
     if (!erc_in_window(win, &at, &gap) || gap > kSB) return 0u;
@@ -174,7 +198,7 @@ __device__ __noinline__ uint32_t long_token(uint32_t win, const StreamHead& hd, 
     }
     if (index == 0u || index >= hd.nlev) return 0u;
     const uint32_t negative = (win >> 30) & 1u;
-    return at | (1u << kGapShift) | (hd.levelset == kLevelsUniform ? uniform_symbol(index, negative) : exp_symbol(index, negative, s));
+    return at | (1u << kGapShift) | (hd.levelset == kLevelsUniform ? Symbol<Sym>::uniform(index, negative) : Symbol<Sym>::exponential(index, negative, s));
 }
 
 // What a lane knows of its chain.
@@ -209,7 +233,7 @@ __device__ __forceinline__ uint32_t walk_body(uint32_t copy, uint32_t from, uint
         if (GAPS) {
             const uint32_t behind = hi << (e & kLenMask), cw = code[(behind << 1) >> (32u - kMaxCodedS)];
             const uint32_t len = (e & kLenMask) + 1u + (cw >> 8), index = cw & 0xffu, negative = behind >> 31;
-            const uint32_t sym = hd.levelset == kLevelsUniform ? uniform_symbol(index, negative) : exp_symbol(index, negative, s);
+            const uint32_t sym = hd.levelset == kLevelsUniform ? Symbol<Sym>::uniform(index, negative) : Symbol<Sym>::exponential(index, negative, s);
             e = e != 0u && cw != 0u ? len | (e & (0xffu << kGapShift)) | sym : 0u;
         }
     };
@@ -226,7 +250,7 @@ __device__ __forceinline__ uint32_t walk_body(uint32_t copy, uint32_t from, uint
         for (;;) {
             if (e == 0u) {
                 if ((int32_t)(q - c) <= 0) break;
-                e = long_token(hi, hd, code, GAPS, s);
+                e = long_token<Sym>(hi, hd, code, GAPS, s);
                 if (e == 0u) {
                     good = false;
                     break;
@@ -238,9 +262,13 @@ __device__ __forceinline__ uint32_t walk_body(uint32_t copy, uint32_t from, uint
                 at = min(at, row_end);
                 // (no symbol: a part of a gap, or a lane that stands still)
                 if (sizeof(Sym) == 1)
-                    asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.u32 p, %1, 0;\n\t@p st.shared.u8 [%0], %1;\n\t}" ::"r"(at), "r"(e >> kSymShift) : "memory");
+                    asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.u32 p, %1, 0;\n\t@p st.shared.u8 [%0], %1;\n\t}" ::"r"(at), "r"(e >> Symbol<Sym>::kShift) : "memory");
                 else
-                    asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.u32 p, %1, 0;\n\t@p st.shared.u16 [%0], %1;\n\t}" ::"r"(at), "r"((int32_t)e >> kSymShift) : "memory");
+                    asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.u32 p, %1, 0;\n\t@p st.shared.u16 [%0], %1;\n\t}" ::"r"(at), "r"((int32_t)e >> Symbol<Sym>::kShift) : "memory");
+                if (kPairs<Sym> && !GAPS) {
+                    const uint32_t gap2 = (e >> kGap2Shift) & kMaxGap2;
+                    asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.u32 p, %1, 0;\n\t@p st.shared.u8 [%0], %2;\n\t}" ::"r"(at - gap2), "r"(gap2), "r"(e >> kFirstShift) : "memory");
+                }
                 hi = __funnelshift_l(lo, hi, e);
                 lo = __funnelshift_l(0u, lo, e);
                 q -= e & kLenMask;
@@ -487,7 +515,7 @@ __device__ __forceinline__ void fields_of_width(const DecodeParams& P, const Str
 template <class Sym, bool MANY, bool CALLED>
 __device__ __forceinline__ void decode_streams(const DecodeParams& P) {
     extern __shared__ __align__(128) unsigned char dsm[];
-    __shared__ uint32_t s_kind, s_alike, s_fields;
+    __shared__ uint32_t s_kind, s_alike, s_fields, s_words[kMaxCodedS + 1];
     const Geometry& G = P.geo;
     const uint32_t K = P.K, tid = threadIdx.x, lane = tid & 31u, warp = tid >> 5;
     uint32_t* const table = reinterpret_cast<uint32_t*>(dsm);
@@ -502,34 +530,66 @@ __device__ __forceinline__ void decode_streams(const DecodeParams& P) {
         for (uint32_t i = 16u * lane; i < 32u * Row<Sym>::kPitch; i += 512u)
             asm volatile("st.shared.v4.u32 [%0], {%1, %1, %1, %1};" ::"r"(rows + i), "r"(0u) : "memory");
     };
-    // The token table for streams of kind `kind` (`code`: their level code, kTabCoded only).
+    using Symbols = Symbol<Sym>;
+    // the entry of a gap's code joined with the streams' level code
+    auto coded_token = [&](uint32_t e, uint32_t i, const uint16_t* code) {
+        const uint32_t at = e & kLenMask, low = e & 0xffffu;
+        if (at == 0u) return 0u;
+        const uint32_t rest = i << (32u - kTokBits + at), c = code[(rest << 1) >> (32u - kMaxCodedS)];
+        const uint32_t len = at + 1u + (c >> 8);
+        if (c != 0u && len <= kTokBits) return len | (low & (0xffu << kGapShift)) | Symbols::exponential(c & 0xffu, rest >> 31, G.s);
+        return at > 1u ? (at - 1u) | ((low & (0xffu << kGapShift)) - (1u << kGapShift)) : 0u;
+    };
+    // The token table for streams of kind `kind` (`code`: their level code, kTabCoded only), in pairs but for a level code's.
     auto build_table = [&](uint32_t kind, const uint16_t* code) {
-        const uint4* src = reinterpret_cast<const uint4*>(g_token_tables[kind == kTabErc || kind == kTabUniform ? kTabErc : kTabGaps]);
+        const bool erc = kind == kTabErc || kind == kTabUniform;
+        const uint4* src = reinterpret_cast<const uint4*>(g_token_tables[!erc ? kTabGaps : kPairs<Sym> ? kTabPairs : kTabErc]);
         const uint32_t top = kind == kTabUniform ? 1u << G.s : G.s + 1u;
         auto entry = [&](uint32_t e, uint32_t i) {
             if (kind == kTabGaps) return e;
-            const uint32_t at = e & kLenMask, low = e & 0xffffu;
-            if (kind == kTabCoded) {                        // the gap's entry joined with the streams' level code
-                if (at == 0u) return 0u;
-                const uint32_t rest = i << (32u - kTokBits + at), c = code[(rest << 1) >> (32u - kMaxCodedS)];
-                const uint32_t len = at + 1u + (c >> 8);
-                if (c != 0u && len <= kTokBits) return len | (low & (0xffu << kGapShift)) | exp_symbol(c & 0xffu, rest >> 31, G.s);
-                return at > 1u ? (at - 1u) | ((low & (0xffu << kGapShift)) - (1u << kGapShift)) : 0u;
-            }
-            const uint32_t index = (e >> kSymShift) & 0x1ffu, negative = e >> 31;
+            if (kind == kTabCoded) return coded_token(e, i, code);
+            const uint32_t index = (e >> kIndexShift) & 0x1ffu, negative = e >> 31;
             if (index == 0u) return e;
             if (index > top) return 0u;
-            return low | (kind == kTabUniform ? uniform_symbol(index, negative) : exp_symbol(index, negative, G.s));
+            return (e & 0xffffu) | (kind == kTabUniform ? Symbols::uniform(index, negative) : Symbols::exponential(index, negative, G.s));
+        };
+        // a ready-made pair with this call's symbols; 0 where there is no such index (long_token takes the first one then, if that exists)
+        auto ready = [&](uint32_t e) {
+            const uint32_t first = (e >> kFirstShift) & 31u, last = (e >> 24) & 31u;
+            if (first > top || last > top) return 0u;
+            if (last == 0u) return e;
+            if (kind == kTabErc) return e + ((e & 0x1f1f0000u) * 3u) + ((14u - G.s) << 26) + (first ? (14u - G.s) << (kFirstShift + 2u) : 0u);
+            const uint32_t f = e & 1u << 23 ? 0u - first : first, l = e >> 31 ? 0u - last : last;
+            return (e & 0xffffu) | (f & 0xffu) << kFirstShift | l << 24;
         };
 #pragma unroll 4
         for (uint32_t i = tid; i < kTokEntries / 4u; i += blockDim.x) {
             uint4 e = __ldg(src + i);
-            e.x = entry(e.x, 4u * i);
-            e.y = entry(e.y, 4u * i + 1u);
-            e.z = entry(e.z, 4u * i + 2u);
-            e.w = entry(e.w, 4u * i + 3u);
+            if (kPairs<Sym> && erc) {
+                e = make_uint4(ready(e.x), ready(e.y), ready(e.z), ready(e.w));
+            } else {
+                e = make_uint4(entry(e.x, 4u * i), entry(e.y, 4u * i + 1u), entry(e.z, 4u * i + 2u), entry(e.w, 4u * i + 3u));
+            }
             reinterpret_cast<uint4*>(table)[i] = e;
         }
+    };
+    // ... and a level code's in pairs, by way of the table of single tokens at `singles`: a token and the one behind it, if that is a
+    // whole one and near enough.  (The bits behind the prefix are taken for zeros; they do not matter to a token that ends within it.)
+    // The entry behind prefix i is that of i moved up by a token's length, for neighbouring i a power of two apart: entries are
+    // kept within 32 by the sum of their five-bit digits, which keeps them in different banks (2 us of 15 otherwise).
+    auto build_pairs = [&](const uint16_t* code, uint32_t* singles) {
+        auto place = [](uint32_t i) { return i ^ ((i >> 5 ^ i >> 10) & 31u); };
+#pragma unroll 8
+        for (uint32_t i = tid; i < kTokEntries; i += blockDim.x) singles[place(i)] = coded_token(__ldg(g_token_tables[kTabGaps] + i), i, code);
+        __syncthreads();
+#pragma unroll 8
+        for (uint32_t i = tid; i < kTokEntries; i += blockDim.x) {
+            const uint32_t e = singles[place(i)], then = singles[place((i << (e & kLenMask)) & (kTokEntries - 1u))];
+            const uint32_t len = (e & kLenMask) + (then & kLenMask), gap2 = (then >> kGapShift) & 0xffu;
+            const bool two = e >> 24 != 0u && then >> 24 != 0u && len <= kTokBits && gap2 <= kMaxGap2;
+            table[i] = two ? len | gap2 << kGap2Shift | ((e & 0xff00u) + (gap2 << kGapShift)) | (e >> 24) << kFirstShift | (then & 0xff000000u) : e;
+        }
+        __syncthreads();
     };
 
     // The kernel is launched with programmatic stream serialization: its CTAs take the SMs as the kernel in front leaves
@@ -582,6 +642,7 @@ __device__ __forceinline__ void decode_streams(const DecodeParams& P) {
                 if (__any_sync(0xffffffffu, in_code && (w0 != first0 || w1 != first1))) found |= kSeveralCodes;
             }
         }
+        if ((found & kCoded) && lane <= min(G.s, kMaxCodedS)) s_words[lane] = level_word(first0, first1, G.s, lane);
         if (lane == 0) {
             s_kind = found & kCoded ? (found & (kErc | kSeveralCodes) ? kTabGaps : kTabCoded)
                      : found & kUniform ? (found & kOther ? kTabGaps : kTabUniform) : kTabErc;
@@ -595,6 +656,10 @@ __device__ __forceinline__ void decode_streams(const DecodeParams& P) {
         return;
     }
     if (CALLED) clear_rows();
+    const uint32_t S = P.unit_subs;                         // sub-blocks of a unit
+    const uint32_t nsub = (uint32_t)((G.d + kSB - 1u) / kSB), nunits = (uint32_t)(((uint64_t)nsub + S - 1u) / S), stride = gridDim.x * (blockDim.x >> 5);
+    // A level code's table is built when the headers have been read, and its pairs take a microsecond more: not where no warp has a
+    // second unit (65 536 elements 11.6 us without, 12.6 with them; 8 x 10^6, K = 4: 27.3 and 26.0).
     const uint32_t kind = s_kind, all_alike = s_alike == 3u && s_kind == kTabGaps ? 2u : s_alike;
     if (kind != P.likely_table || kind == kTabGaps || kind == kTabCoded || all_alike >= 2u) {
         uint32_t first = K;                                 // the first token stream (all have the same code in the coded mode)
@@ -605,7 +670,8 @@ __device__ __forceinline__ void decode_streams(const DecodeParams& P) {
             if (kind == kTabGaps || (kind == kTabCoded && first == K)) {   // level index by the next 7 bits
                 for (uint32_t i = tid; i < (1u << kMaxCodedS); i += blockDim.x) {
                     uint32_t c = 0, at = 0, index = 0;
-                    if (hd.mode == kModeCoded) c = coded_entry(hd, G.s, i);
+                    if (kind == kTabCoded) c = coded_entry([](uint32_t j) { return s_words[j]; }, G.s, i);     // (all streams have this code)
+                    else if (hd.mode == kModeCoded) c = coded_entry([&](uint32_t j) { return level_word(hd.hdr[hd.hwords - 2u], hd.hdr[hd.hwords - 1u], G.s, j); }, G.s, i);
                     else if (erc_in_window(i << (32u - kMaxCodedS) | 0x01ffffffu, &at, &index) && at <= kMaxCodedS && index < hd.nlev) c = index | (at << 8);
                     code[i] = (uint16_t)c;
                 }
@@ -616,7 +682,13 @@ __device__ __forceinline__ void decode_streams(const DecodeParams& P) {
             if (first == K) first = k;
         }
         if (kind == kTabCoded) __syncthreads();
-        if (kind != P.likely_table || kind == kTabCoded) build_table(kind, reinterpret_cast<const uint16_t*>(codes + (first == K ? 0u : first) * kCodeBytes));
+        const uint16_t* const code = reinterpret_cast<const uint16_t*>(codes + (first == K ? 0u : first) * kCodeBytes);
+        if (kPairs<Sym> && kind == kTabCoded && nunits > stride) {         // the single tokens where the rows will be
+            build_pairs(code, reinterpret_cast<uint32_t*>(dsm + chain_fixed_bytes(K)));
+            clear_rows();
+        } else if (kind != P.likely_table || kind == kTabCoded) {
+            build_table(kind, code);
+        }
         __syncthreads();
         if (all_alike == 3u) {                              // levels by symbol, sign included (the codes are no longer needed)
             for (uint32_t i = tid; i < 64u * K; i += blockDim.x) {
@@ -630,8 +702,6 @@ __device__ __forceinline__ void decode_streams(const DecodeParams& P) {
     // from here on warps run alone
 
     const uint32_t tab = smem_u32(table);
-    const uint32_t S = P.unit_subs;                         // sub-blocks of a unit
-    const uint32_t nsub = (uint32_t)((G.d + kSB - 1u) / kSB), nunits = (uint32_t)(((uint64_t)nsub + S - 1u) / S), stride = gridDim.x * (blockDim.x >> 5);
     const uint32_t spb = G.bucket <= kBLK ? G.sb_per_block : 32u;   // sub-blocks of a coding block
     const uint32_t lj = lane / S, lq = lane - lj * S;
     const uint32_t ngroups = MANY ? (K + 31u) / 32u : 1u;   // of up to 32 streams (S = 1 when there are several)
@@ -752,15 +822,18 @@ __device__ __forceinline__ void decode_streams(const DecodeParams& P) {
         uint32_t left = ch.len;
         if (!long_chain) {
             put_ones();
-            left -= kind == kTabGaps ? walk_rare<Sym, false, true>(copy, ch.bit, left, tab, row, row_end, my_head, my_code, G.s, good)
-                                     : walk_body<Sym, false, false>(copy, ch.bit, left, tab, row, row_end, my_head, my_code, G.s, good);
+            if (kind == kTabGaps) left -= walk_rare<Sym, false, true>(copy, ch.bit, left, tab, row, row_end, my_head, my_code, G.s, good);
+            else left -= walk_body<Sym, false, false>(copy, ch.bit, left, tab, row, row_end, my_head, my_code, G.s, good);
         } else {
             // chains longer than a lane's copy: one copy after the other, each walked up to 96 bits before its end
             while (__any_sync(0xffffffffu, left != 0u)) {
                 const uint32_t room = 32u * kChunkWords - ch.bit;
                 const uint32_t bits = fits(ch) ? left : room - 96u;
-                uint32_t took = kind == kTabGaps ? walk_rare<Sym, true, true>(copy, ch.bit, bits, tab, row, row_end, my_head, my_code, G.s, good)
-                                                 : walk_rare<Sym, true, false>(copy, ch.bit, bits, tab, row, row_end, my_head, my_code, G.s, good);
+                // (a pair of tokens must not reach into the chain behind: it may pass the point by 12 bits)
+                if (ch.bit + ch.len <= 32u * (kChunkWords - 2u)) put_ones();
+                uint32_t took;
+                if (kind == kTabGaps) took = walk_rare<Sym, true, true>(copy, ch.bit, bits, tab, row, row_end, my_head, my_code, G.s, good);
+                else took = walk_rare<Sym, true, false>(copy, ch.bit, bits, tab, row, row_end, my_head, my_code, G.s, good);
                 if (!good || took > left) {
                     good = false;
                     took = left;
@@ -865,11 +938,6 @@ static DecodeKernel fields_kernel(uint32_t s, uint32_t levelset) {
 
 template <class Sym>
 static cudaError_t launch_chains(const DecodeParams& P, int sms, cudaStream_t stream) {
-    const DecodeKernel kernel = P.likely_table == kTabFields ? fields_kernel(P.geo.s, P.likely_levels)
-                                : P.K > 32u ? decode_chains_kernel<Sym, true> : decode_chains_kernel<Sym, false>;
-    static std::map<DecodeKernel, OncePerDevice> prepared;
-    const cudaError_t e = prepared[kernel]([=] { return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kChainSmem); });
-    if (e != cudaSuccess) return e;
     const size_t fixed = chain_fixed_bytes(P.K);
     size_t warps = (kChainSmem - fixed) / Row<Sym>::kWarpBytes;
     if (warps > kChainMaxWarps) warps = kChainMaxWarps;
@@ -882,6 +950,11 @@ static cudaError_t launch_chains(const DecodeParams& P, int sms, cudaStream_t st
     if (share < Q.unit_subs) Q.unit_subs = (uint32_t)share;
     const uint64_t units = (nsub + Q.unit_subs - 1u) / Q.unit_subs;
     Q.let_next = units > 2u * (uint64_t)sms * warps ? 1u : 0u;
+    DecodeKernel kernel = P.K > 32u ? decode_chains_kernel<Sym, true> : decode_chains_kernel<Sym, false>;
+    if (P.likely_table == kTabFields) kernel = fields_kernel(P.geo.s, P.likely_levels);
+    static std::map<DecodeKernel, OncePerDevice> prepared;
+    const cudaError_t e = prepared[kernel]([=] { return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kChainSmem); });
+    if (e != cudaSuccess) return e;
     cudaLaunchConfig_t cfg = cudaLaunchConfig_t{};
     cudaLaunchAttribute attr[1];
     cfg.gridDim = dim3((unsigned)(units < (uint64_t)sms ? units : (uint64_t)sms));

@@ -81,6 +81,26 @@ def test_sums_of_streams_with_different_codes_and_level_sets():
     _same_sums(streams + tables, d, bucket, s)
 
 
+@pytest.mark.parametrize("kind", ["normal", "sparse", "dense", "mixed", "ends"])
+@pytest.mark.parametrize("weights", [[9, 5, 3, 2, 1], [1, 1, 1, 1, 1], [1, 2, 4, 8, 16, 32, 64]])
+def test_sums_of_coded_streams_where_warps_have_several_units(kind, weights):
+    """A level code's table holds pairs of tokens there (32 streams: a unit is one sub-block)."""
+    d, bucket, s = 2500 * 256 + 77, 1024, len(weights) - 1
+    O.set_level_code(O.huffman_lengths(weights))
+    streams = [_container(kind, d, bucket, s, O.NORM_L2, O.LEVELS_EXP, O.MODE_CODED, k) for k in range(2)]
+    _same_sums(streams * 16, d, bucket, s)
+
+
+@pytest.mark.parametrize("ls,s,less", [(O.LEVELS_EXP, 6, 3), (O.LEVELS_EXP, 5, 4), (O.LEVELS_UNIFORM, 4, 2), (O.LEVELS_UNIFORM, 4, 3)])
+def test_symbols_beyond_the_last_level_are_refused(ls, s, less):
+    """Containers whose header claims fewer levels than they use: many such symbols follow a good one within a table's prefix."""
+    d, bucket = 20001, 1024
+    c = _container("normal", d, bucket, s, O.NORM_LINF, ls, O.MODE_ERC, 4)
+    c[5] = less
+    assert O.decode_accumulate([c], d, bucket, less)[0] != 0
+    gpu_decode([c], d, bucket, less, expect_status=-3)
+
+
 def test_missing_symbols_and_values_that_are_not_finite_in_fixed_width_streams():
     require_cuda()
     d, bucket, s = 5000, 1024, 3                                    # 5 levels in 3 bits: 5, 6 and 7 do not exist
