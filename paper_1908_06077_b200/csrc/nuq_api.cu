@@ -141,7 +141,8 @@ uint32_t token_bits_bound(const Geometry& G, uint32_t elems, uint32_t buckets, b
 // words of shared-memory staging the records of one ERC tile can need
 uint32_t stage_words_for(const Geometry& G, bool norms_are_ours) {
     uint32_t head = 1u + (G.sb_per_block + 1u) / 2u + 1u;          // norm, lengths, padding
-    return G.blocks_per_tile * head + (token_bits_bound(G, kBLK, G.blocks_per_tile, norms_are_ours) + 31u) / 32u;
+    const uint32_t elems = G.bucket <= kBLK ? G.tile_elems : kBLK;
+    return G.blocks_per_tile * head + (token_bits_bound(G, elems, G.blocks_per_tile, norms_are_ours) + 31u) / 32u;
 }
 
 uint64_t bound_bytes(const Geometry& G) {
@@ -235,7 +236,7 @@ static int occupancy(const EncodeParams& P, int dev, bool clusters) {
     const uint64_t key = (uint64_t)encode_smem_bytes(P) | (uint64_t)G.levelset << 32 | (uint64_t)G.mode << 34 |
                          (uint64_t)(fixed4_applies(G) ? 1u + fixed4_variant(G) : 0u) << 36 |
                          (uint64_t)(P.warps >> 3) << 42 |
-                         (uint64_t)(clusters ? P.cluster : 0) << 38 | (uint64_t)(uint32_t)dev << 44;
+                         (uint64_t)(clusters ? P.cluster : 0) << 38 | (uint64_t)(uint32_t)dev << 44 | (uint64_t)(P.tile != kBLK) << 63;
     const auto it = known.find(key);
     if (it != known.end()) return it->second;
     const int n = clusters ? encode_max_clusters(P) : encode_blocks_per_sm(P);
@@ -245,24 +246,36 @@ static int occupancy(const EncodeParams& P, int dev, bool clusters) {
 
 static EncodePlan plan_encode(EncodeParams& P, int dev, uint32_t flags) {
     const int sms = device_sms(dev);
-    const Geometry& G = P.geo;
+    Geometry& G = P.geo;
     const bool norms_are_ours = (flags & NUQ_TEST_NORMS) == 0;
     EncodePlan pl;
-    pl.state_bytes = sizeof(Workspace) + 8 * (G.ntiles + (G.ntiles + 31) / 32);
     pl.norms_bytes = G.bucket > kBLK ? 4 * G.nb : 0;
     // a look-back wait polls this often (with a pause in between: tens of ms in all) before it gives up
     P.patience = (flags & NUQ_TEST_SHORT_PATIENCE) ? 2u : 1u << 16;
     P.window_words = 0;
     P.stage_words = 0;
-    // A call that gives an SM two tiles at most (a tile's latency counts there, not the SM's throughput): twice the warps
-    // per tile.  65536 elements 11.0 -> 10.0 us, 10^6 elements 16.4 -> 12.7 us; from three tiles per SM on 8 warps are
-    // faster.  With clusters 10^6 elements 20.9 -> 17.7 us,
-    // a single cluster 13 to 15 us with either.  (The fixed-width encoders have no such variant.)
-    P.warps = G.mode != kModeFixed && G.ntiles <= 2u * (uint64_t)sms ? kEncMaxWarps : kEncWarps;
+    // Small calls: a tile's latency counts there, not the SM's throughput.  (The fixed-width encoders have no such variants.)
+    // Up to one tile per SM, with buckets of which a small tile holds one at least: a quarter of a tile, one sub-block per
+    // warp.  65 536 elements 10.5 us in whole tiles of 16 warps, 9.0 in small ones (uniform levels 13.1 and 9.3), 10^6 elements
+    // with coded indices 15.5 and 13.6; 2 x 10^6 15.8 and 18.2.
+    // Up to three tiles per SM: twice the warps per tile.  10^6 elements 16.4 -> 12.7 us, 3 x 10^6 18.7 -> 16.8 (uniform levels
+    // 24.5 -> 21.3), 4 x 10^6 19.5 and 19.8.  With clusters 10^6 elements 20.9 -> 17.7, a single cluster 13 to 15 us with either.
+    const bool tokens = G.mode != kModeFixed;
+    P.warps = tokens && G.ntiles <= 3u * (uint64_t)sms ? kEncMaxWarps : kEncWarps;
+    P.tile = kBLK;
+    if (tokens && G.bucket <= kSmallTile && G.ntiles <= (uint64_t)sms) {
+        P.tile = kSmallTile;
+        P.warps = kEncWarps;
+        G.blocks_per_tile = kSmallTile / G.bucket;
+        G.tile_elems = G.blocks_per_tile * G.bucket;
+        G.ntiles = (G.nb + G.blocks_per_tile - 1) / G.blocks_per_tile;
+    }
+    // (the tiles' number is what it will be from here on)
+    pl.state_bytes = sizeof(Workspace) + 8 * (G.ntiles + (G.ntiles + 31) / 32);
     if (G.mode != kModeFixed) {
         P.stage_words = (stage_words_for(G, norms_are_ours) + 3u) & ~3u;
         // a warp's elements lie in at most this many buckets
-        const uint32_t warp_elems = kBLK / P.warps;
+        const uint32_t warp_elems = P.tile / P.warps;
         // (tiles start at bucket boundaries and a warp's part at a multiple of its size)
         const uint32_t warp_buckets = G.bucket >= warp_elems ? (G.bucket % warp_elems == 0 ? 1u : 2u)
                                                              : (warp_elems % G.bucket == 0 ? warp_elems / G.bucket : warp_elems / G.bucket + 1u);
@@ -503,7 +516,7 @@ nuq_status nuq_level_histogram(const float* g, uint64_t d, uint32_t bucket, uint
         P.round_keys[2 * r] = (uint32_t)seed + r * 0x9E3779B9u;
         P.round_keys[2 * r + 1] = (uint32_t)(seed >> 32) + r * 0xBB67AE85u;
     }
-    P.stage_words = P.window_words = P.patience = P.grid = P.cluster = P.overlap = P.let_next = P.warps = 0;
+    P.stage_words = P.window_words = P.patience = P.grid = P.cluster = P.overlap = P.let_next = P.warps = P.tile = 0;
     if (cudaMemsetAsync(hist, 0, 8 * (s + 2), stream) != cudaSuccess) return NUQ_ERR_CUDA;
     if (launch_level_histogram(P, hist, device_sms(dev), stream) != cudaSuccess) return NUQ_ERR_CUDA;
     return NUQ_OK;

@@ -16,6 +16,7 @@ constexpr uint32_t kMaxK = 64;
 constexpr int kEncThreads = 256;          // 8 warps share a tile, 1024 elements each
 constexpr int kEncWarps = kEncThreads / 32;
 constexpr int kEncMaxWarps = 16;          // ... in small calls, 512 elements each
+constexpr uint32_t kSmallTile = 8 * kSB;  // elements of a tile in small calls with small buckets
 constexpr int kEncMinBlocks = 4;          // resident CTAs per SM the encoder is compiled for (register cap) ...
 constexpr int kEncMaxBlocks = 4;          // ... and the most it is launched with
 
@@ -84,6 +85,7 @@ struct EncodeParams {
     uint32_t window_words;   // ERC: shared-memory token string of one warp and tile; a warp holds two
     uint32_t patience;       // polls a look-back wait may take before it gives up
     uint32_t warps;          // worker warps per CTA: kEncWarps, or kEncMaxWarps
+    uint32_t tile;           // elements a CTA has room for: kBLK, or kSmallTile
     uint32_t grid;           // CTAs to launch
     uint32_t cluster;        // CTAs per thread-block cluster: the blocks of one wide bucket (0: no clusters)
     uint32_t overlap;        // launched so that its CTAs are set up while the kernel before it in the stream ends

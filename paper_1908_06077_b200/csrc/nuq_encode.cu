@@ -562,9 +562,9 @@ __device__ void flush_pending(const EncodeParams& P, Pending& pd, CtaTotals& tot
 }
 
 // CLUSTERS: the call's buckets are wider than a tile and each is encoded by a thread-block cluster (see below).
-// W: worker warps, 8 as a rule.  Calls that give an SM two tiles at most take 16 (half the sub-blocks per warp): there a
-// tile's own latency is what counts.
-template <uint32_t LEVELSET, uint32_t MODE, bool CLUSTERS, uint32_t W>
+// W: worker warps, 8 as a rule, TILE: elements a CTA takes at a time.  Small calls take 16 (half the sub-blocks per warp) or, with
+// small buckets, small tiles (one sub-block per warp): there a tile's own latency is what counts.
+template <uint32_t LEVELSET, uint32_t MODE, bool CLUSTERS, uint32_t W, uint32_t TILE>
 __global__ void __launch_bounds__(MODE == kModeErc ? all_threads(W) : 32u * W, W == 8u ? kEncMinBlocks : 2)
 encode_kernel(const __grid_constant__ EncodeParams P) {
     extern __shared__ __align__(128) uint32_t smem[];
@@ -591,12 +591,12 @@ encode_kernel(const __grid_constant__ EncodeParams P) {
     __shared__ unsigned long long s_bucket[4];             // buckets of the iterations to come, handed out by the cluster's first CTA
 
     using S = Sym<LEVELSET>;
-    constexpr uint32_t kAll = all_threads(W), kWarpElems = kBLK / W, kQ = kWarpElems / kSB;   // elements and sub-blocks of a tile per warp
+    constexpr uint32_t kAll = all_threads(W), kWarpElems = TILE / W, kQ = kWarpElems / kSB;   // elements and sub-blocks of a tile per warp
     const Geometry& G = P.geo;
     const uint32_t tid = threadIdx.x, lane = tid & 31u;
     const uint32_t warp = __shfl_sync(0xffffffffu, tid >> 5, 0);      // (the same in all lanes, and known to be)
-    float* const data = reinterpret_cast<float*>(smem);                         // kBLK floats: the tile
-    uint32_t* const images = smem + kBLK;                                       // [2][stage_words]: staged tile records
+    float* const data = reinterpret_cast<float*>(smem);                         // TILE floats: the tile
+    uint32_t* const images = smem + TILE;                                       // [2][stage_words]: staged tile records
     uint32_t* const windows = images + 2u * P.stage_words;                      // [2][W][window_words]: token strings
     uint64_t* tile_state = reinterpret_cast<uint64_t*>(P.ws + 1);
     uint64_t* group_state = tile_state + G.ntiles;
@@ -1106,7 +1106,7 @@ encode_kernel(const __grid_constant__ EncodeParams P) {
             cum = __reduce_add_sync(0xffffffffu, cum);
             const uint32_t next_start = __shfl_down_sync(0xffffffffu, string_start, 1);
             if (lane < kQ) {                                // lane q: sub-block q of the warp
-                meta->sb_bits[warp * kQ + lane] = (lane < kQ - 1u ? next_start : bits) - string_start;
+                meta->sb_bits[warp * kQ + lane] = (lane + 1u < kQ ? next_start : bits) - string_start;
                 meta->sb_src[warp * kQ + lane] = string_start;
             }
             if (lane == 0) {
@@ -1264,7 +1264,7 @@ cudaError_t launch_level_histogram(const EncodeParams& P, uint64_t* hist, int sm
 // shared memory of one CTA: the tile buffers and, in the ERC mode, two staged tile images and two sets of per-warp token windows
 size_t encode_smem_bytes(const EncodeParams& P) {
     if (fixed4_applies(P.geo)) return 0;                    // that kernel's tile buffer is static
-    size_t words = kBLK;
+    size_t words = P.tile;
     if (P.geo.mode != kModeFixed) words += 2u * (size_t)P.stage_words + 2u * (size_t)P.warps * P.window_words;
     return 4u * words;
 }
@@ -1276,12 +1276,23 @@ static cudaError_t prepare_kernel() {
     static OncePerDevice prepared;
     return prepared([] {
         constexpr cudaFuncAttribute kSmem = cudaFuncAttributeMaxDynamicSharedMemorySize;
-        cudaError_t e = cudaFuncSetAttribute(encode_kernel<L, M, false, 8>, kSmem, kEncMaxDynSmem);
-        if (e == cudaSuccess) e = cudaFuncSetAttribute(encode_kernel<L, M, true, 8>, kSmem, kEncMaxDynSmem);
-        if (M == kModeErc && e == cudaSuccess) e = cudaFuncSetAttribute(encode_kernel<L, kModeErc, false, kEncMaxWarps>, kSmem, kEncMaxDynSmem);
-        if (M == kModeErc && e == cudaSuccess) e = cudaFuncSetAttribute(encode_kernel<L, kModeErc, true, kEncMaxWarps>, kSmem, kEncMaxDynSmem);
+        cudaError_t e = cudaFuncSetAttribute(encode_kernel<L, M, false, 8, kBLK>, kSmem, kEncMaxDynSmem);
+        if (e == cudaSuccess) e = cudaFuncSetAttribute(encode_kernel<L, M, true, 8, kBLK>, kSmem, kEncMaxDynSmem);
+        if (M == kModeErc && e == cudaSuccess) e = cudaFuncSetAttribute(encode_kernel<L, kModeErc, false, kEncMaxWarps, kBLK>, kSmem, kEncMaxDynSmem);
+        if (M == kModeErc && e == cudaSuccess) e = cudaFuncSetAttribute(encode_kernel<L, kModeErc, true, kEncMaxWarps, kBLK>, kSmem, kEncMaxDynSmem);
+        if (M == kModeErc && e == cudaSuccess) e = cudaFuncSetAttribute(encode_kernel<L, kModeErc, false, 8, kSmallTile>, kSmem, kEncMaxDynSmem);
         return e;
     });
+}
+
+using EncodeKernel = void (*)(EncodeParams);
+// the kernel of a call (clusters: the instance for buckets wider than a tile)
+template <uint32_t L, uint32_t M>
+static EncodeKernel kernel_of(const EncodeParams& P, bool clusters) {
+    if (M == kModeErc && P.tile == kSmallTile) return encode_kernel<L, kModeErc, false, 8, kSmallTile>;
+    if (M == kModeErc && P.warps == (uint32_t)kEncMaxWarps)
+        return clusters ? encode_kernel<L, kModeErc, true, kEncMaxWarps, kBLK> : encode_kernel<L, kModeErc, false, kEncMaxWarps, kBLK>;
+    return clusters ? encode_kernel<L, M, true, 8, kBLK> : encode_kernel<L, M, false, 8, kBLK>;
 }
 
 template <uint32_t M>
@@ -1292,9 +1303,7 @@ static int blocks_per_sm(const EncodeParams& P) {
     if (prepare_kernel<L, M>() != cudaSuccess) return 0;
     int n = 0;
     const size_t smem = encode_smem_bytes(P);
-    const cudaError_t e = M == kModeErc && P.warps == (uint32_t)kEncMaxWarps
-        ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, encode_kernel<L, kModeErc, false, kEncMaxWarps>, threads_of<M>(P), smem)
-        : cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, encode_kernel<L, M, false, 8>, threads_of<M>(P), smem);
+    const cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, kernel_of<L, M>(P, false), threads_of<M>(P), smem);
     return e == cudaSuccess ? n : 0;
 }
 
@@ -1345,11 +1354,7 @@ static cudaError_t launch_one(const EncodeParams& P, cudaStream_t stream) {
     if (smem > (size_t)kEncMaxDynSmem || P.grid == 0 || (P.cluster > 1u && P.grid % P.cluster != 0)) return cudaErrorInvalidValue;
     EncodeLaunch cfg;
     fill_launch<M>(&cfg, P, P.grid, stream);
-    if (M == kModeErc && P.warps == (uint32_t)kEncMaxWarps)
-        return P.cluster > 1u ? cudaLaunchKernelEx(&cfg.cfg, encode_kernel<L, kModeErc, true, kEncMaxWarps>, P)
-                              : cudaLaunchKernelEx(&cfg.cfg, encode_kernel<L, kModeErc, false, kEncMaxWarps>, P);
-    if (P.cluster > 1u) return cudaLaunchKernelEx(&cfg.cfg, encode_kernel<L, M, true, 8>, P);
-    return cudaLaunchKernelEx(&cfg.cfg, encode_kernel<L, M, false, 8>, P);
+    return cudaLaunchKernelEx(&cfg.cfg, kernel_of<L, M>(P, P.cluster > 1u), P);
 }
 
 // clusters of P.cluster CTAs the device holds at once (0 on error)
@@ -1359,9 +1364,7 @@ static int max_clusters(const EncodeParams& P) {
     EncodeLaunch cfg;
     fill_launch<M>(&cfg, P, P.cluster, nullptr);
     int n = 0;
-    const cudaError_t e = M == kModeErc && P.warps == (uint32_t)kEncMaxWarps
-        ? cudaOccupancyMaxActiveClusters(&n, encode_kernel<L, kModeErc, true, kEncMaxWarps>, &cfg.cfg)
-        : cudaOccupancyMaxActiveClusters(&n, encode_kernel<L, M, true, 8>, &cfg.cfg);
+    const cudaError_t e = cudaOccupancyMaxActiveClusters(&n, kernel_of<L, M>(P, true), &cfg.cfg);
     if (e != cudaSuccess) {
         cudaGetLastError();
         return 0;

@@ -137,6 +137,24 @@ def test_containers_at_the_encoders_edges(kind, d, bucket, s, ls):
         assert free_bits == want_bits and np.array_equal(free, want)
 
 
+@pytest.mark.parametrize("kind", ["normal", "mixed"])
+@pytest.mark.parametrize("tiles,bucket", [(1, 256), (1, 768), (1, 2048), (1, 2304), (3, 512), (3, 8192), (3, 16384)])
+def test_containers_where_small_tiles_and_more_warps_end(kind, tiles, bucket):
+    """One tile of 8192 elements (whole buckets of it) per SM is encoded in small tiles, three with more warps."""
+    torch, _ = require_cuda()
+    tile = 8192 if bucket > 8192 else 8192 // bucket * bucket
+    last = tiles * torch.cuda.get_device_properties(0).multi_processor_count * tile
+    for d in (last, last + 1):
+        g = _vector(kind, d, 3)
+        norms = O.bucket_norms(g, bucket, O.NORM_L2)
+        want, want_bits = O.encode(g, bucket, 4, 0, seed=5, offset=9, norms=norms)
+        got, got_bits = gpu_encode(g, bucket, 4, 0, seed=5, offset=9, norms=norms)
+        assert got_bits == want_bits and np.array_equal(got, want)
+        free, _ = gpu_encode(g, bucket, 4, 0, seed=5, offset=9)
+        _, _, _, taken = O.decode_symbols(free, d, bucket, 4)
+        assert np.array_equal(free, O.encode(g, bucket, 4, 0, seed=5, offset=9, norms=taken)[0])
+
+
 @pytest.mark.parametrize("mode", [O.MODE_ERC, O.MODE_FIXED])
 @pytest.mark.parametrize("ls,s,K", [(O.LEVELS_UNIFORM, 4, 3), (O.LEVELS_UNIFORM, 8, 3), (O.LEVELS_TABLE, 5, 3), (O.LEVELS_TABLE, 8, 2), (O.LEVELS_TABLE, 3, 40)])
 def test_products_are_rounded_before_they_are_added(ls, s, K, mode):
