@@ -509,6 +509,126 @@ __device__ __forceinline__ void fields_of_width(const DecodeParams& P, const Str
     }
 }
 
+template <class Sym>
+__device__ __forceinline__ void clear_rows(uint32_t rows) {
+    for (uint32_t i = 16u * lane_id(); i < 32u * Row<Sym>::kPitch; i += 512u)
+        asm volatile("st.shared.v4.u32 [%0], {%1, %1, %1, %1};" ::"r"(rows + i), "r"(0u) : "memory");
+}
+
+// The token table for ERC streams of one level set (kTabErc, kTabUniform), by all threads of the CTA.
+template <class Sym>
+__device__ __forceinline__ void build_erc_table(uint32_t* table, uint32_t kind, uint32_t s) {
+    using Symbols = Symbol<Sym>;
+    const uint4* src = reinterpret_cast<const uint4*>(g_token_tables[kPairs<Sym> ? kTabPairs : kTabErc]);
+    const uint32_t top = kind == kTabUniform ? 1u << s : s + 1u;
+    auto entry = [&](uint32_t e) {
+        const uint32_t index = (e >> kIndexShift) & 0x1ffu, negative = e >> 31;
+        if (index == 0u) return e;
+        if (index > top) return 0u;
+        return (e & 0xffffu) | (kind == kTabUniform ? Symbols::uniform(index, negative) : Symbols::exponential(index, negative, s));
+    };
+    // a ready-made pair with this call's symbols; 0 where there is no such index (long_token takes the first one then, if that exists)
+    auto ready = [&](uint32_t e) {
+        const uint32_t first = (e >> kFirstShift) & 31u, last = (e >> 24) & 31u;
+        if (first > top || last > top) return 0u;
+        if (last == 0u) return e;
+        if (kind == kTabErc) return e + ((e & 0x1f1f0000u) * 3u) + ((14u - s) << 26) + (first ? (14u - s) << (kFirstShift + 2u) : 0u);
+        const uint32_t f = e & 1u << 23 ? 0u - first : first, l = e >> 31 ? 0u - last : last;
+        return (e & 0xffffu) | (f & 0xffu) << kFirstShift | l << 24;
+    };
+    // (rolled up: where the call comes behind other work its code has to be fetched, which takes longer than the loads: K = 4
+    // ResNet-18 containers behind their encodes 38.9 us, 37.0 rolled up)
+#pragma unroll 1
+    for (uint32_t i = threadIdx.x; i < kTokEntries / 4u; i += blockDim.x) {
+        uint4 e = __ldg(src + i);
+        if (kPairs<Sym>) e = make_uint4(ready(e.x), ready(e.y), ready(e.z), ready(e.w));
+        else e = make_uint4(entry(e.x), entry(e.y), entry(e.z), entry(e.w));
+        reinterpret_cast<uint4*>(table)[i] = e;
+    }
+}
+
+// Whatever table the streams need and the kernel has not prepared, with their level codes and level tables; all threads of the CTA.
+// `words`: the level code of all streams (kTabCoded).  `several`: some warp has more than one unit.
+template <class Sym>
+__device__ __forceinline__ void prepare_tables(const DecodeParams& P, unsigned char* dsm, const uint32_t* words, uint32_t kind, uint32_t all_alike, bool several) {
+    using Symbols = Symbol<Sym>;
+    const Geometry& G = P.geo;
+    const uint32_t K = P.K, tid = threadIdx.x;
+    uint32_t* const table = reinterpret_cast<uint32_t*>(dsm);
+    const Layout<Sym> at(dsm, K);
+    unsigned char *const codes = at.codes, *const levels = at.levels;
+    uint32_t first = K;                                     // the first token stream (all have the same code in the coded mode)
+    for (uint32_t k = 0; k < K; ++k) {
+        const StreamHead& hd = at.heads[k];
+        if (!hd.ok || hd.mode == kModeFixed) continue;
+        uint16_t* const code = reinterpret_cast<uint16_t*>(codes + k * kCodeBytes);
+        if (kind == kTabGaps || (kind == kTabCoded && first == K)) {   // level index by the next 7 bits
+            for (uint32_t i = tid; i < (1u << kMaxCodedS); i += blockDim.x) {
+                uint32_t c = 0, at = 0, index = 0;
+                if (kind == kTabCoded) c = coded_entry([&](uint32_t j) { return words[j]; }, G.s, i);     // (all streams have this code)
+                else if (hd.mode == kModeCoded) c = coded_entry([&](uint32_t j) { return level_word(hd.hdr[hd.hwords - 2u], hd.hdr[hd.hwords - 1u], G.s, j); }, G.s, i);
+                else if (erc_in_window(i << (32u - kMaxCodedS) | 0x01ffffffu, &at, &index) && at <= kMaxCodedS && index < hd.nlev) c = index | (at << 8);
+                code[i] = (uint16_t)c;
+            }
+        }
+        if (hd.levelset == kLevelsTable && tid <= G.s)
+            reinterpret_cast<float*>(levels + k * kLevelBytes)[tid] = tid < G.s ? __uint_as_float(hd.hdr[kHeaderWords + tid]) : 1.0f;
+        if (first == K) first = k;
+    }
+    if (kind == kTabCoded) __syncthreads();
+    const uint16_t* const code = reinterpret_cast<const uint16_t*>(codes + (first == K ? 0u : first) * kCodeBytes);
+    // the entry of the gap's code at prefix i joined with the streams' level code
+    auto coded_token = [&](uint32_t e, uint32_t i) {
+        const uint32_t at = e & kLenMask, low = e & 0xffffu;
+        if (at == 0u) return 0u;
+        const uint32_t rest = i << (32u - kTokBits + at), c = code[(rest << 1) >> (32u - kMaxCodedS)];
+        const uint32_t len = at + 1u + (c >> 8);
+        if (c != 0u && len <= kTokBits) return len | (low & (0xffu << kGapShift)) | Symbols::exponential(c & 0xffu, rest >> 31, G.s);
+        return at > 1u ? (at - 1u) | ((low & (0xffu << kGapShift)) - (1u << kGapShift)) : 0u;
+    };
+    if (kPairs<Sym> && kind == kTabCoded && several) {
+        // A level code's table in pairs, by way of the table of single tokens (kept where the rows will be): a token and the one behind it, if
+        // that is a whole one and near enough.  (The bits behind the prefix are taken for zeros; they do not matter to a token that ends
+        // within it.)  The entry behind prefix i is that of i moved up by a token's length, for neighbouring i a power of two
+        // apart: entries are kept within 32 by the sum of their five-bit digits, which keeps them in different banks (2 us of 15
+        // otherwise).  All this takes a microsecond more than single tokens: not where no warp has a second unit (65 536 elements 11.2 us
+        // without, 12.6 with them; 8 x 10^6, K = 4: 27.3 and 26.0).
+        uint32_t* const singles = reinterpret_cast<uint32_t*>(dsm + chain_fixed_bytes(K));
+        auto place = [](uint32_t i) { return i ^ ((i >> 5 ^ i >> 10) & 31u); };
+#pragma unroll 4
+        for (uint32_t i = tid; i < kTokEntries; i += blockDim.x) singles[place(i)] = coded_token(__ldg(g_token_tables[kTabGaps] + i), i);
+        __syncthreads();
+#pragma unroll 4
+        for (uint32_t i = tid; i < kTokEntries; i += blockDim.x) {
+            const uint32_t e = singles[place(i)], then = singles[place((i << (e & kLenMask)) & (kTokEntries - 1u))];
+            const uint32_t len = (e & kLenMask) + (then & kLenMask), gap2 = (then >> kGapShift) & 0xffu;
+            const bool two = e >> 24 != 0u && then >> 24 != 0u && len <= kTokBits && gap2 <= kMaxGap2;
+            table[i] = two ? len | gap2 << kGap2Shift | ((e & 0xff00u) + (gap2 << kGapShift)) | (e >> 24) << kFirstShift | (then & 0xff000000u) : e;
+        }
+        __syncthreads();
+        clear_rows<Sym>(at.rows);
+    } else if (kind == kTabCoded || kind == kTabGaps) {
+        const uint4* const gaps = reinterpret_cast<const uint4*>(g_token_tables[kTabGaps]);
+#pragma unroll 1
+        for (uint32_t i = tid; i < kTokEntries / 4u; i += blockDim.x) {
+            uint4 e = __ldg(gaps + i);
+            if (kind == kTabCoded) e = make_uint4(coded_token(e.x, 4u * i), coded_token(e.y, 4u * i + 1u), coded_token(e.z, 4u * i + 2u), coded_token(e.w, 4u * i + 3u));
+            reinterpret_cast<uint4*>(table)[i] = e;
+        }
+    } else if (kind != P.likely_table) {
+        build_erc_table<Sym>(table, kind, G.s);
+    }
+    __syncthreads();
+    if (all_alike == 3u) {                                  // levels by symbol, sign included (the codes are no longer needed)
+        for (uint32_t i = tid; i < 64u * K; i += blockDim.x) {
+            const uint32_t k = i >> 6, index = (i & 31u) + G.s - 14u;
+            const float l = index >= 1u && index <= G.s + 1u ? reinterpret_cast<const float*>(levels + k * kLevelBytes)[index - 1u] : 0.0f;
+            reinterpret_cast<float*>(codes + k * kCodeBytes)[i & 63u] = i & 32u ? -l : l;
+        }
+        __syncthreads();
+    }
+}
+
 // Streams of any kind.  MANY: more than 32 of them, in groups (the sums of a unit are kept in registers from group to group:
 // an instance of its own, since these and the counters of groups cost the common one 2 % of its time in the walk).
 // CALLED: from the kernel for fixed-width streams, where those the call was made for are not; fields are then added one by one.
@@ -526,72 +646,6 @@ __device__ __forceinline__ void decode_streams(const DecodeParams& P) {
     const uint32_t norms = rows + 32u * Row<Sym>::kPitch;   // one per lane's chain
     const uint32_t copy = norms + 128u + lane * (4u * kChunkWords);   // this lane's words of its chain
 
-    auto clear_rows = [&] {
-        for (uint32_t i = 16u * lane; i < 32u * Row<Sym>::kPitch; i += 512u)
-            asm volatile("st.shared.v4.u32 [%0], {%1, %1, %1, %1};" ::"r"(rows + i), "r"(0u) : "memory");
-    };
-    using Symbols = Symbol<Sym>;
-    // the entry of a gap's code joined with the streams' level code
-    auto coded_token = [&](uint32_t e, uint32_t i, const uint16_t* code) {
-        const uint32_t at = e & kLenMask, low = e & 0xffffu;
-        if (at == 0u) return 0u;
-        const uint32_t rest = i << (32u - kTokBits + at), c = code[(rest << 1) >> (32u - kMaxCodedS)];
-        const uint32_t len = at + 1u + (c >> 8);
-        if (c != 0u && len <= kTokBits) return len | (low & (0xffu << kGapShift)) | Symbols::exponential(c & 0xffu, rest >> 31, G.s);
-        return at > 1u ? (at - 1u) | ((low & (0xffu << kGapShift)) - (1u << kGapShift)) : 0u;
-    };
-    // The token table for streams of kind `kind` (`code`: their level code, kTabCoded only), in pairs but for a level code's.
-    auto build_table = [&](uint32_t kind, const uint16_t* code) {
-        const bool erc = kind == kTabErc || kind == kTabUniform;
-        const uint4* src = reinterpret_cast<const uint4*>(g_token_tables[!erc ? kTabGaps : kPairs<Sym> ? kTabPairs : kTabErc]);
-        const uint32_t top = kind == kTabUniform ? 1u << G.s : G.s + 1u;
-        auto entry = [&](uint32_t e, uint32_t i) {
-            if (kind == kTabGaps) return e;
-            if (kind == kTabCoded) return coded_token(e, i, code);
-            const uint32_t index = (e >> kIndexShift) & 0x1ffu, negative = e >> 31;
-            if (index == 0u) return e;
-            if (index > top) return 0u;
-            return (e & 0xffffu) | (kind == kTabUniform ? Symbols::uniform(index, negative) : Symbols::exponential(index, negative, G.s));
-        };
-        // a ready-made pair with this call's symbols; 0 where there is no such index (long_token takes the first one then, if that exists)
-        auto ready = [&](uint32_t e) {
-            const uint32_t first = (e >> kFirstShift) & 31u, last = (e >> 24) & 31u;
-            if (first > top || last > top) return 0u;
-            if (last == 0u) return e;
-            if (kind == kTabErc) return e + ((e & 0x1f1f0000u) * 3u) + ((14u - G.s) << 26) + (first ? (14u - G.s) << (kFirstShift + 2u) : 0u);
-            const uint32_t f = e & 1u << 23 ? 0u - first : first, l = e >> 31 ? 0u - last : last;
-            return (e & 0xffffu) | (f & 0xffu) << kFirstShift | l << 24;
-        };
-#pragma unroll 4
-        for (uint32_t i = tid; i < kTokEntries / 4u; i += blockDim.x) {
-            uint4 e = __ldg(src + i);
-            if (kPairs<Sym> && erc) {
-                e = make_uint4(ready(e.x), ready(e.y), ready(e.z), ready(e.w));
-            } else {
-                e = make_uint4(entry(e.x, 4u * i), entry(e.y, 4u * i + 1u), entry(e.z, 4u * i + 2u), entry(e.w, 4u * i + 3u));
-            }
-            reinterpret_cast<uint4*>(table)[i] = e;
-        }
-    };
-    // ... and a level code's in pairs, by way of the table of single tokens at `singles`: a token and the one behind it, if that is a
-    // whole one and near enough.  (The bits behind the prefix are taken for zeros; they do not matter to a token that ends within it.)
-    // The entry behind prefix i is that of i moved up by a token's length, for neighbouring i a power of two apart: entries are
-    // kept within 32 by the sum of their five-bit digits, which keeps them in different banks (2 us of 15 otherwise).
-    auto build_pairs = [&](const uint16_t* code, uint32_t* singles) {
-        auto place = [](uint32_t i) { return i ^ ((i >> 5 ^ i >> 10) & 31u); };
-#pragma unroll 8
-        for (uint32_t i = tid; i < kTokEntries; i += blockDim.x) singles[place(i)] = coded_token(__ldg(g_token_tables[kTabGaps] + i), i, code);
-        __syncthreads();
-#pragma unroll 8
-        for (uint32_t i = tid; i < kTokEntries; i += blockDim.x) {
-            const uint32_t e = singles[place(i)], then = singles[place((i << (e & kLenMask)) & (kTokEntries - 1u))];
-            const uint32_t len = (e & kLenMask) + (then & kLenMask), gap2 = (then >> kGapShift) & 0xffu;
-            const bool two = e >> 24 != 0u && then >> 24 != 0u && len <= kTokBits && gap2 <= kMaxGap2;
-            table[i] = two ? len | gap2 << kGap2Shift | ((e & 0xff00u) + (gap2 << kGapShift)) | (e >> 24) << kFirstShift | (then & 0xff000000u) : e;
-        }
-        __syncthreads();
-    };
-
     // The kernel is launched with programmatic stream serialization: its CTAs take the SMs as the kernel in front leaves
     // them, build the table that the call is likely to need and clear their rows, and wait here until that kernel has ended.
     // Nothing before the wait touches memory that another kernel writes.  The kernel behind is let in early only by calls
@@ -599,8 +653,8 @@ __device__ __forceinline__ void decode_streams(const DecodeParams& P) {
     // left and is packed onto a few SMs, four CTAs each (a step of 10^6 elements, K = 3: 66 -> 74 us).
     if (!CALLED) {
         if (P.let_next) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-        if (P.likely_table == kTabErc || P.likely_table == kTabUniform) build_table(P.likely_table, nullptr);
-        clear_rows();
+        if (P.likely_table == kTabErc || P.likely_table == kTabUniform) build_erc_table<Sym>(table, P.likely_table, G.s);
+        clear_rows<Sym>(rows);
         asm volatile("griddepcontrol.wait;" ::: "memory");
     }
 
@@ -655,50 +709,12 @@ __device__ __forceinline__ void decode_streams(const DecodeParams& P) {
         fields_of_width<Sym, MANY>(P, heads, at.field_tables, rows, s_fields);
         return;
     }
-    if (CALLED) clear_rows();
+    if (CALLED) clear_rows<Sym>(rows);
     const uint32_t S = P.unit_subs;                         // sub-blocks of a unit
     const uint32_t nsub = (uint32_t)((G.d + kSB - 1u) / kSB), nunits = (uint32_t)(((uint64_t)nsub + S - 1u) / S), stride = gridDim.x * (blockDim.x >> 5);
-    // A level code's table is built when the headers have been read, and its pairs take a microsecond more: not where no warp has a
-    // second unit (65 536 elements 11.6 us without, 12.6 with them; 8 x 10^6, K = 4: 27.3 and 26.0).
     const uint32_t kind = s_kind, all_alike = s_alike == 3u && s_kind == kTabGaps ? 2u : s_alike;
-    if (kind != P.likely_table || kind == kTabGaps || kind == kTabCoded || all_alike >= 2u) {
-        uint32_t first = K;                                 // the first token stream (all have the same code in the coded mode)
-        for (uint32_t k = 0; k < K; ++k) {
-            const StreamHead& hd = heads[k];
-            if (!hd.ok || hd.mode == kModeFixed) continue;
-            uint16_t* const code = reinterpret_cast<uint16_t*>(codes + k * kCodeBytes);
-            if (kind == kTabGaps || (kind == kTabCoded && first == K)) {   // level index by the next 7 bits
-                for (uint32_t i = tid; i < (1u << kMaxCodedS); i += blockDim.x) {
-                    uint32_t c = 0, at = 0, index = 0;
-                    if (kind == kTabCoded) c = coded_entry([](uint32_t j) { return s_words[j]; }, G.s, i);     // (all streams have this code)
-                    else if (hd.mode == kModeCoded) c = coded_entry([&](uint32_t j) { return level_word(hd.hdr[hd.hwords - 2u], hd.hdr[hd.hwords - 1u], G.s, j); }, G.s, i);
-                    else if (erc_in_window(i << (32u - kMaxCodedS) | 0x01ffffffu, &at, &index) && at <= kMaxCodedS && index < hd.nlev) c = index | (at << 8);
-                    code[i] = (uint16_t)c;
-                }
-            }
-            if (hd.levelset == kLevelsTable && tid <= G.s)
-                reinterpret_cast<float*>(levels + k * kLevelBytes)[tid] =
-                    tid < G.s ? __uint_as_float(hd.hdr[kHeaderWords + tid]) : 1.0f;
-            if (first == K) first = k;
-        }
-        if (kind == kTabCoded) __syncthreads();
-        const uint16_t* const code = reinterpret_cast<const uint16_t*>(codes + (first == K ? 0u : first) * kCodeBytes);
-        if (kPairs<Sym> && kind == kTabCoded && nunits > stride) {         // the single tokens where the rows will be
-            build_pairs(code, reinterpret_cast<uint32_t*>(dsm + chain_fixed_bytes(K)));
-            clear_rows();
-        } else if (kind != P.likely_table || kind == kTabCoded) {
-            build_table(kind, code);
-        }
-        __syncthreads();
-        if (all_alike == 3u) {                              // levels by symbol, sign included (the codes are no longer needed)
-            for (uint32_t i = tid; i < 64u * K; i += blockDim.x) {
-                const uint32_t k = i >> 6, index = (i & 31u) + G.s - 14u;
-                const float l = index >= 1u && index <= G.s + 1u ? reinterpret_cast<const float*>(levels + k * kLevelBytes)[index - 1u] : 0.0f;
-                reinterpret_cast<float*>(codes + k * kCodeBytes)[i & 63u] = i & 32u ? -l : l;
-            }
-            __syncthreads();
-        }
-    }
+    if (kind != P.likely_table || kind == kTabGaps || kind == kTabCoded || all_alike >= 2u)
+        prepare_tables<Sym>(P, dsm, s_words, kind, all_alike, nunits > stride);
     // from here on warps run alone
 
     const uint32_t tab = smem_u32(table);
@@ -870,7 +886,7 @@ __device__ __forceinline__ void decode_streams(const DecodeParams& P) {
 #pragma unroll 1
         for (; q0 < S; ++q0) add_block<Sym, 1, MANY>(P, ap, q0, e0 + 256u * q0, carry);
         __syncwarp();
-        clear_rows();
+        clear_rows<Sym>(rows);
         __syncwarp();
         ch = after;
         next = next2;
