@@ -91,6 +91,14 @@ def test_sums_of_coded_streams_where_warps_have_several_units(kind, weights):
     _same_sums(streams * 16, d, bucket, s)
 
 
+@pytest.mark.parametrize("bucket,mode", [(256, O.MODE_ERC), (768, O.MODE_ERC), (1024, O.MODE_ERC), (1024, O.MODE_FIXED), (1280, O.MODE_ERC)])
+def test_sums_of_short_blocks_where_warps_have_more_than_two_units(bucket, mode):
+    """Buckets of up to 1024 elements have a kernel of their own there; fixed-width streams of unknown origin are a call in it."""
+    d, s = 4800 * 256 + 77, 4
+    streams = [_container(kind, d, bucket, s, O.NORM_L2, O.LEVELS_EXP, mode, 3) for kind in ("mixed", "normal")]
+    _same_sums(streams * 16, d, bucket, s)
+
+
 @pytest.mark.parametrize("ls,s,less", [(O.LEVELS_EXP, 6, 3), (O.LEVELS_EXP, 5, 4), (O.LEVELS_UNIFORM, 4, 2), (O.LEVELS_UNIFORM, 4, 3)])
 def test_symbols_beyond_the_last_level_are_refused(ls, s, less):
     """Containers whose header claims fewer levels than they use: many such symbols follow a good one within a table's prefix."""
