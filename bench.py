@@ -573,7 +573,7 @@ def run_gpu(args):
 # had left the 126 MB L2 when the kernel ended (a container or the sums of C3 fit in it), so the
 # totals of the decoders and of the fixed-width encoder lie below the algorithmic bytes.
 ENCODE_TRAFFIC_BYTES = {"c3": 102_311_680 + 3_371_264, "c3-fixed": 102_297_088 + 5_346_304}
-DECODE_TRAFFIC_BYTES = {"c3": 24_697_856 + 43_226_880, "c3-fixed": 102_395_648 + 49_322_496}
+DECODE_TRAFFIC_BYTES = {"c3": 24_697_600 + 44_290_560, "c3-fixed": 102_395_648 + 49_322_496}
 # the encode kernel that does the work of a call, where it is not the general one
 ENCODE_KERNEL = {"c3-fixed": "encode_fixed4_kernel"}
 

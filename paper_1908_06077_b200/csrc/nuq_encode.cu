@@ -5,8 +5,8 @@
 // A persistent CTA takes tiles of up to 8192 consecutive elements (whole buckets, or
 // one 8192-element coding block of a wider bucket) by ticket.  The tile's bytes are
 // brought into shared memory by bulk asynchronous copies (TMA, completion on an
-// mbarrier), one per warp: the worker warps (eight, or sixteen in small calls) own an equal
-// part of the tile's 256-element coding sub-blocks each, and a warp starts the copy of its
+// mbarrier), one per warp: the worker warps (eight, or sixteen in small calls; the smallest
+// calls take tiles of 2048 elements) own an equal part of the tile's 256-element coding sub-blocks each, and a warp starts the copy of its
 // part of the next tile as soon as it is done with its part of this one.  Per tile a worker
 //   1. adds up the squares of its elements per sub-block (eight per lane in fp32,
 //      everything beyond that in fp64); whichever warp is done last turns the partial
