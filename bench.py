@@ -97,42 +97,61 @@ def variance_bounds(bucket, s, flags):
 
 
 class ClockSampler:
-    """samples nvidia-smi clocks and throttle reasons while the timed region runs"""
+    """samples nvidia-smi clocks and throttle reasons while the timed region runs: start() ahead of the warm-up returns when
+    the first sample is there (nvidia-smi takes longer to start than the region lasts), mark() begins the region"""
     Q = ("clocks.sm,clocks.max.sm,clocks_event_reasons.hw_slowdown,clocks_event_reasons.hw_thermal_slowdown,"
          "clocks_event_reasons.sw_thermal_slowdown,clocks_event_reasons.sw_power_cap")
+    PERIOD_MS = 20
 
-    def __init__(self, index):
-        self.index, self.rows, self.proc = index, [], None
+    def __init__(self, index, patience=10.0):
+        self.index, self.patience, self.rows, self.first, self.proc, self.note = index, patience, [], 0, None, None
 
     def start(self):
         try:
             self.proc = subprocess.Popen(["nvidia-smi", "-i", str(self.index), f"--query-gpu={self.Q}",
-                                          "--format=csv,noheader,nounits", "-lms", "100"],
+                                          "--format=csv,noheader,nounits", "-lms", str(self.PERIOD_MS)],
                                          stdout=subprocess.PIPE, stderr=subprocess.DEVNULL, text=True)
-            threading.Thread(target=self._read, daemon=True).start()
-        except Exception:
-            self.proc = None
+        except OSError as e:
+            self.note = f"nvidia-smi unavailable: {e}"
+            return
+        threading.Thread(target=self._read, daemon=True).start()
+        self._wait_for_rows(1, self.patience)
+
+    def mark(self):
+        self.first = len(self.rows)
 
     def _read(self):
         for line in self.proc.stdout:
             self.rows.append([x.strip() for x in line.split(",")])
 
+    def _wait_for_rows(self, n, seconds):
+        end = time.monotonic() + seconds
+        while len(self.rows) < n and self.proc.poll() is None and time.monotonic() < end:
+            time.sleep(0.002)
+
     def stop(self):
+        """the samples since mark(), at least one (the first behind a region shorter than the period was taken at its end)"""
         if self.proc is None:
-            return {"sm_mhz": None, "sm_max_mhz": None, "reasons": ["nvidia-smi unavailable"]}
-        time.sleep(0.15)
+            return {"sm_mhz": None, "sm_max_mhz": None, "reasons": [], "note": self.note or "not started"}
+        self._wait_for_rows(self.first + 1, 1.0)
+        rows, exit_code = self.rows[self.first:], self.proc.poll()
         self.proc.terminate()
+        self.proc.wait()
         sm, mx, reasons = [], None, set()
         names = ["hw_slowdown", "hw_thermal_slowdown", "sw_thermal_slowdown", "sw_power_cap"]
-        for r in self.rows:
+        for r in rows:
             try:
                 sm.append(float(r[0])); mx = float(r[1])
-            except Exception:
+            except (ValueError, IndexError):
                 continue
             for n, v in zip(names, r[2:6]):
                 if v.lower().startswith("active"):
                     reasons.add(n)
-        return {"sm_mhz": statistics.median(sm) if sm else None, "sm_max_mhz": mx, "reasons": sorted(reasons)}
+        record = {"sm_mhz": statistics.median(sm) if sm else None, "sm_max_mhz": mx, "reasons": sorted(reasons), "samples": len(sm)}
+        if not sm:
+            record["note"] = (f"nvidia-smi ended with status {exit_code}" if exit_code is not None else
+                              f"nvidia-smi gave no sample in time ({len(self.rows)} before the timed region, {len(rows)} unreadable in it)")
+        return record
 
 
 def max_over_ranks(values, device):
@@ -454,7 +473,7 @@ def run_gpu(args):
         if world > 1:
             dist.barrier()
         torch.cuda.synchronize()
-        sampler.start()
+        sampler.mark()
 
     clocks = {}
 
@@ -463,6 +482,7 @@ def run_gpu(args):
             dist.barrier()
         clocks.update(sampler.stop())
 
+    sampler.start()
     enc_ms, dec_ms = w.timed(steps, warmup, flush, before, after)
     t_enc, t_dec = sum(enc_ms) / steps, sum(dec_ms) / steps                # ms per step: K encodes, one decode
     t_step = t_enc + t_dec
