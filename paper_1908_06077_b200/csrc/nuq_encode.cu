@@ -895,7 +895,8 @@ encode_kernel(const __grid_constant__ EncodeParams P) {
             if (__shfl_sync(0xffffffffu, last, 0)) {
                 __threadfence_block();
                 // lane = sub-block of the tile; the lanes of one bucket all do the same sum, in the same order
-                const uint32_t bi = lane / spb, sb0 = bi * spb;
+                const SubBlocks mine = bucket_of_lane<TILE / kSB>(lane, spb);
+                const uint32_t bi = lane / spb, sb0 = mine.from;
                 float norm;
                 if (P.norms_in != nullptr) {
                     const uint64_t nb_idx = narrow ? ti.first_block + bi : ti.bucket_idx;
@@ -930,13 +931,13 @@ encode_kernel(const __grid_constant__ EncodeParams P) {
                     }
                 } else if (G.norm_kind == kNormL2) {
                     double a = 0.0;
-                    if (coarse) for (uint32_t j = sb0 + kQ - 1u; j < sb0 + spb; j += kQ) a += s_partial[j];     // one partial per warp
-                    else for (uint32_t j = sb0; j < sb0 + spb; ++j) a += s_partial[j];
+                    if (coarse) for (uint32_t j = sb0 + kQ - 1u; j < mine.to; j += kQ) a += s_partial[j];     // one partial per warp
+                    else for (uint32_t j = sb0; j < mine.to; ++j) a += s_partial[j];
                     norm = (float)sqrt(a);
                 } else {
                     uint32_t mxb = 0;
-                    if (coarse) for (uint32_t j = sb0 + kQ - 1u; j < sb0 + spb; j += kQ) mxb = max(mxb, s_maxbits[j]);
-                    else for (uint32_t j = sb0; j < sb0 + spb; ++j) mxb = max(mxb, s_maxbits[j]);
+                    if (coarse) for (uint32_t j = sb0 + kQ - 1u; j < mine.to; j += kQ) mxb = max(mxb, s_maxbits[j]);
+                    else for (uint32_t j = sb0; j < mine.to; ++j) mxb = max(mxb, s_maxbits[j]);
                     norm = __uint_as_float(mxb);
                 }
                 if (norm != norm) norm = __uint_as_float(0x7fc00000u);     // one NaN pattern in the stream

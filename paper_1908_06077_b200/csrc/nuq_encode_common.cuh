@@ -126,6 +126,19 @@ __device__ __forceinline__ void cluster_sync_all() {
     asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
 
+// Where the norms are worked out a lane stands for a sub-block of the tile and adds up the sums of all sub-blocks of its bucket,
+// [from, to), spb of them.  A tile has sums for SUBS sub-blocks; its buckets need not fill them, and the lanes behind the last
+// bucket must not read on behind the sums.  (Those of sub-blocks that the tile does not have are 0.  A limit by the tile's number
+// of buckets, which is no constant, cost the 4-bit encoder 1 %: this is on the path that a tile's warps wait for.)
+struct SubBlocks {
+    uint32_t from, to;
+};
+template <uint32_t SUBS>
+__host__ __device__ __forceinline__ SubBlocks bucket_of_lane(uint32_t lane, uint32_t spb) {
+    const uint32_t from = lane / spb * spb, to = from + spb;
+    return SubBlocks{from, to < SUBS ? to : SUBS};
+}
+
 // Geometry of a tile, worked out once by the thread that took its ticket.
 struct TileInfo {
     unsigned long long tile;                               // >= ntiles: there is no such tile
