@@ -130,7 +130,8 @@ typedef struct nuq_info {
  * captured size, and a decode call, on the stream first; without them the captured
  * call returns NUQ_ERR_CUDA (and the capture may be invalid).  A graph holds the
  * workspace's address: it must not be replayed once a larger call on the stream
- * has made the workspace grow, or after nuq_shutdown.
+ * has made the workspace grow, or after nuq_shutdown.  ("Size" and "larger" are the
+ * number of elements d alone: its room goes by d, whatever bucket, s and mode are.)
  */
 nuq_status nuq_encode(const float* g, uint64_t d, uint32_t bucket, uint32_t s, uint32_t norm_kind, uint64_t seed,
                       uint64_t offset, void* out, uint64_t* out_bits, void* stream);

@@ -161,6 +161,18 @@ int device_sms(int dev) {
     return sms;
 }
 
+// Room for the scan state of `ntiles` tiles behind the control block: one look-back word per tile and per group of 32 tiles.
+size_t scan_state_bytes(uint64_t ntiles) { return sizeof(Workspace) + 8 * (ntiles + (ntiles + 31) / 32); }
+
+// The most tiles that an encode call of up to d elements has, whatever its buckets and its mode: tiles of more than kBLK / 2
+// elements (whole buckets, as many as fit), or of more than kSmallTile / 2 in calls of up to one tile of kBLK per SM.  A stream's
+// workspace is made for that number and not for the call's own, which small tiles and short buckets raise: a call with fewer
+// elements than an earlier one must not make the workspace grow (it may be captured, and a graph may hold the workspace's address).
+uint64_t most_tiles(uint64_t d, int sms) {
+    const uint64_t whole = d / (kBLK / 2) + 2, few = (uint64_t)sms * kBLK, small = (d < few ? d : few) / (kSmallTile / 2) + 2;
+    return whole > small ? whole : small;
+}
+
 // Workspace of (current device, stream), grown to `bytes`.  Growing synchronises the stream.
 nuq_status get_workspace(cudaStream_t stream, size_t bytes, Workspace** out, int* dev_out) {
     int dev = 0;
@@ -271,7 +283,7 @@ static EncodePlan plan_encode(EncodeParams& P, int dev, uint32_t flags) {
         G.ntiles = (G.nb + G.blocks_per_tile - 1) / G.blocks_per_tile;
     }
     // (the tiles' number is what it will be from here on)
-    pl.state_bytes = sizeof(Workspace) + 8 * (G.ntiles + (G.ntiles + 31) / 32);
+    pl.state_bytes = scan_state_bytes(G.ntiles);
     if (G.mode != kModeFixed) {
         P.stage_words = (stage_words_for(G, norms_are_ours) + 3u) & ~3u;
         // a warp's elements lie in at most this many buckets
@@ -543,7 +555,7 @@ nuq_status nuq_encode(const float* g, uint64_t d, uint32_t bucket, uint32_t s, u
     P.grid = pl.want_grid;
     Workspace* ws = nullptr;
     WsEntry& e = g_ws[std::make_pair(dev, stream)];
-    nuq_status st = get_workspace(stream, pl.state_bytes, &ws, &dev);
+    nuq_status st = get_workspace(stream, scan_state_bytes(most_tiles(d, device_sms(dev))), &ws, &dev);
     if (st == NUQ_OK && pl.norms_bytes && !(norm_kind & NUQ_TEST_NORMS)) st = get_norms(stream, pl.norms_bytes, e);
     if (st != NUQ_OK) return st;
     return enqueue_encode(P, pl, g, norm_kind, seed, offset, out, out_bits, ws, e.norms, &e, dev, stream);

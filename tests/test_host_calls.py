@@ -109,3 +109,19 @@ def test_every_device_is_told_how_much_shared_memory_the_kernels_take(lib, kind,
         for d in (100000, 10000000):
             assert _encode(lib, d=d, bucket=bucket, s=5, kind=kind) == 0 and _decode(lib, d=d, bucket=bucket, s=5) == 0
             assert _decode(lib, d=d, bucket=bucket, s=7) == 0                           # (16-bit symbols)
+
+
+@pytest.mark.parametrize("kinds", [(ERC,), (FIXED,), (2 << 16,), (ERC, FIXED, 2 << 16)])
+@pytest.mark.parametrize("d", [1212417, 2000000, 5000000, 10000000])
+def test_a_call_with_fewer_elements_than_the_one_before_never_allocates(lib, d, kinds):
+    """whatever its buckets, mode and tiles are: it may be captured, and a graph may hold the workspace's address"""
+    assert lib.nuq_set_level_code((C.c_uint8 * 5)(1, 2, 3, 4, 4), 4) == 0
+    assert _encode(lib, d=d, bucket=8192) == 0
+    lib.fake_capture(1)
+    for kind in kinds:
+        for bucket in (256, 768, 1024, 1280, 2048, 4352, 8192, 16384):
+            if kind == FIXED and bucket > 8192:
+                continue                                    # (norms of their own)
+            for n in (65536, 148 * 2048, 4 * 148 * 1024, 1200000, 148 * 8192, d):
+                assert n > d or _encode(lib, d=n, bucket=bucket, s=4, kind=kind) == 0, (n, bucket)
+    assert "refused" not in lib.fake_events().decode()
