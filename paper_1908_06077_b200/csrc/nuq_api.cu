@@ -205,8 +205,11 @@ nuq_status get_workspace(cudaStream_t stream, size_t bytes, Workspace** out, int
     return NUQ_OK;
 }
 
-// Room for `bytes` of bucket norms behind the workspace of (current device, stream).  Growing synchronises the stream.
-nuq_status get_norms(cudaStream_t stream, size_t bytes, WsEntry& e) {
+// Room for the bucket norms of a call of d elements in the stream's current device, for the shortest buckets there are: like the
+// workspace it goes by d alone (a pass over wide buckets that is captured, a histogram over short ones behind it).  Growing
+// synchronises the stream.
+nuq_status get_norms(cudaStream_t stream, uint64_t d, WsEntry& e) {
+    const size_t bytes = 4 * ((d + kSB - 1) / kSB);
     if (e.norms_bytes >= bytes) return NUQ_OK;
     if (e.norms) {
         if (cudaStreamSynchronize(stream) != cudaSuccess) return NUQ_ERR_CUDA;
@@ -511,7 +514,7 @@ nuq_status nuq_level_histogram(const float* g, uint64_t d, uint32_t bucket, uint
         Workspace* ws = nullptr;
         WsEntry& e = g_ws[std::make_pair(dev, stream)];
         nuq_status st = get_workspace(stream, sizeof(Workspace), &ws, &dev);
-        if (st == NUQ_OK) st = get_norms(stream, 4 * G.nb, e);
+        if (st == NUQ_OK) st = get_norms(stream, d, e);
         if (st != NUQ_OK) return st;
         if (launch_bucket_norms(g, G.d, G.bucket, G.norm_kind, e.norms, G.nb, stream) != cudaSuccess) return NUQ_ERR_CUDA;
         P.norms_in = e.norms;
@@ -556,7 +559,7 @@ nuq_status nuq_encode(const float* g, uint64_t d, uint32_t bucket, uint32_t s, u
     Workspace* ws = nullptr;
     WsEntry& e = g_ws[std::make_pair(dev, stream)];
     nuq_status st = get_workspace(stream, scan_state_bytes(most_tiles(d, device_sms(dev))), &ws, &dev);
-    if (st == NUQ_OK && pl.norms_bytes && !(norm_kind & NUQ_TEST_NORMS)) st = get_norms(stream, pl.norms_bytes, e);
+    if (st == NUQ_OK && pl.norms_bytes && !(norm_kind & NUQ_TEST_NORMS)) st = get_norms(stream, d, e);
     if (st != NUQ_OK) return st;
     return enqueue_encode(P, pl, g, norm_kind, seed, offset, out, out_bits, ws, e.norms, &e, dev, stream);
 }

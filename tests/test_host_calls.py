@@ -125,3 +125,14 @@ def test_a_call_with_fewer_elements_than_the_one_before_never_allocates(lib, d, 
             for n in (65536, 148 * 2048, 4 * 148 * 1024, 1200000, 148 * 8192, d):
                 assert n > d or _encode(lib, d=n, bucket=bucket, s=4, kind=kind) == 0, (n, bucket)
     assert "refused" not in lib.fake_events().decode()
+
+
+def test_a_pass_for_norms_over_fewer_elements_than_the_one_before_never_allocates(lib):
+    hist = (C.c_uint64 * 8)()
+    assert _encode(lib, d=2000000, bucket=65536, kind=FIXED) == 0
+    lib.fake_capture(1)
+    for bucket in (65536, 32768, 16384):
+        assert _encode(lib, d=2000000, bucket=bucket, kind=FIXED) == 0
+    for bucket in (256, 1024, 8192, 65536):
+        assert lib.nuq_level_histogram(0x1000, 2000000, bucket, 4, 0, 1, 0, C.addressof(hist), STREAM) == 0
+    assert "refused" not in lib.fake_events().decode()
