@@ -270,20 +270,24 @@ static EncodePlan plan_encode(EncodeParams& P, int dev, uint32_t flags) {
     P.window_words = 0;
     P.stage_words = 0;
     // Small calls: a tile's latency counts there, not the SM's throughput.  (The fixed-width encoders have no such variants.)
-    // Up to one tile per SM, with buckets of which a small tile holds one at least: a quarter of a tile, one sub-block per
-    // warp.  65 536 elements 10.5 us in whole tiles of 16 warps, 9.0 in small ones (uniform levels 13.1 and 9.3), 10^6 elements
-    // with coded indices 15.5 and 13.6; 2 x 10^6 15.8 and 18.2.
     // Up to three tiles per SM: twice the warps per tile.  10^6 elements 16.4 -> 12.7 us, 3 x 10^6 18.7 -> 16.8 (uniform levels
     // 24.5 -> 21.3), 4 x 10^6 19.5 and 19.8.  With clusters 10^6 elements 20.9 -> 17.7, a single cluster 13 to 15 us with either.
     const bool tokens = G.mode != kModeFixed;
     P.warps = tokens && G.ntiles <= 3u * (uint64_t)sms ? kEncMaxWarps : kEncWarps;
     P.tile = kBLK;
-    if (tokens && G.bucket <= kSmallTile && G.ntiles <= (uint64_t)sms) {
+    // A quarter of a tile, one sub-block per warp, four to an SM: with fewer whole tiles than SMs, as long as small ones (of whole
+    // buckets too, so that there may be six for a whole one) are no more than 5.5 to an SM.  65 536 elements 10.9 us in whole tiles of 16 warps, 8.8 in
+    // small ones (uniform levels 12.0 and 8.7), 10^6 elements 15.2 and 13.3, coded indices 15.4 and 12.5; 147 whole tiles, buckets of
+    // 512 / 768 / 1536 (3.96, 4.95 and 4.95 small ones to an SM) 15.4 and 13.6, 15.2 and 14.7, 15.4 and 14.9; buckets of 1280 with 5.4
+    // to an SM 15.9 and 15.1, 5.6 15.9 and 16.2.  Whole tiles for all 148 SMs 12.5 and 13.9 (no SM gets two, then).
+    const uint32_t small_blocks = G.bucket <= kSmallTile ? kSmallTile / G.bucket : 1u;
+    const uint64_t small_tiles = (G.nb + small_blocks - 1) / small_blocks;
+    if (tokens && G.bucket <= kSmallTile && G.ntiles < (uint64_t)sms && 2u * small_tiles <= 11u * (uint64_t)sms) {
         P.tile = kSmallTile;
         P.warps = kEncWarps;
-        G.blocks_per_tile = kSmallTile / G.bucket;
-        G.tile_elems = G.blocks_per_tile * G.bucket;
-        G.ntiles = (G.nb + G.blocks_per_tile - 1) / G.blocks_per_tile;
+        G.blocks_per_tile = small_blocks;
+        G.tile_elems = small_blocks * G.bucket;
+        G.ntiles = small_tiles;
     }
     // (the tiles' number is what it will be from here on)
     pl.state_bytes = scan_state_bytes(G.ntiles);

@@ -2,6 +2,7 @@
 that runs nothing (fake_cudart.cpp).  No GPU is needed."""
 import ctypes as C
 import os
+import re
 import shutil
 import subprocess
 
@@ -136,3 +137,22 @@ def test_a_pass_for_norms_over_fewer_elements_than_the_one_before_never_allocate
     for bucket in (256, 1024, 8192, 65536):
         assert lib.nuq_level_histogram(0x1000, 2000000, bucket, 4, 0, 1, 0, C.addressof(hist), STREAM) == 0
     assert "refused" not in lib.fake_events().decode()
+
+
+def _tile_and_warps(lib, d, bucket, s=4, kind=ERC):
+    """elements of a tile and worker warps of the encode kernel that a call launches"""
+    lib.fake_reset()
+    assert _encode(lib, d=d, bucket=bucket, s=s, kind=kind) == 0
+    (name,) = re.findall(r"encode_kernelILj\d+ELj\d+ELb\dELj(\d+)ELj(\d+)E", lib.fake_events().decode())
+    return int(name[1]), int(name[0])
+
+
+SMS = 148                                                   # (of the stand-in)
+
+
+@pytest.mark.parametrize("bucket,last", [(256, (SMS - 1) * 8192), (768, (SMS - 1) * 7680), (1280, 11 * SMS // 2 * 1280), (1536, (SMS - 1) * 7680), (2048, (SMS - 1) * 8192)])
+def test_small_tiles_end_where_sms_would_get_six_or_each_has_a_whole_one(lib, bucket, last):
+    assert _tile_and_warps(lib, 256, bucket) == (2048, 8)
+    assert _tile_and_warps(lib, last, bucket) == (2048, 8)
+    assert _tile_and_warps(lib, last + 1, bucket) == (8192, 16)
+    assert _tile_and_warps(lib, SMS * (8192 // bucket * bucket), bucket) == (8192, 16)
