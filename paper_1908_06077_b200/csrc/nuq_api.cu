@@ -270,10 +270,16 @@ static EncodePlan plan_encode(EncodeParams& P, int dev, uint32_t flags) {
     P.window_words = 0;
     P.stage_words = 0;
     // Small calls: a tile's latency counts there, not the SM's throughput.  (The fixed-width encoders have no such variants.)
-    // Up to three tiles per SM: twice the warps per tile.  10^6 elements 16.4 -> 12.7 us, 3 x 10^6 18.7 -> 16.8 (uniform levels
-    // 24.5 -> 21.3), 4 x 10^6 19.5 and 19.8.  With clusters 10^6 elements 20.9 -> 17.7, a single cluster 13 to 15 us with either.
+    // Twice the warps per tile, two such CTAs to an SM: up to 17/7 tiles per SM as a rule.  2.0 to 2.4 tiles of 8192 (2.4 to 2.9 x 10^6 elements)
+    // take 18 to 20 us instead of 20 to 23; from 2.45 on some SM gets four tiles, and 20 us become 23 to 24 (s = 4 in buckets of 512:
+    // 2.35 tiles 20.3 and 19.1, 2.43 20.3 and 19.5, 2.52 20.4 and 23.9; level tables 25.5 and 25.0, 25.6 and 25.1, 25.7 and 30.0).  Uniform
+    // levels with many symbols (2.5 tiles 24.9 and 22.8, 2.95 25.9 and 24.9) and buckets in clusters of four and eight gain up to three tiles per
+    // SM (buckets of 65536, 2.2 tiles 26.5 and 23.8, 2.9 27.8 and 25.6, level tables 37.9 and 34.6, 43.8 and 37.3; largest-magnitude norms and
+    // uniform levels between 10 % less and 5 % more); clusters of two up to two tiles (2.3 tiles 24.0 and 23.8, but uniform levels with s = 2
+    // 24.5 and 27.2, largest-magnitude norms 25.6 and 27.9).
     const bool tokens = G.mode != kModeFixed;
-    P.warps = tokens && G.ntiles <= 3u * (uint64_t)sms ? kEncMaxWarps : kEncWarps;
+    const uint64_t sevenths = G.bucket == 2u * kBLK ? 14u : G.bucket > kBLK || (G.levelset == kLevelsUniform && G.s >= 4u) ? 21u : 17u;
+    P.warps = tokens && 7u * G.ntiles <= sevenths * (uint64_t)sms ? kEncMaxWarps : kEncWarps;
     P.tile = kBLK;
     // A quarter of a tile, one sub-block per warp, four to an SM: with fewer whole tiles than SMs, as long as small ones (of whole
     // buckets too, so that there may be six for a whole one) are no more than 5.5 to an SM.  65 536 elements 10.9 us in whole tiles of 16 warps, 8.8 in

@@ -156,3 +156,11 @@ def test_small_tiles_end_where_sms_would_get_six_or_each_has_a_whole_one(lib, bu
     assert _tile_and_warps(lib, last, bucket) == (2048, 8)
     assert _tile_and_warps(lib, last + 1, bucket) == (8192, 16)
     assert _tile_and_warps(lib, SMS * (8192 // bucket * bucket), bucket) == (8192, 16)
+
+
+@pytest.mark.parametrize("bucket,s,kind,sevenths", [(512, 4, ERC, 17), (8192, 4, ERC, 17), (8192, 2, 1 << 8, 17), (8192, 4, 1 << 8 | 1, 21), (512, 6, 1 << 8, 21),
+                                                    (16384, 4, ERC, 14), (32768, 4, ERC, 21), (65536, 4, 1 << 8 | 1, 21)])
+def test_sixteen_warps_end_where_an_sm_would_get_four_tiles(lib, bucket, s, kind, sevenths):
+    last = sevenths * SMS // 7 * 8192
+    assert _tile_and_warps(lib, last, bucket, s, kind) == (8192, 16)
+    assert _tile_and_warps(lib, last + 1, bucket, s, kind) == (8192, 8)
