@@ -371,7 +371,9 @@ static nuq_status enqueue_encode(EncodeParams& P, const EncodePlan& pl, const fl
     P.overlap = entry && G.ntiles <= 32ull * P.grid ? 1u : 0u;
     // The kernel behind is let in early, except by a 4-bit fixed-width call that leaves SMs with room for more of its CTAs:
     // the next such call's CTAs would be packed there, four to an SM, instead of spread (10^6 elements 13.0 -> 8.05 us,
-    // 3 x 10^6 13.4 -> 11.3 us).  The token encoders' small calls have two CTAs to an SM at most and gain from it.
+    // 3 x 10^6 13.4 -> 11.3 us).  The token encoders' small calls gain from it although those in small tiles are four to an SM too
+    // (without / with: 65 536 elements 10.2 / 8.8 us, 6 x 10^5 13.2 / 11.0, 9 x 10^5 14.8 / 12.9, from 10^6 on the same; steps of four
+    // workers with 65 536 and 6 x 10^5 elements 49.5 / 44.3 and 65.1 / 56.2).
     P.let_next = P.overlap && !(fixed4_applies(G) && P.grid <= 3u * (uint32_t)device_sms(dev)) ? 1u : 0u;
     P.seed = seed;
     P.offset = offset;
