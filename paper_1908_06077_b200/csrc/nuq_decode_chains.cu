@@ -858,7 +858,7 @@ __device__ __forceinline__ void decode_streams(const DecodeParams& P) {
                 const uint32_t room = 32u * kChunkWords - ch.bit;
                 const uint32_t bits = fits(ch) ? left : room - 96u;
                 // (a pair of tokens must not reach into the chain behind: it may pass the point by 12 bits)
-                if (ch.bit + ch.len <= 32u * (kChunkWords - 2u)) put_ones();
+                if (kPairs<Sym> && ch.bit + ch.len <= 32u * (kChunkWords - 2u)) put_ones();
                 uint32_t took;
                 if (kind == kTabGaps) took = walk_rare<Sym, true, true>(copy, ch.bit, bits, tab, row, row_end, my_head, my_code, G.s, good);
                 else took = walk_rare<Sym, true, false>(copy, ch.bit, bits, tab, row, row_end, my_head, my_code, G.s, good);
