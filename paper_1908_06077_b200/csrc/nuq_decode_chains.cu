@@ -488,24 +488,38 @@ struct Layout {
     }
 };
 
+// An instance of the kernel for token streams.  Whatever makes instances differ is named here, and only here: the functions for
+// fixed-width streams take the whole type as a template argument, so that no two kernels share one (decode_fields_call says why).
+// MANY: more than 32 streams, in groups (the sums of a unit are kept in registers from group to group: an instance of its own,
+// since these and the counters of groups cost the common one 2 % of its time in the walk).
+// SHORT: blocks are of at most four sub-blocks, so that a unit's lengths are in a line of their own as a rule, which no unit before
+// it has read; they are asked for a walk ahead (25 557 032 elements, buckets of 512: K = 8 123.6 -> 119.3 us, with the step 156 -> 148,
+// K = 2 at 2^28 381 -> 362; buckets of 2048 and more gain nothing and lose up to 1 %: an instance of its own).
+template <class SYMBOL, bool MANY_STREAMS, bool SHORT_BLOCKS>
+struct Instance {
+    using Sym = SYMBOL;
+    static constexpr bool kMany = MANY_STREAMS, kShort = SHORT_BLOCKS;
+};
+
 // All streams in the fixed-width mode.  (16-bit symbols: s = 7 or 8, hence fields of 5 bits, or of 9 and 10 with uniform levels.)
-template <class Sym, bool MANY, bool SHORT>
+template <class I>
 __device__ __forceinline__ void fields_of_width(const DecodeParams& P, const StreamHead* heads, unsigned char* tables, uint32_t mine, uint32_t width) {
+    constexpr bool kBytes = sizeof(typename I::Sym) == 1;
     if (heads[0].levelset == kLevelsExp) {
-        if (width == 5u) return decode_fields_call<5, true, Row<Sym>, std::integral_constant<uint32_t, 2u * MANY + SHORT>>(P, heads, tables, mine);
-        if (sizeof(Sym) == 1 && width == 4u) return decode_fields_call<4, true, Row<Sym>, std::integral_constant<uint32_t, 2u * MANY + SHORT>>(P, heads, tables, mine);
-        if (sizeof(Sym) == 1 && width == 3u) return decode_fields_call<3, true, Row<Sym>, std::integral_constant<uint32_t, 2u * MANY + SHORT>>(P, heads, tables, mine);
+        if (width == 5u) return decode_fields_call<5, true, I>(P, heads, tables, mine);
+        if (kBytes && width == 4u) return decode_fields_call<4, true, I>(P, heads, tables, mine);
+        if (kBytes && width == 3u) return decode_fields_call<3, true, I>(P, heads, tables, mine);
     }
-    if (width == 5u) return decode_fields_call<5, false, Row<Sym>, std::integral_constant<uint32_t, 2u * MANY + SHORT>>(P, heads, tables, mine);
-    if (sizeof(Sym) == 1) {
-        if (width == 3u) return decode_fields_call<3, false, Row<Sym>, std::integral_constant<uint32_t, 2u * MANY + SHORT>>(P, heads, tables, mine);
-        if (width == 4u) return decode_fields_call<4, false, Row<Sym>, std::integral_constant<uint32_t, 2u * MANY + SHORT>>(P, heads, tables, mine);
-        if (width == 6u) return decode_fields_call<6, false, Row<Sym>, std::integral_constant<uint32_t, 2u * MANY + SHORT>>(P, heads, tables, mine);
-        if (width == 7u) return decode_fields_call<7, false, Row<Sym>, std::integral_constant<uint32_t, 2u * MANY + SHORT>>(P, heads, tables, mine);
-        if (width == 8u) return decode_fields_call<8, false, Row<Sym>, std::integral_constant<uint32_t, 2u * MANY + SHORT>>(P, heads, tables, mine);
+    if (width == 5u) return decode_fields_call<5, false, I>(P, heads, tables, mine);
+    if (kBytes) {
+        if (width == 3u) return decode_fields_call<3, false, I>(P, heads, tables, mine);
+        if (width == 4u) return decode_fields_call<4, false, I>(P, heads, tables, mine);
+        if (width == 6u) return decode_fields_call<6, false, I>(P, heads, tables, mine);
+        if (width == 7u) return decode_fields_call<7, false, I>(P, heads, tables, mine);
+        if (width == 8u) return decode_fields_call<8, false, I>(P, heads, tables, mine);
     } else {
-        if (width == 9u) return decode_fields_call<9, false, Row<Sym>, std::integral_constant<uint32_t, 2u * MANY + SHORT>>(P, heads, tables, mine);
-        if (width == 10u) return decode_fields_call<10, false, Row<Sym>, std::integral_constant<uint32_t, 2u * MANY + SHORT>>(P, heads, tables, mine);
+        if (width == 9u) return decode_fields_call<9, false, I>(P, heads, tables, mine);
+        if (width == 10u) return decode_fields_call<10, false, I>(P, heads, tables, mine);
     }
 }
 
@@ -629,14 +643,12 @@ __device__ __forceinline__ void prepare_tables(const DecodeParams& P, unsigned c
     }
 }
 
-// Streams of any kind.  MANY: more than 32 of them, in groups (the sums of a unit are kept in registers from group to group:
-// an instance of its own, since these and the counters of groups cost the common one 2 % of its time in the walk).
-// CALLED: from the kernel for fixed-width streams, where those the call was made for are not; fields are then added one by one.
-// SHORT: blocks are of at most four sub-blocks, so that a unit's lengths are in a line of their own as a rule, which no unit before
-// it has read; they are asked for a walk ahead (25 557 032 elements, buckets of 512: K = 8 123.6 -> 119.3 us, with the step 156 -> 148,
-// K = 2 at 2^28 381 -> 362; buckets of 2048 and more gain nothing and lose up to 1 %: an instance of its own).
-template <class Sym, bool MANY, bool SHORT, bool CALLED>
+// Streams of any kind.
+// CALLED: from a kernel for fixed-width streams, where those the call was made for are not; fields are then added one by one.
+template <class I, bool CALLED>
 __device__ __forceinline__ void decode_streams(const DecodeParams& P) {
+    using Sym = typename I::Sym;
+    constexpr bool MANY = I::kMany, SHORT = I::kShort;
     extern __shared__ __align__(128) unsigned char dsm[];
     __shared__ uint32_t s_kind, s_alike, s_fields, s_words[kMaxCodedS + 1];
     const Geometry& G = P.geo;
@@ -709,7 +721,7 @@ __device__ __forceinline__ void decode_streams(const DecodeParams& P) {
     }
     __syncthreads();
     if (!CALLED && s_fields != 0u) {                        // no tokens at all
-        fields_of_width<Sym, MANY, SHORT>(P, heads, at.field_tables, rows, s_fields);
+        fields_of_width<I>(P, heads, at.field_tables, rows, s_fields);
         return;
     }
     if (CALLED) clear_rows<Sym>(rows);
@@ -907,14 +919,16 @@ __device__ __forceinline__ void decode_streams(const DecodeParams& P) {
     }
 }
 
-template <class Sym, bool MANY, bool SHORT>
+template <class I>
 __global__ void __launch_bounds__(32 * kChainMaxWarps, 1) decode_chains_kernel(const __grid_constant__ DecodeParams P) {
-    decode_streams<Sym, MANY, SHORT, false>(P);
+    decode_streams<I, false>(P);
 }
 
+// (One function for all the kernels for fixed-width streams.  Its stores are of 16 bytes, not the wide ones that went wrong in a
+// shared function; each kernel's way through it is tested.)
 template <class Sym>
 __device__ __noinline__ void decode_streams_call(const DecodeParams& P) {
-    decode_streams<Sym, true, false, true>(P);
+    decode_streams<Instance<Sym, true, false>, true>(P);
 }
 
 // Calls whose streams are likely all in the fixed-width mode, with fields of W bits of one level set: a kernel of its own for
@@ -978,9 +992,9 @@ static cudaError_t launch_chains(const DecodeParams& P, int sms, cudaStream_t st
     if (share < Q.unit_subs) Q.unit_subs = (uint32_t)share;
     const uint64_t units = (nsub + Q.unit_subs - 1u) / Q.unit_subs;
     Q.let_next = units > 2u * (uint64_t)sms * warps ? 1u : 0u;
-    DecodeKernel kernel = P.K > 32u ? decode_chains_kernel<Sym, true, false> : decode_chains_kernel<Sym, false, false>;
+    DecodeKernel kernel = P.K > 32u ? decode_chains_kernel<Instance<Sym, true, false>> : decode_chains_kernel<Instance<Sym, false, false>>;
     if constexpr (sizeof(Sym) == 1) {
-        if (P.K <= 32u && P.geo.bucket <= 4u * kSB && Q.let_next) kernel = decode_chains_kernel<Sym, false, true>;
+        if (P.K <= 32u && P.geo.bucket <= 4u * kSB && Q.let_next) kernel = decode_chains_kernel<Instance<Sym, false, true>>;
     }
     if (P.likely_table == kTabFields) kernel = fields_kernel(P.geo.s, P.likely_levels);
     static std::map<DecodeKernel, OncePerDevice> prepared;

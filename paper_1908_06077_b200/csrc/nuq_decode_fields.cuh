@@ -370,9 +370,10 @@ __device__ __forceinline__ void decode_fields(const DecodeParams& P, const Strea
 }
 
 // The same as a function, for the kernels of token streams: inlined there, fields and tokens share registers and the
-// instruction cache.  (Kernel: a function for each of them.  In one that several kernels called, built by nvcc 12.9,
-// the wide store wrote its first element only, in all kernels but one.)
-template <uint32_t W, bool EXACT, class... Kernel>
+// instruction cache.  Kernel: a type of the calling kernel's own, so that each has a function for itself.  (In one that several
+// kernels called, built by nvcc 12.9, store8 wrote its first element only, in all kernels but one.  The source has no reason for
+// that: the same text is right where it is inlined and where one kernel calls it.)
+template <uint32_t W, bool EXACT, class Kernel>
 __device__ __noinline__ void decode_fields_call(const DecodeParams& P, const StreamHead* heads, unsigned char* table_memory, uint32_t mine) {
     decode_fields<W, EXACT>(P, heads, table_memory, false, mine);
 }

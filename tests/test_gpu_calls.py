@@ -209,3 +209,37 @@ def test_fields_of_every_width_where_they_were_encoded_and_elsewhere(ls, s, buck
         y = (1.0 - step * want.double()).float()             # one fused operation: one rounding
         assert nuq.last_status() == 0 and torch.equal(yl, y)
         assert torch.equal(w, ((y - 1.0).double() * 0.5 + y.double()).float())
+
+
+@pytest.mark.parametrize("ls,s", [(O.LEVELS_EXP, s) for s in (1, 2, 3, 6, 7, 8, 14)] + [(O.LEVELS_TABLE, s) for s in (2, 5, 8, 14)] +
+                         [(O.LEVELS_UNIFORM, s) for s in range(1, 9)])
+def test_token_streams_where_fields_of_every_width_were_encoded(ls, s):
+    """Each of the kernels for fixed-width streams hands streams of another kind on to the same function: sums and the fused step
+    come out right from all of them (short blocks and long ones, one unit for a warp and several)."""
+    torch, nuq = require_cuda()
+    if ls == O.LEVELS_TABLE:
+        levels = np.float32([0.7 ** (s + 1 - j) for j in range(1, s + 1)])
+        nuq.set_level_table(levels)
+        O.set_levels(levels)
+    gen = torch.Generator(device="cuda").manual_seed(s)
+    for d, K, bucket in ((3 * 2048 + 11, 9, 2048), (4800 * 256 + 77, 33, 512), (20 * 148 * 256 + 77, 2, 8192)):
+        g = torch.randn(d, generator=gen, device="cuda")
+        erc = O.encode(g.cpu().numpy(), bucket, s, O.make_flags(O.NORM_LINF, ls, O.MODE_ERC), seed=1, offset=0)[0]
+        fixed = O.make_flags(O.NORM_LINF, ls, O.MODE_FIXED)
+        words = max(nuq.encode_bound(d, bucket, s, fixed) // 4, erc.size)
+        outs = [torch.zeros(words, dtype=torch.int32, device="cuda") for _ in range(K)]
+        for out in outs:
+            nuq.encode(g, bucket, s, fixed, out=out)
+            out[: erc.size].copy_(torch.from_numpy(erc.view(np.int32)))
+        rc, want = O.decode_accumulate([erc] * K, d, bucket, s)
+        assert rc == 0
+        want = torch.from_numpy(want).cuda()
+        acc = torch.full((d,), float("nan"), device="cuda")
+        nuq.decode_accumulate(outs, d, bucket, s, acc=acc)
+        assert nuq.last_status() == 0 and torch.equal(acc.view(torch.int32), want.view(torch.int32)), (d, K)
+        w, yl = torch.ones(d, device="cuda"), torch.ones(d, device="cuda")
+        nuq.decode_update(outs, d, bucket, s, w, yl, 0.25, 0.5, 1.0, acc=acc)
+        step = torch.tensor(0.25 / K, dtype=torch.float32, device="cuda").double()
+        y = (1.0 - step * want.double()).float()             # one fused operation: one rounding
+        assert nuq.last_status() == 0 and torch.equal(yl, y)
+        assert torch.equal(w, ((y - 1.0).double() * 0.5 + y.double()).float())
