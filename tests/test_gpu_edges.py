@@ -128,7 +128,8 @@ def test_missing_symbols_and_values_that_are_not_finite_in_fixed_width_streams()
 @pytest.mark.parametrize("d,bucket,s,ls", [
     (1, 256, 4, O.LEVELS_EXP), (8191, 8192, 4, O.LEVELS_EXP), (40000, 512, 6, O.LEVELS_EXP), (40000, 768, 5, O.LEVELS_UNIFORM),
     (65536, 65536, 4, O.LEVELS_EXP), (3 * 16384 + 9000, 16384, 4, O.LEVELS_EXP),      # one cluster, several
-    (2 * 148 * 8192, 8192, 4, O.LEVELS_EXP), (2 * 148 * 8192 + 1, 8192, 4, O.LEVELS_EXP)])      # two tiles per SM, one more
+    (2 * 148 * 8192, 8192, 4, O.LEVELS_EXP), (2 * 148 * 8192 + 1, 8192, 4, O.LEVELS_EXP),       # two tiles per SM, one more
+    (3 * 148 * 8192, 8192, 4, O.LEVELS_EXP), (3 * 148 * 8192 + 1, 8192, 4, O.LEVELS_EXP)])      # three tiles per SM, one more
 def test_containers_at_the_encoders_edges(kind, d, bucket, s, ls):
     g = _vector(kind, d, 3)
     for mode in (O.MODE_ERC, O.MODE_FIXED) + ((O.MODE_CODED,) if ls == O.LEVELS_EXP else ()):
@@ -148,7 +149,7 @@ def test_containers_at_the_encoders_edges(kind, d, bucket, s, ls):
 @pytest.mark.parametrize("kind", ["normal", "mixed"])
 @pytest.mark.parametrize("tiles,bucket", [(1, 256), (1, 768), (1, 2048), (1, 2304), (3, 512), (3, 8192), (3, 16384)])
 def test_containers_where_small_tiles_and_more_warps_end(kind, tiles, bucket):
-    """One tile of 8192 elements (whole buckets of it) per SM is encoded in small tiles, three with more warps."""
+    """One tile of 8192 elements (whole buckets of it) per SM and one more, three and one more."""
     torch, _ = require_cuda()
     tile = 8192 if bucket > 8192 else 8192 // bucket * bucket
     last = tiles * torch.cuda.get_device_properties(0).multi_processor_count * tile
@@ -161,6 +162,33 @@ def test_containers_where_small_tiles_and_more_warps_end(kind, tiles, bucket):
         free, _ = gpu_encode(g, bucket, 4, 0, seed=5, offset=9)
         _, _, _, taken = O.decode_symbols(free, d, bucket, 4)
         assert np.array_equal(free, O.encode(g, bucket, 4, 0, seed=5, offset=9, norms=taken)[0])
+
+
+@pytest.mark.parametrize("ls,s,mode,nk", [(O.LEVELS_EXP, 4, O.MODE_ERC, O.NORM_L2), (O.LEVELS_UNIFORM, 4, O.MODE_ERC, O.NORM_LINF), (O.LEVELS_UNIFORM, 2, O.MODE_ERC, O.NORM_L2),
+                                          (O.LEVELS_TABLE, 4, O.MODE_ERC, O.NORM_LINF), (O.LEVELS_EXP, 4, O.MODE_CODED, O.NORM_LINF)])
+@pytest.mark.parametrize("bucket", [256, 768, 1024, 1280, 8192])
+def test_containers_of_every_kind_at_the_limits_of_small_calls(bucket, ls, s, mode, nk):
+    """Small tiles end where every SM has a whole one, or 5.5 small ones; twice the warps at 17/7 tiles per SM or at three."""
+    torch, nuq = require_cuda()
+    sms, tile, small = torch.cuda.get_device_properties(0).multi_processor_count, 8192 // bucket * bucket, 2048 // bucket * bucket
+    limits = [(sms - 1) * tile, 17 * sms // 7 * tile, 3 * sms * tile] + ([11 * sms // 2 * small] if small else [])
+    if ls == O.LEVELS_TABLE:
+        levels = np.float32([0.6 ** (s + 1 - j) for j in range(1, s + 1)])
+        O.set_levels(levels)
+        nuq.set_level_table(levels)
+    if mode == O.MODE_CODED:
+        lengths = list(O.huffman_lengths([9, 5, 3, 2, 1]))
+        O.set_level_code(lengths)
+        nuq.set_level_code(lengths)
+    flags = O.make_flags(nk, ls, mode)
+    for d in [n + more for n in limits for more in (0, 1)] + [70001]:
+        g = _vector("normal", d, 3)
+        free, bits = gpu_encode(g, bucket, s, flags, seed=5, offset=9)
+        norms = O.decode_symbols(free, d, bucket, s)[3]
+        if nk == O.NORM_LINF:                               # (exact)
+            assert np.array_equal(norms, O.bucket_norms(g, bucket, nk))
+        want, want_bits = O.encode(g, bucket, s, flags, seed=5, offset=9, norms=norms)
+        assert bits == want_bits and np.array_equal(free, want), d
 
 
 @pytest.mark.parametrize("mode", [O.MODE_ERC, O.MODE_FIXED])

@@ -70,10 +70,12 @@ def _step_and_compare(torch, nuq, dev_streams, host_streams, d, bucket, s, w0, y
     (2, 8192 * 3 + 17, 8192, 3, O.MODE_ERC),
     (4, 100037, 8192, 4, O.MODE_ERC),         # four streams side by side, sums in shared memory
     (8, 200000, 8192, 4, O.MODE_ERC),
-    (9, 50000, 512, 4, O.MODE_ERC),           # two groups of streams
+    (9, 50000, 512, 4, O.MODE_ERC),           # nine lanes of a warp with a chain
     (8, 100000, 8192, 4, O.MODE_FIXED),       # the fixed-width kernel, 4-bit fields
     (3, 70001, 768, 2, O.MODE_FIXED),         # the fixed-width kernel, other widths
     (3, 200000, 65536, 4, O.MODE_ERC),        # buckets wider than a tile
+    (32, 4800 * 256 + 77, 512, 4, O.MODE_ERC),    # short blocks where warps have more than two units, one sub-block each ...
+    (16, 9600 * 256 + 77, 1024, 3, O.MODE_ERC),   # ... and two
 ])
 @pytest.mark.parametrize("alpha,mu,l", [(0.1, 0.0, 0.0), (0.05, 0.9, 0.0), (0.05, 0.9, 1.0), (0.3, 0.5, 0.25)])
 def test_decode_update_matches_the_oracle(K, d, bucket, s, mode, alpha, mu, l):
