@@ -141,8 +141,7 @@ uint32_t token_bits_bound(const Geometry& G, uint32_t elems, uint32_t buckets, b
 // words of shared-memory staging the records of one ERC tile can need
 uint32_t stage_words_for(const Geometry& G, bool norms_are_ours) {
     uint32_t head = 1u + (G.sb_per_block + 1u) / 2u + 1u;          // norm, lengths, padding
-    const uint32_t elems = G.bucket <= kBLK ? G.tile_elems : kBLK;
-    return G.blocks_per_tile * head + (token_bits_bound(G, elems, G.blocks_per_tile, norms_are_ours) + 31u) / 32u;
+    return G.blocks_per_tile * head + (token_bits_bound(G, G.tile_elems, G.blocks_per_tile, norms_are_ours) + 31u) / 32u;
 }
 
 uint64_t bound_bytes(const Geometry& G) {
