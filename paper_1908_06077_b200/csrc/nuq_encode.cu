@@ -895,7 +895,7 @@ encode_kernel(const __grid_constant__ EncodeParams P) {
             if (__shfl_sync(0xffffffffu, last, 0)) {
                 __threadfence_block();
                 // lane = sub-block of the tile; the lanes of one bucket all do the same sum, in the same order
-                const SubBlocks mine = bucket_of_lane<TILE / kSB>(lane, spb);
+                const SubBlocks mine = bucket_of_lane(lane, spb);
                 const uint32_t bi = lane / spb, sb0 = mine.from;
                 float norm;
                 if (P.norms_in != nullptr) {
@@ -929,6 +929,8 @@ encode_kernel(const __grid_constant__ EncodeParams P) {
                         for (uint32_t r = 0; r < cl; ++r) mxb = max(mxb, (uint32_t)s_xchg[xp][r]);
                         norm = __uint_as_float(mxb);
                     }
+                } else if (lane >= nsb_tile) {
+                    norm = 0.0f;
                 } else if (G.norm_kind == kNormL2) {
                     double a = 0.0;
                     if (coarse) for (uint32_t j = sb0 + kQ - 1u; j < mine.to; j += kQ) a += s_partial[j];     // one partial per warp

@@ -127,19 +127,17 @@ __device__ __forceinline__ void cluster_sync_all() {
 }
 
 // Where the norms are worked out a lane stands for a sub-block of the tile and adds up the sums of all sub-blocks of its bucket,
-// [from, to), spb of them.  A tile has sums for SUBS sub-blocks; its buckets need not fill them, and the lanes behind the last
-// bucket must not read on behind the sums: there is nothing for them.  (Those of sub-blocks that the tile does not have are 0.
-// This is on the path that a tile's warps wait for, and the form of the limit shows: 25 557 032 elements, ERC, buckets of 512 / 1024 /
-// 1280 / 8192 without a limit 96.4, 90.9, 98.7, 68.3 us, with this one 95.8, 90.5, 100.6, 68.2; `to` at most SUBS: 95.9, 90.1, 101.3, 68.5;
-// `from` at most SUBS - spb: 96.9, 91.8, 98.5, 68.5; with longer arrays 97.0, 91.8, 98.4, 68.4 and buckets of 2048 83.6 -> 86.0.
-// Uniform levels in buckets of 8192: 102.3 without, 101.1 so, 102.4 to 102.7 the other ways.)
+// [from, to), spb of them.  (Those of sub-blocks that the tile does not have are 0.)  Only lanes whose sub-block the tile has may ask:
+// for those behind, the range may lie behind the sums.
+// This is on the path that a tile's warps wait for, and the form of that limit shows: 25 557 032 elements, ERC, buckets of 1024 / 1280 /
+// 8192 without it 90.9, 98.7, 68.2 us, a branch around the sums 91.6, 98.0, 68.2, loops that end at the last of the sums 90.1, 101.3,
+// 68.6, loops that are empty behind it 90.7, 100.2, 68.6 (ResNet-18 step 193.4 with either of the first two, 196.2 with the last).
 struct SubBlocks {
     uint32_t from, to;
 };
-template <uint32_t SUBS>
 __host__ __device__ __forceinline__ SubBlocks bucket_of_lane(uint32_t lane, uint32_t spb) {
     const uint32_t from = lane / spb * spb;
-    return SubBlocks{from, from + spb <= SUBS ? from + spb : from};
+    return SubBlocks{from, from + spb};
 }
 
 // Geometry of a tile, worked out once by the thread that took its ticket.

@@ -219,12 +219,14 @@ __global__ void __launch_bounds__(kEncThreads, kEncMinBlocks) encode_fixed4_kern
             if (__shfl_sync(0xffffffffu, last, 0)) {
                 __threadfence_block();
                 // lane = sub-block of the tile; the lanes of one bucket all do the same sum, in the same order
-                const SubBlocks mine = bucket_of_lane<32u>(lane, spb);
+                const SubBlocks mine = bucket_of_lane(lane, spb);
                 const uint32_t bi = lane / spb, sb0 = mine.from;
                 float norm;
                 if (P.norms_in != nullptr) {
                     const uint64_t nb_idx = narrow ? ti.first_block + bi : ti.bucket_idx;
                     norm = nb_idx < G.nb ? P.norms_in[nb_idx] : 0.0f;
+                } else if (lane >= nsb_tile) {
+                    norm = 0.0f;
                 } else if (G.norm_kind == kNormL2) {
                     double a = 0.0;
                     for (uint32_t j = sb0; j < mine.to; j += COARSE ? 4u : 1u) a += s_partial[j];

@@ -9,8 +9,8 @@ from paper_1908_06077_b200 import build as cuda_build
 
 SOURCE = """
 #include "nuq_encode_common.cuh"
-extern "C" void bucket_of_lane(uint32_t subs, uint32_t lane, uint32_t spb, uint32_t* out) {
-    const nuq::SubBlocks b = subs == 8 ? nuq::bucket_of_lane<8>(lane, spb) : nuq::bucket_of_lane<32>(lane, spb);
+extern "C" void bucket_of_lane(uint32_t lane, uint32_t spb, uint32_t* out) {
+    const nuq::SubBlocks b = nuq::bucket_of_lane(lane, spb);
     out[0] = b.from;
     out[1] = b.to;
 }
@@ -28,11 +28,16 @@ def lib(tmp_path_factory):
 
 @pytest.mark.parametrize("subs", [32, 8])
 def test_norms_are_summed_over_the_tile_s_own_sub_blocks(lib, subs):
-    """Every sub-block of a tile gets the sum of its own bucket's; nobody reads where no sum of this tile is."""
+    """Every sub-block of a tile, which is of whole buckets or the vector's end, gets the sum of its own bucket's, and finds it within
+    the tile's sums; lanes behind the tile's last sub-block may not ask."""
     out = (C.c_uint32 * 2)()
+    beyond = 0
     for spb in range(1, subs + 1):
         for lane in range(32):
-            lib.bucket_of_lane(subs, lane, spb, out)
+            lib.bucket_of_lane(lane, spb, out)
+            assert tuple(out) == (lane // spb * spb, lane // spb * spb + spb)
             if lane < subs // spb * spb:
-                assert tuple(out) == (lane // spb * spb, lane // spb * spb + spb)
-            assert out[0] >= out[1] or out[1] <= subs, (spb, lane, tuple(out))
+                assert out[1] <= subs, (spb, lane)
+            else:
+                beyond += out[1] > subs
+    assert beyond > 0
