@@ -281,7 +281,7 @@ static EncodePlan plan_encode(EncodeParams& P, int dev, uint32_t flags) {
     P.warps = tokens && 7u * G.ntiles <= sevenths * (uint64_t)sms ? kEncMaxWarps : kEncWarps;
     P.tile = kBLK;
     // A quarter of a tile, one sub-block per warp, four to an SM: with fewer whole tiles than SMs, as long as small ones (of whole
-    // buckets too, so that there may be six for a whole one) are no more than 5.5 to an SM.  65 536 elements 10.9 us in whole tiles of 16 warps, 8.8 in
+    // buckets too, so that there may be six for a whole one) are no more than 5.5 to an SM.  65 536 elements 10.2 us in whole tiles of 16 warps, 8.4 in
     // small ones (uniform levels 12.0 and 8.7), 10^6 elements 15.2 and 13.3, coded indices 15.4 and 12.5; 147 whole tiles, buckets of
     // 512 / 768 / 1536 (3.96, 4.95 and 4.95 small ones to an SM) 15.4 and 13.6, 15.2 and 14.7, 15.4 and 14.9; buckets of 1280 with 5.4
     // to an SM 15.9 and 15.1, 5.6 15.9 and 16.2.  Whole tiles for all 148 SMs 12.5 and 13.9 (no SM gets two, then).

@@ -64,7 +64,8 @@ struct Row {
 // With symbols of one byte an entry may stand for two tokens (pairs): the gap is then that of both together, bits 5-7 are the
 // second one's (0: one token), bits 16-23 the first one's symbol.  Dense symbols take 5 bits a token and most look-ups give two;
 // sparse ones (8 bits and more) one in four, and gain next to nothing (K = 8 ResNet-50 containers: largest-magnitude norms with uniform
-// levels 193 -> 150 us, s = 4 in buckets of 512 149 -> 125, 8192 83.4 -> 81.1, s = 3 there 72.2 -> 72.6).
+// levels 193 -> 150 us, s = 4 in buckets of 512 149 -> 125, 8192 83.4 -> 81.1, s = 3 there 72.2 -> 72.6, s = 2 69.6 -> 70.5; with what came
+// since 72.0 and 69.7; 33 streams of 6 x 10^6 elements with s = 3 are 1.2 % slower than without, 114.6 and 116.0).
 constexpr uint32_t kLenMask = 31u, kGap2Shift = 5u, kMaxGap2 = 7u, kGapShift = 8u, kFirstShift = 16u;
 template <class Sym>
 constexpr bool kPairs = sizeof(Sym) == 1;
